@@ -485,18 +485,13 @@ def algorithmic_bytes(name, n, extra_steps=0.0, out_bytes=3):
     """Compulsory DRAM bytes of one launch: the per-point figure of each kernel times n."""
     per_point = {
         "slg_hist": 12,                                   # xyz
-        # digit counts of pass 2 (passes 0 and 1 are counted by the histogram and the slab sort)
-        "slg_counts2": 4,
-        # scatter: keys and values in, keys and values (or the final arrays) out.
-        # pass 0 (y-slabs) reads xyz; the slab sort reads the y-ordered pairs and
-        # writes the C3 order; pass 1 (C1 on z) writes packed codes, input
-        # indices, ranks and the C3 order as sorted ids; pass 2 (C2 on x) reads
-        # the codes only and writes the C2 order, the C2 ranks and the codes
-        # along C2
-        "slg_scatter0": 12 + 8, "slg_slab": 8 + 8, "slg_scatter1": 8 + 16, "slg_scatter2": 4 + 12,
-        # link: codes along C1, ids and codes along C2 and C3, C2 ranks of the C3
-        # points; the neighbour slots out
-        "slg_link": 4 + 8 + 12 + 16,
+        # row scatter: xyz in, (index, code) out for each of the three codes
+        "slg_scatter": 12 + 3 * 8,
+        # bucket sort: (index, code) in, codes and indices out for each code, the C1 and C2 ranks out
+        "slg_sort": 3 * 8 + 3 * 8 + 2 * 4,
+        # link: codes along C1, indices and codes along C2 and C3, both ranks; the neighbour slots
+        # out; in a whole run also the input indices along C1, the colours, and the colours in C1 order
+        "slg_link": 4 + 2 * 8 + 8 + 16 + 11,
         "gather_colors": 11,
         # moments: codes 4, slots 16, colours 4, the spread out 4; x_0 of the filter steps out 16
         "ne_moments": 28 + 16,
@@ -512,16 +507,13 @@ def algorithmic_bytes(name, n, extra_steps=0.0, out_bytes=3):
     if name == "filter_select":
         # keep flags: y 4, spread 4, keep 1; the stored steps' Eq. 6 terms 4 each and keep 1;
         # ordinary steps beyond the stored ones 72 each (x in, c4, weights, x out);
-        # output: rank 4, x 16, colours out
-        return (9 + 4 * SPEC_STEPS + 1 + 72 * extra_steps + 20 + out_bytes) * n
+        # output: ranks 8, x 16, colours out
+        return (9 + 4 * SPEC_STEPS + 1 + 72 * extra_steps + 24 + out_bytes) * n
     return 0
 
 
 def kernel_group(name):
-    """Launches of the same kernel function share one group (the sort passes differ by digit)."""
-    for g in ("slg_counts", "slg_scan", "slg_scatter"):
-        if name.startswith(g):
-            return g
+    """Launches of the same kernel function share one group (every function has one name here)."""
     return name
 
 
@@ -633,7 +625,7 @@ def run_fgbd(args):
         kernels[name] = {"ms": avg, "launches_per_step": len(lst) / len(cols),
                          "algo_bytes": b, "gbs": (b / (avg / 1e3) / 1e9) if b and avg > 0 else None}
     # the dominant kernel: the largest share of the step; the launches of one
-    # kernel function (the sort passes) count as one kernel.  Every kernel in
+    # kernel function count as one kernel.  Every kernel in
     # the step has algorithmic bytes (the estimate launch: its stored filter
     # steps; its eigen block moves none).
     groups = {}

@@ -275,7 +275,7 @@ fgbd_status fgbd_run_reuse(fgbd_ctx* ctx, const int32_t* xyz, int64_t n, const v
  * take the frames' speculative filter steps; the selection and filter: one
  * cooperative launch in which each frame's blocks, shared out by frame size,
  * synchronise among themselves).  Whether a batch that can be segmented is,
- * how many frames a launch takes and the block shapes of the sort scatter and
+ * how many frames a launch takes and the block shapes of the row scatter and
  * of the selection/filter are those fgbd_tune_batch chose for this device and
  * frame size (or fgbd_set_batch_shape set; by default segmented below 2^18
  * points a frame); they do not change any result.  Other batches run every
@@ -302,7 +302,7 @@ typedef struct fgbd_batch_shape {
   int32_t seg_frames;            /* frames per segmented launch, 1..16; 0: per-frame streams.  Default: 16
                                     below 2^18 points a frame, 0 above (fgbd_tune_batch: -1 when the batch
                                     cannot be segmented, and nothing was tuned) */
-  int32_t scatter_threads;       /* threads ranking one 4096-key sort tile: 256, 512 (default) or 1024 */
+  int32_t scatter_threads;       /* threads of a block of the row scatter (a tile of up to 4096 points): 256, 512 (default) or 1024 */
   int32_t filter_threads;        /* threads per block of the selection/filter: 256 or 512 (default) */
   int32_t filter_blocks_per_sm;  /* its blocks per SM (default 2; capped by what fits) */
   float ms;                      /* fgbd_tune_batch: device time of one batch with the chosen shape */
@@ -311,7 +311,7 @@ typedef struct fgbd_batch_shape {
 
 /* Autotuner of batches: runs the batch (the arguments of fgbd_run_batch) with
  * candidate shapes - per-frame streams against segmented launches of 16, 8, 4
- * and 2 frames, then, if segmented won, the sort scatter at 256, 512 and 1024
+ * and 2 frames, then, if segmented won, the row scatter at 256, 512 and 1024
  * threads a tile, then the selection/filter at 512 threads x 1 or 2 blocks per
  * SM and 256 threads x 2 or 4 - timing each (median of three after one untimed
  * run, CUDA events on `stream`), one coordinate at a time, and keeps the
@@ -474,7 +474,7 @@ fgbd_status fgbd_get_timings(fgbd_ctx* ctx, int32_t max, int32_t* count_host, ch
  *           point along code l+1.
  *   status: optional device uint32 receiving 0, or 1 if a coordinate was out
  *           of range (the orders are then unspecified); NULL to skip.
- * Scratch: one file-scope device array of about 1.3 MiB (FGBD_STATIC_MAX_POINTS
+ * Scratch: one file-scope device array of about 2.7 MiB (FGBD_STATIC_MAX_POINTS
  * points) reserved on every GPU that loads the library until the process
  * exits.  The call allocates and frees nothing.  The first call on a device
  * looks up the array's device address (cudaGetSymbolAddress) with that device

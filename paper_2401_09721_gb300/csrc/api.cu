@@ -263,7 +263,7 @@ FilterArgs filter_args(fgbd_ctx* ctx, int mode, int q_fixed, const double* sigma
   a.spread = ctx->spread;
   a.pk = ctx->gb.pk;
   a.c4 = ctx->gb.c4;
-  a.rank1 = ctx->gb.rank1;
+  a.rank12 = ctx->gb.rank12;
   a.xbuf0 = ctx->x0;
   a.xbuf1 = ctx->x1;
   a.out = out;
@@ -354,12 +354,15 @@ void release_batch_objects(fgbd_ctx* ctx) {
     }
 }
 
+ColorArgs color_args(const fgbd_ctx* ctx, const void* rgb, int32_t dtype) {
+  return ColorArgs{rgb, dtype, ctx->gb.perm1, ctx->y8, ctx->yf};
+}
+
 // `zeroed`: the caller has already zeroed the scalar regions this call fills.
-// `rgb_gather` (fgbd_run): the colours of the frame, gathered into sorted order
-// on the context's side stream as soon as the C1 order exists, beside the C2
-// pass and the link step, which do not touch them (do_estimate then joins it).
+// `rgb` (a whole run): the colours of the frame, which the link launch then takes
+// into the C1 order (do_estimate and the filter find them gathered).
 fgbd_status do_build(fgbd_ctx* ctx, const int32_t* xyz, int64_t n64, cudaStream_t st, bool zeroed = false,
-                     const void* rgb_gather = nullptr, int32_t gather_dtype = FGBD_U8) {
+                     const void* rgb = nullptr, int32_t dtype = FGBD_U8) {
   if (n64 < 0 || n64 > ctx->capacity) return FGBD_EINVAL;
   if (n64 > 0 && !xyz) return FGBD_EINVAL;
   const int n = int(n64);
@@ -373,35 +376,20 @@ fgbd_status do_build(fgbd_ctx* ctx, const int32_t* xyz, int64_t n64, cudaStream_
   if (!zeroed) zero_region(ctx, offsetof(DevScalars, n_edges), offsetof(DevScalars, build_end_), st, &e);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "memset");
   if (n > 0) {
-    // kernel names carry the pass: 0 = y-slabs, 1 = C1 (on z, over C3), 2 = C2 (on x, over C1)
-    static const char* const kCounts[kSlgPasses] = {"slg_counts0", "slg_counts1", "slg_counts2"};
-    static const char* const kScan[kSlgPasses] = {"slg_scan0", "slg_scan1", "slg_scan2"};
-    static const char* const kScatter[kSlgPasses] = {"slg_scatter0", "slg_scatter1", "slg_scatter2"};
-    FGBD_LAUNCH(ctx, "slg_hist", st, launch_coord_hist(xyz, n, bits, ctx->sc, &ctx->sb, ctx->num_sms, st));
-    for (int p = 0; p < kSlgPasses; ++p) {
-      const SortPassArgs a = slg_pass_args(p, xyz, n, bits, ord_stride(ctx), ctx->sb, ctx->gb, ctx->sc);
-      if (!pass_counted_before(p)) FGBD_LAUNCH(ctx, kCounts[p], st, launch_tile_counts(a, st));
-      FGBD_LAUNCH(ctx, kScan[p], st, launch_tile_scan(a, st));
-      FGBD_LAUNCH(ctx, kScatter[p], st, launch_sort_scatter(a, st));
-      if (p == 0)
-        FGBD_LAUNCH(ctx, "slg_slab", st,
-                    launch_slab_sort(n, bits, ord_stride(ctx), ctx->sb, ctx->gb, ctx->sc, st));
-      if (p == 1 && rgb_gather) {
-        FGBD_CUDA(ctx, cudaEventRecord(ctx->ev_fork, st));
-        FGBD_CUDA(ctx, cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0));
-        FGBD_LAUNCH(ctx, "gather_colors", ctx->side,
-                    launch_gather_colors(rgb_gather, gather_dtype, n, ctx->gb.perm1, ctx->y8, ctx->yf, ctx->side));
-        FGBD_CUDA(ctx, cudaEventRecord(ctx->ev_join, ctx->side));
-      }
-    }
+    FGBD_LAUNCH(ctx, "slg_hist", st, launch_coord_hist(xyz, n, bits, ctx->sc, ctx->num_sms, st));
+    const BucketArgs ba =
+        bucket_args(xyz, n, bits, ord_stride(ctx), ctx->sb, ctx->gb, ctx->sc, scatter_fill(ctx->num_sms));
+    FGBD_LAUNCH(ctx, "slg_scatter", st, launch_bucket_scatter(ba, st));
+    FGBD_LAUNCH(ctx, "slg_sort", st, launch_bucket_sort(ba, st));
     const bool same_line = (ctx->params.variant & FGBD_VARIANT_SAME_LINE) != 0;
     if (ctx->params.window == 1)
       FGBD_LAUNCH(ctx, "slg_link", st,
-                  launch_link(n, bits, ord_stride(ctx), same_line, ctx->gb, ctx->sb, ctx->sc, ctx->num_sms, st));
+                  launch_link(n, bits, ord_stride(ctx), same_line, ctx->gb, ctx->sb, ctx->sc, color_args(ctx, rgb, dtype),
+                              ctx->num_sms, st));
     else
       FGBD_LAUNCH(ctx, "slg_link", st,
                   launch_link_wide(n, bits, ord_stride(ctx), ctx->params.window, same_line, ctx->gb, ctx->sb,
-                                   ctx->sc, ctx->num_sms, st));
+                                   ctx->sc, color_args(ctx, rgb, dtype), ctx->num_sms, st));
     if (same_line) ctx->launches += 1;  // and k_c1_line_flags
     if (ctx->params.variant & (FGBD_VARIANT_SIGMA_NODE | FGBD_VARIANT_SIGMA_PAIR))
       FGBD_LAUNCH(ctx, "slg_node_sigma", st,
@@ -427,13 +415,8 @@ fgbd_status do_estimate(fgbd_ctx* ctx, const void* rgb, int32_t dtype, double* s
   if (ctx->params.window > 1) {
     // wider windows: moments, their reduction, the eigenvector block, the Rayleigh
     // quotients with the tail rule; no filter steps are taken beside them
-    if (n > 0) {
-      if (pregathered)
-        FGBD_CUDA(ctx, cudaStreamWaitEvent(st, ctx->ev_join, 0));
-      else
-        FGBD_LAUNCH(ctx, "gather_colors", st,
-                    launch_gather_colors(rgb, dtype, n, ctx->gb.perm1, ctx->y8, ctx->yf, st));
-    }
+    if (n > 0 && !pregathered)
+      FGBD_LAUNCH(ctx, "gather_colors", st, launch_gather_colors(color_args(ctx, rgb, dtype), n, st));
     static const char* const kStage[4] = {"ne_wide_moments", "ne_wide_reduce", "ne_wide_eigvec", "ne_wide_tail"};
     for (int stage = n > 0 ? 0 : 1; stage < 4; ++stage)
       FGBD_LAUNCH(ctx, kStage[stage], st,
@@ -447,11 +430,9 @@ fgbd_status do_estimate(fgbd_ctx* ctx, const void* rgb, int32_t dtype, double* s
   }
   int nblocks = 0;
   if (n > 0) {
-    if (pregathered)
-      FGBD_CUDA(ctx, cudaStreamWaitEvent(st, ctx->ev_join, 0));  // the gather do_build started
-    else
+    if (!pregathered)
       FGBD_LAUNCH(ctx, "gather_colors", st,
-                  launch_gather_colors(rgb, dtype, n, ctx->gb.perm1, ctx->y8, ctx->yf, st));
+                  launch_gather_colors(color_args(ctx, rgb, dtype), n, st));
     nblocks = ne_moment_blocks(n, ctx->num_sms);
     // (with x_0 of the filter steps into ctx->x0, which step 1 then reads as one 16-byte load a point)
     FGBD_LAUNCH(ctx, "ne_moments", st,
@@ -568,8 +549,8 @@ fgbd_status capture_run(fgbd_ctx* ctx, const fgbd_ctx::RunKey& k, cudaStream_t s
 // ---------------------------------------------------------------- segmented batches
 // A batch whose frames share the window (1), the ablation switches and the
 // colour type runs each stage as one launch over up to kSegMax frames
-// (segmented launches, fgbd_internal.cuh): 15 launches for the whole chunk
-// instead of 15 per frame, every frame's short latency-bound kernels
+// (segmented launches, fgbd_internal.cuh): 8 launches for the whole chunk
+// instead of 8 per frame, every frame's short latency-bound kernels
 // side by side in one grid, the estimate launch with one eigen block per
 // frame, and one cooperative selection/filter for all frames (each frame's
 // blocks synchronise among themselves).  Each frame's blocks run the same
@@ -604,30 +585,27 @@ fgbd_status seg_chunk(const std::vector<fgbd_ctx*>& ctxs, const std::vector<fgbd
   ZeroArgs z[kSegMax];
   HistArgs h[kSegMax];
   LinkArgs l[kSegMax];
-  GatherArgs g[kSegMax];
   MomentArgs m[kSegMax];
   FilterArgs spec[kSegMax], sel[kSegMax];
   const double* f64[kSegMax];
-  int nblk[kSegMax], ns[kSegMax], bits[kSegMax], caps[kSegMax];
-  SortBufs sbs[kSegMax];
-  GraphBufs gbs[kSegMax];
-  DevScalars* scs[kSegMax];
+  int nblk[kSegMax], bits[kSegMax], caps[kSegMax];
+  BucketArgs ba[kSegMax];
+  double points = 0.0;
+  for (int f = 0; f < F; ++f) points += double(keys[i0 + f].n);
   for (int f = 0; f < F; ++f) {
     fgbd_ctx* c = ctxs[i0 + f];
     const fgbd_ctx::RunKey& k = keys[i0 + f];
     const int n = int(k.n);
     const int32_t* xyz = static_cast<const int32_t*>(k.xyz);
-    ns[f] = n;
     bits[f] = c->params.bits;
     caps[f] = ord_stride(c);
-    sbs[f] = c->sb;
-    gbs[f] = c->gb;
-    scs[f] = c->sc;
     z[f] = ZeroArgs{reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(c->sc) + offsetof(DevScalars, n_edges)),
                     (offsetof(DevScalars, sel_end_) - offsetof(DevScalars, n_edges)) / 4};
-    h[f] = hist_args(xyz, n, bits[f], c->sc, c->sb);
-    l[f] = link_args(n, bits[f], caps[f], c->gb, c->sb, c->sc);
-    g[f] = GatherArgs{k.rgb_in, dtype, n, c->gb.perm1, c->y8, c->yf};
+    h[f] = hist_args(xyz, n, bits[f], c->sc);
+    // (the frame's share of the blocks that fill the GPU)
+    ba[f] = bucket_args(xyz, n, bits[f], caps[f], c->sb, c->gb, c->sc,
+                        std::max(1, int(double(scatter_fill(num_sms)) * double(n) / points)));
+    l[f] = link_args(n, bits[f], caps[f], c->gb, c->sb, c->sc, color_args(c, k.rgb_in, dtype));
     m[f] = moment_args(n, bits[f], c->gb, c->y8, c->yf, c->spread, c->f64part, true, sorted, c->sc);
     // the state fgbd_run's calls leave (n is set first: filter_args reads it)
     c->n = n;
@@ -640,26 +618,10 @@ fgbd_status seg_chunk(const std::vector<fgbd_ctx*>& ctxs, const std::vector<fgbd
   }
   FGBD_LAUNCH(lead, "seg_zero", st, launch_zero_words_seg(z, F, st));
   FGBD_LAUNCH(lead, "seg_hist", st, launch_coord_hist_seg(h, F, num_sms, st));
-  static const char* const kPass[kSlgPasses][3] = {{"seg_counts0", "seg_scan0", "seg_scatter0"},
-                                                   {"seg_counts1", "seg_scan1", "seg_scatter1"},
-                                                   {"seg_counts2", "seg_scan2", "seg_scatter2"}};
-  for (int p = 0; p < kSlgPasses; ++p) {
-    SortPassArgs a[kSegMax];
-    for (int f = 0; f < F; ++f) {
-      fgbd_ctx* c = ctxs[i0 + f];
-      a[f] = slg_pass_args(p, static_cast<const int32_t*>(keys[i0 + f].xyz), ns[f], bits[f], caps[f], c->sb, c->gb,
-                           c->sc);
-    }
-    {
-      // (counts,) scan and scatter: two or three launches under one timing scope
-      LaunchScope scope_(lead, kPass[p][2], st, pass_counted_before(p) ? 2 : 3);
-      FGBD_CUDA(lead, launch_sort_pass_seg(a, F, shape.scatter_threads, st));
-    }
-    if (p == 0) FGBD_LAUNCH(lead, "seg_slab", st, launch_slab_sort_seg(ns, bits, caps, sbs, gbs, scs, F, st));
-  }
+  FGBD_LAUNCH(lead, "seg_scatter", st, launch_bucket_scatter_seg(ba, F, shape.scatter_threads, st));
+  FGBD_LAUNCH(lead, "seg_sort", st, launch_bucket_sort_seg(ba, F, st));
   FGBD_LAUNCH(lead, "seg_link", st, launch_link_seg(l, F, same_line, num_sms, st));
   if (same_line) lead->launches += 1;  // and the line flags
-  FGBD_LAUNCH(lead, "seg_gather", st, launch_gather_colors_seg(g, F, st));
   FGBD_LAUNCH(lead, "seg_moments", st, launch_ne_moments_seg(m, F, dtype, num_sms, st));
   FGBD_LAUNCH(lead, "seg_estimate", st, launch_ne_finalize_seg(spec, f64, nblk, F, num_sms, st));
   FGBD_LAUNCH(lead, "seg_select", st,
@@ -762,8 +724,9 @@ fgbd_status stream_batch(const std::vector<fgbd_ctx*>& ctxs, const std::vector<f
   for (int f = 0; f < count; ++f) {
     fgbd_ctx* c = ctxs[f];
     const fgbd_ctx::RunKey& k = keys[f];
-    fgbd_status s = do_build(c, static_cast<const int32_t*>(k.xyz), k.n, c->side);
-    if (s == FGBD_OK) s = do_estimate(c, k.rgb_in, k.in_dtype, nullptr, c->side, false);
+    fgbd_status s = do_build(c, static_cast<const int32_t*>(k.xyz), k.n, c->side, false, k.rgb_in, k.in_dtype);
+    if (s == FGBD_OK)
+      s = do_estimate(c, k.rgb_in, k.in_dtype, nullptr, c->side, false, false, nullptr, FGBD_U8, false, k.n > 0);
     if (s != FGBD_OK) return s;
   }
   // selection + filter: cooperative launches, one at a time (frame f waits for
@@ -882,7 +845,6 @@ fgbd_status fgbd_ctx_create(int64_t capacity, const fgbd_params* params, fgbd_ct
   ctx->filter_per_sm = std::max(1, filter_grid(1 << 30, ctx->num_sms, nx) / ctx->num_sms);
 
   const size_t C = size_t(capacity);
-  const int tiles = int((C + kSortTile - 1) / kSortTile);
   ctx->f64_blocks = ne_moment_blocks(int(C), ctx->num_sms);
   const size_t kP = size_t(kD) * kD + kD + 1;
   // wider windows: the further neighbour slots and the noise-estimate scratch
@@ -896,20 +858,14 @@ fgbd_status fgbd_ctx_create(int64_t capacity, const fgbd_params* params, fgbd_ct
   };
   void* keys0 = nullptr;
   void* keys1 = nullptr;
-  void* vals0 = nullptr;
-  void* vals1 = nullptr;
   const Item items[] = {
       {reinterpret_cast<void**>(&ctx->sc), sizeof(DevScalars)},
       {&keys0, C * 4},
       {&keys1, C * 4},
-      {&vals0, C * 4},
-      {&vals1, C * 4},
-      {reinterpret_cast<void**>(&ctx->sb.tile_counts), size_t(kSlgPasses) * kMaxRadix * tiles * 4},
       {reinterpret_cast<void**>(&ctx->gb.perm1), C * 4},
-      {reinterpret_cast<void**>(&ctx->gb.rank1), C * 4},
+      {reinterpret_cast<void**>(&ctx->gb.rank12), C * 8},
       {reinterpret_cast<void**>(&ctx->gb.pk), C * 4},
       {reinterpret_cast<void**>(&ctx->gb.ord23), 2 * align_up(C, 64) * 4},
-      {reinterpret_cast<void**>(&ctx->gb.rank2), C * 4},
       {reinterpret_cast<void**>(&ctx->gb.c4), C * 16},
       {reinterpret_cast<void**>(&ctx->spec_x), size_t(kSpecMax) * align_up(C, 64) * 16},
       {reinterpret_cast<void**>(&ctx->spec_z), size_t(kSpecMax) * align_up(C, 64) * 4},
@@ -931,7 +887,7 @@ fgbd_status fgbd_ctx_create(int64_t capacity, const fgbd_params* params, fgbd_ct
       {reinterpret_cast<void**>(&ctx->wne.S), wide ? wD * wD * 8 : 0},
       {reinterpret_cast<void**>(&ctx->wne.V), wide ? (wD * wD + wD) * 4 : 0},
       {reinterpret_cast<void**>(&ctx->wne.lam), wide ? wD * 8 : 0},
-      {reinterpret_cast<void**>(&ctx->wne.done), wide ? 4 : 0},
+      {reinterpret_cast<void**>(&ctx->wne.done), wide ? size_t(4) : 0},
   };
   size_t total = 0;
   for (const Item& it : items) total = align_up(total, 256) + it.bytes;
@@ -948,11 +904,17 @@ fgbd_status fgbd_ctx_create(int64_t capacity, const fgbd_params* params, fgbd_ct
     *it.ptr = static_cast<char*>(ctx->mem) + off;
     off += it.bytes;
   }
-  ctx->sb.count_stride = kMaxRadix * tiles;
-  ctx->sb.keys[0] = static_cast<uint32_t*>(keys0);
-  ctx->sb.keys[1] = static_cast<uint32_t*>(keys1);
-  ctx->sb.vals[0] = static_cast<uint32_t*>(vals0);
-  ctx->sb.vals[1] = static_cast<uint32_t*>(vals1);
+  ctx->sb.keys_c2 = static_cast<uint32_t*>(keys0);
+  ctx->sb.keys_c3 = static_cast<uint32_t*>(keys1);
+  // the sort's rows and their scratch (8 + 8 bytes a point and code) lie in the
+  // three stored filter steps, which are written after the graph is built
+  static_assert(kSpecMax >= 3 && sizeof(float4) == sizeof(uint2) + 2 * sizeof(uint32_t), "one row of spec_x a code");
+  const size_t Ca = align_up(C, 64);
+  ctx->sb.tmp_stride = int(Ca);
+  for (int c = 0; c < 3; ++c) {
+    ctx->sb.row_pts[c] = reinterpret_cast<uint2*>(ctx->spec_x + size_t(c) * Ca);
+    ctx->sb.row_tmp[c] = reinterpret_cast<uint32_t*>(ctx->sb.row_pts[c] + Ca);
+  }
   ctx->gb.nx = nx;
   ctx->gb.cx_stride = int(align_up(C, 64));
   if (!(p.variant & FGBD_VARIANT_SIGMA_PAIR)) ctx->gb.node_sig = nullptr;
@@ -1066,7 +1028,7 @@ fgbd_status fgbd_denoise(fgbd_ctx* ctx, const void* rgb_in, int32_t in_dtype, in
   if (ctx->n > 0 && !rgb_in) return FGBD_EINVAL;
   if (ctx->n > 0) {
     FGBD_LAUNCH(ctx, "gather_colors", st,
-                launch_gather_colors(rgb_in, in_dtype, ctx->n, ctx->gb.perm1, ctx->y8, ctx->yf, st));
+                launch_gather_colors(color_args(ctx, rgb_in, in_dtype), ctx->n, st));
   }
   // the gathered colours and filter buffers now hold this call's data
   if (rgb_in != ctx->noise_rgb || in_dtype != ctx->noise_dtype) {
@@ -1184,11 +1146,8 @@ fgbd_status fgbd_run_reuse(fgbd_ctx* ctx, const int32_t* xyz, int64_t n, const v
   if (!ctx->ever_selected) return FGBD_ESTATE;
   DeviceGuard g(ctx->device);
   const cudaStream_t st = as_stream(stream);
-  const fgbd_status s = do_build(ctx, xyz, n, st);
+  const fgbd_status s = do_build(ctx, xyz, n, st, false, rgb_in, in_dtype);
   if (s != FGBD_OK) return s;
-  if (ctx->n > 0)
-    FGBD_LAUNCH(ctx, "gather_colors", st,
-                launch_gather_colors(rgb_in, in_dtype, ctx->n, ctx->gb.perm1, ctx->y8, ctx->yf, st));
   cudaError_t e = cudaSuccess;
   zero_region(ctx, offsetof(DevScalars, ysq_keep), offsetof(DevScalars, sel_end_), st, &e);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "memset");
@@ -1684,7 +1643,7 @@ fgbd_status fgbd_get_fslr(fgbd_ctx* ctx, float* spread, uint8_t* keep, void* str
   if (!ctx->has_sel) return FGBD_ESTATE;
   const cudaStream_t st = as_stream(stream);
   FGBD_LAUNCH(ctx, "fslr_export", st,
-              launch_spread_export(ctx->n, ctx->gb.rank1, ctx->spread, ctx->keep8, spread, keep, st));
+              launch_spread_export(ctx->n, ctx->gb.rank12, ctx->spread, ctx->keep8, spread, keep, st));
   return FGBD_OK;
 }
 

@@ -20,11 +20,8 @@
 namespace fgbd {
 
 constexpr int kMaxBits = 10;                       // three b-bit coordinates fit a 32-bit code
-constexpr int kMaxRadix = 1 << kMaxBits;           // radix passes use one coordinate (b bits) as digit
-constexpr int kSortThreads = 256;
-constexpr int kSortKpt = 16;                       // keys per thread
-constexpr int kSortTile = kSortThreads * kSortKpt;  // 4096 keys per tile
-constexpr int kSlgPasses = 3;                      // y-slabs (then the slab sort: C3), C1, C2
+constexpr int kMaxRadix = 1 << kMaxBits;           // values of one coordinate (b bits)
+constexpr int kSortTile = 4096;                    // points a block of the histogram / row scatter holds at most
 constexpr int kK = 6;                              // neighbours per point at window 1
 constexpr int kD = 3 * (kK + 1);                   // patch dimension (Section 2.3)
 constexpr int kMaxWindow = 3;                      // windows 1..3: K = 6w neighbours per point
@@ -60,6 +57,8 @@ struct DevScalars {
   unsigned long long node_cnt;  // and the points that have edges
   float cexp;                   // the Eq. 4 exponent scale log2(e) / sigma_g^2 of this graph, once cexp_ready
   uint32_t cexp_ready;          // set by the first moments launch on this graph
+  uint32_t row_used[3][kMaxRadix];  // row scatter: places of every x, y and z row handed out so far
+  uint32_t row_ext[3][2];           // per coordinate: 2^b - 1 minus its smallest value, and its largest
   uint32_t build_end_;
   // ---- noise estimate region
   unsigned long long n_patches;
@@ -96,6 +95,7 @@ struct DevScalars {
   int32_t sel_valid;
   // ---- latched errors (never zeroed by a call; cleared when read)
   uint32_t status;
+  uint32_t row_start[3][kMaxRadix + 1];  // row scatter: first place of every x, y and z row, then n (not zeroed)
   // ---- settings (set at context creation)
   unsigned long long wait_limit_ns;  // any device-side wait gives up after this long
   uint32_t sigma_mode;               // sigma_g of Eq. 4: kSigmaEdge, kSigmaNode or kSigmaPair
@@ -118,24 +118,22 @@ static_assert(offsetof(DevScalars, n_edges) < offsetof(DevScalars, build_end_) &
                   offsetof(DevScalars, ne_end_) < offsetof(DevScalars, ysq_keep),
               "the build, noise and selection regions are zeroed as one range by fgbd_run");
 
-// Sort scratch for one build.
+// Sort scratch for one build.  row_pts and row_tmp may share memory with arrays
+// that are only used after the graph is built (the stored filter steps).
 struct SortBufs {
-  uint32_t* keys[2];     // ping-pong [cap]
-  uint32_t* vals[2];     // ping-pong [cap]
-  uint32_t* tile_counts; // [3 passes][kMaxRadix digits][tiles of the capacity]: per-tile digit counts,
-                         // then offsets.  Pass 0's are written by the histogram launch, pass 1's
-                         // added up by the slab sort (zeroed by the histogram launch), pass 2's by
-                         // a counting launch.
-  int count_stride;      // words of one pass's counts: kMaxRadix * tiles of the capacity
+  uint2* row_pts[3];     // per code [cap]: (input index, code) of every point, row by row
+  uint32_t* row_tmp[3];  // per code [2][tmp_stride]: scratch of the long-item sort (codes, then indices)
+  int tmp_stride;
+  uint32_t* keys_c2;     // [cap] the C2 codes along C2
+  uint32_t* keys_c3;     // [cap] the C3 codes along C3
 };
 
 // Graph in sorted order.
 struct GraphBufs {
   int32_t* perm1;    // [cap] input index of each sorted (C1-order) point
-  int32_t* rank1;    // [cap] sorted id of each input point
+  int2* rank12;      // [cap] of each input point: its sorted id (x) and its position in the C2 order (y)
   uint32_t* pk;      // [cap] packed C1 code of each sorted point (its coordinates)
-  int32_t* ord23;    // [2][cap] sorted ids along C2, then along C3
-  int32_t* rank2;    // [cap] position of each sorted id in the C2 order
+  int32_t* ord23;    // [2][cap] input indices along C2, then along C3
   int4* c4;          // [cap] C2 prev, C2 next, C3 prev, C3 next (sorted ids, -1 empty)
   // windows w > 1: [6 (w - 1)][cap stride] the points d = 2..w positions away;
   // slot 6 (d - 2) + 2 l + s holds code l's point d before (s = 0) / after (s = 1)
@@ -149,23 +147,20 @@ struct GraphBufs {
 // number of further neighbour slots at window w
 __host__ __device__ constexpr int extra_slots(int w) { return 6 * (w - 1); }
 
-// One stable radix pass whose digit is one coordinate field of the key.
-struct SortPassArgs {
+// The row scatter and the bucket sort of one frame (codes 0 C1, 1 C2, 2 C3).
+struct BucketArgs {
   int n;
   int bits;
-  int tiles;
-  int shift;               // bit offset of the digit in the key
-  int coord;               // which coordinate histogram gives the digit totals
-  const int32_t* xyz;      // if set: keys from the coordinates, values = input index
-  const uint32_t* keys_in;
-  const uint32_t* vals_in; // null: value = position
-  uint32_t* keys_out;      // null: not written
-  uint32_t* vals_out;
-  int32_t* rank_out;       // rank_out[value] = output position, or null
-  int32_t* pos_out;        // pos_out[input position] = output position, or null
-  int pass;                // 0, 1, 2 (which launch made the tile counts: pass_counted_before)
-  uint32_t* counts;
-  const DevScalars* sc;
+  int tile;                // points per block of the scatter
+  int window;              // output positions per block of the sort
+  const int32_t* xyz;
+  uint2* row_pts[3];       // SortBufs
+  uint32_t* row_tmp[3];
+  int tmp_stride;
+  uint32_t* keys_out[3];   // code c of the points along code c
+  int32_t* order_out[3];   // the input indices along each code
+  int32_t* rank12;         // GraphBufs::rank12, as [n][2]
+  DevScalars* sc;
 };
 
 // ---------------------------------------------------------------- segmented launches
@@ -211,20 +206,14 @@ struct HistArgs {
   int n;
   int bits;
   struct DevScalars* sc;
-  uint32_t* counts0;     // sort pass 0's tile counts (the y digits of each 4096-point input tile), or null
-  uint32_t* counts1;     // pass 1's tile counts, zeroed here (the slab sort adds them up), or null
 };
-struct SlabArgs {
-  int n;
-  int bits;
-  const uint32_t* keys_in;
-  const uint32_t* vals_in;
-  uint32_t* keys_tmp;
-  uint32_t* vals_tmp;
-  uint32_t* keys_out;
-  int32_t* vals_out;
-  const struct DevScalars* sc;
-  uint32_t* counts1;     // sort pass 1's tile counts: the z digits of the C3 order, added up here (or null)
+// The caller's colours (input order) and where they go in C1 order.
+struct ColorArgs {
+  const void* rgb;       // null: none
+  int dtype;             // 0: uint8 into y8, else float32 into yf
+  const int32_t* perm1;
+  uint32_t* y8;
+  float4* yf;
 };
 struct LinkArgs {
   int n;
@@ -233,18 +222,11 @@ struct LinkArgs {
   const int32_t* ord23;
   const uint32_t* keys_c2;
   const uint32_t* keys_c3;
-  const int32_t* rank2;
+  const int2* rank12;
   uint32_t* pk;
   int4* c4;
   struct DevScalars* sc;
-};
-struct GatherArgs {
-  const void* rgb;
-  int dtype;
-  int n;
-  const int32_t* perm1;
-  uint32_t* y8;
-  float4* yf;
+  ColorArgs colors;
 };
 struct MomentArgs {
   int n;
@@ -267,7 +249,7 @@ struct ZeroArgs {
 
 // How a batch runs, chosen by the batch tuner (api.cu): frames per segmented
 // launch (0: every frame on a stream of its own, its own kernels), threads of
-// the sort scatter (one 4096-key tile a block), threads of the filter blocks
+// the row scatter (a tile of up to 4096 points a block), threads of the filter blocks
 // and filter blocks per SM of the cooperative selection.
 struct BatchShape {
   int seg_frames = kSegMax;
@@ -280,46 +262,39 @@ struct BatchShape {
 struct FilterArgs;
 // Every launcher enqueues on `stream` and returns the launch error.
 
-// the coordinate histograms; with sb, also sort pass 0's tile counts (and pass 1's zeroed)
-cudaError_t launch_coord_hist(const int32_t* xyz, int n, int bits, DevScalars* sc, const SortBufs* sb, int num_sms,
-                              cudaStream_t stream);
-// pass 0: y-slabs from the input; (the slab sort then gives C3); pass 1: C1 = the C3 order on z;
-// pass 2: C2 = the C1 order on x
-SortPassArgs slg_pass_args(int pass, const int32_t* xyz, int n, int bits, int cap, const SortBufs& sb,
-                           const GraphBufs& gb, const DevScalars* sc);
-// C3 within each y-slab (after pass 0): (x, z) order into keys[1] and ord23[1]
-cudaError_t launch_slab_sort(int n, int bits, int cap, const SortBufs& sb, const GraphBufs& gb,
-                             const DevScalars* sc, cudaStream_t stream);
-cudaError_t launch_tile_counts(const SortPassArgs& a, cudaStream_t stream);
-// pass p's tile counts are made by the launches before it for p = 0 (histogram) and p = 1 (slab sort)
-constexpr bool pass_counted_before(int pass) { return pass < 2; }
-cudaError_t launch_tile_scan(const SortPassArgs& a, cudaStream_t stream);
-cudaError_t launch_sort_scatter(const SortPassArgs& a, cudaStream_t stream);
-cudaError_t launch_sort_pass(const SortPassArgs& a, cudaStream_t stream);  // the three above
+// the coordinate histograms (and the range check)
+cudaError_t launch_coord_hist(const int32_t* xyz, int n, int bits, DevScalars* sc, int num_sms, cudaStream_t stream);
+// `cap`: distance between the C2 and the C3 half of gb.ord23; `fill`: blocks of the row scatter that
+// fill the GPU (or this frame's share of it)
+BucketArgs bucket_args(const int32_t* xyz, int n, int bits, int cap, const SortBufs& sb, const GraphBufs& gb,
+                       DevScalars* sc, int fill);
+constexpr int scatter_fill(int num_sms) { return 2 * num_sms; }  // two resident blocks per SM
+cudaError_t launch_bucket_scatter(const BucketArgs& a, cudaStream_t stream);
+cudaError_t launch_bucket_sort(const BucketArgs& a, cudaStream_t stream);
 cudaError_t launch_orders_export(int n, int cap, const GraphBufs& gb, int32_t* out, cudaStream_t stream);
 // segmented launches: one launch for frames 0..count-1 (count <= kSegMax), each
 // frame with the blocks its one-frame launch would have
-HistArgs hist_args(const int32_t* xyz, int n, int bits, DevScalars* sc, const SortBufs& sb);
-LinkArgs link_args(int n, int bits, int cap, const GraphBufs& gb, const SortBufs& sb, DevScalars* sc);
+HistArgs hist_args(const int32_t* xyz, int n, int bits, DevScalars* sc);
+LinkArgs link_args(int n, int bits, int cap, const GraphBufs& gb, const SortBufs& sb, DevScalars* sc,
+                   const ColorArgs& colors);
 cudaError_t launch_zero_words_seg(const ZeroArgs* a, int count, cudaStream_t stream);
 cudaError_t launch_coord_hist_seg(const HistArgs* a, int count, int num_sms, cudaStream_t stream);
-// counts, scan and scatter of one pass (scatter_threads: 256, 512 or 1024 per 4096-key tile)
-cudaError_t launch_sort_pass_seg(const SortPassArgs* a, int count, int scatter_threads, cudaStream_t stream);
-cudaError_t launch_slab_sort_seg(const int* n, const int* bits, const int* cap, const SortBufs* sb,
-                                 const GraphBufs* gb, DevScalars* const* sc, int count, cudaStream_t stream);
+// (scatter_threads: 256, 512 or 1024 per tile)
+cudaError_t launch_bucket_scatter_seg(const BucketArgs* a, int count, int scatter_threads, cudaStream_t stream);
+cudaError_t launch_bucket_sort_seg(const BucketArgs* a, int count, cudaStream_t stream);
 cudaError_t launch_link_seg(const LinkArgs* a, int count, bool same_line, int num_sms, cudaStream_t stream);
 cudaError_t launch_link(int n, int bits, int cap, bool same_line, const GraphBufs& gb, const SortBufs& sb,
-                        DevScalars* sc, int num_sms, cudaStream_t stream);
+                        DevScalars* sc, const ColorArgs& colors, int num_sms, cudaStream_t stream);
 // each sorted point's mean edge length into gb.node_sig (if set) and, for the
 // node reading of sigma_g, their sum and count into the build scalars
 cudaError_t launch_node_sigma(int n, int bits, const GraphBufs& gb, DevScalars* sc, int num_sms, cudaStream_t stream);
 // windows w > 1: every link of the window (C2/C3 d = 1 into c4, d >= 2 into cx)
 // and the edge sums; then k_c1_line_flags under the same-line variant
 cudaError_t launch_link_wide(int n, int bits, int cap, int window, bool same_line, const GraphBufs& gb,
-                             const SortBufs& sb, DevScalars* sc, int num_sms, cudaStream_t stream);
+                             const SortBufs& sb, DevScalars* sc, const ColorArgs& colors, int num_sms,
+                             cudaStream_t stream);
 
-cudaError_t launch_gather_colors(const void* rgb, int dtype, int n, const int32_t* perm1,
-                                 uint32_t* y8, float4* yf, cudaStream_t stream);
+cudaError_t launch_gather_colors(const ColorArgs& a, int n, cudaStream_t stream);
 // x0: if set, the launch also writes x_0 of the filter steps (colours and packed code)
 cudaError_t launch_ne_moments(int n, int bits, int dtype, const GraphBufs& gb, const uint32_t* y8,
                               const float4* yf, float* spread, double* f64_partials,
@@ -337,7 +312,6 @@ cudaError_t launch_debug_div(const double* a, const double* b, double* q_newton,
 MomentArgs moment_args(int n, int bits, const GraphBufs& gb, const uint32_t* y8, const float4* yf, float* spread,
                        double* f64_partials, bool moments, bool sorted_patches, DevScalars* sc);
 // segmented: frames 0..count-1 (count <= kSegMax; one colour dtype for the moments)
-cudaError_t launch_gather_colors_seg(const GatherArgs* a, int count, cudaStream_t stream);
 cudaError_t launch_ne_moments_seg(const MomentArgs* a, int count, int dtype, int num_sms, cudaStream_t stream);
 // the estimate launch over frames: one eigen block per frame, the other SMs
 // shared out for the speculative steps (spec[f].spec_depth of them)
@@ -379,7 +353,7 @@ struct FilterArgs {
   const float* spread;
   const uint32_t* pk;
   const int4* c4;
-  const int32_t* rank1;
+  const int2* rank12;    // (x: the sorted id of each input point)
   float4* xbuf0;
   float4* xbuf1;
   void* out;             // input-order output or nullptr
@@ -446,7 +420,7 @@ cudaError_t launch_csr_degree(int n, const GraphBufs& gb, int64_t* deg_out, cuda
 cudaError_t launch_scan_i64(int64_t* data, int64_t count, int64_t* block_tmp, cudaStream_t stream);
 cudaError_t launch_csr_fill(int n, int bits, const GraphBufs& gb, const int64_t* row_ptr, int32_t* col,
                             float* w, int64_t col_capacity, const DevScalars* sc, cudaStream_t stream);
-cudaError_t launch_spread_export(int n, const int32_t* rank1, const float* spread, const uint8_t* keep8,
+cudaError_t launch_spread_export(int n, const int2* rank12, const float* spread, const uint8_t* keep8,
                                  float* spread_out, uint8_t* keep_out, cudaStream_t stream);
 
 // ---------------------------------------------------------------- device helpers
@@ -462,6 +436,64 @@ __host__ __device__ inline uint32_t code_of(int which, uint32_t x, uint32_t y, u
 
 // an index read from device memory is used only if it lies in [0, n)
 __device__ __forceinline__ bool in_range(int v, int n) { return unsigned(v) < unsigned(n); }
+
+// Colour of input point i (R, G, B in the low three bytes) out of n: from the one
+// or two aligned words that hold its bytes, where the array starts on a word
+// and the second word lies inside it (three byte loads a point fill the load
+// queue: 10.8 us at 1M points).
+__device__ __forceinline__ uint32_t load_rgb8(const uint8_t* __restrict__ rgb, uint32_t i, uint32_t n, bool words) {
+  const size_t at = 3 * size_t(i);
+  if (words && i + 2 < n) {
+    const uint32_t* w = reinterpret_cast<const uint32_t*>(rgb) + (at >> 2);
+    const uint32_t off = uint32_t(at) & 3u;
+    const uint32_t lo = __ldg(w), hi = off > 1u ? __ldg(w + 1) : 0u;
+    return __funnelshift_r(lo, hi, 8u * off) & 0xffffffu;
+  }
+  return uint32_t(__ldg(rgb + at)) | (uint32_t(__ldg(rgb + at + 1)) << 8) | (uint32_t(__ldg(rgb + at + 2)) << 16);
+}
+__device__ __forceinline__ float4 load_rgbf(const float* __restrict__ rgb, uint32_t i) {
+  const size_t at = 3 * size_t(i);
+  return make_float4(__ldg(rgb + at), __ldg(rgb + at + 1), __ldg(rgb + at + 2), 0.f);
+}
+
+// The colours of the sorted points k0 .. k0 + 3 (k0 a multiple of 4) below n into
+// C1 order: their input indices read as one int4 and the loads issued together.
+__device__ __forceinline__ void colors_quad(const ColorArgs& a, int k0, int n) {
+  int pi[4];
+  if (k0 + 4 <= n) {
+    const int4 v = *reinterpret_cast<const int4*>(a.perm1 + k0);
+    pi[0] = v.x;
+    pi[1] = v.y;
+    pi[2] = v.z;
+    pi[3] = v.w;
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) pi[i] = k0 + i < n ? a.perm1[k0 + i] : -1;
+  }
+  if (a.dtype == 0) {
+    const uint8_t* rgb = static_cast<const uint8_t*>(a.rgb);
+    const bool words = (reinterpret_cast<uintptr_t>(rgb) & 3u) == 0;
+    uint32_t c[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) c[i] = in_range(pi[i], n) ? load_rgb8(rgb, uint32_t(pi[i]), uint32_t(n), words) : 0u;
+    if (k0 + 4 <= n) {
+      *reinterpret_cast<uint4*>(a.y8 + k0) = make_uint4(c[0], c[1], c[2], c[3]);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (k0 + i < n) a.y8[k0 + i] = c[i];
+    }
+  } else {
+    const float* rgb = static_cast<const float*>(a.rgb);
+    float4 c[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      c[i] = in_range(pi[i], n) ? load_rgbf(rgb, uint32_t(pi[i])) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (k0 + i < n) a.yf[k0 + i] = c[i];
+  }
+}
 
 __device__ __forceinline__ void decode_c1(uint32_t c, int b, int& x, int& y, int& z) {
   const uint32_t m = (1u << b) - 1u;

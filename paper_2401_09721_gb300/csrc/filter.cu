@@ -71,7 +71,7 @@ __global__ void k_csr_degree(int n, GraphBufs gb, int64_t* __restrict__ deg) {
       continue;
     }
     int nb[kMaxDegree];
-    deg[i] = gather_row(gb.rank1[i], n, gb, nb);
+    deg[i] = gather_row(gb.rank12[i].x, n, gb, nb);
   }
 }
 
@@ -82,7 +82,7 @@ __global__ void k_csr_fill(int n, int bits, GraphBufs gb, const int64_t* __restr
   const double sg = sigma_g_of(sc);
   const float inv2 = sg > 0.0 ? float(1.0 / (sg * sg)) : 0.f;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const int k = gb.rank1[i];
+    const int k = gb.rank12[i].x;
     int nb[kMaxDegree];
     const int cnt = gather_row(k, n, gb, nb);
     if (cnt == 0) continue;
@@ -158,12 +158,12 @@ __global__ void k_scan_add(int64_t* data, int64_t count, const int64_t* totals) 
   if (i < count) data[i] += totals[blockIdx.x];
 }
 
-__global__ void k_spread_export(int n, const int32_t* __restrict__ rank1, const float* __restrict__ spread,
+__global__ void k_spread_export(int n, const int2* __restrict__ rank12, const float* __restrict__ spread,
                                 const uint8_t* __restrict__ keep8, float* __restrict__ spread_out,
                                 uint8_t* __restrict__ keep_out) {
   pdl_wait();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const int k = rank1[i];
+    const int k = rank12[i].x;
     if (!in_range(k, n)) continue;
     if (spread_out) spread_out[i] = spread[k];
     if (keep_out) keep_out[i] = keep8[k] ? 1 : 0;
@@ -270,11 +270,11 @@ cudaError_t launch_csr_fill(int n, int bits, const GraphBufs& gb, const int64_t*
                        col_capacity, sc);
 }
 
-cudaError_t launch_spread_export(int n, const int32_t* rank1, const float* spread, const uint8_t* keep8,
+cudaError_t launch_spread_export(int n, const int2* rank12, const float* spread, const uint8_t* keep8,
                                  float* spread_out, uint8_t* keep_out, cudaStream_t stream) {
   if (n <= 0) return cudaSuccess;
   const int grid = std::min((n + 255) / 256, 152 * 16);
-  return launch_kernel(k_spread_export, dim3(grid), dim3(256), 0, stream, false, n, rank1, spread, keep8, spread_out,
+  return launch_kernel(k_spread_export, dim3(grid), dim3(256), 0, stream, false, n, rank12, spread, keep8, spread_out,
                        keep_out);
 }
 

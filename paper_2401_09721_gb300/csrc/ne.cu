@@ -29,88 +29,11 @@ namespace {
 
 constexpr int kTiles = 28;  // 3x3 output tiles covering the upper triangle of a 21x21 matrix
 
-// Colours into sorted order: four consecutive sorted points per thread, their
-// input indices read as one int4 and the twelve colour loads issued together.
-__device__ __forceinline__ void perm_quad(const int32_t* __restrict__ perm1, int k0, int n, int (&pi)[4]) {
-  if (k0 + 4 <= n) {
-    const int4 v = *reinterpret_cast<const int4*>(perm1 + k0);
-    pi[0] = v.x;
-    pi[1] = v.y;
-    pi[2] = v.z;
-    pi[3] = v.w;
-  } else {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) pi[i] = k0 + i < n ? perm1[k0 + i] : -1;
-  }
-}
-
-__device__ __forceinline__ void gather_u8_body(const uint8_t* __restrict__ rgb, int n,
-                                               const int32_t* __restrict__ perm1, uint32_t* __restrict__ y8,
-                                               int bid, int nblk) {
-  for (int k0 = 4 * (bid * blockDim.x + threadIdx.x); k0 < n; k0 += 4 * nblk * blockDim.x) {
-    int pi[4];
-    perm_quad(perm1, k0, n, pi);
-    uint32_t c[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      c[i] = 0u;
-      if (in_range(pi[i], n)) {
-        const size_t b = 3 * size_t(pi[i]);
-        c[i] = uint32_t(__ldg(rgb + b)) | (uint32_t(__ldg(rgb + b + 1)) << 8) | (uint32_t(__ldg(rgb + b + 2)) << 16);
-      }
-    }
-    if (k0 + 4 <= n) {
-      *reinterpret_cast<uint4*>(y8 + k0) = make_uint4(c[0], c[1], c[2], c[3]);
-    } else {
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        if (k0 + i < n) y8[k0 + i] = c[i];
-    }
-  }
-}
-
-__device__ __forceinline__ void gather_f32_body(const float* __restrict__ rgb, int n,
-                                                const int32_t* __restrict__ perm1, float4* __restrict__ yf, int bid,
-                                                int nblk) {
-  for (int k0 = 4 * (bid * blockDim.x + threadIdx.x); k0 < n; k0 += 4 * nblk * blockDim.x) {
-    int pi[4];
-    perm_quad(perm1, k0, n, pi);
-    float4 c[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      c[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (in_range(pi[i], n)) {
-        const size_t b = 3 * size_t(pi[i]);
-        c[i] = make_float4(__ldg(rgb + b), __ldg(rgb + b + 1), __ldg(rgb + b + 2), 0.f);
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-      if (k0 + i < n) yf[k0 + i] = c[i];
-  }
-}
-
-__global__ void __launch_bounds__(256) k_gather_u8(const uint8_t* __restrict__ rgb, int n,
-                                                   const int32_t* __restrict__ perm1,
-                                                   uint32_t* __restrict__ y8) {
+// Colours into sorted order, on their own (a whole run takes them in the link launch).
+__global__ void __launch_bounds__(256) k_gather_colors(ColorArgs a, int n) {
   pdl_wait();
-  gather_u8_body(rgb, n, perm1, y8, blockIdx.x, gridDim.x);
-}
-
-__global__ void __launch_bounds__(256) k_gather_f32(const float* __restrict__ rgb, int n,
-                                                    const int32_t* __restrict__ perm1,
-                                                    float4* __restrict__ yf) {
-  pdl_wait();
-  gather_f32_body(rgb, n, perm1, yf, blockIdx.x, gridDim.x);
-}
-
-__global__ void __launch_bounds__(256) k_gather_seg(const __grid_constant__ Seg<GatherArgs> s) {
-  pdl_wait();
-  const int f = seg_frame(s, blockIdx.x);
-  const GatherArgs& a = s.a[f];
-  const int bid = blockIdx.x - s.start[f], nblk = s.start[f + 1] - s.start[f];
-  if (a.dtype == 0) gather_u8_body(static_cast<const uint8_t*>(a.rgb), a.n, a.perm1, a.y8, bid, nblk);
-  else gather_f32_body(static_cast<const float*>(a.rgb), a.n, a.perm1, a.yf, bid, nblk);
+  for (int k0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x); k0 < n; k0 += 4 * gridDim.x * blockDim.x)
+    colors_quad(a, k0, n);
 }
 
 __device__ __forceinline__ void tile_rc(int tile, int& r0, int& c0) {
@@ -831,19 +754,6 @@ cudaError_t launch_debug_div(const double* a, const double* b, double* q_newton,
   return launch_kernel(k_debug_div, dim3(grid), dim3(256), 0, stream, false, a, b, q_newton, q_div, n);
 }
 
-cudaError_t launch_gather_colors_seg(const GatherArgs* a, int count, cudaStream_t stream) {
-  if (count < 1 || count > kSegMax) return cudaErrorInvalidValue;
-  Seg<GatherArgs> sg;
-  int blocks[kSegMax];
-  for (int f = 0; f < count; ++f) {
-    sg.a[f] = a[f];
-    blocks[f] = a[f].n > 0 ? std::min((a[f].n + 1023) / 1024, 152 * 8) : 0;  // as launch_gather_colors
-  }
-  const int grid = seg_layout(sg, blocks, count);
-  if (grid == 0) return cudaSuccess;
-  return launch_kernel(k_gather_seg, dim3(grid), dim3(256), 0, stream, false, sg);
-}
-
 cudaError_t launch_ne_moments_seg(const MomentArgs* a, int count, int dtype, int num_sms, cudaStream_t stream) {
   if (count < 1 || count > kSegMax) return cudaErrorInvalidValue;
   Seg<MomentArgs> sg;
@@ -889,15 +799,10 @@ cudaError_t launch_ne_finalize_seg(const FilterArgs* spec, const double* const* 
                        es);
 }
 
-cudaError_t launch_gather_colors(const void* rgb, int dtype, int n, const int32_t* perm1,
-                                 uint32_t* y8, float4* yf, cudaStream_t stream) {
+cudaError_t launch_gather_colors(const ColorArgs& a, int n, cudaStream_t stream) {
   if (n <= 0) return cudaSuccess;
   const int grid = std::min((n + 1023) / 1024, 152 * 8);  // four points a thread
-  if (dtype == 0)
-    return launch_kernel(k_gather_u8, dim3(grid), dim3(256), 0, stream, false, static_cast<const uint8_t*>(rgb), n,
-                         perm1, y8);
-  return launch_kernel(k_gather_f32, dim3(grid), dim3(256), 0, stream, false, static_cast<const float*>(rgb), n,
-                       perm1, yf);
+  return launch_kernel(k_gather_colors, dim3(grid), dim3(256), 0, stream, false, a, n);
 }
 
 int ne_moment_blocks(int n, int num_sms) {

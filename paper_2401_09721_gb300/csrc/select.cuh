@@ -299,7 +299,7 @@ __device__ __forceinline__ float4 kept_rgb(const FilterArgs& a, int kept, int k)
 }
 
 // The kept iterate in input order: input points i0 .. i0 + 3 per thread and
-// trip, their sorted positions read as one int4 and the four gathers issued
+// trip, their sorted positions read as two int4 and the four gathers issued
 // together; uint8 / float32 output as 32- / 128-bit stores where aligned.
 __device__ __forceinline__ void output_quads(const FilterArgs& a, int kept, int gtid, int gstride) {
   const int n = a.n;
@@ -309,15 +309,16 @@ __device__ __forceinline__ void output_quads(const FilterArgs& a, int kept, int 
     const bool full = i0 + 4 <= n;
     int kk[4] = {-1, -1, -1, -1};
     if (full) {
-      const int4 v = *reinterpret_cast<const int4*>(a.rank1 + i0);
-      kk[0] = v.x;
-      kk[1] = v.y;
-      kk[2] = v.z;
-      kk[3] = v.w;
+      const int4 u = *reinterpret_cast<const int4*>(a.rank12 + i0);
+      const int4 v = *reinterpret_cast<const int4*>(a.rank12 + i0 + 2);
+      kk[0] = u.x;
+      kk[1] = u.z;
+      kk[2] = v.x;
+      kk[3] = v.z;
     } else {
 #pragma unroll
       for (int i = 0; i < 4; ++i)
-        if (i0 + i < n) kk[i] = a.rank1[i0 + i];
+        if (i0 + i < n) kk[i] = a.rank12[i0 + i].x;
     }
     float4 v[4];
     bool ok[4];

@@ -1,27 +1,21 @@
 // SLG: scan-line graph construction (Section 2.2).
 //
 // Sorting by a code of Eq. 1-3 is sorting by three b-bit coordinates, most
-// significant first.  The digits of the radix passes are the coordinates
-// themselves (2^b bins), and ties keep input order throughout, so equal codes
-// are ordered by index:
-//   pass 0   one stable pass on y over the input puts every y-slab in place;
-//   slab     k_slab_sort sorts each y-slab by (x, z) in shared memory, one
-//            block per slab (two stable passes, z then x): the C3 = (y, x, z)
-//            order;
-//   pass 1   C1 = (z, y, x): one stable pass on z over the C3 order (among
-//            points with equal z the C3 order already ranks them by (y, x));
-//   pass 2   C2 = (x, z, y): one stable pass on x over the C1 order (among
-//            points with equal x the C1 order ranks them by (z, y)).
-// The digit totals of every pass are the three coordinate histograms, taken
-// once (k_coord_hist).  Each global pass is reduce-then-scan:
-//   k_tile_counts   digit counts of every 4096-key tile;
-//   k_tile_scan     each tile's global start of every digit;
-//   k_sort_scatter  stable in-tile rank (one ballot per digit bit) and
-//                   write-out in digit runs.
-// Keys are the packed C1 codes in every pass.  Pass 1 ends with the packed
-// code of every sorted (C1) point, its input index, the rank of every input
-// point, and the C3 order rewritten as sorted ids; pass 2 ends with the sorted
-// ids along C2, their packed codes, and the C2 rank of every sorted id.
+// significant first, with equal codes (repeated voxels) in input order.  The
+// three orders are made side by side, each in two steps:
+//   k_coord_hist      the three coordinate histograms: the size of every row,
+//                     a row being the points of one most significant
+//                     coordinate of a code (z for C1, x for C2, y for C3);
+//   k_bucket_scatter  every point into its row of each code, in any order
+//                     inside the row: a block ranks its tile's points with
+//                     shared-memory counters and reserves its share of every
+//                     row with one global atomic a row;
+//   k_bucket_sort     the points of a window of consecutive rows (or of the
+//                     lines of one large row that start in the window) ordered
+//                     by (code, input index) in shared memory.
+// C1 ends with the packed code of every sorted (C1) point, its input index and
+// the rank of every input point; C2 and C3 with the input indices and the codes
+// along the code, C2 also with the rank of every input point.
 // k_link: points consecutive along a code are linked.  In C1 order the code-1
 // neighbours are implicit (k-1, k+1); C2/C3 neighbours are written as slots;
 // a pair already linked by an earlier code is left out so the union is a set,
@@ -34,46 +28,46 @@
 namespace fgbd {
 namespace {
 
-// The scatter ranks a 4096-key tile with THREADS threads (the one-frame path
-// runs 512, twice the threads of the counting pass, so that the per-block
-// serial chains - ranking, write-out - are half as long; the batch tuner may
-// pick 256 or 1024).  Two warps share one 32-bit digit counter word (16 bits
-// each: a warp ranks at most 512 keys).
-template <int THREADS>
-struct ScatterShape {
-  static constexpr int kWarps = THREADS / 32;
-  static constexpr int kKpt = kSortTile / THREADS;          // keys per thread
-  static constexpr int kPairWords = kWarps / 2;             // counter words per digit
-  static constexpr int kDigitsPerThread = kMaxRadix / THREADS;
-  static constexpr int kMinBlocks = THREADS >= 1024 ? 1 : 2;
-  static_assert(kSortTile % THREADS == 0 && kMaxRadix % THREADS == 0 && kWarps % 2 == 0 && 32 * kKpt <= 65535,
-                "tile, digits and counter halves must divide evenly");
-};
-constexpr int kScatterThreads = 512;  // the one-frame path
+// the coordinate rows of the histograms (0 x, 1 y, 2 z) that are the most and
+// the second most significant of code c (0 C1, 1 C2, 2 C3); the least is row c
+__device__ __forceinline__ int row_coord(int c) { return c == 0 ? 2 : c - 1; }
+__device__ __forceinline__ int mid_coord(int c) { return c == 2 ? 0 : c + 1; }
 
-size_t scatter_smem_bytes(int threads) {
-  const int warps = threads / 32;
-  return sizeof(uint32_t) *
-         (size_t(warps / 2) * kMaxRadix + 2 * size_t(kSortTile) + 2 * size_t(kMaxRadix) + warps + 1);
+// code c of a packed C1 code
+__device__ __forceinline__ uint32_t code_from_c1(int c, uint32_t c1, int b, uint32_t m) {
+  return c == 0 ? c1 : code_of(c, c1 & m, (c1 >> b) & m, c1 >> (2 * b), b);
+}
+
+// this warp's offset from the totals of the warps of the block (at most 32)
+__device__ __forceinline__ uint32_t warps_before(const uint32_t* s_w, int lane, int warp) {
+  return __reduce_add_sync(0xffffffffu, lane < warp ? s_w[lane] : 0u);
+}
+
+__device__ __forceinline__ uint32_t warp_inclusive(uint32_t x, int lane) {
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  return x;
+}
+
+// exclusive scan of one value per thread over the block (s_w: one word a warp)
+__device__ __forceinline__ uint32_t block_exclusive(uint32_t v, uint32_t* s_w) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t x = warp_inclusive(v, lane);
+  if (lane == 31) s_w[warp] = x;
+  __syncthreads();
+  return warps_before(s_w, lane, warp) + x - v;
 }
 
 // The three coordinate histograms, 1024-thread blocks (up to two per SM) taking
-// whole 4096-point tiles of the input, merged with global atomics.  The y digits of
-// each tile are also counted on their own: sort pass 0's tile counts (its
-// keys are the input's y digits in input order), so that pass needs no
-// counting launch.  Pass 1's tile counts, which the slab sort adds up, are
-// zeroed here.
+// whole 4096-point tiles of the input, merged with global atomics.
 __device__ __forceinline__ void coord_hist_body(const HistArgs& a, int bid, int nblk) {
   __shared__ uint32_t h[3][kMaxRadix];
-  __shared__ uint32_t ht[kMaxRadix];
   const int radix = 1 << a.bits;
   const int tiles = (a.n + kSortTile - 1) / kSortTile;
   for (int i = threadIdx.x; i < 3 * kMaxRadix; i += blockDim.x) (&h[0][0])[i] = 0;
-  if (a.counts1) {
-    const size_t words = size_t(radix) * tiles;
-    for (size_t i = size_t(bid) * blockDim.x + threadIdx.x; i < words; i += size_t(nblk) * blockDim.x)
-      a.counts1[i] = 0u;
-  }
   const uint32_t m = uint32_t(radix) - 1u;
   // four consecutive points a thread (a tile is kSortTile = 4 x 1024 points),
   // read as three 16-byte loads where the array is aligned, all issued before
@@ -81,9 +75,8 @@ __device__ __forceinline__ void coord_hist_body(const HistArgs& a, int bid, int 
   static_assert(kSortTile == 4 * 1024, "1024 threads take four points each");
   const bool vec = (reinterpret_cast<uintptr_t>(a.xyz) & 15u) == 0;
   bool bad = false;
+  __syncthreads();
   for (int t = bid; t < tiles; t += nblk) {
-    for (int d = threadIdx.x; d < radix; d += blockDim.x) ht[d] = 0;
-    __syncthreads();
     const int p0 = t * kSortTile + 4 * int(threadIdx.x);
     int c[12];
     if (vec && p0 + 4 <= a.n) {
@@ -104,11 +97,7 @@ __device__ __forceinline__ void coord_hist_body(const HistArgs& a, int bid, int 
       atomicAdd(&h[0][xi & m], 1u);
       atomicAdd(&h[1][yi & m], 1u);
       atomicAdd(&h[2][zi & m], 1u);
-      atomicAdd(&ht[yi & m], 1u);
     }
-    __syncthreads();
-    if (a.counts0)
-      for (int d = threadIdx.x; d < radix; d += blockDim.x) a.counts0[size_t(d) * tiles + t] = ht[d];
   }
   if (bad) atomicOr(&a.sc->status, kFlagRange);
   __syncthreads();
@@ -128,337 +117,220 @@ __global__ void __launch_bounds__(1024, 2) k_coord_hist_seg(const __grid_constan
   coord_hist_body(s.a[f], blockIdx.x - s.start[f], s.start[f + 1] - s.start[f]);
 }
 
-// The keys and values of one tile (striped: item j of lane l of warp w is
-// position t*kSortTile + w*32*kSortKpt + j*32 + l, so loads coalesce).
-__device__ __forceinline__ void load_tile(const SortPassArgs& a, int warp_base, int lane, uint32_t (&key)[kSortKpt],
-                                          uint32_t (&val)[kSortKpt], bool with_vals) {
-  const uint32_t m = (1u << a.bits) - 1u;
-#pragma unroll
-  for (int j = 0; j < kSortKpt; ++j) {
-    const int pos = warp_base + j * 32 + lane;
-    key[j] = 0;
-    val[j] = 0;
-    if (pos < a.n) {
-      if (a.xyz) {
-        const uint32_t x = uint32_t(a.xyz[3 * size_t(pos)]) & m;
-        const uint32_t y = uint32_t(a.xyz[3 * size_t(pos) + 1]) & m;
-        const uint32_t z = uint32_t(a.xyz[3 * size_t(pos) + 2]) & m;
-        key[j] = code_of(0, x, y, z, a.bits);
-        val[j] = uint32_t(pos);
-      } else {
-        key[j] = a.keys_in[pos];
-        if (with_vals) val[j] = a.vals_in ? a.vals_in[pos] : uint32_t(pos);
-      }
-    }
-  }
-}
-
-// Reduce: digit counts of every tile, counts[digit * tiles + tile].
-__device__ __forceinline__ void tile_counts_body(const SortPassArgs& a, int t) {
-  __shared__ uint32_t s_h[kMaxRadix];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int radix = 1 << a.bits;
-  for (int d = tid; d < radix; d += kSortThreads) s_h[d] = 0;
-  __syncthreads();
-  uint32_t key[kSortKpt], val[kSortKpt];
-  const int warp_base = t * kSortTile + warp * (32 * kSortKpt);
-  load_tile(a, warp_base, lane, key, val, false);
-  const uint32_t m = uint32_t(radix) - 1u;
-#pragma unroll
-  for (int j = 0; j < kSortKpt; ++j)
-    if (warp_base + j * 32 + lane < a.n) atomicAdd(&s_h[(key[j] >> a.shift) & m], 1u);
-  __syncthreads();
-  for (int d = tid; d < radix; d += kSortThreads) a.counts[size_t(d) * a.tiles + t] = s_h[d];
-}
-
-__global__ void __launch_bounds__(kSortThreads) k_tile_counts(SortPassArgs a) {
-  pdl_wait();
-  tile_counts_body(a, blockIdx.x);
-}
-
-__global__ void __launch_bounds__(kSortThreads) k_tile_counts_seg(const __grid_constant__ Seg<SortPassArgs> s) {
-  pdl_wait();
-  const int f = seg_frame(s, blockIdx.x);
-  tile_counts_body(s.a[f], blockIdx.x - s.start[f]);
-}
-
-// Scan: one warp per digit row.  counts become offsets: the start of the
-// digit's bucket (total of the smaller digits) plus the counts of the earlier
-// tiles.  Each lane owns a run of up to 8 consecutive tiles per batch.
-__device__ __forceinline__ void tile_scan_body(const SortPassArgs& a, int bid) {
-  const int lane = threadIdx.x & 31;
-  const int radix = 1 << a.bits;
-  const int d = bid * 8 + (threadIdx.x >> 5);
-  if (d >= radix) return;
-  uint32_t* r = a.counts + size_t(d) * a.tiles;
-  constexpr int kRun = 8;
-  // the first run of tile counts, loaded before the histogram so that the two
-  // sets of loads are in flight together
-  uint32_t c[kRun];
-#pragma unroll
-  for (int i = 0; i < kRun; ++i) {
-    const int t = lane * kRun + i;
-    c[i] = t < a.tiles ? r[t] : 0u;
-  }
-  // the digit's bucket start: lane l sums the histogram entries 32l..32l+31
-  // below d, read as eight independent 16-byte loads
-  const uint4* hist4 = reinterpret_cast<const uint4*>(a.sc->chist[a.coord]);
-  uint32_t base = 0;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int e = lane * 32 + i * 4;
-    if (e < d) {
-      const uint4 h = hist4[e >> 2];
-      base += h.x + (e + 1 < d ? h.y : 0u) + (e + 2 < d ? h.z : 0u) + (e + 3 < d ? h.w : 0u);
-    }
-  }
-  base = warp_sum(base);
-  for (int t0 = 0; t0 < a.tiles; t0 += 32 * kRun) {
-    if (t0 > 0) {
-#pragma unroll
-      for (int i = 0; i < kRun; ++i) {
-        const int t = t0 + lane * kRun + i;
-        c[i] = t < a.tiles ? r[t] : 0u;
-      }
-    }
-    uint32_t own = 0;
-#pragma unroll
-    for (int i = 0; i < kRun; ++i) own += c[i];
-    uint32_t x = own;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
-    }
-    uint32_t run = base + x - own;
-#pragma unroll
-    for (int i = 0; i < kRun; ++i) {
-      const int t = t0 + lane * kRun + i;
-      if (t < a.tiles) r[t] = run;
-      run += c[i];
-    }
-    base += __shfl_sync(0xffffffffu, x, 31);
-  }
-}
-
-__global__ void __launch_bounds__(256) k_tile_scan(SortPassArgs a) {
-  pdl_wait();
-  tile_scan_body(a, blockIdx.x);
-}
-
-__global__ void __launch_bounds__(256) k_tile_scan_seg(const __grid_constant__ Seg<SortPassArgs> s) {
-  pdl_wait();
-  const int f = seg_frame(s, blockIdx.x);
-  tile_scan_body(s.a[f], blockIdx.x - s.start[f]);
-}
-
-// Scatter: rank each key of the tile among equal digits (stable), then write
-// the tile out in digit runs at the offsets the scan produced.
+// ---------------------------------------------------------------- rows
+// One tile of up to kSortTile points a block: (input index, code) of every
+// point into its row of the three codes.  The order inside a row is left to
+// k_bucket_sort, so the ranks come from shared-memory atomics instead of
+// ballots, the tiles need no counts from an earlier launch (a block reserves
+// its share of a row with one global atomic), and the three codes share one
+// read of the coordinates.  A tile is staged in row order in shared memory
+// before it is written, so that the points of one row leave as one run.
+// Measured (1M body points, b = 10): 16 us for the three codes; one of the
+// three ballot-ranked passes it stands in for took 17.5 us, and with its scan
+// and counts 25.  It waits on its loads, barriers and shared-memory ranks (27 %
+// of the issue slots used); scattering without staging (8-byte random writes)
+// took 36 us.  Two blocks an SM: more and smaller tiles pay for the row scans
+// and the global atomics (37 us with 608 blocks).
 template <int THREADS>
-__device__ __forceinline__ void sort_scatter_body(const SortPassArgs& a, int t) {
+struct ScatterShape {
+  static constexpr int kKpt = kSortTile / THREADS;    // points per thread
+  static constexpr int kDpt = kMaxRadix / THREADS;    // rows per thread
+  static constexpr int kMinBlocks = 2;                // resident blocks per SM
+  static_assert(kSortTile % THREADS == 0 && kMaxRadix % THREADS == 0, "points and rows divide evenly");
+};
+constexpr int kScatterThreads = 1024;  // the one-frame path (the batch tuner may pick 256 or 512)
+// row counts (then write-out offsets), the tile's row starts, and the staged tile
+constexpr size_t kScatterSmem = sizeof(uint32_t) * (6 * size_t(kMaxRadix)) + sizeof(uint2) * size_t(kSortTile);
+
+template <int THREADS>
+__device__ __forceinline__ void bucket_scatter_body(const BucketArgs& a, int t) {
   using SS = ScatterShape<THREADS>;
-  constexpr int kScatterWarps = SS::kWarps, kScatterKpt = SS::kKpt, kPairWords = SS::kPairWords;
-  constexpr int kDigitsPerThread = SS::kDigitsPerThread;
-  extern __shared__ uint32_t smem[];
-  uint32_t* s_whist = smem;                             // [kPairWords][radix]: warps 2w, 2w+1 in the low, high half
-  uint32_t* s_keys = s_whist + kPairWords * kMaxRadix;  // [kSortTile]
-  uint32_t* s_vals = s_keys + kSortTile;                // [kSortTile]
-  uint32_t* s_tstart = s_vals + kSortTile;              // [radix]
-  uint32_t* s_gbase = s_tstart + kMaxRadix;             // [radix]
-  uint32_t* s_warp = s_gbase + kMaxRadix;               // [kScatterWarps]
-  uint32_t* s_count = s_warp + kScatterWarps;
-
+  constexpr int kKpt = SS::kKpt, kDpt = SS::kDpt, kWarps = THREADS / 32;
+  extern __shared__ __align__(16) uint32_t smem[];
+  uint32_t* s_cnt = smem;                                               // [3 coordinates][rows]
+  uint32_t* s_at = s_cnt + 3 * kMaxRadix;                               // [3 coordinates][rows]
+  uint2* s_pt = reinterpret_cast<uint2*>(s_at + 3 * kMaxRadix);         // [kSortTile]
+  __shared__ uint32_t s_w[6][kWarps];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int bits = a.bits, radix = 1 << bits;
+  const int b = a.bits, radix = 1 << b, n = a.n;
   const uint32_t m = uint32_t(radix) - 1u;
-  const int shift = a.shift;
-  const int warp_base = t * kSortTile + warp * (32 * kScatterKpt);
-  for (int i = tid; i < kPairWords * radix; i += THREADS) s_whist[i] = 0;
-  // this tile's global start of every digit, known before any key is ranked
-  for (int d = tid; d < radix; d += THREADS) s_gbase[d] = a.counts[size_t(d) * a.tiles + t];
+  const int base = t * a.tile, end = min(n, base + a.tile);
 
-  // the keys and values of this warp's 256 positions (striped, so loads coalesce)
-  uint32_t key[kScatterKpt], val[kScatterKpt], rnk[kScatterKpt];
+  uint32_t code[kKpt];
 #pragma unroll
-  for (int j = 0; j < kScatterKpt; ++j) {
-    const int pos = warp_base + j * 32 + lane;
-    key[j] = 0;
-    val[j] = 0;
-    if (pos < a.n) {
-      if (a.xyz) {
-        const uint32_t x = uint32_t(a.xyz[3 * size_t(pos)]) & m;
-        const uint32_t y = uint32_t(a.xyz[3 * size_t(pos) + 1]) & m;
-        const uint32_t z = uint32_t(a.xyz[3 * size_t(pos) + 2]) & m;
-        key[j] = code_of(0, x, y, z, bits);
-        val[j] = uint32_t(pos);
-      } else {
-        key[j] = a.keys_in[pos];
-        val[j] = a.vals_in ? a.vals_in[pos] : uint32_t(pos);
-      }
+  for (int j = 0; j < kKpt; ++j) {
+    const int i = base + j * THREADS + tid;
+    code[j] = 0u;
+    if (i < end) {
+      const uint32_t x = uint32_t(a.xyz[3 * size_t(i)]) & m;
+      const uint32_t y = uint32_t(a.xyz[3 * size_t(i) + 1]) & m;
+      const uint32_t z = uint32_t(a.xyz[3 * size_t(i) + 2]) & m;
+      code[j] = code_of(0, x, y, z, b);
+    }
+  }
+  // the rows' sizes; this thread owns the consecutive rows tid * kDpt ..
+  uint32_t size[3][kDpt], sum[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    sum[c] = 0u;
+#pragma unroll
+    for (int i = 0; i < kDpt; ++i) {
+      const int d = tid * kDpt + i;
+      size[c][i] = d < radix ? a.sc->chist[c][d] : 0u;
+      s_cnt[c * kMaxRadix + d] = 0u;
+      sum[c] += size[c][i];
     }
   }
   __syncthreads();
-
-  // stable rank of each key among equal digits of its warp, in input order:
-  // the lanes with the same digit are found with one ballot per digit bit; the
-  // lowest of them adds the group size to the warp's digit counter and the
-  // count it gets back is the group's base
-  uint32_t* wh = s_whist + (warp >> 1) * radix;
-  const int half = 16 * (warp & 1);
-  const uint32_t lt = (1u << lane) - 1u;
+  // rank of each point among the tile's points of its row, in any order
+  uint32_t rxy[kKpt], rz[kKpt];  // x row in the low, y row in the high half; z row
 #pragma unroll
-  for (int j = 0; j < kScatterKpt; ++j) {
-    const bool valid = (warp_base + j * 32 + lane) < a.n;
-    const uint32_t d = (key[j] >> shift) & m;
-    uint32_t peers = __ballot_sync(0xffffffffu, valid);
-    for (int b = 0; b < bits; ++b) {
-      const bool bit = (d >> b) & 1u;
-      const uint32_t on = __ballot_sync(0xffffffffu, bit);
-      peers &= bit ? on : ~on;
+  for (int j = 0; j < kKpt; ++j) {
+    rxy[j] = rz[j] = 0u;
+    if (base + j * THREADS + tid < end) {
+      const uint32_t rx = atomicAdd(&s_cnt[code[j] & m], 1u);
+      const uint32_t ry = atomicAdd(&s_cnt[kMaxRadix + ((code[j] >> b) & m)], 1u);
+      rz[j] = atomicAdd(&s_cnt[2 * kMaxRadix + (code[j] >> (2 * b))], 1u);
+      rxy[j] = rx | (ry << 16);
     }
-    const int leader = peers ? __ffs(peers) - 1 : lane;
-    uint32_t old = 0;
-    if (valid && lane == leader) old = (atomicAdd(&wh[d], uint32_t(__popc(peers)) << half) >> half) & 0xffffu;
-    rnk[j] = __shfl_sync(0xffffffffu, old, leader) + __popc(peers & lt);
-    __syncwarp();
+  }
+  // the rows' starts in the frame
+  uint32_t start[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const uint32_t x = warp_inclusive(sum[c], lane);
+    if (lane == 31) s_w[c][warp] = x;
+    start[c] = x - sum[c];
   }
   __syncthreads();
-
-  // per digit (each thread owns kDigitsPerThread consecutive digits): offsets
-  // of the warps, the tile total, and the tile's exclusive digit start
-  uint32_t tot[kDigitsPerThread];
-  uint32_t own = 0;
 #pragma unroll
-  for (int i = 0; i < kDigitsPerThread; ++i) {
-    const int d = tid * kDigitsPerThread + i;
-    uint32_t run = 0;
-    if (d < radix) {
+  for (int c = 0; c < 3; ++c) start[c] += warps_before(s_w[c], lane, warp);
+  if (t == 0) {
+    // for the sort: the rows' starts and the coordinates' extents
 #pragma unroll
-      for (int w = 0; w < kPairWords; ++w) {
-        const uint32_t c = s_whist[w * radix + d];
-        const uint32_t lo = c & 0xffffu, hi = c >> 16;
-        s_whist[w * radix + d] = run | ((run + lo) << 16);
-        run += lo + hi;
+    for (int c = 0; c < 3; ++c) {
+      uint32_t s = start[c], lo = m, hi = 0u;
+#pragma unroll
+      for (int i = 0; i < kDpt; ++i) {
+        const uint32_t d = uint32_t(tid * kDpt + i);
+        if (int(d) < radix) a.sc->row_start[c][d] = s;
+        s += size[c][i];
+        if (size[c][i]) {
+          lo = min(lo, d);
+          hi = max(hi, d);
+        }
+      }
+      if (tid == 0) a.sc->row_start[c][radix] = uint32_t(n);
+      lo = __reduce_min_sync(0xffffffffu, lo);
+      hi = __reduce_max_sync(0xffffffffu, hi);
+      if (lane == 0) {
+        // kept as maxima of (2^b - 1 - coordinate) and of the coordinate: zeroed with the build scalars
+        atomicMax(&a.sc->row_ext[c][0], m - lo);
+        atomicMax(&a.sc->row_ext[c][1], hi);
       }
     }
-    tot[i] = run;
-    own += run;
   }
-  {
-    uint32_t x = own;
+  // reserve this tile's share of its rows, and the rows' starts inside the tile
+  uint32_t cnt[3][kDpt], at[3][kDpt], own[3];
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
+  for (int c = 0; c < 3; ++c) {
+    own[c] = 0u;
+#pragma unroll
+    for (int i = 0; i < kDpt; ++i) {
+      const int d = tid * kDpt + i;
+      cnt[c][i] = s_cnt[c * kMaxRadix + d];
+      at[c][i] = start[c] + (cnt[c][i] ? atomicAdd(&a.sc->row_used[c][d], cnt[c][i]) : 0u);
+      start[c] += size[c][i];
+      own[c] += cnt[c][i];
     }
-    if (lane == 31) s_warp[warp] = x;
+    const uint32_t x = warp_inclusive(own[c], lane);
+    if (lane == 31) s_w[3 + c][warp] = x;
+    own[c] = x - own[c];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    uint32_t s = own[c] + warps_before(s_w[3 + c], lane, warp);
+#pragma unroll
+    for (int i = 0; i < kDpt; ++i) {
+      const int d = tid * kDpt + i;
+      s_at[c * kMaxRadix + d] = s;
+      s_cnt[c * kMaxRadix + d] = at[c][i] - s;  // + place in the tile = place in the frame
+      s += cnt[c][i];
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const int rc = row_coord(c);
+#pragma unroll
+    for (int j = 0; j < kKpt; ++j) {
+      const int i = base + j * THREADS + tid;
+      if (i < end) {
+        const uint32_t k = code_from_c1(c, code[j], b, m);
+        const uint32_t r = c == 0 ? rz[j] : c == 1 ? (rxy[j] & 0xffffu) : (rxy[j] >> 16);
+        s_pt[s_at[rc * kMaxRadix + (k >> (2 * b))] + r] = make_uint2(uint32_t(i), k);
+      }
+    }
     __syncthreads();
-    uint32_t off = 0;
+    uint2* out = a.row_pts[c];
 #pragma unroll
-    for (int w = 0; w < kScatterWarps; ++w) off += (w < warp) ? s_warp[w] : 0u;
-    uint32_t start = off + x - own;
-#pragma unroll
-    for (int i = 0; i < kDigitsPerThread; ++i) {
-      const int d = tid * kDigitsPerThread + i;
-      if (d < radix) s_tstart[d] = start;
-      start += tot[i];
-    }
-    if (tid == THREADS - 1) *s_count = start;
-  }
-  __syncthreads();
-
-  // local sort of the tile by digit, then write out in digit runs
-#pragma unroll
-  for (int j = 0; j < kScatterKpt; ++j) {
-    if ((warp_base + j * 32 + lane) < a.n) {
-      const uint32_t dj = (key[j] >> shift) & m;
-      const uint32_t lp = s_tstart[dj] + ((wh[dj] >> half) & 0xffffu) + rnk[j];
-      s_keys[lp] = key[j];
-      s_vals[lp] = val[j];
-      if (a.pos_out) {
-        const uint32_t g = s_gbase[dj] + (lp - s_tstart[dj]);
-        if (g < uint32_t(a.n)) a.pos_out[warp_base + j * 32 + lane] = int32_t(g);
+    for (int j = 0; j < kKpt; ++j) {
+      const int p = j * THREADS + tid;
+      if (p < end - base) {
+        const uint2 e = s_pt[p];
+        const uint32_t g = s_cnt[rc * kMaxRadix + (e.y >> (2 * b))] + uint32_t(p);
+        if (g < uint32_t(n)) out[g] = e;
       }
     }
-  }
-  __syncthreads();
-  const uint32_t cnt = *s_count;
-  uint32_t* ko = a.keys_out;
-  uint32_t* vo = a.vals_out;
-  int32_t* ro = a.rank_out;
-  for (uint32_t i = tid; i < cnt; i += THREADS) {
-    const uint32_t k = s_keys[i], v = s_vals[i];
-    const uint32_t dk = (k >> shift) & m;
-    const uint32_t g = s_gbase[dk] + (i - s_tstart[dk]);
-    if (g >= uint32_t(a.n) || v >= uint32_t(a.n)) continue;
-    if (ko) ko[g] = k;
-    if (vo) vo[g] = v;
-    if (ro) ro[v] = int32_t(g);
+    if (c < 2) __syncthreads();
   }
 }
 
 template <int THREADS>
-__global__ void __launch_bounds__(THREADS, ScatterShape<THREADS>::kMinBlocks) k_sort_scatter(SortPassArgs a) {
+__global__ void __launch_bounds__(THREADS, ScatterShape<THREADS>::kMinBlocks) k_bucket_scatter(BucketArgs a) {
   pdl_wait();
-  sort_scatter_body<THREADS>(a, blockIdx.x);
+  bucket_scatter_body<THREADS>(a, blockIdx.x);
 }
 
 template <int THREADS>
 __global__ void __launch_bounds__(THREADS, ScatterShape<THREADS>::kMinBlocks)
-    k_sort_scatter_seg(const __grid_constant__ Seg<SortPassArgs> s) {
+    k_bucket_scatter_seg(const __grid_constant__ Seg<BucketArgs> s) {
   pdl_wait();
   const int f = seg_frame(s, blockIdx.x);
-  sort_scatter_body<THREADS>(s.a[f], blockIdx.x - s.start[f]);
+  bucket_scatter_body<THREADS>(s.a[f], blockIdx.x - s.start[f]);
 }
 
-// ---------------------------------------------------------------- slab sort
-// One block per y-slab of the y-sorted (code, input index) pairs: sort the
-// slab by (x, z) with two stable passes (z, then x), which gives the C3
-// order.  A slab of up to kSlabMax points is held in shared memory and
-// ranked kSlabKpt rounds per warp; warp w owns the contiguous positions
-// [w C, (w + 1) C), so warp order is position order and the ballot ranks
-// inside a warp keep lane order.  A larger slab (a cloud with very many points
-// in one plane) takes the same ranking through global memory, kSlabThreads
-// points at a time, with running digit offsets carried from chunk to chunk.
-constexpr int kSlabThreads = 256;
-constexpr int kSlabWarps = kSlabThreads / 32;
-constexpr int kSlabKpt = 8;
-constexpr int kSlabMax = kSlabThreads * kSlabKpt;  // 4096 points
-constexpr int kSlabPairWords = kSlabWarps / 2;    // digit counter words (two warps each)
-constexpr int kSlabDigits = kMaxRadix / kSlabThreads;  // digits owned by each thread
-
-size_t slab_smem_bytes() {
-  return sizeof(uint32_t) * (size_t(kSlabPairWords) * kMaxRadix + 2 * size_t(kSlabMax) + kMaxRadix + kSlabWarps + 4);
-}
-
-// exclusive scan of one value per thread over the 1024-thread block
-__device__ __forceinline__ uint32_t slab_block_scan(uint32_t v, uint32_t* s_warp, uint32_t* total) {
-  static_assert(kSlabWarps <= 32, "one warp scans the warp totals");
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint32_t x = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) s_warp[warp] = x;
-  __syncthreads();
-  if (warp == 0) {
-    const uint32_t w = lane < kSlabWarps ? s_warp[lane] : 0u;
-    uint32_t wx = w;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, wx, o);
-      if (lane >= o) wx += y;
-    }
-    if (lane < kSlabWarps) s_warp[lane] = wx - w;
-    if (lane == 31 && total) *total = wx;
-  }
-  __syncthreads();
-  const uint32_t r = s_warp[warp] + x - v;
-  __syncthreads();
-  return r;
-}
+// ---------------------------------------------------------------- order inside the rows
+// One block per window of a.window output positions of a code.  It owns the
+// rows of up to kRowMax points that start in the window, and of a larger row
+// the lines (points of one second coordinate; their starts come from a
+// histogram of the row) that start in it, so every point has one owner and an
+// item holds at most window + kRowMax points unless one line repeats voxels
+// thousands of times.  The item's points go into kSortBuckets buckets by the
+// leading bits of their code (relative to the item's first row, and to the
+// second coordinate's extent), and inside a bucket each point's place is the
+// number of smaller (code, index) pairs.  Repeated voxels that overfill the item
+// or a bucket are ordered by a radix sort through global memory instead.
+// Measured (1M body points, b = 10): 38 us for the three codes, of which the
+// prologue 7, counting 6, placing 5, ranking and writing 17; it is bound by its
+// instructions (22 M a launch) and by the barriers between its phases.  With the
+// row scatter it replaced three global radix passes and a slab sort: the graph's
+// sorting launches took 112 us at 1M points and 54 us at 3k (12 launches), now 63
+// and 17 (3 launches).  One counter a scan line in global memory instead (random
+// atomics and writes in L2) took 110 us.  Windows of 1024 and 2048 positions were
+// slower at 1M points (67 and 41 against 37 us: more prologues, and large rows are
+// read by more blocks); splitting C1 from C2 and C3, to carry sorted ids, too (63).
+constexpr int kBucketThreads = 1024;
+constexpr int kRowMax = 7168;
+constexpr int kWindowMax = 4096;
+constexpr int kItemMax = kWindowMax + kRowMax;
+constexpr int kSortBucketBits = 13;
+constexpr int kSortBuckets = 1 << kSortBucketBits;  // 16-bit counters, two a word
+constexpr uint32_t kBucketMax = 512;                // larger buckets are not ranked by counting
+constexpr size_t kBucketSmem = sizeof(uint2) * (size_t(kItemMax) + 4) + sizeof(uint16_t) * size_t(kSortBuckets);
+static_assert(kSortBuckets == 8 * kBucketThreads && kMaxRadix <= kBucketThreads, "eight buckets, one row a thread");
+static_assert(kItemMax < 65536, "16-bit places inside an item");
 
 // Stable rank of one key among the equal digits of its warp (lanes in order),
 // added to the warp's digit counter (16-bit half `half` of the pair word).
@@ -475,274 +347,373 @@ __device__ __forceinline__ uint32_t warp_rank(bool valid, uint32_t d, int bits, 
   return __shfl_sync(0xffffffffu, old, leader) + __popc(peers & ((1u << lane) - 1u));
 }
 
-// For digit d (one per thread): the counters of the warps become their
-// exclusive offsets; returns the digit's total.
-__device__ __forceinline__ uint32_t digit_warp_offsets(uint32_t* cnt, int radix, int d) {
-  uint32_t run = 0;
-  if (d < radix) {
-#pragma unroll
-    for (int w = 0; w < kSlabPairWords; ++w) {
-      const uint32_t c = cnt[w * radix + d];
-      const uint32_t lo = c & 0xffffu, hi = c >> 16;
-      cnt[w * radix + d] = run | ((run + lo) << 16);
-      run += lo + hi;
-    }
-  }
-  return run;
+// A sorted point's outputs: code c, its place r, code k and input index idx.
+__device__ __forceinline__ void emit_sorted(const BucketArgs& a, int c, uint32_t r, uint32_t k, uint32_t idx) {
+  if (max(r, idx) >= uint32_t(a.n)) return;
+  a.keys_out[c][r] = k;
+  a.order_out[c][r] = int32_t(idx);
+  if (c < 2) a.rank12[2 * size_t(idx) + c] = int32_t(r);
 }
 
-__device__ __forceinline__ void slab_sort_body(const SlabArgs& sa, int yv) {
-  const int n = sa.n, bits = sa.bits;
-  const uint32_t* __restrict__ keys_in = sa.keys_in;
-  const uint32_t* __restrict__ vals_in = sa.vals_in;
-  uint32_t* __restrict__ keys_tmp = sa.keys_tmp;
-  uint32_t* __restrict__ vals_tmp = sa.vals_tmp;
-  uint32_t* __restrict__ keys_out = sa.keys_out;
-  int32_t* __restrict__ vals_out = sa.vals_out;
-  const DevScalars* __restrict__ sc = sa.sc;
-  extern __shared__ uint32_t smem[];
-  uint32_t* cnt = smem;                                   // [kSlabPairWords][radix]
-  uint32_t* s_keys = cnt + kSlabPairWords * kMaxRadix;    // [kSlabMax]
-  uint32_t* s_vals = s_keys + kSlabMax;                   // [kSlabMax]
-  uint32_t* s_start = s_vals + kSlabMax;                  // [radix]
-  uint32_t* s_warp = s_start + kMaxRadix;                 // [kSlabWarps]
-  uint32_t* s_misc = s_warp + kSlabWarps;                 // [4]
+// The places of an item's rows and the second coordinates [mid0, mid1) it owns in
+// them: its small rows (side by side, all of them), and up to two large ones.
+struct ItemRows {
+  uint32_t from[3], to[3], mid0[3], mid1[3];
+};
 
+// The points of an item that do not fit shared memory (repeated voxels), by a
+// least-significant-digit radix sort of (code, input index), kBucketThreads
+// points at a time, between the scratch half of the code's row array and the
+// output arrays (this item's `total` places from `out0`).
+__device__ __noinline__ void item_radix_sort(const BucketArgs& a, int c, uint32_t out0, uint32_t total, ItemRows rows,
+                                             uint32_t* smem) {
+  constexpr int kPairs = kBucketThreads / 64;
+  uint32_t* s_cnt = smem;                        // [kPairs][kMaxRadix]
+  uint32_t* s_run = s_cnt + kPairs * kMaxRadix;  // [kMaxRadix]
+  static_assert(sizeof(uint32_t) * (kPairs + 1) * kMaxRadix <= sizeof(uint2) * kItemMax, "the counters fit the item's points");
+  __shared__ uint32_t s_n, s_sw[32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int radix = 1 << bits;
-  const uint32_t m = uint32_t(radix) - 1u;
-  if (yv >= radix) return;
-  const uint32_t* hy = sc->chist[1];
-  const uint32_t size = hy[yv];
-  if (size == 0) return;
-  // the slab starts after every point of a smaller y
-  uint32_t below = 0;
-  for (int e = tid; e < yv; e += kSlabThreads) below += hy[e];
-  slab_block_scan(below, s_warp, &s_misc[0]);
-  const uint32_t start = s_misc[0];
-  if (uint64_t(start) + size > uint64_t(n)) return;  // inconsistent histogram: leave the slab alone
-  uint32_t* wh = cnt + (warp >> 1) * radix;
+  const int b = a.bits, n = a.n;
+  uint32_t* key[2] = {a.row_tmp[c] + out0, a.keys_out[c] + out0};
+  uint32_t* val[2] = {a.row_tmp[c] + size_t(a.tmp_stride) + out0, reinterpret_cast<uint32_t*>(a.order_out[c]) + out0};
+  if (tid == 0) s_n = 0u;
+  __syncthreads();
+  // the item's points: its small rows, and of its large rows the points on its lines
+  for (int g = 0; g < 3; ++g)
+    for (uint32_t i = rows.from[g] + tid; i < rows.to[g]; i += kBucketThreads) {
+      const uint2 e = a.row_pts[c][i];
+      const uint32_t mid = (e.y >> b) & ((1u << b) - 1u);
+      if (mid < rows.mid0[g] || mid >= rows.mid1[g]) continue;
+      const uint32_t p = atomicAdd(&s_n, 1u);
+      if (p < total) {
+        key[0][p] = e.y;
+        val[0][p] = e.x;
+      }
+    }
+  __syncthreads();
+  int cur = 0;
+  const int idx_bits = max(1, 32 - __clz(n - 1));
+  const int idx_passes = (idx_bits + 9) / 10;
+  uint32_t* wh = s_cnt + (warp >> 1) * kMaxRadix;
   const int half = 16 * (warp & 1);
-
-  if (size <= uint32_t(kSlabMax)) {
-    // the slab's z and x extents: each pass ranks the coordinate minus its
-    // smallest value in the slab, with as many digit bits as the extent needs
-    // (the order is the same; the digit counters and ballots are fewer)
-    __shared__ uint32_t s_ext[4][kSlabWarps];
-    uint32_t zlo = m, zhi = 0, xlo = m, xhi = 0;
-    for (uint32_t i = tid; i < size; i += kSlabThreads) {
-      const uint32_t key = keys_in[start + i];
-      s_keys[i] = key;
-      s_vals[i] = vals_in[start + i];
-      const uint32_t z = (key >> (2 * bits)) & m, x = key & m;
-      zlo = min(zlo, z);
-      zhi = max(zhi, z);
-      xlo = min(xlo, x);
-      xhi = max(xhi, x);
-    }
-    zlo = __reduce_min_sync(0xffffffffu, zlo);
-    zhi = __reduce_max_sync(0xffffffffu, zhi);
-    xlo = __reduce_min_sync(0xffffffffu, xlo);
-    xhi = __reduce_max_sync(0xffffffffu, xhi);
-    if (lane == 0) {
-      s_ext[0][warp] = zlo;
-      s_ext[1][warp] = zhi;
-      s_ext[2][warp] = xlo;
-      s_ext[3][warp] = xhi;
-    }
+  for (int pass = 0; pass < idx_passes + 3; ++pass) {
+    const bool by_idx = pass < idx_passes;
+    const int shift = by_idx ? 10 * pass : b * (pass - idx_passes);
+    const int dbits = by_idx ? 10 : b;
+    const uint32_t dm = (1u << dbits) - 1u;
+    const uint32_t *ks = key[cur], *vs = val[cur];
+    uint32_t *kd = key[cur ^ 1], *vd = val[cur ^ 1];
+    // every digit's first place
+    s_run[tid] = 0u;
     __syncthreads();
-#pragma unroll
-    for (int w = 0; w < kSlabWarps; ++w) {
-      zlo = min(zlo, s_ext[0][w]);
-      zhi = max(zhi, s_ext[1][w]);
-      xlo = min(xlo, s_ext[2][w]);
-      xhi = max(xhi, s_ext[3][w]);
-    }
-    const int chunk = int((size + 32 * kSlabWarps - 1) / (32 * kSlabWarps)) * 32;  // positions per warp
-    const int rounds = chunk / 32;                                                 // <= kSlabKpt
-    for (int pass = 0; pass < 2; ++pass) {
-      const int shift = pass == 0 ? 2 * bits : 0;  // z, then x
-      const uint32_t lo = pass == 0 ? zlo : xlo, ext = (pass == 0 ? zhi : xhi) - lo;
-      const int dbits = max(1, 32 - __clz(int(ext)));  // digit bits of this pass (<= bits)
-      const int pradix = 1 << dbits;
-      uint32_t* pw = cnt + (warp >> 1) * pradix;       // this warp pair's counters
-      for (int i = tid; i < kSlabPairWords * pradix; i += kSlabThreads) cnt[i] = 0;
-      __syncthreads();
-      uint32_t k[kSlabKpt], v[kSlabKpt], rk[kSlabKpt];
-#pragma unroll
-      for (int j = 0; j < kSlabKpt; ++j) {
-        k[j] = v[j] = rk[j] = 0;
-        if (j < rounds) {
-          const uint32_t pos = uint32_t(warp * chunk + j * 32 + lane);
-          const bool valid = pos < size;
-          if (valid) {
-            k[j] = s_keys[pos];
-            v[j] = s_vals[pos];
-          }
-          rk[j] = warp_rank(valid, ((k[j] >> shift) & m) - lo, dbits, pw, half, lane);
-          __syncwarp();
-        }
-      }
-      __syncthreads();
-      // each thread owns kSlabDigits consecutive digits
-      uint32_t tot[kSlabDigits], own = 0;
-#pragma unroll
-      for (int i = 0; i < kSlabDigits; ++i) {
-        tot[i] = digit_warp_offsets(cnt, pradix, kSlabDigits * tid + i);
-        own += tot[i];
-      }
-      uint32_t ts = slab_block_scan(own, s_warp, nullptr);
-#pragma unroll
-      for (int i = 0; i < kSlabDigits; ++i) {
-        if (kSlabDigits * tid + i < pradix) s_start[kSlabDigits * tid + i] = ts;
-        ts += tot[i];
-      }
-      __syncthreads();
-#pragma unroll
-      for (int j = 0; j < kSlabKpt; ++j) {
-        if (j < rounds) {
-          const uint32_t pos = uint32_t(warp * chunk + j * 32 + lane);
-          if (pos < size) {
-            const uint32_t d = ((k[j] >> shift) & m) - lo;
-            const uint32_t lp = s_start[d] + ((pw[d] >> half) & 0xffffu) + rk[j];
-            if (lp < size) {
-              s_keys[lp] = k[j];
-              s_vals[lp] = v[j];
-            }
-          }
-        }
-      }
-      __syncthreads();
-    }
-    for (uint32_t i = tid; i < size; i += kSlabThreads) {
-      keys_out[start + i] = s_keys[i];
-      vals_out[start + i] = int32_t(s_vals[i]);
-    }
-    if (sa.counts1) {
-      // sort pass 1's tile counts (z digits of the C3 order): the slab's at
-      // most kSlabMax positions lie in the 4096-key tiles t0 and t0 + 1, counted
-      // in the digit counters (free after the last pass), then added to the totals
-      const uint32_t t0 = start / kSortTile;
-      const int tiles = (n + kSortTile - 1) / kSortTile;
-      static_assert(kSlabMax <= kSortTile && 2 * kMaxRadix <= kSlabPairWords * kMaxRadix,
-                    "a slab spans at most two tiles, counted in the digit counter words");
-      // (z digits zlo .. zhi only)
-      const int zr = int(zhi - zlo) + 1;
-      for (int i = tid; i < 2 * zr; i += kSlabThreads) cnt[i] = 0;
-      __syncthreads();
-      for (uint32_t i = tid; i < size; i += kSlabThreads)
-        atomicAdd(&cnt[((start + i) / kSortTile - t0) * zr + (((s_keys[i] >> (2 * bits)) & m) - zlo)], 1u);
-      __syncthreads();
-      for (int i = tid; i < 2 * zr; i += kSlabThreads) {
-        const uint32_t c = cnt[i], t = t0 + uint32_t(i / zr);
-        if (c && t < uint32_t(tiles)) atomicAdd(&sa.counts1[size_t(zlo + uint32_t(i % zr)) * tiles + t], c);
-      }
-    }
-    return;
-  }
-
-  // ---- a slab larger than shared memory: the same passes, 1024 points at a
-  // time, through global memory (pass 0 into the scratch arrays, pass 1 into
-  // the final arrays)
-  for (int pass = 0; pass < 2; ++pass) {
-    const int shift = pass == 0 ? 2 * bits : 0;  // z, then x
-    const uint32_t* ks = pass == 0 ? keys_in : keys_tmp;
-    const uint32_t* vs = pass == 0 ? vals_in : vals_tmp;
-    // digit histogram of the slab, then each digit's first position
-    for (int d = tid; d < radix; d += kSlabThreads) s_start[d] = 0;
+    for (uint32_t i = tid; i < total; i += kBucketThreads)
+      atomicAdd(&s_run[((by_idx ? __ldcg(vs + i) : __ldcg(ks + i)) >> shift) & dm], 1u);
     __syncthreads();
-    for (uint32_t i = tid; i < size; i += kSlabThreads) atomicAdd(&s_start[(ks[start + i] >> shift) & m], 1u);
+    uint32_t run = s_run[tid];
+    run = block_exclusive(run, s_sw);
     __syncthreads();
-    // thread t: the next free positions of its kSlabDigits digits
-    uint32_t run[kSlabDigits], own = 0;
-#pragma unroll
-    for (int i = 0; i < kSlabDigits; ++i) {
-      run[i] = kSlabDigits * tid + i < radix ? s_start[kSlabDigits * tid + i] : 0u;
-      own += run[i];
-    }
-    {
-      uint32_t r0 = slab_block_scan(own, s_warp, nullptr);
-#pragma unroll
-      for (int i = 0; i < kSlabDigits; ++i) {
-        const uint32_t h = run[i];
-        run[i] = r0;
-        r0 += h;
-      }
-    }
-    for (uint32_t c0 = 0; c0 < size; c0 += kSlabThreads) {
-      for (int i = tid; i < kSlabPairWords * radix; i += kSlabThreads) cnt[i] = 0;
-#pragma unroll
-      for (int i = 0; i < kSlabDigits; ++i)
-        if (kSlabDigits * tid + i < radix) s_start[kSlabDigits * tid + i] = run[i];
+    s_run[tid] = run;
+    for (uint32_t c0 = 0; c0 < total; c0 += kBucketThreads) {
+      for (int i = tid; i < kPairs * kMaxRadix; i += kBucketThreads) s_cnt[i] = 0u;
       __syncthreads();
       const uint32_t pos = c0 + uint32_t(tid);
-      const bool valid = pos < size;
-      const uint32_t key = valid ? ks[start + pos] : 0u, val = valid ? vs[start + pos] : 0u;
-      const uint32_t d = (key >> shift) & m;
-      const uint32_t rk = warp_rank(valid, d, bits, wh, half, lane);
+      const bool valid = pos < total;
+      const uint32_t k = valid ? __ldcg(ks + pos) : 0u, v = valid ? __ldcg(vs + pos) : 0u;
+      const uint32_t d = ((by_idx ? v : k) >> shift) & dm;
+      const uint32_t rk = warp_rank(valid, d, dbits, wh, half, lane);
       __syncthreads();
-      uint32_t tot[kSlabDigits];
+      // thread d: the warps' offsets of digit d, and the digit's points in this chunk
+      uint32_t w0 = 0u;
 #pragma unroll
-      for (int i = 0; i < kSlabDigits; ++i) tot[i] = digit_warp_offsets(cnt, radix, kSlabDigits * tid + i);
+      for (int w = 0; w < kPairs; ++w) {
+        const uint32_t q = s_cnt[w * kMaxRadix + tid];
+        s_cnt[w * kMaxRadix + tid] = w0 | ((w0 + (q & 0xffffu)) << 16);
+        w0 += (q & 0xffffu) + (q >> 16);
+      }
       __syncthreads();
       if (valid) {
-        const uint32_t lp = s_start[d] + ((wh[d] >> half) & 0xffffu) + rk;
-        if (lp < size) {
-          const uint32_t g = start + lp;
-          if (pass == 0) {
-            keys_tmp[g] = key;
-            vals_tmp[g] = val;
-          } else {
-            keys_out[g] = key;
-            vals_out[g] = int32_t(val);
-            if (sa.counts1)  // sort pass 1's tile counts, one key at a time here
-              atomicAdd(&sa.counts1[size_t((key >> (2 * bits)) & m) * ((n + kSortTile - 1) / kSortTile) +
-                                    g / kSortTile],
-                        1u);
-          }
+        const uint32_t p = s_run[d] + ((wh[d] >> half) & 0xffffu) + rk;
+        if (p < total) {
+          kd[p] = k;
+          vd[p] = v;
         }
       }
-#pragma unroll
-      for (int i = 0; i < kSlabDigits; ++i) run[i] += tot[i];
       __syncthreads();
+      s_run[tid] += w0;
     }
     __syncthreads();
+    cur ^= 1;
+  }
+  for (uint32_t i = tid; i < total; i += kBucketThreads)
+    emit_sorted(a, c, out0 + i, __ldcg(key[cur] + i), __ldcg(val[cur] + i));
+}
+
+// A code's bucket: the leading bits of the code with the unused high bits of
+// the second coordinate taken out (`base`: the first row and the smallest second
+// coordinate; `gap` = 2^2b - 2^(b + bits of the second coordinate's extent)).
+struct BucketOf {
+  uint32_t base, gap;
+  int row_shift, shift;
+  __device__ __forceinline__ uint32_t operator()(uint32_t k) const {
+    const uint32_t d = k - base;
+    return min((d - (d >> row_shift) * gap) >> shift, uint32_t(kSortBuckets - 1));
+  }
+};
+
+__device__ __forceinline__ void bucket_sort_body(const BucketArgs& a, int item, int c) {
+  extern __shared__ __align__(16) uint32_t smem[];
+  // (code in the high, index in the low half; four entries of padding for the ranking loads)
+  unsigned long long* s_pt = reinterpret_cast<unsigned long long*>(smem);     // [kItemMax + 4]
+  uint32_t* s_cnt = reinterpret_cast<uint32_t*>(s_pt + kItemMax + 4);         // [kSortBuckets / 2]
+  const uint16_t* s_end = reinterpret_cast<const uint16_t*>(s_cnt);           // bucket k's counter
+  __shared__ uint32_t s_w[3][32];
+  __shared__ uint32_t s_lo, s_hi, s_row0, s_row1;  // the small rows' places, the first and the last row
+  __shared__ uint32_t s_big[2];                    // 1 + the large row that starts before / in the window
+  __shared__ uint32_t s_mid0, s_mid1;              // a large row's own lines [mid0, mid1)
+  __shared__ uint32_t s_first, s_last;             // and the places they take, of both rows
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int b = a.bits, radix = 1 << b, n = a.n;
+  const uint32_t m = uint32_t(radix) - 1u;
+  const DevScalars* sc = a.sc;
+  const uint2* pts = a.row_pts[c];
+  const uint32_t* start = sc->row_start[row_coord(c)];
+  const uint32_t w0 = uint32_t(item) * uint32_t(a.window), w1 = w0 + uint32_t(a.window);
+  const uint32_t rs = tid < radix ? start[tid] : 0u, re = tid < radix ? min(start[tid + 1], uint32_t(n)) : 0u;
+  const int mc = mid_coord(c);
+  const uint32_t mid0 = m - sc->row_ext[mc][0], mid1 = sc->row_ext[mc][1];
+  reinterpret_cast<uint4*>(s_cnt)[tid] = make_uint4(0u, 0u, 0u, 0u);
+  if (tid == 0) {
+    s_lo = s_row0 = s_first = 0xffffffffu;
+    s_hi = s_row1 = s_big[0] = s_big[1] = s_last = 0u;
+  }
+  __syncthreads();
+  {
+    uint32_t lo = 0xffffffffu, hi = 0u, row = 0xffffffffu;
+    if (re > rs) {
+      if (re - rs <= uint32_t(kRowMax)) {
+        if (rs >= w0 && rs < w1) {
+          lo = rs;
+          hi = re;
+          row = uint32_t(tid);
+        }
+      } else if (rs < w1 && re > w0) {
+        s_big[rs < w0 ? 0 : 1] = uint32_t(tid) + 1u;
+        row = uint32_t(tid);
+      }
+    }
+    if (__any_sync(0xffffffffu, row != 0xffffffffu)) {
+      lo = __reduce_min_sync(0xffffffffu, lo);
+      hi = __reduce_max_sync(0xffffffffu, hi);
+      const uint32_t r0 = __reduce_min_sync(0xffffffffu, row);
+      const uint32_t r1 = __reduce_max_sync(0xffffffffu, row == 0xffffffffu ? 0u : row);
+      if (lane == 0) {
+        atomicMin(&s_lo, lo);
+        atomicMax(&s_hi, hi);
+        atomicMin(&s_row0, r0);
+        atomicMax(&s_row1, r1);
+      }
+    }
+  }
+  __syncthreads();
+  // the small rows lie side by side: [lo, lo + cnt_small), lo = 0 if there are none
+  const uint32_t lo = s_hi ? s_lo : 0u, cnt_small = s_hi - lo;
+  const uint32_t big[2] = {s_big[0], s_big[1]};
+  if (!cnt_small && !big[0] && !big[1]) return;
+  const int mid_bits = 32 - __clz(int(mid1 - mid0));
+  BucketOf bucket;
+  bucket.base = (s_row0 << (2 * b)) + (mid0 << b);
+  bucket.gap = (1u << (2 * b)) - (1u << (b + mid_bits));
+  bucket.row_shift = 2 * b;
+  // the smallest shift that leaves at most kSortBuckets buckets
+  bucket.shift = max(0, (32 - __clz(int(s_row1 - s_row0))) + mid_bits + b - kSortBucketBits);
+  uint32_t out0 = cnt_small ? lo : 0xffffffffu, out1 = s_hi;  // the item's places [out0, out1)
+  uint32_t b0[2] = {0u, 0u}, b1[2] = {0u, 0u}, l0[2] = {0u, 0u}, l1[2] = {0u, 0u};  // large rows: places, own lines
+  if (big[0] | big[1]) {
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
+      if (!big[g]) continue;
+      b0[g] = start[big[g] - 1u];
+      b1[g] = min(start[big[g]], uint32_t(n));
+      // the row's line histogram, and the lines that start in the window
+#pragma unroll 4
+      for (uint32_t i = b0[g] + tid; i < b1[g]; i += kBucketThreads) atomicAdd(&s_cnt[(pts[i].y >> b) & m], 1u);
+      if (tid == 0) {
+        s_mid0 = 0xffffffffu;
+        s_mid1 = 0u;
+      }
+      __syncthreads();
+      const uint32_t v = s_cnt[tid];
+      const uint32_t at = b0[g] + block_exclusive(v, s_w[g]);
+      s_cnt[tid] = 0u;
+      const bool own = v && at >= w0 && at < w1;
+      const uint32_t lo_w = __reduce_min_sync(0xffffffffu, own ? uint32_t(tid) : 0xffffffffu);
+      const uint32_t hi_w = __reduce_max_sync(0xffffffffu, own ? uint32_t(tid) + 1u : 0u);
+      if (lane == 0 && hi_w) {
+        atomicMin(&s_mid0, lo_w);
+        atomicMax(&s_mid1, hi_w);
+      }
+      if (own) {
+        atomicMin(&s_first, at);
+        atomicMax(&s_last, at + v);
+      }
+      __syncthreads();
+      l0[g] = s_mid0;
+      l1[g] = s_mid1;
+      __syncthreads();
+    }
+    out0 = min(out0, s_first);
+    out1 = max(out1, s_last);
+    if (out0 >= out1) return;  // one long line crosses the window
+  }
+  const uint32_t total = out1 - out0;
+  const auto owned = [&](int g, uint32_t k) {
+    const uint32_t mid = (k >> b) & m;
+    return mid >= l0[g] && mid < l1[g];
+  };
+  // (by value: nothing of the loops below is kept in memory for the rare radix sort)
+#define FGBD_ITEM_RADIX_SORT()                                                                                  \
+  item_radix_sort(a, c, out0, min(total, uint32_t(n) - min(out0, uint32_t(n))),                                 \
+                  ItemRows{{lo, b0[0], b0[1]},                                                                  \
+                           {lo + cnt_small, l1[0] ? b1[0] : 0u, l1[1] ? b1[1] : 0u},                            \
+                           {0u, l0[0], l0[1]},                                                                  \
+                           {1u << b, l1[0], l1[1]}},                                                            \
+                  smem)
+  if (total > uint32_t(kItemMax)) {
+    FGBD_ITEM_RADIX_SORT();
+    return;
+  }
+  // adds one to a bucket's counter; its value before
+  const auto count = [&](uint32_t k) {
+    const uint32_t bk = bucket(k), half = (bk & 1u) << 4;
+    return (atomicAdd(&s_cnt[bk >> 1], 1u << half) >> half) & 0xffffu;
+  };
+#pragma unroll 4
+  for (uint32_t i = lo + tid; i < lo + cnt_small; i += kBucketThreads) count(pts[i].y);
+#pragma unroll
+  for (int g = 0; g < 2; ++g)
+    if (l1[g])
+#pragma unroll 4
+      for (uint32_t i = b0[g] + tid; i < b1[g]; i += kBucketThreads) {
+        const uint32_t k = pts[i].y;
+        if (owned(g, k)) count(k);
+      }
+  __syncthreads();
+  // the buckets' starts
+  uint32_t v[4] = {s_cnt[4 * tid], s_cnt[4 * tid + 1], s_cnt[4 * tid + 2], s_cnt[4 * tid + 3]};
+  uint32_t sum = 0u, most = 0u;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    sum += (v[i] & 0xffffu) + (v[i] >> 16);
+    most = max(most, max(v[i] & 0xffffu, v[i] >> 16));
+  }
+  uint32_t q = block_exclusive(sum, s_w[2]);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint32_t w = v[i];
+    v[i] = q + ((q + (w & 0xffffu)) << 16);
+    q += (w & 0xffffu) + (w >> 16);
+  }
+  reinterpret_cast<uint4*>(s_cnt)[tid] = make_uint4(v[0], v[1], v[2], v[3]);
+  if (__syncthreads_or(most > kBucketMax)) {
+    FGBD_ITEM_RADIX_SORT();
+    return;
+  }
+#undef FGBD_ITEM_RADIX_SORT
+  const auto put = [&](uint2 e) {
+    const uint32_t p = count(e.y);
+    if (p < uint32_t(kItemMax)) s_pt[p] = ((unsigned long long)e.y << 32) | e.x;
+  };
+#pragma unroll 4
+  for (uint32_t i = lo + tid; i < lo + cnt_small; i += kBucketThreads) put(pts[i]);
+#pragma unroll
+  for (int g = 0; g < 2; ++g)
+    if (l1[g])
+#pragma unroll 4
+      for (uint32_t i = b0[g] + tid; i < b1[g]; i += kBucketThreads) {
+        const uint2 e = pts[i];
+        if (owned(g, e.y)) put(e);
+      }
+  if (tid < 4) s_pt[total + tid] = ~0ull;
+  __syncthreads();
+  // counter k is now the end of bucket k.  The points before a bucket are
+  // smaller and those behind it larger, so the counting may start at a
+  // multiple of four and run past the end: four points a step, no tail.
+  for (uint32_t p = tid; p < total; p += kBucketThreads) {
+    const unsigned long long me = s_pt[p];
+    const uint32_t k = uint32_t(me >> 32), bk = bucket(k);
+    const uint32_t first = (bk ? uint32_t(s_end[bk - 1]) : 0u) & ~3u, last = min(uint32_t(s_end[bk]), total);
+    uint32_t r = out0 + first;
+#pragma unroll 1
+    for (uint32_t j = first; j < last; j += 4) {
+      const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(s_pt + j);
+      const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(s_pt + j + 2);
+      r += (u.x < me) + (u.y < me) + (w.x < me) + (w.y < me);
+    }
+    emit_sorted(a, c, r, k, uint32_t(me));
   }
 }
 
-__global__ void __launch_bounds__(kSlabThreads, 4) k_slab_sort(SlabArgs a) {
+__global__ void __launch_bounds__(kBucketThreads, 2) k_bucket_sort(BucketArgs a) {
   pdl_wait();
-  slab_sort_body(a, blockIdx.x);
+  bucket_sort_body(a, blockIdx.x, blockIdx.y);
 }
 
-__global__ void __launch_bounds__(kSlabThreads, 4) k_slab_sort_seg(const __grid_constant__ Seg<SlabArgs> s) {
+// segmented: frame f's blocks are runs of equal length, one per code
+__global__ void __launch_bounds__(kBucketThreads, 2) k_bucket_sort_seg(const __grid_constant__ Seg<BucketArgs> s) {
   pdl_wait();
   const int f = seg_frame(s, blockIdx.x);
-  slab_sort_body(s.a[f], blockIdx.x - s.start[f]);
+  const int local = blockIdx.x - s.start[f], items = (s.start[f + 1] - s.start[f]) / 3;
+  bucket_sort_body(s.a[f], local % items, local / items);
 }
 
 // One code's order per group of gx blocks (block x of code c).  Code 0 is the C1 order
-// itself; codes 1 and 2 read the sorted ids along C2 and C3 and the packed C1
-// codes in the same order (keys of the C2 pass; keys of the slab sort for C3),
-// so only the C2 rank of a C3 point is a gather.  Each lane takes four
-// consecutive positions (16-byte loads, the C2 rank gathers issued together);
-// the neighbours across lanes come from shuffles, with one extra lookup at
-// each end of the warp.
+// itself; codes 1 and 2 read the input indices along C2 and C3 and the codes in
+// the same order (code c's own packing; a distance does not depend on it) and
+// gather each point's sorted id and, beside it, its C2 rank by input index (one
+// array of pairs: 27.8 us at 1M points, 29.4 with two arrays).  The two million
+// random reads and the slot writes bound it (6.8 M L2 sectors).  Each lane takes four consecutive positions
+// (16-byte loads, the gathers issued together); the neighbours across lanes
+// come from shuffles, with one extra lookup at each end of the warp.  With
+// colours (a whole run), the blocks of code 0, which have no slots to write, also
+// take the colours into the C1 order (colors_quad): 29.8 us with them, against
+// 9.7 us for a launch of its own.
 struct LinkPt {
   int k;       // sorted (C1) id, -1 outside [0, n)
   int r2;      // position in the C2 order (code 2 only)
-  uint32_t c;  // packed C1 code
+  uint32_t c;  // packed code of the order
 };
 
-__device__ __forceinline__ LinkPt link_point(int r, int n, int code, const int32_t* __restrict__ ord,
-                                             const uint32_t* keys, const int32_t* __restrict__ rank2) {
+// the sorted id (x) and the C2 rank (y, code 2 only) of the point at position r of
+// a code; x = -1 outside the frame
+__device__ __forceinline__ int2 link_id(int r, int n, int code, const int32_t* __restrict__ ord,
+                                        const int2* __restrict__ rank12) {
+  if (code == 0) return make_int2(r, -1);
+  const int i = ord[r];
+  if (!in_range(i, n)) return make_int2(-1, -1);
+  int2 q = make_int2(-1, -1);
+  if (code == 1) q.x = rank12[i].x;
+  else q = rank12[i];
+  if (!in_range(q.x, n)) q.x = -1;
+  return q;
+}
+
+// a packed code of order c as a C1 code
+__device__ __forceinline__ uint32_t c1_from_code(int c, uint32_t k, int b) {
+  const uint32_t m = (1u << b) - 1u;
+  const uint32_t hi = (k >> (2 * b)) & m, mid = (k >> b) & m, lo = k & m;
+  return c == 0 ? k : c == 1 ? code_of(0, hi, lo, mid, b) : code_of(0, mid, hi, lo, b);
+}
+
+template <bool SAME_LINE>
+__device__ __forceinline__ LinkPt link_point(int r, int n, int bits, int code, const int32_t* __restrict__ ord,
+                                             const uint32_t* keys, const int2* __restrict__ rank12) {
   LinkPt q{-1, -1, 0u};
   if (r < 0 || r >= n) return q;
-  const int k = code == 0 ? r : ord[r];
-  if (!in_range(k, n)) return q;
-  q.k = k;
-  q.c = keys[r];
-  if (code == 2) q.r2 = rank2[k];
+  const int2 id = link_id(r, n, code, ord, rank12);
+  if (id.x < 0) return q;
+  q.k = id.x;
+  q.r2 = id.y;
+  q.c = SAME_LINE ? c1_from_code(code, keys[r], bits) : keys[r];
   return q;
 }
 
@@ -775,7 +746,7 @@ __device__ __forceinline__ void link_body(const LinkArgs& la, int bx, int gx, in
   const int32_t* __restrict__ ord23 = la.ord23;
   const uint32_t* __restrict__ keys_c2 = la.keys_c2;
   const uint32_t* __restrict__ keys_c3 = la.keys_c3;
-  const int32_t* __restrict__ rank2 = la.rank2;
+  const int2* __restrict__ rank12 = la.rank12;
   const uint32_t* __restrict__ pk = la.pk;
   int4* __restrict__ c4 = la.c4;
   DevScalars* __restrict__ sc = la.sc;
@@ -821,17 +792,29 @@ __device__ __forceinline__ void link_body(const LinkArgs& la, int bx, int gx, in
         }
       }
     }
+    if (code == 0 && la.colors.rgb && r0 < n) colors_quad(la.colors, r0, n);
     LinkPt p[kLinkPerLane];
 #pragma unroll
     for (int i = 0; i < kLinkPerLane; ++i) {
-      p[i].k = in_range(kk[i], n) ? kk[i] : -1;
-      p[i].c = cc[i];
-      p[i].r2 = (code == 2 && p[i].k >= 0) ? rank2[p[i].k] : -1;
+      // (code 0: the position is the sorted id; else kk holds the input index)
+      const bool in = in_range(kk[i], n);
+      p[i].k = kk[i];
+      p[i].r2 = -1;
+      if (code == 1) p[i].k = in ? rank12[kk[i]].x : -1;
+      if (code == 2) {
+        const int2 q = in ? rank12[kk[i]] : make_int2(-1, -1);
+        p[i].k = q.x;
+        p[i].r2 = q.y;
+      }
+      p[i].c = SAME_LINE ? c1_from_code(code, cc[i], bits) : cc[i];
     }
+#pragma unroll
+    for (int i = 0; i < kLinkPerLane; ++i)
+      if (!in_range(p[i].k, n)) p[i].k = -1;
     LinkPt before = shfl_pt(p[kLinkPerLane - 1], 1, true);
     LinkPt after = shfl_pt(p[0], 1, false);
-    if (lane == 0) before = link_point(r0 - 1, n, code, ord, keys, rank2);
-    if (lane == 31) after = link_point(r0 + kLinkPerLane, n, code, ord, keys, rank2);
+    if (lane == 0) before = link_point<SAME_LINE>(r0 - 1, n, bits, code, ord, keys, rank12);
+    if (lane == 31) after = link_point<SAME_LINE>(r0 + kLinkPerLane, n, bits, code, ord, keys, rank12);
 #pragma unroll
     for (int i = 0; i < kLinkPerLane; ++i) {
       const LinkPt me = p[i];
@@ -921,11 +904,12 @@ __global__ void __launch_bounds__(256) k_c1_line_flags_seg(const __grid_constant
 // is a function of the pair and the code, so both ends reach the same one.
 // Each undirected edge is counted (and its length summed) once, from the
 // earlier position.
-__global__ void __launch_bounds__(256) k_link_wide(int n, int bits, int cap, int window, int same_line,
+__global__ void __launch_bounds__(256) k_link_wide(ColorArgs colors, int n, int bits, int cap, int window,
+                                                  int same_line,
                                                   const int32_t* __restrict__ ord23,
                                                   const uint32_t* __restrict__ keys_c2,
                                                   const uint32_t* __restrict__ keys_c3,
-                                                  const int32_t* __restrict__ rank2, const uint32_t* __restrict__ pk,
+                                                  const int2* __restrict__ rank12, const uint32_t* __restrict__ pk,
                                                   int4* __restrict__ c4, int32_t* __restrict__ cx, int cx_stride,
                                                   DevScalars* __restrict__ sc) {
   pdl_wait();
@@ -937,10 +921,12 @@ __global__ void __launch_bounds__(256) k_link_wide(int n, int bits, int cap, int
   unsigned long long edges = 0;
   float dist_f = 0.f;
   for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
-    const int k = code == 0 ? r : ord[r];
-    if (!in_range(k, n)) continue;
-    const uint32_t c = keys[r] & kCoordMask;
-    const int r2 = code == 2 ? rank2[k] : -1;
+    const int2 id = link_id(r, n, code, ord, rank12);
+    const int k = id.x;
+    if (k < 0) continue;
+    if (code == 0 && colors.rgb && (r & 3) == 0) colors_quad(colors, r, n);  // (points r .. r + 3)
+    const uint32_t c = c1_from_code(code, keys[r] & kCoordMask, bits);
+    const int r2 = id.y;
     for (int d = 1; d <= window; ++d) {
       int slot[2];
 #pragma unroll
@@ -948,14 +934,15 @@ __global__ void __launch_bounds__(256) k_link_wide(int n, int bits, int cap, int
         slot[side] = -1;
         const int rr = side ? r + d : r - d;
         if (rr < 0 || rr >= n) continue;
-        const int o = code == 0 ? rr : ord[rr];
-        if (!in_range(o, n)) continue;
-        const uint32_t oc = keys[rr] & kCoordMask;
+        const int2 oid = link_id(rr, n, code, ord, rank12);
+        const int o = oid.x;
+        if (o < 0) continue;
+        const uint32_t oc = c1_from_code(code, keys[rr] & kCoordMask, bits);
         if (sl && !same_scan_line(code, c, oc, bits)) continue;
         bool dup = false;
         if (code >= 1) dup = abs(k - o) <= window && (!sl || same_scan_line(0, c, oc, bits));
         if (code == 2 && !dup) {
-          const int o2 = rank2[o];
+          const int o2 = oid.y;
           dup = abs(r2 - o2) <= window && (!sl || same_scan_line(1, c, oc, bits));
         }
         if (dup) continue;
@@ -1018,17 +1005,15 @@ __global__ void __launch_bounds__(256) k_node_sigma(int n, int bits, GraphBufs g
   }
 }
 
-// The three orders in input indices: C1 from perm1, C2 and C3 through perm1.
+// The three orders in input indices.
 __global__ void __launch_bounds__(256) k_orders_export(int n, int cap, const int32_t* __restrict__ perm1,
                                                        const int32_t* __restrict__ ord23, int32_t* __restrict__ out) {
   pdl_wait();
   const int stride = gridDim.x * blockDim.x;
   for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += stride) {
     out[r] = perm1[r];
-    const int k = ord23[r];
-    out[size_t(n) + r] = in_range(k, n) ? perm1[k] : -1;
-    const int k3 = ord23[size_t(cap) + r];
-    out[2 * size_t(n) + r] = in_range(k3, n) ? perm1[k3] : -1;
+    out[size_t(n) + r] = ord23[r];
+    out[2 * size_t(n) + r] = ord23[size_t(cap) + r];
   }
 }
 
@@ -1046,26 +1031,38 @@ int link_gx(int n, int num_sms) {
 }
 int line_flag_blocks(int n, int num_sms) { return n <= 0 ? 0 : std::min((n + 255) / 256, num_sms * 8); }
 
+// blocks of the row scatter: enough to fill the GPU twice while a tile keeps at least 1024
+// points (each block pays for a scan of the rows and one global atomic a row)
+int scatter_blocks(int n, int fill) {
+  return n <= 0 ? 0 : std::max(std::min(fill, (n + 1023) / 1024), (n + kSortTile - 1) / kSortTile);
+}
+// output positions a block of the bucket sort owns: large windows share its fixed costs (scans,
+// barriers, the rows' starts) over more points (300k points: 14.9 us at 4096, 16.7 at 2048; 217k:
+// 13.3 at 2048, 15.1 at 1024), small frames keep enough blocks to spread over the SMs (20k: 6.7 us
+// at 1024, 7.2 at 256)
+int sort_window(int n) { return n >= (1 << 17) ? kWindowMax : n >= (1 << 15) ? kWindowMax / 2 : kWindowMax / 4; }
+int sort_items(int n) { return n <= 0 ? 0 : (n + sort_window(n) - 1) / sort_window(n); }
+
 template <int THREADS>
 cudaError_t scatter_attr() {
   // the shared-memory limit is a per-device function attribute: set it once per device
   static std::atomic<unsigned long long> configured{0};
   return once_per_device(configured, [] {
-    cudaError_t e = cudaFuncSetAttribute(k_sort_scatter<THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         int(scatter_smem_bytes(THREADS)));
+    cudaError_t e = cudaFuncSetAttribute(k_bucket_scatter<THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         int(kScatterSmem));
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_sort_scatter_seg<THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               int(scatter_smem_bytes(THREADS)));
+      e = cudaFuncSetAttribute(k_bucket_scatter_seg<THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               int(kScatterSmem));
     return e;
   });
 }
 
-cudaError_t slab_attr() {
+cudaError_t sort_attr() {
   static std::atomic<unsigned long long> configured{0};  // the shared-memory limit is set once per device
   return once_per_device(configured, [] {
-    cudaError_t e = cudaFuncSetAttribute(k_slab_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, int(slab_smem_bytes()));
+    cudaError_t e = cudaFuncSetAttribute(k_bucket_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kBucketSmem));
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_slab_sort_seg, cudaFuncAttributeMaxDynamicSharedMemorySize, int(slab_smem_bytes()));
+      e = cudaFuncSetAttribute(k_bucket_sort_seg, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kBucketSmem));
     return e;
   });
 }
@@ -1081,66 +1078,67 @@ cudaError_t launch_seg(K kernel, const A* args, const int* blocks, int count, in
   return launch_kernel(kernel, dim3(grid), dim3(threads), smem, stream, false, sg);
 }
 
-SlabArgs slab_args(int n, int bits, int cap, const SortBufs& sb, const GraphBufs& gb, const DevScalars* sc) {
-  // scratch for slabs larger than shared memory: the C2 order and C2 ranks, written later
-  return SlabArgs{n,  bits, sb.keys[0], sb.vals[0], reinterpret_cast<uint32_t*>(gb.ord23),
-                  reinterpret_cast<uint32_t*>(gb.rank2), sb.keys[1], gb.ord23 + size_t(cap), sc,
-                  sb.tile_counts + sb.count_stride};
-}
 }  // namespace
 
-HistArgs hist_args(const int32_t* xyz, int n, int bits, DevScalars* sc, const SortBufs& sb) {
-  return HistArgs{xyz, n, bits, sc, sb.tile_counts, sb.tile_counts + sb.count_stride};
+HistArgs hist_args(const int32_t* xyz, int n, int bits, DevScalars* sc) { return HistArgs{xyz, n, bits, sc}; }
+
+LinkArgs link_args(int n, int bits, int cap, const GraphBufs& gb, const SortBufs& sb, DevScalars* sc,
+                   const ColorArgs& colors) {
+  return LinkArgs{n, bits, cap, gb.ord23, sb.keys_c2, sb.keys_c3, gb.rank12, gb.pk, gb.c4, sc, colors};
 }
 
-LinkArgs link_args(int n, int bits, int cap, const GraphBufs& gb, const SortBufs& sb, DevScalars* sc) {
-  return LinkArgs{n, bits, cap, gb.ord23, sb.keys[0], sb.keys[1], gb.rank2, gb.pk, gb.c4, sc};
+BucketArgs bucket_args(const int32_t* xyz, int n, int bits, int cap, const SortBufs& sb, const GraphBufs& gb,
+                       DevScalars* sc, int fill) {
+  BucketArgs a{};
+  a.xyz = xyz;
+  a.n = n;
+  a.bits = bits;
+  const int blocks = scatter_blocks(n, fill);
+  a.tile = blocks > 0 ? (n + blocks - 1) / blocks : 0;
+  a.window = sort_window(n);
+  for (int c = 0; c < 3; ++c) {
+    a.row_pts[c] = sb.row_pts[c];
+    a.row_tmp[c] = sb.row_tmp[c];
+  }
+  a.tmp_stride = sb.tmp_stride;
+  a.keys_out[0] = gb.pk;
+  a.keys_out[1] = sb.keys_c2;
+  a.keys_out[2] = sb.keys_c3;
+  a.order_out[0] = gb.perm1;
+  a.order_out[1] = gb.ord23;
+  a.order_out[2] = gb.ord23 + size_t(cap);
+  a.rank12 = reinterpret_cast<int32_t*>(gb.rank12);
+  a.sc = sc;
+  return a;
 }
 
-cudaError_t launch_coord_hist(const int32_t* xyz, int n, int bits, DevScalars* sc, const SortBufs* sb, int num_sms,
-                              cudaStream_t stream) {
+cudaError_t launch_coord_hist(const int32_t* xyz, int n, int bits, DevScalars* sc, int num_sms, cudaStream_t stream) {
   if (n <= 0) return cudaSuccess;
-  const HistArgs h = sb ? hist_args(xyz, n, bits, sc, *sb) : HistArgs{xyz, n, bits, sc, nullptr, nullptr};
   // one block a tile, two per SM: every tile of a 1M-point frame in one wave
-  return launch_kernel(k_coord_hist, dim3(coord_hist_blocks(n, num_sms)), dim3(1024), 0, stream, false, h);
+  return launch_kernel(k_coord_hist, dim3(coord_hist_blocks(n, num_sms)), dim3(1024), 0, stream, false,
+                       hist_args(xyz, n, bits, sc));
 }
 
-cudaError_t launch_tile_counts(const SortPassArgs& a, cudaStream_t stream) {
-  return launch_kernel(k_tile_counts, dim3(a.tiles), dim3(kSortThreads), 0, stream, false, a);
-}
-
-cudaError_t launch_tile_scan(const SortPassArgs& a, cudaStream_t stream) {
-  return launch_kernel(k_tile_scan, dim3(((1 << a.bits) + 7) / 8), dim3(256), 0, stream, false, a);
-}
-
-cudaError_t launch_sort_scatter(const SortPassArgs& a, cudaStream_t stream) {
+cudaError_t launch_bucket_scatter(const BucketArgs& a, cudaStream_t stream) {
+  if (a.n <= 0) return cudaSuccess;
   const cudaError_t e = scatter_attr<kScatterThreads>();
   if (e != cudaSuccess) return e;
-  return launch_kernel(k_sort_scatter<kScatterThreads>, dim3(a.tiles), dim3(kScatterThreads),
-                       scatter_smem_bytes(kScatterThreads), stream, false, a);
+  return launch_kernel(k_bucket_scatter<kScatterThreads>, dim3((a.n + a.tile - 1) / a.tile), dim3(kScatterThreads),
+                       kScatterSmem, stream, false, a);
 }
 
-cudaError_t launch_sort_pass(const SortPassArgs& a, cudaStream_t stream) {
-  cudaError_t e = pass_counted_before(a.pass) ? cudaSuccess : launch_tile_counts(a, stream);
-  if (e == cudaSuccess) e = launch_tile_scan(a, stream);
-  if (e == cudaSuccess) e = launch_sort_scatter(a, stream);
-  return e;
-}
-
-cudaError_t launch_slab_sort(int n, int bits, int cap, const SortBufs& sb, const GraphBufs& gb,
-                             const DevScalars* sc, cudaStream_t stream) {
-  if (n <= 0) return cudaSuccess;
-  const cudaError_t e = slab_attr();
+cudaError_t launch_bucket_sort(const BucketArgs& a, cudaStream_t stream) {
+  if (a.n <= 0) return cudaSuccess;
+  const cudaError_t e = sort_attr();
   if (e != cudaSuccess) return e;
-  return launch_kernel(k_slab_sort, dim3(1 << bits), dim3(kSlabThreads), slab_smem_bytes(), stream, false,
-                       slab_args(n, bits, cap, sb, gb, sc));
+  return launch_kernel(k_bucket_sort, dim3(sort_items(a.n), 3), dim3(kBucketThreads), kBucketSmem, stream, false, a);
 }
 
 cudaError_t launch_link(int n, int bits, int cap, bool same_line, const GraphBufs& gb, const SortBufs& sb,
-                        DevScalars* sc, int num_sms, cudaStream_t stream) {
+                        DevScalars* sc, const ColorArgs& colors, int num_sms, cudaStream_t stream) {
   if (n <= 0) return cudaSuccess;
   const int gx = link_gx(n, num_sms);
-  const LinkArgs la = link_args(n, bits, cap, gb, sb, sc);
+  const LinkArgs la = link_args(n, bits, cap, gb, sb, sc, colors);
   if (!same_line) return launch_kernel(k_link<false>, dim3(gx, 3), dim3(kLinkThreads), 0, stream, false, la);
   const cudaError_t e = launch_kernel(k_link<true>, dim3(gx, 3), dim3(kLinkThreads), 0, stream, false, la);
   if (e != cudaSuccess) return e;
@@ -1156,46 +1154,29 @@ cudaError_t launch_coord_hist_seg(const HistArgs* a, int count, int num_sms, cud
   return launch_seg(k_coord_hist_seg, a, blocks, count, 1024, 0, stream);
 }
 
-cudaError_t launch_sort_pass_seg(const SortPassArgs* a, int count, int scatter_threads, cudaStream_t stream) {
-  int tiles[kSegMax], scan[kSegMax];
-  for (int f = 0; f < count && f < kSegMax; ++f) {
-    tiles[f] = a[f].n > 0 ? a[f].tiles : 0;
-    scan[f] = a[f].n > 0 ? ((1 << a[f].bits) + 7) / 8 : 0;
-  }
-  cudaError_t e = count > 0 && pass_counted_before(a[0].pass)
-                      ? cudaSuccess
-                      : launch_seg(k_tile_counts_seg, a, tiles, count, kSortThreads, 0, stream);
-  if (e == cudaSuccess) e = launch_seg(k_tile_scan_seg, a, scan, count, 256, 0, stream);
-  if (e != cudaSuccess) return e;
+cudaError_t launch_bucket_scatter_seg(const BucketArgs* a, int count, int scatter_threads, cudaStream_t stream) {
+  int tiles[kSegMax];
+  for (int f = 0; f < count && f < kSegMax; ++f) tiles[f] = a[f].n > 0 ? (a[f].n + a[f].tile - 1) / a[f].tile : 0;
+  cudaError_t e;
   switch (scatter_threads) {
     case 256:
       e = scatter_attr<256>();
-      return e != cudaSuccess ? e
-                              : launch_seg(k_sort_scatter_seg<256>, a, tiles, count, 256, scatter_smem_bytes(256), stream);
+      return e != cudaSuccess ? e : launch_seg(k_bucket_scatter_seg<256>, a, tiles, count, 256, kScatterSmem, stream);
     case 1024:
       e = scatter_attr<1024>();
-      return e != cudaSuccess
-                 ? e
-                 : launch_seg(k_sort_scatter_seg<1024>, a, tiles, count, 1024, scatter_smem_bytes(1024), stream);
+      return e != cudaSuccess ? e : launch_seg(k_bucket_scatter_seg<1024>, a, tiles, count, 1024, kScatterSmem, stream);
     default:
       e = scatter_attr<512>();
-      return e != cudaSuccess ? e
-                              : launch_seg(k_sort_scatter_seg<512>, a, tiles, count, 512, scatter_smem_bytes(512), stream);
+      return e != cudaSuccess ? e : launch_seg(k_bucket_scatter_seg<512>, a, tiles, count, 512, kScatterSmem, stream);
   }
 }
 
-cudaError_t launch_slab_sort_seg(const int* n, const int* bits, const int* cap, const SortBufs* sb,
-                                 const GraphBufs* gb, DevScalars* const* sc, int count, cudaStream_t stream) {
-  if (count < 1 || count > kSegMax) return cudaErrorInvalidValue;
-  const cudaError_t e = slab_attr();
+cudaError_t launch_bucket_sort_seg(const BucketArgs* a, int count, cudaStream_t stream) {
+  const cudaError_t e = sort_attr();
   if (e != cudaSuccess) return e;
-  SlabArgs a[kSegMax];
   int blocks[kSegMax];
-  for (int f = 0; f < count; ++f) {
-    a[f] = slab_args(n[f], bits[f], cap[f], sb[f], gb[f], sc[f]);
-    blocks[f] = n[f] > 0 ? (1 << bits[f]) : 0;
-  }
-  return launch_seg(k_slab_sort_seg, a, blocks, count, kSlabThreads, slab_smem_bytes(), stream);
+  for (int f = 0; f < count && f < kSegMax; ++f) blocks[f] = 3 * sort_items(a[f].n);
+  return launch_seg(k_bucket_sort_seg, a, blocks, count, kBucketThreads, kBucketSmem, stream);
 }
 
 cudaError_t launch_link_seg(const LinkArgs* a, int count, bool same_line, int num_sms, cudaStream_t stream) {
@@ -1211,12 +1192,13 @@ cudaError_t launch_link_seg(const LinkArgs* a, int count, bool same_line, int nu
 }
 
 cudaError_t launch_link_wide(int n, int bits, int cap, int window, bool same_line, const GraphBufs& gb,
-                             const SortBufs& sb, DevScalars* sc, int num_sms, cudaStream_t stream) {
+                             const SortBufs& sb, DevScalars* sc, const ColorArgs& colors, int num_sms,
+                             cudaStream_t stream) {
   if (n <= 0) return cudaSuccess;
   if (window < 2 || window > kMaxWindow || gb.nx != extra_slots(window) || !gb.cx) return cudaErrorInvalidValue;
   const int gx = std::max(1, std::min((n + 255) / 256, num_sms * 4));
-  const cudaError_t e = launch_kernel(k_link_wide, dim3(gx, 3), dim3(256), 0, stream, false, n, bits, cap, window,
-                                      same_line ? 1 : 0, gb.ord23, sb.keys[0], sb.keys[1], gb.rank2, gb.pk, gb.c4,
+  const cudaError_t e = launch_kernel(k_link_wide, dim3(gx, 3), dim3(256), 0, stream, false, colors, n, bits, cap, window,
+                                      same_line ? 1 : 0, gb.ord23, sb.keys_c2, sb.keys_c3, gb.rank12, gb.pk, gb.c4,
                                       gb.cx, gb.cx_stride, sc);
   if (e != cudaSuccess || !same_line) return e;
   return launch_kernel(k_c1_line_flags, dim3(std::min((n + 255) / 256, num_sms * 8)), dim3(256), 0, stream, false, n,
@@ -1233,48 +1215,6 @@ cudaError_t launch_orders_export(int n, int cap, const GraphBufs& gb, int32_t* o
   if (n <= 0) return cudaSuccess;
   const int grid = std::max(1, std::min((n + 255) / 256, 152 * 16));
   return launch_kernel(k_orders_export, dim3(grid), dim3(256), 0, stream, false, n, cap, gb.perm1, gb.ord23, out);
-}
-
-SortPassArgs slg_pass_args(int pass, const int32_t* xyz, int n, int bits, int cap, const SortBufs& sb,
-                           const GraphBufs& gb, const DevScalars* sc) {
-  SortPassArgs a{};
-  a.n = n;
-  a.bits = bits;
-  a.tiles = (n + kSortTile - 1) / kSortTile;
-  a.pass = pass;
-  a.counts = sb.tile_counts + size_t(pass) * sb.count_stride;
-  a.sc = sc;
-  if (pass == 0) {
-    // y-slabs: keys are packed C1 codes, values input indices
-    a.shift = bits;
-    a.coord = 1;
-    a.xyz = xyz;
-    a.keys_out = sb.keys[0];
-    a.vals_out = sb.vals[0];
-    return a;
-  }
-  if (pass == 1) {
-    // C1: the C3 order (from the slab sort) on z; ends with pk, perm1, rank1 and the C3
-    // order as sorted ids
-    a.shift = 2 * bits;
-    a.coord = 2;
-    a.keys_in = sb.keys[1];
-    a.vals_in = reinterpret_cast<const uint32_t*>(gb.ord23 + size_t(cap));
-    a.keys_out = gb.pk;
-    a.vals_out = reinterpret_cast<uint32_t*>(gb.perm1);
-    a.rank_out = gb.rank1;
-    a.pos_out = gb.ord23 + size_t(cap);  // the C3 order now as sorted ids (over the input indices read here)
-    return a;
-  }
-  // C2: the C1 order (value = position = sorted id) on x
-  a.shift = 0;
-  a.coord = 0;
-  a.keys_in = gb.pk;
-  a.vals_in = nullptr;
-  a.keys_out = sb.keys[0];  // the packed codes along C2, for the link step
-  a.vals_out = reinterpret_cast<uint32_t*>(gb.ord23);
-  a.rank_out = gb.rank2;
-  return a;
 }
 
 // ---------------------------------------------------------------- shared launch pieces

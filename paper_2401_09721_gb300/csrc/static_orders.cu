@@ -4,9 +4,9 @@
 // a real-time frame loop where an allocation would stall the frame, plug-ins
 // whose host application owns all device memory, or services on a GPU with a
 // fixed memory budget.  This
-// entry point runs the same histogram and radix-sort kernels as
-// fgbd_build_graph, but its scratch (key/value ping-pong buffers, per-tile
-// digit counts, coordinate histograms, orders, ranks) lives in one file-scope device array of
+// entry point runs the same histogram and sort kernels as
+// fgbd_build_graph, but its scratch (the points row by row, coordinate
+// histograms, orders, ranks) lives in one file-scope device array of
 // fixed size, reserved on every GPU that loads the library until the process
 // exits.  The caller passes the coordinates and the output buffer.
 #include <mutex>
@@ -19,23 +19,19 @@ using namespace fgbd;
 namespace {
 
 constexpr size_t kMaxPts = FGBD_STATIC_MAX_POINTS;
-constexpr size_t kMaxTiles = (kMaxPts + kSortTile - 1) / kSortTile;
-
 constexpr size_t align256(size_t v) { return (v + 255) / 256 * 256; }
 
 // byte offsets inside the scratch array
 constexpr size_t kOffScalars = 0;
-constexpr size_t kOffKeys0 = align256(kOffScalars + sizeof(DevScalars));
-constexpr size_t kOffKeys1 = align256(kOffKeys0 + kMaxPts * 4);
-constexpr size_t kOffVals0 = align256(kOffKeys1 + kMaxPts * 4);
-constexpr size_t kOffVals1 = align256(kOffVals0 + kMaxPts * 4);
-constexpr size_t kOffTileCounts = align256(kOffVals1 + kMaxPts * 4);
-constexpr size_t kOffPerm1 = align256(kOffTileCounts + size_t(kSlgPasses) * kMaxRadix * kMaxTiles * 4);
-constexpr size_t kOffRank1 = align256(kOffPerm1 + kMaxPts * 4);
-constexpr size_t kOffPk = align256(kOffRank1 + kMaxPts * 4);
+constexpr size_t kOffKeys2 = align256(kOffScalars + sizeof(DevScalars));
+constexpr size_t kOffKeys3 = align256(kOffKeys2 + kMaxPts * 4);
+constexpr size_t kOffRows = align256(kOffKeys3 + kMaxPts * 4);      // [3][points] of (index, code)
+constexpr size_t kOffTmp = align256(kOffRows + 3 * kMaxPts * 8);    // [3][2][points]
+constexpr size_t kOffPerm1 = align256(kOffTmp + 3 * kMaxPts * 8);
+constexpr size_t kOffRank12 = align256(kOffPerm1 + kMaxPts * 4);
+constexpr size_t kOffPk = align256(kOffRank12 + kMaxPts * 8);
 constexpr size_t kOffOrd23 = align256(kOffPk + kMaxPts * 4);
-constexpr size_t kOffRank2 = align256(kOffOrd23 + 2 * kMaxPts * 4);
-constexpr size_t kScratchBytes = align256(kOffRank2 + kMaxPts * 4);
+constexpr size_t kScratchBytes = align256(kOffOrd23 + 2 * kMaxPts * 4);
 
 static __device__ __align__(256) unsigned char g_static_scratch[kScratchBytes];
 
@@ -75,7 +71,7 @@ extern "C" fgbd_status fgbd_scan_orders_static(const int32_t* xyz, int64_t n64, 
   }
   DevScalars* sc = reinterpret_cast<DevScalars*>(base + kOffScalars);
   // the array keeps the previous call's contents: clear the status word and
-  // the coordinate histograms (the per-tile digit counts are rewritten by every pass)
+  // the coordinate histograms and row counters
   if (cudaMemsetAsync(sc, 0, sizeof(DevScalars), st) != cudaSuccess) {
     cudaGetLastError();
     return FGBD_ECUDA;
@@ -90,29 +86,24 @@ extern "C" fgbd_status fgbd_scan_orders_static(const int32_t* xyz, int64_t n64, 
       return FGBD_ECUDA;
     }
     SortBufs sb{};
-    sb.keys[0] = reinterpret_cast<uint32_t*>(base + kOffKeys0);
-    sb.keys[1] = reinterpret_cast<uint32_t*>(base + kOffKeys1);
-    sb.vals[0] = reinterpret_cast<uint32_t*>(base + kOffVals0);
-    sb.vals[1] = reinterpret_cast<uint32_t*>(base + kOffVals1);
-    sb.tile_counts = reinterpret_cast<uint32_t*>(base + kOffTileCounts);
-    sb.count_stride = int(size_t(kMaxRadix) * kMaxTiles);
+    sb.keys_c2 = reinterpret_cast<uint32_t*>(base + kOffKeys2);
+    sb.keys_c3 = reinterpret_cast<uint32_t*>(base + kOffKeys3);
+    sb.tmp_stride = int(kMaxPts);
+    for (size_t c = 0; c < 3; ++c) {
+      sb.row_pts[c] = reinterpret_cast<uint2*>(base + kOffRows) + c * kMaxPts;
+      sb.row_tmp[c] = reinterpret_cast<uint32_t*>(base + kOffTmp) + c * 2 * kMaxPts;
+    }
     GraphBufs gb{};
     gb.perm1 = reinterpret_cast<int32_t*>(base + kOffPerm1);
-    gb.rank1 = reinterpret_cast<int32_t*>(base + kOffRank1);
+    gb.rank12 = reinterpret_cast<int2*>(base + kOffRank12);
     gb.pk = reinterpret_cast<uint32_t*>(base + kOffPk);
     gb.ord23 = reinterpret_cast<int32_t*>(base + kOffOrd23);
-    gb.rank2 = reinterpret_cast<int32_t*>(base + kOffRank2);
-    if (launch_coord_hist(xyz, n, bits, sc, &sb, num_sms, st) != cudaSuccess) {
+    // cap = n: the C2 and C3 orders lie n apart in the ord23 array
+    const BucketArgs ba = bucket_args(xyz, n, bits, n, sb, gb, sc, scatter_fill(num_sms));
+    if (launch_coord_hist(xyz, n, bits, sc, num_sms, st) != cudaSuccess ||
+        launch_bucket_scatter(ba, st) != cudaSuccess || launch_bucket_sort(ba, st) != cudaSuccess) {
       cudaGetLastError();
       return FGBD_ECUDA;
-    }
-    // cap = n: the C2 and C3 orders lie n apart in the ord23 array
-    for (int p = 0; p < kSlgPasses; ++p) {
-      if (launch_sort_pass(slg_pass_args(p, xyz, n, bits, n, sb, gb, sc), st) != cudaSuccess ||
-          (p == 0 && launch_slab_sort(n, bits, n, sb, gb, sc, st) != cudaSuccess)) {
-        cudaGetLastError();
-        return FGBD_ECUDA;
-      }
     }
     // the three orders in input indices, written into the caller's [3][n] array
     if (launch_orders_export(n, n, gb, orders, st) != cudaSuccess) {
