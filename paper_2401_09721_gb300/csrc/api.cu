@@ -846,7 +846,7 @@ fgbd_status fgbd_ctx_create(int64_t capacity, const fgbd_params* params, fgbd_ct
 
   const size_t C = size_t(capacity);
   ctx->f64_blocks = ne_moment_blocks(int(C), ctx->num_sms);
-  const size_t kP = size_t(kD) * kD + kD + 1;
+  const size_t kP = size_t(kD) * kD + kD + 1;  // (at least the sums of a moment block)
   // wider windows: the further neighbour slots and the noise-estimate scratch
   const bool wide = p.window > 1;
   const size_t wD = size_t(3 * (6 * p.window + 1));

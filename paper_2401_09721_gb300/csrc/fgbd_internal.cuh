@@ -30,6 +30,8 @@ constexpr int kQCap = 256;                         // largest q_max accepted
 constexpr int kSqShift = 8;                        // fixed point of squared colours (2^-8)
 constexpr int kDistShift = 20;                     // fixed point of edge lengths
 constexpr int kNeThreads = 256;
+constexpr int kNeGroup = 32;                       // float colours: moment blocks whose sums their last block adds up
+constexpr int kNeGroups = 32;                      // at most kNeGroup * kNeGroups moment blocks
 constexpr int kFilterThreads = 512;
 constexpr int kSpecMax = 3;                        // filter steps taken while sigma_est is computed
 constexpr uint32_t kCoordMask = 0x3FFFFFFFu;       // low 30 bits: packed C1 code
@@ -64,6 +66,7 @@ struct DevScalars {
   unsigned long long n_patches;
   long long s1[kD];             // sum of (a - 128)
   long long s2[kD * kD];        // sum of (a - 128)(a - 128)^T (upper triangle filled)
+  uint32_t ne_groups[kNeGroups];  // float colours: blocks of each group that have written their moments
   uint32_t spec_barrier;        // grid barrier of the speculative filter steps
   int32_t spec_done;            // filter steps stored by the noise-estimate kernel
   uint32_t sigma_ready;         // set (release) once sigma_est of this estimate is written

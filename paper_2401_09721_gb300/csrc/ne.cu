@@ -47,6 +47,14 @@ __device__ __forceinline__ void tile_rc(int tile, int& r0, int& c0) {
   c0 = 3 * (ti + rem);
 }
 
+// Float colours: the moments of a block or a group, the kTiles tiles (row-major),
+// sum a, then the patch count; and where entry (r, c), r <= c, of sum a a^T is.
+constexpr int kNeSums = 9 * kTiles + kD + 1;
+__device__ __forceinline__ int tile_entry(int r, int c) {
+  const int ti = r / 3, tj = c / 3;
+  return 9 * (ti * 7 - ti * (ti - 1) / 2 + (tj - ti)) + 3 * (r % 3) + c % 3;
+}
+
 // one neighbour of a patch: sort key (d^2, dz, dy, dx packed so that integer
 // order is lexicographic), its sorted id (input order among repeated voxels)
 // and its colour, carried through the sort
@@ -73,8 +81,7 @@ constexpr int kNeWarps = kNeThreads / 32;
 // row (80-byte rows: the eight rows of an ldmatrix tile fall in distinct banks)
 constexpr int kHRow = 40;
 constexpr int kHRows = 32;
-constexpr int kRowFloats = 33;  // 32 float entries, padded likewise
-constexpr int kFirstLanes = 32 - kTiles;  // lanes 28..31 sum the first moments
+constexpr int kRowFloats = 36;  // 32 float entries and padding: rows start on 16 bytes, four banks apart
 
 // Per point: FSLR spread over the point and its neighbours (written to
 // spread[k]) and, for a point with exactly 6 neighbours, its patch (the point
@@ -252,10 +259,13 @@ __device__ __forceinline__ bool point_patch(int k, int n, int bits, int lane, co
 // pipe (gram_mma.cuh): per 16 patches four m16n8k16 products cover the upper
 // triangle of the 22 x 22 Gram matrix of (a, 1), moved to exact int64 sums
 // every kGramFlushPatches patches.  Float colours: lanes 0..27 own one 3x3
-// tile of the upper triangle of sum a a^T, lanes 28..31 rows of sum a, in
-// fp32 over 4 batches, then float64.  The block combines its warps through
-// shared atomics and adds its totals to the context (uint8) or writes them
-// (float).
+// tile of the upper triangle of sum a a^T, four patches a load, and lanes 0..20
+// one entry of sum a, in fp32 over 4 batches, then float64.  The block combines
+// its warps through shared atomics and adds its totals to the context (uint8) or
+// writes them (float); the last block of a group of kNeGroup to do so adds up the
+// group's sums in block order, so that the eigen step reads a few rows instead of
+// one a block (adding 608 rows there, one load after another, made the estimate
+// launch 146 us at 217k points; with the groups it is 41 us).
 template <int DT>
 __device__ __forceinline__ void ne_moments_body(const MomentArgs& ma, int bid, int nblk) {
   const int n = ma.n, bits = ma.bits, moments = ma.moments, sorted_patches = ma.sorted_patches;
@@ -271,15 +281,13 @@ __device__ __forceinline__ void ne_moments_body(const MomentArgs& ma, int bid, i
   __shared__ __align__(16) __half s_h[DT == 0 ? kNeWarps : 1][kHRows * kHRow];
   __shared__ __align__(16) float s_atf[DT == 1 ? kNeWarps : 1][kD * kRowFloats];
   __shared__ unsigned long long s_tot8[DT == 0 ? kP : 1];
-  __shared__ double s_totf[DT == 1 ? kP : 1];
+  // (float: the warps' sums take the place of their patches when those are done)
+  static_assert(sizeof(double) * kNeSums <= sizeof(float) * kD * kRowFloats, "a warp's sums fit its patch block");
 
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (moments) {
-    for (int i = threadIdx.x; i < kP; i += kNeThreads) {
-      if (DT == 0) s_tot8[i] = 0ull;
-      else s_totf[i] = 0.0;
-    }
-    if (DT == 0) {
+  if (moments && DT == 0) {
+    for (int i = threadIdx.x; i < kP; i += kNeThreads) s_tot8[i] = 0ull;
+    {
       // the warp's staging block: all zero (rows 22..31 stay so)
       uint32_t* hw = reinterpret_cast<uint32_t*>(&s_h[warp][0]);
       for (int i = lane; i < kHRows * kHRow / 2; i += 32) hw[i] = 0u;
@@ -293,18 +301,11 @@ __device__ __forceinline__ void ne_moments_body(const MomentArgs& ma, int bid, i
     sc->cexp_ready = 1u;
   }
   __syncthreads();
-  int r0 = 0, c0 = 0, rb = 0, re = 0;
-  if (DT == 1) {
-    if (lane < kTiles) {
-      tile_rc(lane, r0, c0);
-    } else {
-      rb = ((lane - kTiles) * kD) / kFirstLanes;
-      re = ((lane - kTiles + 1) * kD) / kFirstLanes;
-    }
-  }
+  int r0 = 0, c0 = 0;
+  if (DT == 1 && lane < kTiles) tile_rc(lane, r0, c0);
   float gc[4][4] = {};  // uint8: the Gram blocks (m0, n0), (m0, n1), (m0, n2), (m1, n2)
-  float accf[9] = {};
-  double accd[9] = {};
+  float accf[9] = {}, acc1f = 0.f;
+  double accd[9] = {}, acc1d = 0.0;
   unsigned long long npatch = 0;
   int since_flush = 0;
   __half* ath = &s_h[DT == 0 ? warp : 0][0];
@@ -352,29 +353,37 @@ __device__ __forceinline__ void ne_moments_body(const MomentArgs& ma, int bid, i
       }
     } else {
       if (lane < kTiles) {
-#pragma unroll 4
-        for (int p = 0; p < 32; ++p) {
-          float a[3], b[3];
+#pragma unroll 2
+        for (int p = 0; p < 32; p += 4) {
+          float4 a[3], b[3];
 #pragma unroll
           for (int i = 0; i < 3; ++i) {
-            a[i] = atf[(r0 + i) * kRowFloats + p];
-            b[i] = atf[(c0 + i) * kRowFloats + p];
+            a[i] = *reinterpret_cast<const float4*>(atf + (r0 + i) * kRowFloats + p);
+            b[i] = *reinterpret_cast<const float4*>(atf + (c0 + i) * kRowFloats + p);
           }
 #pragma unroll
           for (int i = 0; i < 3; ++i)
 #pragma unroll
-            for (int j = 0; j < 3; ++j) accf[3 * i + j] = fmaf(a[i], b[j], accf[3 * i + j]);
+            for (int j = 0; j < 3; ++j) {
+              float t = accf[3 * i + j];
+              t = fmaf(a[i].x, b[j].x, t);
+              t = fmaf(a[i].y, b[j].y, t);
+              t = fmaf(a[i].z, b[j].z, t);
+              accf[3 * i + j] = fmaf(a[i].w, b[j].w, t);
+            }
         }
-      } else {
+      }
+      if (lane < kD) {
+        float sum = 0.f;
 #pragma unroll
-        for (int t = 0; t < 6; ++t) {
-          const int r = rb + t;
-          if (r < re) {
-            float sum = 0.f;
-            for (int p = 0; p < 32; ++p) sum += atf[r * kRowFloats + p];
-            accf[t] += sum;
-          }
+        for (int p = 0; p < 32; p += 4) {
+          const float4 a = *reinterpret_cast<const float4*>(atf + lane * kRowFloats + p);
+          sum += a.x;
+          sum += a.y;
+          sum += a.z;
+          sum += a.w;
         }
+        acc1f += sum;
       }
       if (++since_flush == 4) {
 #pragma unroll
@@ -382,6 +391,8 @@ __device__ __forceinline__ void ne_moments_body(const MomentArgs& ma, int bid, i
           accd[i] += double(accf[i]);
           accf[i] = 0.f;
         }
+        acc1d += double(acc1f);
+        acc1f = 0.f;
         since_flush = 0;
       }
     }
@@ -394,37 +405,46 @@ __device__ __forceinline__ void ne_moments_body(const MomentArgs& ma, int bid, i
     gram_flush(gc[1], 0, 1, kD + 1, lane, s_tot8, s_tot8 + kD * kD);
     gram_flush(gc[2], 0, 2, kD + 1, lane, s_tot8, s_tot8 + kD * kD);
     gram_flush(gc[3], 1, 2, kD + 1, lane, s_tot8, s_tot8 + kD * kD);
-  } else {
-#pragma unroll
-    for (int i = 0; i < 9; ++i) accd[i] += double(accf[i]);
-    if (lane < kTiles) {
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) atomicAdd(&s_totf[(r0 + i) * kD + (c0 + j)], accd[3 * i + j]);
-    } else {
-#pragma unroll
-      for (int t = 0; t < 6; ++t) {
-        const int r = rb + t;
-        if (r < re) atomicAdd(&s_totf[kD * kD + r], accd[t]);
-      }
-    }
-  }
-  if (lane == 0) {
-    if (DT == 0) atomicAdd(&s_tot8[kD * kD + kD], npatch);
-    else atomicAdd(&s_totf[kD * kD + kD], double(npatch));
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < kP; i += kNeThreads) {
-    if (DT == 0) {
+    if (lane == 0) atomicAdd(&s_tot8[kD * kD + kD], npatch);
+    __syncthreads();
+    for (int i = threadIdx.x; i < kP; i += kNeThreads) {
       const unsigned long long v = s_tot8[i];
       if (v == 0) continue;
       if (i < kD * kD) atomicAdd(reinterpret_cast<unsigned long long*>(&sc->s2[i]), v);
       else if (i < kD * kD + kD) atomicAdd(reinterpret_cast<unsigned long long*>(&sc->s1[i - kD * kD]), v);
       else atomicAdd(&sc->n_patches, v);
-    } else {
-      f64_partials[size_t(bid) * kP + i] = s_totf[i];
     }
+    return;
+  }
+  double* own = reinterpret_cast<double*>(atf);
+  if (lane < kTiles) {
+#pragma unroll
+    for (int i = 0; i < 9; ++i) own[9 * lane + i] = accd[i] + double(accf[i]);
+  }
+  if (lane < kD) own[9 * kTiles + lane] = acc1d + double(acc1f);
+  if (lane == 0) own[9 * kTiles + kD] = double(npatch);
+  __syncthreads();
+  double* row = f64_partials + size_t(bid) * kNeSums;
+  for (int i = threadIdx.x; i < kNeSums; i += kNeThreads) {
+    double t = 0.0;
+#pragma unroll
+    for (int w = 0; w < kNeWarps; ++w) t += reinterpret_cast<const double*>(&s_atf[DT == 1 ? w : 0][0])[i];
+    row[i] = t;
+  }
+  // the last block of the group adds up its rows, in block order, into the first
+  const int g = bid / kNeGroup, b0 = g * kNeGroup, members = min(kNeGroup, nblk - b0);
+  __shared__ int s_last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(&sc->ne_groups[g], 1u) == uint32_t(members - 1);
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  for (int i = threadIdx.x; i < kNeSums; i += kNeThreads) {
+    double t = 0.0;
+#pragma unroll 8
+    for (int b = 0; b < members; ++b) t += __ldcg(&f64_partials[size_t(b0 + b) * kNeSums + i]);
+    f64_partials[size_t(b0) * kNeSums + i] = t;
   }
 }
 
@@ -585,9 +605,9 @@ __device__ __noinline__ void finalize_block(int dtype, const double* __restrict_
   __shared__ double S[kD * kD];
   __shared__ float Sf[kD * kD];  // Sigma rounded to float32 once, for the float32 work
   __shared__ double s_sum[kD * kD + kD + 1];
+  __shared__ double s_tile[kNeSums];
 
   const int tid = threadIdx.x;
-  constexpr int kP = kD * kD + kD + 1;
   constexpr int kT = kD / 3;  // points of a patch: the pooled dimension
   // gather the moments
   double npd;
@@ -596,11 +616,18 @@ __device__ __noinline__ void finalize_block(int dtype, const double* __restrict_
     for (int i = tid; i < kD; i += kFinThreads) s_sum[kD * kD + i] = double(sc->s1[i]);
     if (tid == 0) s_sum[kD * kD + kD] = double(sc->n_patches);
   } else {
-    for (int i = tid; i < kP; i += kFinThreads) {
-      double t = 0.0;
-      for (int b = 0; b < nblocks; ++b) t += f64_partials[size_t(b) * kP + i];
-      s_sum[i] = t;
+    for (int i = tid; i < kNeSums; i += kFinThreads) {
+      double t = 0.0;  // the groups' sums, each in its first block's row
+#pragma unroll 8
+      for (int b = 0; b < nblocks; b += kNeGroup) t += f64_partials[size_t(b) * kNeSums + i];
+      s_tile[i] = t;
     }
+    fin_bar();
+    for (int i = tid; i < kD * kD; i += kFinThreads) {
+      const int r = i / kD, c = i % kD;
+      s_sum[i] = r <= c ? s_tile[tile_entry(r, c)] : 0.0;
+    }
+    for (int i = tid; i <= kD; i += kFinThreads) s_sum[kD * kD + i] = s_tile[9 * kTiles + i];
   }
   fin_bar();
   npd = s_sum[kD * kD + kD];
@@ -816,7 +843,7 @@ int ne_moment_blocks(int n, int num_sms) {
     cudaGetLastError();
     return std::min(a, b);
   }();
-  return std::max(1, std::min((n + kNeThreads - 1) / kNeThreads, num_sms * per_sm));
+  return std::max(1, std::min({(n + kNeThreads - 1) / kNeThreads, num_sms * per_sm, kNeGroup * kNeGroups}));
 }
 
 MomentArgs moment_args(int n, int bits, const GraphBufs& gb, const uint32_t* y8, const float4* yf, float* spread,
