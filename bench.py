@@ -490,10 +490,11 @@ def algorithmic_bytes(name, n, extra_steps=0.0, out_bytes=3):
         # bucket sort: (index, code) in, codes and indices out for each code, the C1 and C2 ranks out
         "slg_sort": 3 * 8 + 3 * 8 + 2 * 4,
         # link: codes along C1, indices and codes along C2 and C3, both ranks; the neighbour slots
-        # out; in a whole run also the input indices along C1, the colours, and the colours in C1 order
-        "slg_link": 4 + 2 * 8 + 8 + 16 + 11,
+        # out; in a whole run also the input indices along C1, the colours, and the colours (alone and
+        # beside their codes) in C1 order
+        "slg_link": 4 + 2 * 8 + 8 + 16 + 19,
         "gather_colors": 11,
-        # moments: codes 4, slots 16, colours 4, the spread out 4; x_0 of the filter steps out 16
+        # moments: (code, colour) 8, slots 16, the spread out 4; x_0 of the filter steps out 16
         "ne_moments": 28 + 16,
     }
     if name in per_point:

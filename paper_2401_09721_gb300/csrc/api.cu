@@ -39,6 +39,8 @@ struct fgbd_ctx {
   float4* yf = nullptr;
   float* spread = nullptr;
   float4* x0 = nullptr;
+  uint2* pc = nullptr;      // window 1: (packed code, uint8 colour) per sorted point
+  bool x0_kept = false;  // x0 holds x_0 of the uint8 colours as the moments launch wrote it (later steps overwrite it)
   float4* x1 = nullptr;
   float4* xbest = nullptr;  // the global reading of the q search: the best iterate (else null)
   float4* w4 = nullptr;     // window 1: normalised Eq. 4 weights of the slots (FilterArgs::w4, w2)
@@ -265,6 +267,7 @@ FilterArgs filter_args(fgbd_ctx* ctx, int mode, int q_fixed, const double* sigma
   a.c4 = ctx->gb.c4;
   a.rank12 = ctx->gb.rank12;
   a.xbuf0 = ctx->x0;
+  a.x0 = ctx->params.window != 1 ? nullptr : dtype == FGBD_F32 ? ctx->yf : ctx->x0_kept ? ctx->x0 : nullptr;
   a.xbuf1 = ctx->x1;
   a.out = out;
   a.out_dtype = out_dtype;
@@ -355,7 +358,14 @@ void release_batch_objects(fgbd_ctx* ctx) {
 }
 
 ColorArgs color_args(const fgbd_ctx* ctx, const void* rgb, int32_t dtype) {
-  return ColorArgs{rgb, dtype, ctx->gb.perm1, ctx->y8, ctx->yf};
+  const bool codes = ctx->params.window == 1;
+  return ColorArgs{rgb, dtype, ctx->gb.perm1, ctx->y8, ctx->yf, codes && dtype == FGBD_U8 ? ctx->pc : nullptr,
+                   codes ? ctx->gb.pk : nullptr};
+}
+
+MomentArgs moment_args(const fgbd_ctx* ctx, int n) {
+  const int sorted = (ctx->params.variant & FGBD_VARIANT_UNSORTED_PATCH) == 0 ? 1 : 0;
+  return MomentArgs{n, ctx->params.bits, ctx->pc, ctx->yf, ctx->x0, ctx->gb.c4, ctx->spread, ctx->f64part, sorted, ctx->sc};
 }
 
 // `zeroed`: the caller has already zeroed the scalar regions this call fills.
@@ -368,6 +378,7 @@ fgbd_status do_build(fgbd_ctx* ctx, const int32_t* xyz, int64_t n64, cudaStream_
   const int n = int(n64);
   const int bits = ctx->params.bits;
   ctx->has_graph = ctx->has_noise = ctx->has_sel = false;
+  ctx->x0_kept = false;
   ctx->spec_depth = 0;
   ctx->noise_rgb = nullptr;
   ctx->n = n;
@@ -430,21 +441,17 @@ fgbd_status do_estimate(fgbd_ctx* ctx, const void* rgb, int32_t dtype, double* s
   }
   int nblocks = 0;
   if (n > 0) {
-    if (!pregathered)
-      FGBD_LAUNCH(ctx, "gather_colors", st,
-                  launch_gather_colors(color_args(ctx, rgb, dtype), n, st));
-    nblocks = ne_moment_blocks(n, ctx->num_sms);
-    // (with x_0 of the filter steps into ctx->x0, which step 1 then reads as one 16-byte load a point)
+    if (!pregathered) {
+      FGBD_LAUNCH(ctx, "gather_colors", st, launch_gather_colors(color_args(ctx, rgb, dtype), n, st));
+    }
+    nblocks = ne_moment_blocks(n, ctx->num_sms, dtype);
     FGBD_LAUNCH(ctx, "ne_moments", st,
-                launch_ne_moments(n, ctx->params.bits, dtype, ctx->gb, ctx->y8, ctx->yf, ctx->spread, ctx->f64part,
-                                  ctx->sc, ctx->num_sms, true,
-                                  (ctx->params.variant & FGBD_VARIANT_UNSORTED_PATCH) == 0, st,
-                                  speculate ? ctx->x0 : nullptr));
+                launch_ne_moments(moment_args(ctx, n), dtype, ctx->num_sms, st));
+    ctx->x0_kept = true;
   }
   // the same launch stores the first filter steps of these colours on the other SMs
   FilterArgs spec = filter_args(ctx, 0, 0, nullptr, fuse ? fuse_out : nullptr, fuse ? fuse_out_dtype : 0, dtype);
   spec.spec_depth = speculate ? std::min(kSpecMax, int(ctx->params.q_max)) : 0;
-  spec.x0 = speculate && n > 0 ? ctx->x0 : nullptr;
   ctx->spec_depth = n > 0 && ctx->num_sms >= 2 ? spec.spec_depth : 0;
   const bool fused = fuse && ctx->spec_depth > 0;
   spec.fuse = fused ? 1 : 0;
@@ -458,6 +465,7 @@ fgbd_status do_estimate(fgbd_ctx* ctx, const void* rgb, int32_t dtype, double* s
   ctx->noise_rgb = rgb;
   ctx->noise_dtype = dtype;
   if (fused) {
+    ctx->x0_kept = false;
     ctx->has_sel = true;
     ctx->ever_selected = true;
   }
@@ -476,6 +484,7 @@ fgbd_status do_select(fgbd_ctx* ctx, const void* rgb, int32_t dtype, const doubl
   FilterArgs a = filter_args(ctx, 0, 0, sigma_est, out, out_dtype, dtype);
   a.spec_depth = ctx->spec_depth;  // the kernel checks that they were all stored
   FGBD_LAUNCH(ctx, "filter_select", st, launch_filter(a, filter_grid_for(ctx, ctx->n), st));
+  ctx->x0_kept = false;
   if (q_out) FGBD_CUDA(ctx, cudaMemcpyAsync(q_out, &ctx->sc->q_sel, sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
   ctx->has_sel = true;
   ctx->ever_selected = true;
@@ -503,6 +512,7 @@ void mark_run_done(fgbd_ctx* ctx, const fgbd_ctx::RunKey& k, int64_t launches) {
   ctx->n = int(k.n);
   ctx->graph_gen += 1;
   ctx->has_graph = ctx->has_noise = ctx->has_sel = true;
+  ctx->x0_kept = false;
   ctx->ever_selected = true;
   ctx->noise_rgb = k.rgb_in;
   ctx->noise_dtype = k.in_dtype;
@@ -581,7 +591,6 @@ fgbd_status seg_chunk(const std::vector<fgbd_ctx*>& ctxs, const std::vector<fgbd
   const int num_sms = lead->num_sms;
   const int dtype = keys[i0].in_dtype;
   const bool same_line = (lead->params.variant & FGBD_VARIANT_SAME_LINE) != 0;
-  const bool sorted = (lead->params.variant & FGBD_VARIANT_UNSORTED_PATCH) == 0;
   ZeroArgs z[kSegMax];
   HistArgs h[kSegMax];
   LinkArgs l[kSegMax];
@@ -606,7 +615,8 @@ fgbd_status seg_chunk(const std::vector<fgbd_ctx*>& ctxs, const std::vector<fgbd
     ba[f] = bucket_args(xyz, n, bits[f], caps[f], c->sb, c->gb, c->sc,
                         std::max(1, int(double(scatter_fill(num_sms)) * double(n) / points)));
     l[f] = link_args(n, bits[f], caps[f], c->gb, c->sb, c->sc, color_args(c, k.rgb_in, dtype));
-    m[f] = moment_args(n, bits[f], c->gb, c->y8, c->yf, c->spread, c->f64part, true, sorted, c->sc);
+    m[f] = moment_args(c, n);
+    c->x0_kept = true;
     // the state fgbd_run's calls leave (n is set first: filter_args reads it)
     c->n = n;
     spec[f] = filter_args(c, 0, 0, nullptr, nullptr, 0, dtype);
@@ -614,7 +624,7 @@ fgbd_status seg_chunk(const std::vector<fgbd_ctx*>& ctxs, const std::vector<fgbd
     sel[f] = filter_args(c, 0, 0, nullptr, k.rgb_out, k.out_dtype, dtype);
     sel[f].spec_depth = spec[f].spec_depth;
     f64[f] = c->f64part;
-    nblk[f] = ne_moment_blocks(n, num_sms);
+    nblk[f] = ne_moment_blocks(n, num_sms, dtype);
   }
   FGBD_LAUNCH(lead, "seg_zero", st, launch_zero_words_seg(z, F, st));
   FGBD_LAUNCH(lead, "seg_hist", st, launch_coord_hist_seg(h, F, num_sms, st));
@@ -845,7 +855,7 @@ fgbd_status fgbd_ctx_create(int64_t capacity, const fgbd_params* params, fgbd_ct
   ctx->filter_per_sm = std::max(1, filter_grid(1 << 30, ctx->num_sms, nx) / ctx->num_sms);
 
   const size_t C = size_t(capacity);
-  ctx->f64_blocks = ne_moment_blocks(int(C), ctx->num_sms);
+  ctx->f64_blocks = ne_moment_blocks(int(C), ctx->num_sms, FGBD_F32);
   const size_t kP = size_t(kD) * kD + kD + 1;  // (at least the sums of a moment block)
   // wider windows: the further neighbour slots and the noise-estimate scratch
   const bool wide = p.window > 1;
@@ -880,6 +890,7 @@ fgbd_status fgbd_ctx_create(int64_t capacity, const fgbd_params* params, fgbd_ct
       {reinterpret_cast<void**>(&ctx->gb.cx), size_t(nx) * align_up(C, 64) * 4},
       {reinterpret_cast<void**>(&ctx->gb.node_sig), (p.variant & FGBD_VARIANT_SIGMA_PAIR) ? C * 4 : 0},
       {reinterpret_cast<void**>(&ctx->xbest), (p.variant & FGBD_VARIANT_GLOBAL_Q) ? C * 16 : 0},
+      {reinterpret_cast<void**>(&ctx->pc), wide ? 0 : C * 8},
       {reinterpret_cast<void**>(&ctx->w4), wide ? 0 : C * 16},
       {reinterpret_cast<void**>(&ctx->w2), wide ? 0 : C * 8},
       {reinterpret_cast<void**>(&ctx->wne.part), wide ? size_t(w_blocks) * wP * 8 : 0},
@@ -920,6 +931,7 @@ fgbd_status fgbd_ctx_create(int64_t capacity, const fgbd_params* params, fgbd_ct
   if (!(p.variant & FGBD_VARIANT_SIGMA_PAIR)) ctx->gb.node_sig = nullptr;
   if (!(p.variant & FGBD_VARIANT_GLOBAL_Q)) ctx->xbest = nullptr;
   if (wide) {
+    ctx->pc = nullptr;
     ctx->w4 = nullptr;
     ctx->w2 = nullptr;
   }
@@ -1029,6 +1041,7 @@ fgbd_status fgbd_denoise(fgbd_ctx* ctx, const void* rgb_in, int32_t in_dtype, in
   if (ctx->n > 0) {
     FGBD_LAUNCH(ctx, "gather_colors", st,
                 launch_gather_colors(color_args(ctx, rgb_in, in_dtype), ctx->n, st));
+    ctx->x0_kept = false;
   }
   // the gathered colours and filter buffers now hold this call's data
   if (rgb_in != ctx->noise_rgb || in_dtype != ctx->noise_dtype) {
@@ -1042,6 +1055,7 @@ fgbd_status fgbd_denoise(fgbd_ctx* ctx, const void* rgb_in, int32_t in_dtype, in
   if (e != cudaSuccess) return cuda_fail(ctx, e, "memset");
   const FilterArgs a = filter_args(ctx, 1, q, nullptr, rgb_out, out_dtype, in_dtype);
   FGBD_LAUNCH(ctx, "filter_fixed", st, launch_filter(a, filter_grid_for(ctx, ctx->n), st));
+  ctx->x0_kept = false;
   return FGBD_OK;
 }
 
@@ -1154,6 +1168,7 @@ fgbd_status fgbd_run_reuse(fgbd_ctx* ctx, const int32_t* xyz, int64_t n, const v
   FilterArgs a = filter_args(ctx, 1, 0, nullptr, rgb_out, out_dtype, in_dtype);
   a.q_src = &ctx->sc->q_sel;
   FGBD_LAUNCH(ctx, "filter_reuse", st, launch_filter(a, filter_grid_for(ctx, ctx->n), st));
+  ctx->x0_kept = false;
   return FGBD_OK;
 }
 

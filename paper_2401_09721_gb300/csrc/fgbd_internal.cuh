@@ -217,6 +217,9 @@ struct ColorArgs {
   const int32_t* perm1;
   uint32_t* y8;
   float4* yf;
+  uint2* pc;             // window 1, uint8: also (packed code, colour) of every sorted point, which the moments
+                         // launch gathers as one word pair; null: not written
+  const uint32_t* pk;    // window 1: the packed codes of the sorted points, the fourth word of yf (null: zero)
 };
 struct LinkArgs {
   int n;
@@ -234,16 +237,14 @@ struct LinkArgs {
 struct MomentArgs {
   int n;
   int bits;
-  const uint32_t* pk;
+  const uint2* pc;   // uint8: (packed code, colour) per sorted point
+  const float4* yf;  // float: (R, G, B, packed code) per sorted point
+  float4* x0;        // uint8: x_0 of the filter steps, (R, G, B, packed code), written here
   const int4* c4;
-  const uint32_t* y8;
-  const float4* yf;
   float* spread;
   double* f64_partials;
-  int moments;
   int sorted_patches;
   struct DevScalars* sc;
-  float4* x0;  // if set: also x_0 of the filter steps, (r, g, b, packed code) per sorted point
 };
 struct ZeroArgs {
   uint32_t* p;
@@ -298,22 +299,16 @@ cudaError_t launch_link_wide(int n, int bits, int cap, int window, bool same_lin
                              cudaStream_t stream);
 
 cudaError_t launch_gather_colors(const ColorArgs& a, int n, cudaStream_t stream);
-// x0: if set, the launch also writes x_0 of the filter steps (colours and packed code)
-cudaError_t launch_ne_moments(int n, int bits, int dtype, const GraphBufs& gb, const uint32_t* y8,
-                              const float4* yf, float* spread, double* f64_partials,
-                              DevScalars* sc, int num_sms, bool moments, bool sorted_patches,
-                              cudaStream_t stream, float4* x0 = nullptr);
+cudaError_t launch_ne_moments(const MomentArgs& a, int dtype, int num_sms, cudaStream_t stream);
 // spec: if not null (and spec->spec_depth > 0), the same launch also takes the
 // first spec_depth filter steps on the other SMs (one block per SM)
 cudaError_t launch_ne_finalize(int dtype, const double* f64_partials, int nblocks,
                                DevScalars* sc, double* sigma_out, const FilterArgs* spec, int num_sms,
                                cudaStream_t stream);
-int ne_moment_blocks(int n, int num_sms);
+int ne_moment_blocks(int n, int num_sms, int dtype);
 // testing: div_newton and CUDA's division of n operand pairs
 cudaError_t launch_debug_div(const double* a, const double* b, double* q_newton, double* q_div, int64_t n,
                              cudaStream_t stream);
-MomentArgs moment_args(int n, int bits, const GraphBufs& gb, const uint32_t* y8, const float4* yf, float* spread,
-                       double* f64_partials, bool moments, bool sorted_patches, DevScalars* sc);
 // segmented: frames 0..count-1 (count <= kSegMax; one colour dtype for the moments)
 cudaError_t launch_ne_moments_seg(const MomentArgs* a, int count, int dtype, int num_sms, cudaStream_t stream);
 // the estimate launch over frames: one eigen block per frame, the other SMs
@@ -364,7 +359,8 @@ struct FilterArgs {
   DevScalars* sc;
   // select mode: the first spec_depth steps were stored before sigma_est was known
   int spec_depth;          // 0: none
-  const float4* x0;        // x_0 as the moments launch wrote it (r, g, b, packed code), or null: from y8/yf, pk
+  const float4* x0;        // x_0 (r, g, b, packed code): float colours themselves, or as the moments launch wrote
+                           // it into xbuf0; null: from y8, pk
   float4* spec_x;          // [kSpecMax][cap]: x_1 .. x_S
   int32_t* spec_z;         // [kSpecMax][cap]: per point sum_c x_q^2, fixed point
   int cap;                 // row stride of spec_x / spec_z, a multiple of 64
@@ -473,6 +469,20 @@ __device__ __forceinline__ void colors_quad(const ColorArgs& a, int k0, int n) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) pi[i] = k0 + i < n ? a.perm1[k0 + i] : -1;
   }
+  uint32_t p[4] = {0u, 0u, 0u, 0u};
+  if (a.pk) {
+    if (k0 + 4 <= n) {
+      const uint4 v = *reinterpret_cast<const uint4*>(a.pk + k0);
+      p[0] = v.x;
+      p[1] = v.y;
+      p[2] = v.z;
+      p[3] = v.w;
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (k0 + i < n) p[i] = a.pk[k0 + i];
+    }
+  }
   if (a.dtype == 0) {
     const uint8_t* rgb = static_cast<const uint8_t*>(a.rgb);
     const bool words = (reinterpret_cast<uintptr_t>(rgb) & 3u) == 0;
@@ -481,10 +491,18 @@ __device__ __forceinline__ void colors_quad(const ColorArgs& a, int k0, int n) {
     for (int i = 0; i < 4; ++i) c[i] = in_range(pi[i], n) ? load_rgb8(rgb, uint32_t(pi[i]), uint32_t(n), words) : 0u;
     if (k0 + 4 <= n) {
       *reinterpret_cast<uint4*>(a.y8 + k0) = make_uint4(c[0], c[1], c[2], c[3]);
+      if (a.pc) {
+        uint4* pc = reinterpret_cast<uint4*>(a.pc + k0);
+        pc[0] = make_uint4(p[0], c[0], p[1], c[1]);
+        pc[1] = make_uint4(p[2], c[2], p[3], c[3]);
+      }
     } else {
 #pragma unroll
       for (int i = 0; i < 4; ++i)
-        if (k0 + i < n) a.y8[k0 + i] = c[i];
+        if (k0 + i < n) {
+          a.y8[k0 + i] = c[i];
+          if (a.pc) a.pc[k0 + i] = make_uint2(p[i], c[i]);
+        }
     }
   } else {
     const float* rgb = static_cast<const float*>(a.rgb);
@@ -494,7 +512,7 @@ __device__ __forceinline__ void colors_quad(const ColorArgs& a, int k0, int n) {
       c[i] = in_range(pi[i], n) ? load_rgbf(rgb, uint32_t(pi[i])) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int i = 0; i < 4; ++i)
-      if (k0 + i < n) a.yf[k0 + i] = c[i];
+      if (k0 + i < n) a.yf[k0 + i] = make_float4(c[i].x, c[i].y, c[i].z, __uint_as_float(p[i]));
   }
 }
 

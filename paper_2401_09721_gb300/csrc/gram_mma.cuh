@@ -31,6 +31,13 @@ __device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t (&r)[4]) {
                : "r"(addr));
 }
 
+// the same tiles transposed
+__device__ __forceinline__ void ldsm_x4_trans(uint32_t addr, uint32_t (&r)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr));
+}
+
 // c += A (16x16, row) * B (16x8, col), float16 inputs, float32 accumulation
 __device__ __forceinline__ void mma_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
   asm volatile(
@@ -68,6 +75,43 @@ __device__ __forceinline__ void gram_flush(float (&c)[4], int mt, int nt, int De
     if (v == 0 || r > col || r >= D || col > D) continue;
     if (col < D) atomicAdd(&s2[r * D + col], (unsigned long long)v);
     else atomicAdd(&s1[r], (unsigned long long)v);
+  }
+}
+
+// ---- patch-major staging (window 1): one row of `stride` halves a patch, node i's
+// colours in columns 4i .. 4i + 2, the constant 1 of a valid patch in column 3,
+// zeros in column 4i + 3 of the neighbours and beyond the last node.  A node is
+// one 8-byte store wherever its rank puts it; transposed 16 x 16 tiles of the
+// rows are the operands that the entry-major tiles above are.
+
+// Shared address of this lane's row for the transposed ldmatrix.x4 of entries
+// [col0, col0 + 16) of patches [row0, row0 + 16): entries 0-7 and 8-15 of patches
+// 0-7, then of patches 8-15 (the order of gram_tile_addr).
+__device__ __forceinline__ uint32_t gram_patch_addr(uint32_t base, int row0, int col0, int stride, int lane) {
+  const int row = row0 + (lane & 7) + (lane >> 4) * 8;
+  const int col = col0 + ((lane >> 3) & 1) * 8;
+  return base + uint32_t(row * stride + col) * 2u;
+}
+
+// gram_flush for those columns: block (mt, nt) of the Gram matrix of Nodes nodes
+// into s2[r * D + c] (r <= c), s1[r] and the patch count, D = 3 Nodes.
+template <int Nodes>
+__device__ __forceinline__ void gram_flush_nodes(float (&c)[4], int mt, int nt, int lane, unsigned long long* s2,
+                                                 unsigned long long* s1, unsigned long long* count) {
+  constexpr int D = 3 * Nodes;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const int r = 16 * mt + (lane >> 2) + 8 * (e >> 1);
+    const int col = 8 * nt + 2 * (lane & 3) + (e & 1);
+    const long long v = __float2ll_rz(c[e]);
+    c[e] = 0.f;
+    // (a column 4i + 3, i > 0, is zero: so are its products)
+    if (v == 0 || r > col || col >= 4 * Nodes) continue;
+    const int rd = 3 * (r >> 2) + (r & 3), cd = 3 * (col >> 2) + (col & 3);
+    unsigned long long* to = &s2[rd * D + cd];
+    if (col == 3) to = r == 3 ? count : &s1[rd];
+    else if (r == 3) to = &s1[cd];
+    atomicAdd(to, (unsigned long long)v);
   }
 }
 

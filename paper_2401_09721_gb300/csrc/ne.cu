@@ -18,6 +18,7 @@
 //   tail rule gives sigma_est.
 #include <algorithm>
 #include <atomic>
+#include <climits>
 
 #include "eigen.cuh"
 #include "gram_mma.cuh"
@@ -55,210 +56,172 @@ __device__ __forceinline__ int tile_entry(int r, int c) {
   return 9 * (ti * 7 - ti * (ti - 1) / 2 + (tj - ti)) + 3 * (r % 3) + c % 3;
 }
 
-// one neighbour of a patch: sort key (d^2, dz, dy, dx packed so that integer
-// order is lexicographic), its sorted id (input order among repeated voxels)
-// and its colour, carried through the sort
-template <int DT>
-struct NbKey;
-template <>
-struct NbKey<0> {
-  unsigned long long key;
-  int idx;
-  uint32_t col;  // packed R, G, B bytes
-};
-template <>
-struct NbKey<1> {
-  unsigned long long key;
-  int idx;
-  float r, g, b;
-};
-
-
 constexpr int kNeWarps = kNeThreads / 32;
-// uint8 colours: the batch's patches as float16, entry-major: rows 0..20 the
-// entries, row 21 the constant 1 of each valid patch, rows 22..31 zero (the
-// second 16-row block of the mma tiles); 32 patches and 8 halves of padding a
-// row (80-byte rows: the eight rows of an ldmatrix tile fall in distinct banks)
+// uint8 colours: one row of float16 a patch (gram_mma.cuh, patch-major): 28 columns
+// of the seven nodes, four of zeros, and eight of padding (80-byte rows: the eight
+// rows of an ldmatrix tile fall in distinct banks)
 constexpr int kHRow = 40;
-constexpr int kHRows = 32;
+constexpr int kHPatches = 32;
 constexpr int kRowFloats = 36;  // 32 float entries and padding: rows start on 16 bytes, four banks apart
 
 // Per point: FSLR spread over the point and its neighbours (written to
 // spread[k]) and, for a point with exactly 6 neighbours, its patch (the point
-// then its neighbours by (d^2, dz, dy, dx, index)) written to column `lane`
-// of the warp's transposed patch block.  Returns whether a patch was written.
-template <int DT>
-__device__ __forceinline__ bool point_patch(int k, int n, int bits, int lane, const uint32_t* __restrict__ pk,
-                                            const int4* __restrict__ c4, const uint32_t* __restrict__ y8,
-                                            const float4* __restrict__ yf, float* __restrict__ spread,
-                                            float4* __restrict__ x0, bool moments, bool sorted_patches, __half* ath,
-                                            float* atf) {
-  int nb[6];
-  bool v[6];
-  const uint32_t pkk = pk[k];  // packed code, with the same-line variant's missing-C1-link bits
-  nb[0] = k - 1;
-  v[0] = c1_prev_linked(pkk, k);
-  nb[1] = k + 1;
-  v[1] = c1_next_linked(pkk, k, n);
-  const int4 s = c4[k];
-  nb[2] = s.x;
-  nb[3] = s.y;
-  nb[4] = s.z;
-  nb[5] = s.w;
-  v[2] = in_range(s.x, n);
-  v[3] = in_range(s.y, n);
-  v[4] = in_range(s.z, n);
-  v[5] = in_range(s.w, n);
-  int deg = 0;
-#pragma unroll
-  for (int j = 0; j < 6; ++j) deg += v[j];
-  const bool patch = moments && deg == 6;
-  NbKey<DT> e[6];
-  uint32_t cpk[6];
-#pragma unroll
-  for (int j = 0; j < 6; ++j) {
-    const int q = v[j] ? nb[j] : k;
-    cpk[j] = patch ? pk[q] : 0u;
-    e[j].idx = q;
-    if (DT == 0) {
-      reinterpret_cast<NbKey<0>&>(e[j]).col = y8[q];
-    } else {
-      const float4 c = yf[q];
-      reinterpret_cast<NbKey<1>&>(e[j]).r = c.x;
-      reinterpret_cast<NbKey<1>&>(e[j]).g = c.y;
-      reinterpret_cast<NbKey<1>&>(e[j]).b = c.z;
-    }
-  }
-  float sp;
-  const float cnt = float(deg + 1);
-  uint32_t own8 = 0;
-  float ownr = 0.f, owng = 0.f, ownb = 0.f;
-  if (DT == 0) {
-    own8 = y8[k];
-    if (x0)
-      x0[k] = make_float4(float(own8 & 255u), float((own8 >> 8) & 255u), float((own8 >> 16) & 255u),
-                          __uint_as_float(pkk));
-    int sr = int(own8 & 255u), sg = int((own8 >> 8) & 255u), sb = int((own8 >> 16) & 255u);
-    int qr = sr * sr, qg = sg * sg, qb = sb * sb;
-#pragma unroll
-    for (int j = 0; j < 6; ++j) {
-      if (v[j]) {
-        const uint32_t c = reinterpret_cast<NbKey<0>&>(e[j]).col;
-        const int a = int(c & 255u), b = int((c >> 8) & 255u), d = int((c >> 16) & 255u);
-        sr += a;
-        sg += b;
-        sb += d;
-        qr += a * a;
-        qg += b * b;
-        qb += d * d;
-      }
-    }
-    // cnt^2 times each population variance is an exact integer; the mean of
-    // the three standard deviations is (sum of their roots) / (3 cnt), with one
-    // rounded reciprocal instead of four divisions (a few ulp in all, far
-    // inside the band in which the selection decides exactly)
-    const int nn = deg + 1;
-    const float vr = float(nn * qr - sr * sr), vg = float(nn * qg - sg * sg), vb = float(nn * qb - sb * sb);
-    sp = (sqrtf(vr) + sqrtf(vg) + sqrtf(vb)) * __frcp_rn(3.0f * cnt);
-  } else {
-    const float4 o = yf[k];
-    ownr = o.x;
-    owng = o.y;
-    ownb = o.z;
-    if (x0) x0[k] = make_float4(ownr, owng, ownb, __uint_as_float(pkk));
-    float mr = ownr, mg = owng, mb = ownb;
-#pragma unroll
-    for (int j = 0; j < 6; ++j) {
-      if (v[j]) {
-        const NbKey<1>& f = reinterpret_cast<NbKey<1>&>(e[j]);
-        mr += f.r;
-        mg += f.g;
-        mb += f.b;
-      }
-    }
-    const float icnt = __frcp_rn(cnt);
-    mr *= icnt;
-    mg *= icnt;
-    mb *= icnt;
-    float vr = (ownr - mr) * (ownr - mr), vg = (owng - mg) * (owng - mg), vb = (ownb - mb) * (ownb - mb);
-#pragma unroll
-    for (int j = 0; j < 6; ++j) {
-      if (v[j]) {
-        const NbKey<1>& f = reinterpret_cast<NbKey<1>&>(e[j]);
-        vr += (f.r - mr) * (f.r - mr);
-        vg += (f.g - mg) * (f.g - mg);
-        vb += (f.b - mb) * (f.b - mb);
-      }
-    }
-    sp = (sqrtf(vr * icnt) + sqrtf(vg * icnt) + sqrtf(vb * icnt)) * (1.0f / 3.0f);
-  }
-  spread[k] = sp;
-  if (!patch) return false;
-
+// then its neighbours by (d^2, dz, dy, dx, index)) written to the warp's patch
+// block: row `lane` of float16 (uint8), column `lane` of float32 rows (float).
+// Returns whether a patch was written.  Equal distances are ordered by sorted id
+// alone: the C1 order is that of (z, y, x, input index).
+// a patch place per neighbour, four bits each: its rank in the strict order (d^2,
+// sorted id) from the 15 pairwise comparisons.  Starts from the link order, which
+// the "w/o sort" ablation keeps: C1 prev, C1 next, C2 prev, C2 next, C3 prev, C3
+// next.
+__device__ __forceinline__ uint32_t patch_ranks(uint32_t wk, const uint32_t (&code)[6], const int (&nb)[6], int bits,
+                                                bool sorted) {
+  uint32_t ranks = 0x543210u;
+  if (!sorted) return ranks;
   int kx, ky, kz;
-  decode_c1(pkk, bits, kx, ky, kz);
+  decode_c1(wk, bits, kx, ky, kz);
+  unsigned long long key[6];
 #pragma unroll
   for (int j = 0; j < 6; ++j) {
     int x, y, z;
-    decode_c1(cpk[j], bits, x, y, z);
+    decode_c1(code[j], bits, x, y, z);
     const int dx = x - kx, dy = y - ky, dz = z - kz;
-    const unsigned long long d2 = (unsigned long long)(dx * dx + dy * dy + dz * dz);
-    e[j].key = (d2 << 33) | ((unsigned long long)(dz + 1024) << 22) | ((unsigned long long)(dy + 1024) << 11) |
-               (unsigned long long)(dx + 1024);
+    key[j] = ((unsigned long long)uint32_t(dx * dx + dy * dy + dz * dz) << 32) | uint32_t(nb[j]);
   }
-  // the place of each neighbour in the patch: its rank in the strict order
-  // (key, index), from the 15 pairwise comparisons, so the colours are written
-  // straight to their rows (the unique sorted order).  Without sorting (the
-  // "w/o sort" ablation) the entries stay in link order: C1 prev, C1 next,
-  // C2 prev, C2 next, C3 prev, C3 next.
-  int rk[6] = {0, 1, 2, 3, 4, 5};
-  if (sorted_patches) {
 #pragma unroll
-    for (int j = 0; j < 6; ++j) rk[j] = 0;
+  for (int i = 0; i < 6; ++i)
 #pragma unroll
-    for (int i = 0; i < 6; ++i)
+    for (int j = i + 1; j < 6; ++j)
+      if (key[j] < key[i]) ranks += (1u << (4 * i)) - (1u << (4 * j));
+  return ranks;
+}
+
+// a node of a float16 patch: the colours of a packed word centred on 128 and `last`
+// (0 or 1), from the bytes put into the fraction of 1024 (exact: 1024 + c - 1152)
+__device__ __forceinline__ uint2 patch_node(uint32_t c, uint32_t last) {
+  const __half2 off = __halves2half2(__ushort_as_half(0x6480), __ushort_as_half(0x6480));  // 1152
+  const uint32_t a = __byte_perm(c, 0x64646464u, 0x4140), b = __byte_perm(c, 0x64806464u + (last << 16), 0x7642);
+  const __half2 ha = __hsub2(*reinterpret_cast<const __half2*>(&a), off);
+  const __half2 hb = __hsub2(*reinterpret_cast<const __half2*>(&b), off);
+  return make_uint2(*reinterpret_cast<const uint32_t*>(&ha), *reinterpret_cast<const uint32_t*>(&hb));
+}
+
+// uint8 colours
+__device__ __forceinline__ bool point_patch_u8(const MomentArgs& ma, int k, int lane, __half* ath) {
+  const int n = ma.n, bits = ma.bits;
+  const uint2 own = ma.pc[k];
+  const int4 s = ma.c4[k];
+  const uint32_t wk = own.x;  // packed code, with the same-line variant's missing-C1-link bits
+  int nb[6];
+  bool v[6];
+  slots6(k, n, wk, s, nb, v);
+  uint32_t code[6], c[6];
+  int deg = 0;
 #pragma unroll
-      for (int j = i + 1; j < 6; ++j) {
-        const bool j_first = (e[j].key < e[i].key) || (e[j].key == e[i].key && e[j].idx < e[i].idx);
-        rk[i] += j_first;
-        rk[j] += !j_first;
-      }
+  for (int j = 0; j < 6; ++j) {
+    const uint2 q = v[j] ? ma.pc[nb[j]] : make_uint2(0u, 0u);  // (an absent neighbour adds nothing below)
+    code[j] = q.x;
+    c[j] = q.y;
+    deg += v[j];
   }
-  if (DT == 0) {
-    // entry r of the patch, centred on 128 (exact in float16)
-    ath[0 * kHRow + lane] = __int2half_rn(int(own8 & 255u) - 128);
-    ath[1 * kHRow + lane] = __int2half_rn(int((own8 >> 8) & 255u) - 128);
-    ath[2 * kHRow + lane] = __int2half_rn(int((own8 >> 16) & 255u) - 128);
+  ma.x0[k] = make_float4(float(own.y & 255u), float((own.y >> 8) & 255u), float((own.y >> 16) & 255u),
+                         __uint_as_float(wk));
+  // per channel the seven values in two words, their sum and sum of squares by
+  // byte dot products
+  const uint32_t t0 = __byte_perm(own.y, c[0], 0x5140), t1 = __byte_perm(c[1], c[2], 0x5140),
+                 t2 = __byte_perm(c[3], c[4], 0x5140);  // (R, R, G, G) of two points
+  const uint32_t u0 = __byte_perm(own.y, c[0], 0x7362), u1 = __byte_perm(c[1], c[2], 0x7362),
+                 u2 = __byte_perm(c[3], c[4], 0x7362);  // (B, B, 0, 0)
+  const uint32_t ra = __byte_perm(t0, t1, 0x5410), rb = __byte_perm(t2, c[5], 0x7410);
+  const uint32_t ga = __byte_perm(t0, t1, 0x7632), gb = __byte_perm(t2, c[5], 0x7532);
+  const uint32_t ba = __byte_perm(u0, u1, 0x5410), bb = __byte_perm(u2, c[5], 0x7610);
+  const uint32_t ones = 0x01010101u;
+  const int nn = deg + 1;
+  // nn^2 times a population variance, an exact integer
+  const auto var = [&](uint32_t a, uint32_t b) {
+    const int sum = int(__dp4a(a, ones, __dp4a(b, ones, 0u))), sq = int(__dp4a(a, a, __dp4a(b, b, 0u)));
+    return float(nn * sq - sum * sum);
+  };
+  // the mean of the three standard deviations is (sum of their roots) / (3 nn),
+  // with one rounded reciprocal instead of four divisions (a few ulp in all, far
+  // inside the band in which the selection decides exactly)
+  ma.spread[k] = (sqrtf(var(ra, rb)) + sqrtf(var(ga, gb)) + sqrtf(var(ba, bb))) * __frcp_rn(3.0f * float(nn));
+  if (deg != 6) return false;
+  const uint32_t ranks = patch_ranks(wk, code, nb, bits, ma.sorted_patches != 0);
+  uint2* row = reinterpret_cast<uint2*>(ath + lane * kHRow);
+  row[0] = patch_node(own.y, 1u);
 #pragma unroll
-    for (int j = 0; j < 6; ++j) {
-      const uint32_t c = reinterpret_cast<NbKey<0>&>(e[j]).col;
-      __half* row = ath + (3 + 3 * rk[j]) * kHRow + lane;
-      row[0] = __int2half_rn(int(c & 255u) - 128);
-      row[kHRow] = __int2half_rn(int((c >> 8) & 255u) - 128);
-      row[2 * kHRow] = __int2half_rn(int((c >> 16) & 255u) - 128);
-    }
-  } else {
-    atf[0 * kRowFloats + lane] = ownr - 128.f;
-    atf[1 * kRowFloats + lane] = owng - 128.f;
-    atf[2 * kRowFloats + lane] = ownb - 128.f;
+  for (int j = 0; j < 6; ++j) row[1 + ((ranks >> (4 * j)) & 15u)] = patch_node(c[j], 0u);
+  return true;
+}
+
+// float colours
+__device__ __forceinline__ bool point_patch_f32(const MomentArgs& ma, int k, int lane, float* atf) {
+  const int n = ma.n, bits = ma.bits;
+  const float4 own = ma.yf[k];
+  const int4 s = ma.c4[k];
+  const uint32_t wk = __float_as_uint(own.w);
+  int nb[6];
+  bool v[6];
+  slots6(k, n, wk, s, nb, v);
+  float4 q[6];
 #pragma unroll
-    for (int j = 0; j < 6; ++j) {
-      const NbKey<1>& f = reinterpret_cast<NbKey<1>&>(e[j]);
-      float* row = atf + (3 + 3 * rk[j]) * kRowFloats + lane;
-      row[0] = f.r - 128.f;
-      row[kRowFloats] = f.g - 128.f;
-      row[2 * kRowFloats] = f.b - 128.f;
+  for (int j = 0; j < 6; ++j) q[j] = v[j] ? ma.yf[nb[j]] : own;
+  int deg = 0;
+#pragma unroll
+  for (int j = 0; j < 6; ++j) deg += v[j];
+  float mr = own.x, mg = own.y, mb = own.z;
+#pragma unroll
+  for (int j = 0; j < 6; ++j) {
+    if (v[j]) {
+      mr += q[j].x;
+      mg += q[j].y;
+      mb += q[j].z;
     }
+  }
+  const float icnt = __frcp_rn(float(deg + 1));
+  mr *= icnt;
+  mg *= icnt;
+  mb *= icnt;
+  float vr = (own.x - mr) * (own.x - mr), vg = (own.y - mg) * (own.y - mg), vb = (own.z - mb) * (own.z - mb);
+#pragma unroll
+  for (int j = 0; j < 6; ++j) {
+    if (v[j]) {
+      vr += (q[j].x - mr) * (q[j].x - mr);
+      vg += (q[j].y - mg) * (q[j].y - mg);
+      vb += (q[j].z - mb) * (q[j].z - mb);
+    }
+  }
+  ma.spread[k] = (sqrtf(vr * icnt) + sqrtf(vg * icnt) + sqrtf(vb * icnt)) * (1.0f / 3.0f);
+  if (deg != 6) return false;
+  uint32_t code[6];
+#pragma unroll
+  for (int j = 0; j < 6; ++j) code[j] = __float_as_uint(q[j].w);
+  const uint32_t ranks = patch_ranks(wk, code, nb, bits, ma.sorted_patches != 0);
+  atf[0 * kRowFloats + lane] = own.x - 128.f;
+  atf[1 * kRowFloats + lane] = own.y - 128.f;
+  atf[2 * kRowFloats + lane] = own.z - 128.f;
+#pragma unroll
+  for (int j = 0; j < 6; ++j) {
+    float* row = atf + (3u + 3u * ((ranks >> (4 * j)) & 15u)) * kRowFloats + lane;
+    row[0] = q[j].x - 128.f;
+    row[kRowFloats] = q[j].y - 128.f;
+    row[2 * kRowFloats] = q[j].z - 128.f;
   }
   return true;
 }
 
 // Warp-synchronous: each warp takes 32 points at a time, stages their patches
-// transposed in its own shared-memory block and accumulates the moments with
-// __syncwarp only.  uint8 colours: float16 patches and mma.sync on the tensor
-// pipe (gram_mma.cuh): per 16 patches four m16n8k16 products cover the upper
-// triangle of the 22 x 22 Gram matrix of (a, 1), moved to exact int64 sums
-// every kGramFlushPatches patches.  Float colours: lanes 0..27 own one 3x3
+// in its own shared-memory block and accumulates the moments with __syncwarp
+// only.  The kernel is bound by its instructions (64 % of the issue slots used at 1M
+// points), so neighbours are one 8-byte load of (code, colour), a patch is seven
+// 8-byte stores, sums of squares are byte dot products and equal distances need
+// no tie key: 36 -> 27 us at 1M points (x_0 as 16-byte neighbour loads: 31, and the
+// link launch that writes it 9 us longer).  uint8 colours: float16 patches and
+// mma.sync on the tensor pipe
+// (gram_mma.cuh): per 16 patches six m16n8k16 products cover the upper triangle
+// of the Gram matrix of (a, 1) in its 28 columns, moved to exact int64 sums every
+// kGramFlushPatches patches.  Float colours: lanes 0..27 own one 3x3
 // tile of the upper triangle of sum a a^T, four patches a load, and lanes 0..20
 // one entry of sum a, in fp32 over 4 batches, then float64.  The block combines
 // its warps through shared atomics and adds its totals to the context (uint8) or
@@ -266,32 +229,30 @@ __device__ __forceinline__ bool point_patch(int k, int n, int bits, int lane, co
 // group's sums in block order, so that the eigen step reads a few rows instead of
 // one a block (adding 608 rows there, one load after another, made the estimate
 // launch 146 us at 217k points; with the groups it is 41 us).
+// the six Gram blocks into the block's int64 sums (sum a a^T, sum a, the patch count)
+__device__ __forceinline__ void flush8(float (&gc)[6][4], int lane, unsigned long long* tot) {
+#pragma unroll
+  for (int t = 0; t < 6; ++t)
+    gram_flush_nodes<kK + 1>(gc[t], t / 4, t < 4 ? t : t - 2, lane, tot, tot + kD * kD, tot + kD * kD + kD);
+}
+
 template <int DT>
 __device__ __forceinline__ void ne_moments_body(const MomentArgs& ma, int bid, int nblk) {
-  const int n = ma.n, bits = ma.bits, moments = ma.moments, sorted_patches = ma.sorted_patches;
-  const uint32_t* __restrict__ pk = ma.pk;
-  const int4* __restrict__ c4 = ma.c4;
-  const uint32_t* __restrict__ y8 = ma.y8;
-  const float4* __restrict__ yf = ma.yf;
-  float* __restrict__ spread = ma.spread;
+  const int n = ma.n;
   double* __restrict__ f64_partials = ma.f64_partials;
   DevScalars* __restrict__ sc = ma.sc;
   constexpr int kP = kD * kD + kD + 1;
-  static_assert(kD + 1 <= kHRows && kHRows == 32, "entries, the constant row and the zero rows fill two 16-row blocks");
-  __shared__ __align__(16) __half s_h[DT == 0 ? kNeWarps : 1][kHRows * kHRow];
+  __shared__ __align__(16) __half s_h[DT == 0 ? kNeWarps : 1][kHPatches * kHRow];
   __shared__ __align__(16) float s_atf[DT == 1 ? kNeWarps : 1][kD * kRowFloats];
   __shared__ unsigned long long s_tot8[DT == 0 ? kP : 1];
   // (float: the warps' sums take the place of their patches when those are done)
   static_assert(sizeof(double) * kNeSums <= sizeof(float) * kD * kRowFloats, "a warp's sums fit its patch block");
 
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (moments && DT == 0) {
+  if (DT == 0) {
     for (int i = threadIdx.x; i < kP; i += kNeThreads) s_tot8[i] = 0ull;
-    {
-      // the warp's staging block: all zero (rows 22..31 stay so)
-      uint32_t* hw = reinterpret_cast<uint32_t*>(&s_h[warp][0]);
-      for (int i = lane; i < kHRows * kHRow / 2; i += 32) hw[i] = 0u;
-    }
+    // the columns behind the nodes stay zero
+    *reinterpret_cast<uint2*>(&s_h[warp][lane * kHRow + 4 * (kK + 1)]) = make_uint2(0u, 0u);
   }
   // the graph's Eq. 4 exponent scale, once, for the filter steps that follow
   // (float64 work, here off their critical path)
@@ -303,7 +264,7 @@ __device__ __forceinline__ void ne_moments_body(const MomentArgs& ma, int bid, i
   __syncthreads();
   int r0 = 0, c0 = 0;
   if (DT == 1 && lane < kTiles) tile_rc(lane, r0, c0);
-  float gc[4][4] = {};  // uint8: the Gram blocks (m0, n0), (m0, n1), (m0, n2), (m1, n2)
+  float gc[6][4] = {};  // uint8: the Gram blocks (m0, n0) .. (m0, n3), (m1, n2), (m1, n3)
   float accf[9] = {}, acc1f = 0.f;
   double accd[9] = {}, acc1d = 0.0;
   unsigned long long npatch = 0;
@@ -316,39 +277,34 @@ __device__ __forceinline__ void ne_moments_body(const MomentArgs& ma, int bid, i
   for (int base = (bid * kNeWarps + warp) * 32; base < n; base += nwarps * 32) {
     const int k = base + lane;
     bool has = false;
-    if (k < n)
-      has = point_patch<DT>(k, n, bits, lane, pk, c4, y8, yf, spread, ma.x0, moments != 0, sorted_patches != 0, ath,
-                            atf);
-    if (!moments) continue;
-    if (DT == 0) {
-      if (!has) {
+    if (k < n) has = DT == 0 ? point_patch_u8(ma, k, lane, ath) : point_patch_f32(ma, k, lane, atf);
+    if (!has) {
+      if (DT == 0) {
+        uint2* row = reinterpret_cast<uint2*>(ath + lane * kHRow);
 #pragma unroll
-        for (int r = 0; r < kD; ++r) ath[r * kHRow + lane] = __float2half_rn(0.f);
+        for (int j = 0; j < kK + 1; ++j) row[j] = make_uint2(0u, 0u);
+      } else {
+#pragma unroll
+        for (int r = 0; r < kD; ++r) atf[r * kRowFloats + lane] = 0.f;
       }
-      ath[kD * kHRow + lane] = __float2half_rn(has ? 1.f : 0.f);
-    } else if (!has) {
-#pragma unroll
-      for (int r = 0; r < kD; ++r) atf[r * kRowFloats + lane] = 0.f;
     }
-    const uint32_t hb = __ballot_sync(0xffffffffu, has);
-    npatch += __popc(hb);
+    if (DT == 1) npatch += __popc(__ballot_sync(0xffffffffu, has));
     __syncwarp();
     if (DT == 0) {
 #pragma unroll
       for (int ks = 0; ks < 2; ++ks) {
         uint32_t lo[4], hi[4];
-        ldsm_x4(gram_tile_addr(hbase, 0, 16 * ks, kHRow, lane), lo);
-        ldsm_x4(gram_tile_addr(hbase, 16, 16 * ks, kHRow, lane), hi);
+        ldsm_x4_trans(gram_patch_addr(hbase, 16 * ks, 0, kHRow, lane), lo);
+        ldsm_x4_trans(gram_patch_addr(hbase, 16 * ks, 16, kHRow, lane), hi);
         mma_16816(gc[0], lo, lo[0], lo[2]);
         mma_16816(gc[1], lo, lo[1], lo[3]);
         mma_16816(gc[2], lo, hi[0], hi[2]);
-        mma_16816(gc[3], hi, hi[0], hi[2]);
+        mma_16816(gc[3], lo, hi[1], hi[3]);
+        mma_16816(gc[4], hi, hi[0], hi[2]);
+        mma_16816(gc[5], hi, hi[1], hi[3]);
       }
       if (++since_flush == kGramFlushPatches / 32) {
-        gram_flush(gc[0], 0, 0, kD + 1, lane, s_tot8, s_tot8 + kD * kD);
-        gram_flush(gc[1], 0, 1, kD + 1, lane, s_tot8, s_tot8 + kD * kD);
-        gram_flush(gc[2], 0, 2, kD + 1, lane, s_tot8, s_tot8 + kD * kD);
-        gram_flush(gc[3], 1, 2, kD + 1, lane, s_tot8, s_tot8 + kD * kD);
+        flush8(gc, lane, s_tot8);
         since_flush = 0;
       }
     } else {
@@ -398,14 +354,9 @@ __device__ __forceinline__ void ne_moments_body(const MomentArgs& ma, int bid, i
     }
     __syncwarp();
   }
-  if (!moments) return;
   // combine the warps of the block
   if (DT == 0) {
-    gram_flush(gc[0], 0, 0, kD + 1, lane, s_tot8, s_tot8 + kD * kD);
-    gram_flush(gc[1], 0, 1, kD + 1, lane, s_tot8, s_tot8 + kD * kD);
-    gram_flush(gc[2], 0, 2, kD + 1, lane, s_tot8, s_tot8 + kD * kD);
-    gram_flush(gc[3], 1, 2, kD + 1, lane, s_tot8, s_tot8 + kD * kD);
-    if (lane == 0) atomicAdd(&s_tot8[kD * kD + kD], npatch);
+    flush8(gc, lane, s_tot8);
     __syncthreads();
     for (int i = threadIdx.x; i < kP; i += kNeThreads) {
       const unsigned long long v = s_tot8[i];
@@ -449,13 +400,13 @@ __device__ __forceinline__ void ne_moments_body(const MomentArgs& ma, int bid, i
 }
 
 template <int DT>
-__global__ void __launch_bounds__(kNeThreads, 4) k_ne_moments(MomentArgs a) {
+__global__ void __launch_bounds__(kNeThreads, DT == 0 ? 4 : 3) k_ne_moments(MomentArgs a) {
   pdl_wait();
   ne_moments_body<DT>(a, blockIdx.x, gridDim.x);
 }
 
 template <int DT>
-__global__ void __launch_bounds__(kNeThreads, 4) k_ne_moments_seg(const __grid_constant__ Seg<MomentArgs> s) {
+__global__ void __launch_bounds__(kNeThreads, DT == 0 ? 4 : 3) k_ne_moments_seg(const __grid_constant__ Seg<MomentArgs> s) {
   pdl_wait();
   const int f = seg_frame(s, blockIdx.x);
   ne_moments_body<DT>(s.a[f], blockIdx.x - s.start[f], s.start[f + 1] - s.start[f]);
@@ -785,9 +736,18 @@ cudaError_t launch_ne_moments_seg(const MomentArgs* a, int count, int dtype, int
   if (count < 1 || count > kSegMax) return cudaErrorInvalidValue;
   Seg<MomentArgs> sg;
   int blocks[kSegMax];
+  // uint8 (exact sums, whatever blocks add them): the frames share the blocks that
+  // fill the GPU once, so that a block's set-up and its 275 global atomics serve
+  // several batches of points (16 frames of 20k-100k points: 65 -> 30 us).  Float: as many blocks as the one-frame launch has,
+  // whose sums are the same bits.
+  double total = 0.0;
+  for (int f = 0; f < count; ++f) total += double(std::max(a[f].n, 0));
+  const int fill = ne_moment_blocks(INT_MAX, num_sms, dtype);
   for (int f = 0; f < count; ++f) {
     sg.a[f] = a[f];
-    blocks[f] = a[f].n > 0 ? ne_moment_blocks(a[f].n, num_sms) : 0;
+    blocks[f] = a[f].n > 0 ? ne_moment_blocks(a[f].n, num_sms, dtype) : 0;
+    if (dtype == 0 && blocks[f] > 0)
+      blocks[f] = std::max(1, std::min(blocks[f], int(double(fill) * double(a[f].n) / total)));
   }
   const int grid = seg_layout(sg, blocks, count);
   if (grid == 0) return cudaSuccess;
@@ -832,34 +792,29 @@ cudaError_t launch_gather_colors(const ColorArgs& a, int n, cudaStream_t stream)
   return launch_kernel(k_gather_colors, dim3(grid), dim3(256), 0, stream, false, a, n);
 }
 
-int ne_moment_blocks(int n, int num_sms) {
+int ne_moment_blocks(int n, int num_sms, int dtype) {
   // resident blocks per SM, queried once (the same code runs on every device of one build)
-  static const int per_sm = [] {
+  struct PerSm {
+    int u8 = 1, f32 = 1;
+  };
+  static const PerSm per_sm = [] {
+    PerSm p;
     int a = 0, b = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_ne_moments<0>, kNeThreads, 0) != cudaSuccess || a < 1)
-      a = 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_ne_moments<1>, kNeThreads, 0) != cudaSuccess || b < 1)
-      b = 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_ne_moments<0>, kNeThreads, 0) == cudaSuccess && a > 0)
+      p.u8 = a;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_ne_moments<1>, kNeThreads, 0) == cudaSuccess && b > 0)
+      p.f32 = b;
     cudaGetLastError();
-    return std::min(a, b);
+    return p;
   }();
-  return std::max(1, std::min({(n + kNeThreads - 1) / kNeThreads, num_sms * per_sm, kNeGroup * kNeGroups}));
+  const int need = int((int64_t(n) + kNeThreads - 1) / kNeThreads);
+  if (dtype == 0) return std::max(1, std::min(need, num_sms * per_sm.u8));
+  return std::max(1, std::min({need, num_sms * per_sm.f32, kNeGroup * kNeGroups}));
 }
 
-MomentArgs moment_args(int n, int bits, const GraphBufs& gb, const uint32_t* y8, const float4* yf, float* spread,
-                       double* f64_partials, bool moments, bool sorted_patches, DevScalars* sc) {
-  return MomentArgs{n,  bits,         gb.pk, gb.c4, y8, yf, spread, f64_partials, moments ? 1 : 0, sorted_patches ? 1 : 0,
-                    sc, nullptr};
-}
-
-cudaError_t launch_ne_moments(int n, int bits, int dtype, const GraphBufs& gb, const uint32_t* y8,
-                              const float4* yf, float* spread, double* f64_partials,
-                              DevScalars* sc, int num_sms, bool moments, bool sorted_patches,
-                              cudaStream_t stream, float4* x0) {
-  if (n <= 0) return cudaSuccess;
-  const int grid = ne_moment_blocks(n, num_sms);
-  MomentArgs a = moment_args(n, bits, gb, y8, yf, spread, f64_partials, moments, sorted_patches, sc);
-  a.x0 = x0;
+cudaError_t launch_ne_moments(const MomentArgs& a, int dtype, int num_sms, cudaStream_t stream) {
+  if (a.n <= 0) return cudaSuccess;
+  const int grid = ne_moment_blocks(a.n, num_sms, dtype);
   if (dtype == 0) return launch_kernel(k_ne_moments<0>, dim3(grid), dim3(kNeThreads), 0, stream, false, a);
   return launch_kernel(k_ne_moments<1>, dim3(grid), dim3(kNeThreads), 0, stream, false, a);
 }

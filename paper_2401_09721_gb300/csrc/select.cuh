@@ -6,7 +6,7 @@
 //   phase 0   the FSLR keep flag of each point (spread <= 2 sigma_est) goes to
 //             keep8; the kept power sum y^2 and the kept count are reduced, and
 //             so are the stored steps' per-point power sums x_q^2;
-//             x_0 = y is written unless steps are stored.
+//             x_0 = y is written unless it is there or steps are stored.
 //   J(1..S)   from those sums, by thread 0 of every block (the same values
 //             everywhere: the sums are exact integers).
 //   step t    x_t = x_{t-1}/2 + (sum_j e_j x_{t-1}[j]) / (2 sum_j e_j) with
@@ -417,10 +417,12 @@ __device__ __forceinline__ void select_filter(const FilterArgs& a, int S, int fi
   // Four consecutive points per thread and trip, read with 16-byte loads that
   // are all issued before the first is used.
   unsigned long long acc[kSums] = {};
-  for (int k0 = 4 * gtid; k0 < n; k0 += 4 * gstride) {
+  const bool write_x0 = !S && !a.x0;
+  const bool phase0 = select || write_x0;
+  for (int k0 = 4 * gtid; phase0 && k0 < n; k0 += 4 * gstride) {
     const bool full = k0 + 4 <= n;
     float4 x[4];
-    x0_quad(a, k0, full, !S, x);
+    x0_quad(a, k0, full, write_x0, x);
     float sp[4] = {0.f, 0.f, 0.f, 0.f};
     if (select) {
       if (full) {
@@ -435,7 +437,7 @@ __device__ __forceinline__ void select_filter(const FilterArgs& a, int S, int fi
           if (k0 + i < n) sp[i] = a.spread[k0 + i];
       }
     }
-    if (!S) {
+    if (write_x0) {
 #pragma unroll
       for (int i = 0; i < 4; ++i)
         if (full || k0 + i < n) a.xbuf0[k0 + i] = x[i];
@@ -524,7 +526,7 @@ __device__ __forceinline__ void select_filter(const FilterArgs& a, int S, int fi
       }
     }
   }
-  if (!grid_barrier(bar, &sc->status, members, epoch, &s_ok, sc)) return;
+  if (phase0 && !grid_barrier(bar, &sc->status, members, epoch, &s_ok, sc)) return;
 
   // J(0..S) from the stored terms, by thread 0 of each block (every block
   // reaches the same values: the sums are exact integers).  Under the global
@@ -615,7 +617,8 @@ __device__ __forceinline__ void select_filter(const FilterArgs& a, int S, int fi
   bool copy_best = false;  // this step's source is the best iterate so far: copy it to xbest
   for (int t = S + 1; t <= q_limit && !stopped; ++t) {
     const float4* __restrict__ src =
-        (S > 0 && t == S + 1) ? a.spec_x + size_t(S - 1) * size_t(a.cap) : ((t & 1) ? a.xbuf0 : a.xbuf1);
+        t == 1 && a.x0 ? a.x0
+                       : (S > 0 && t == S + 1) ? a.spec_x + size_t(S - 1) * size_t(a.cap) : ((t & 1) ? a.xbuf0 : a.xbuf1);
     float4* __restrict__ dst = (t & 1) ? a.xbuf1 : a.xbuf0;
     unsigned long long loc = 0;
     for (int k = gtid; k < n; k += gstride) {

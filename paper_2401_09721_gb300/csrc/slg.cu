@@ -874,24 +874,31 @@ __global__ void __launch_bounds__(kLinkThreads, 6) k_link_seg(const __grid_const
 // its packed code, where every kernel that takes k +- 1 as neighbours looks.
 // (A neighbour's word may already carry its own bits when read: the
 // coordinates are decoded through masks, so that does not matter.)
-__device__ __forceinline__ void c1_line_flags_body(int n, int bits, uint32_t* pk, int bid, int nblk) {
+// `colors`: the colours that were taken into C1 order with their codes (rgb null: none).
+__device__ __forceinline__ void c1_line_flags_body(int n, int bits, uint32_t* pk, const ColorArgs& colors, int bid,
+                                                   int nblk) {
   for (int k = bid * blockDim.x + threadIdx.x; k < n; k += nblk * blockDim.x) {
     const uint32_t c = pk[k] & kCoordMask;
     const bool prev_ok = k > 0 && same_scan_line(0, c, pk[k - 1], bits);
     const bool next_ok = k + 1 < n && same_scan_line(0, c, pk[k + 1], bits);
-    pk[k] = c | (prev_ok ? 0u : kNoPrevLink) | (next_ok ? 0u : kNoNextLink);
+    const uint32_t w = c | (prev_ok ? 0u : kNoPrevLink) | (next_ok ? 0u : kNoNextLink);
+    pk[k] = w;
+    if (colors.rgb && colors.pk) {
+      if (colors.dtype != 0) reinterpret_cast<uint32_t*>(colors.yf + k)[3] = w;
+      else if (colors.pc) colors.pc[k].x = w;
+    }
   }
 }
 
-__global__ void __launch_bounds__(256) k_c1_line_flags(int n, int bits, uint32_t* pk) {
+__global__ void __launch_bounds__(256) k_c1_line_flags(int n, int bits, uint32_t* pk, ColorArgs colors) {
   pdl_wait();
-  c1_line_flags_body(n, bits, pk, blockIdx.x, gridDim.x);
+  c1_line_flags_body(n, bits, pk, colors, blockIdx.x, gridDim.x);
 }
 
 __global__ void __launch_bounds__(256) k_c1_line_flags_seg(const __grid_constant__ Seg<LinkArgs> s) {
   pdl_wait();
   const int f = seg_frame(s, blockIdx.x);
-  c1_line_flags_body(s.a[f].n, s.a[f].bits, s.a[f].pk, blockIdx.x - s.start[f], s.start[f + 1] - s.start[f]);
+  c1_line_flags_body(s.a[f].n, s.a[f].bits, s.a[f].pk, s.a[f].colors, blockIdx.x - s.start[f], s.start[f + 1] - s.start[f]);
 }
 
 // Windows w > 1 (Section 2.2 with w points linked on each side): one thread
@@ -1143,7 +1150,7 @@ cudaError_t launch_link(int n, int bits, int cap, bool same_line, const GraphBuf
   const cudaError_t e = launch_kernel(k_link<true>, dim3(gx, 3), dim3(kLinkThreads), 0, stream, false, la);
   if (e != cudaSuccess) return e;
   return launch_kernel(k_c1_line_flags, dim3(line_flag_blocks(n, num_sms)), dim3(256), 0, stream, false, n, bits,
-                       gb.pk);
+                       gb.pk, colors);
 }
 
 // ---- segmented (one launch over the frames of a batch)
@@ -1202,7 +1209,7 @@ cudaError_t launch_link_wide(int n, int bits, int cap, int window, bool same_lin
                                       gb.cx, gb.cx_stride, sc);
   if (e != cudaSuccess || !same_line) return e;
   return launch_kernel(k_c1_line_flags, dim3(std::min((n + 255) / 256, num_sms * 8)), dim3(256), 0, stream, false, n,
-                       bits, gb.pk);
+                       bits, gb.pk, colors);
 }
 
 cudaError_t launch_node_sigma(int n, int bits, const GraphBufs& gb, DevScalars* sc, int num_sms, cudaStream_t stream) {
