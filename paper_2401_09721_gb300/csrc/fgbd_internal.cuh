@@ -244,6 +244,7 @@ struct MomentArgs {
   float* spread;
   double* f64_partials;
   int sorted_patches;
+  int per_sm;        // blocks of the launch on an SM, where they fill the GPU (else 1)
   struct DevScalars* sc;
 };
 struct ZeroArgs {

@@ -21,7 +21,7 @@ __global__ void __launch_bounds__(kFilterThreads, 2) k_filter(FilterArgs a) {
   }
   __syncthreads();
   uint32_t epoch = 0;
-  select_filter<kFilterThreads, NX>(a, s_S, 0, gridDim.x, &a.sc->barrier, epoch);
+  select_filter<kFilterThreads, NX>(a, s_S, 0, gridDim.x, &a.sc->barrier, epoch, 2);
 }
 
 // Segmented (window 1): frame f's blocks [start[f], start[f + 1]) select and
@@ -38,7 +38,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_filter_seg(const __
   }
   __syncthreads();
   uint32_t epoch = 0;
-  select_filter<THREADS, 0>(a, s_S, s.start[f], uint32_t(s.start[f + 1] - s.start[f]), &a.sc->barrier, epoch);
+  select_filter<THREADS, 0>(a, s_S, s.start[f], uint32_t(s.start[f + 1] - s.start[f]), &a.sc->barrier, epoch, 1);
 }
 
 __global__ void __launch_bounds__(256) k_output(FilterArgs a) {

@@ -111,27 +111,43 @@ __device__ __forceinline__ float block_cexp(const DevScalars* sc, float* s_cexp)
 }
 
 // What a step at sorted point k reads before its neighbours: the point's own
-// previous iterate (x_0 built from the colours when src is null) and its C2/C3
+// previous iterate (wider windows: x_0 built from the colours when src is null) and its C2/C3
 // slots.
 struct StepHead {
   float4 xk;
   int4 s;
 };
 
-// An iterate of an earlier step: through L1 (kL1) where every line this SM
-// could hold was final before the launch first read it - the stored steps of
-// the noise-estimate launch, each writing a slice of its own that is only read
-// after the next grid barrier - else from L2 (ping-pong buffers rewritten
-// within one launch, whose stale L1 lines another SM could still hold).
-template <bool kL1>
-__device__ __forceinline__ float4 ld_iterate(const float4* __restrict__ p) {
-  if constexpr (kL1) return __ldca(p);
-  else return __ldcg(p);
+// An iterate of an earlier step, through L1.  It was written by other blocks of
+// this launch or before it: the grid barrier between the steps orders the writes
+// before these loads (release by the writers' thread 0 after its block's barrier,
+// acquire by the readers' thread 0 before theirs; the acquire also drops the
+// lines this SM's L1 holds).  volatile: not moved across the barrier.
+__device__ __forceinline__ float4 ld_iterate(const float4* p) {
+  float4 v;
+  asm volatile("ld.global.ca.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
 }
 
-template <bool kL1 = false>
-__device__ __forceinline__ StepHead step_head(const FilterArgs& a, const float4* __restrict__ src, int k) {
-  return {src ? ld_iterate<kL1>(&src[k]) : x0_of(a, k), a.c4[k]};
+// (the slots are read once a step: from L2, they would only push iterates out of L1)
+__device__ __forceinline__ StepHead step_head(const FilterArgs& a, const float4* src, int k) {
+  return {src ? ld_iterate(&src[k]) : x0_of(a, k), __ldcg(&a.c4[k])};
+}
+
+// The sorted points a block of a step takes: block b of `members` one run of
+// consecutive points, whose neighbours along C1, C2 and mostly C3 (some thousand
+// positions away) lie in the same run and so in the L1 of this SM.  Blocks b and
+// b + members / per_sm, which usually share an SM, take runs side by side.  With
+// blocks taking turns every 1024 points a step moved 6.2 L2 sectors a point, with
+// runs 5.0 (16 frames of 20k-100k points: three stored steps 70 -> 60 us, the
+// selection's steps 111 -> 92 us; 1M points: no change by itself, the steps are bound
+// by latency and instructions there).
+__device__ __forceinline__ int2 step_run(int n, int b, int members, int per_sm) {
+  const int sms = members / per_sm;
+  const int c = per_sm > 1 && sms * per_sm == members ? (b % sms) * per_sm + b / sms : b;
+  const int len = ((n + members - 1) / members + 31) & ~31;
+  const int lo = min(n, c * len);
+  return make_int2(lo, min(n, lo + len));
 }
 
 // The six window-1 slots of sorted point k (C1 k - 1, k + 1, then the C2/C3
@@ -155,16 +171,21 @@ __device__ __forceinline__ void slots6(int k, int n, uint32_t wk, int4 s, int (&
 // neighbours (C1 k - 1, k + 1, the C2/C3 slots), with the weights of Eq. 4
 // normalised by their sum, w_j = e_j / sum_i e_i, e_j = exp(-(d2_j - min d2) /
 // sigma_g^2) (the pair reading: d2_j / (sigma_k sigma_j) in the exponent), from
-// the previous iterate `src` (x_0 built from the colours when src is null;
-// h = step_head(a, src, k)).  A point without neighbours keeps x_k.
+// the previous iterate `src` (h = step_head(a, src, k)).  A point without
+// neighbours keeps x_k.
 // The weights depend on the graph and sigma_g only, so they are computed once:
 // kStore (step 1) computes them and, where a.w4 is set, stores them; the later
 // steps of the same graph load them (kStore false with a.w4 set).  Every kernel
 // that takes a window-1 step uses this function, so a step gives the same bits
 // in all of them.
-template <bool kStore, bool kL1 = false>
-__device__ __forceinline__ float4 eq5_step(const FilterArgs& a, const float4* __restrict__ src, int k, int n,
-                                           float cexp, const StepHead& h) {
+// An empty slot reads the point's own iterate with weight 0, which adds nothing:
+// no predicates on the six loads and their sums.  Only where the own colour is
+// not finite would 0 x_k not be 0; a sum that is not finite is formed again
+// without the empty slots.  (1M points: the launch with three stored steps 48.6 ->
+// 44.7 us.)
+template <bool kStore>
+__device__ __forceinline__ float4 eq5_step(const FilterArgs& a, const float4* src, int k, int n, float cexp,
+                                           const StepHead& h) {
   const float4 xk = h.xk;
   const uint32_t wk = __float_as_uint(xk.w);  // packed code and the missing-C1-link bits
   int nb[6];
@@ -172,7 +193,7 @@ __device__ __forceinline__ float4 eq5_step(const FilterArgs& a, const float4* __
   slots6(k, n, wk, h.s, nb, v);
   float4 xn[6];
 #pragma unroll
-  for (int j = 0; j < 6; ++j) xn[j] = v[j] ? (src ? ld_iterate<kL1>(&src[nb[j]]) : x0_of(a, nb[j])) : xk;
+  for (int j = 0; j < 6; ++j) xn[j] = ld_iterate(src + (v[j] ? nb[j] : k));
   float w[6];
   if (kStore || !a.w4) {
     const uint32_t ck = wk & kCoordMask;
@@ -229,18 +250,25 @@ __device__ __forceinline__ float4 eq5_step(const FilterArgs& a, const float4* __
     w[5] = wb.y;
   }
   float sr = 0.f, sgc = 0.f, sb = 0.f;
-  bool any = false;
 #pragma unroll
   for (int j = 0; j < 6; ++j) {
-    if (v[j]) {
-      sr = fmaf(w[j], xn[j].x, sr);
-      sgc = fmaf(w[j], xn[j].y, sgc);
-      sb = fmaf(w[j], xn[j].z, sb);
-      any = true;
+    sr = fmaf(w[j], xn[j].x, sr);
+    sgc = fmaf(w[j], xn[j].y, sgc);
+    sb = fmaf(w[j], xn[j].z, sb);
+  }
+  if (!(fabsf(sr) + fabsf(sgc) + fabsf(sb) <= 3.0e38f)) {
+    sr = sgc = sb = 0.f;
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+      if (v[j]) {
+        sr = fmaf(w[j], xn[j].x, sr);
+        sgc = fmaf(w[j], xn[j].y, sgc);
+        sb = fmaf(w[j], xn[j].z, sb);
+      }
     }
   }
   float4 xo = xk;
-  if (any) {
+  if (v[0] || v[1] || v[2] || v[3] || v[4] || v[5]) {
     xo.x = 0.5f * xk.x + 0.5f * sr;
     xo.y = 0.5f * xk.y + 0.5f * sgc;
     xo.z = 0.5f * xk.z + 0.5f * sb;
@@ -269,7 +297,7 @@ __device__ __forceinline__ void slot_group(const FilterArgs& a, int k, int n, ui
 // together: a first pass finds min d2 from the packed codes, a second
 // accumulates.
 template <int NX>
-__device__ __forceinline__ float4 eq5_step_wide(const FilterArgs& a, const float4* __restrict__ src, int k, int n,
+__device__ __forceinline__ float4 eq5_step_wide(const FilterArgs& a, const float4* src, int k, int n,
                                                 float cexp, const StepHead& h) {
   const float4 xk = h.xk;
   const uint32_t wk = __float_as_uint(xk.w);
@@ -295,7 +323,7 @@ __device__ __forceinline__ float4 eq5_step_wide(const FilterArgs& a, const float
     float4 xo[6];
 #pragma unroll
     for (int i = 0; i < 6; ++i)
-      xo[i] = o[i] >= 0 ? (src ? __ldcg(&src[o[i]]) : x0_of(a, o[i])) : xk;
+      xo[i] = o[i] >= 0 ? (src ? ld_iterate(&src[o[i]]) : x0_of(a, o[i])) : xk;
 #pragma unroll
     for (int i = 0; i < 6; ++i) {
       if (o[i] < 0) continue;
@@ -319,7 +347,7 @@ __device__ __forceinline__ float4 eq5_step_wide(const FilterArgs& a, const float
 
 // one Eq. 5 step at window 1 (NX = 0) or wider
 template <int NX, bool kStore>
-__device__ __forceinline__ float4 eq5_step_nx(const FilterArgs& a, const float4* __restrict__ src, int k, int n,
+__device__ __forceinline__ float4 eq5_step_nx(const FilterArgs& a, const float4* src, int k, int n,
                                               float cexp, const StepHead& h) {
   if constexpr (NX == 0) return eq5_step<kStore>(a, src, k, n, cexp, h);
   else return eq5_step_wide<NX>(a, src, k, n, cexp, h);
@@ -338,10 +366,11 @@ __device__ __forceinline__ int speculative_steps(const FilterArgs& a, int depth,
                                                  bool until_sigma, uint32_t& epoch, int* s_ok, float* s_cexp,
                                                  int* s_go) {
   const int n = a.n;
-  const int gtid = (blockIdx.x - first) * blockDim.x + threadIdx.x;
-  const int gstride = int(members) * blockDim.x;
+  const int2 run = step_run(n, int(blockIdx.x) - first, int(members), 1);
+  const int stride = int(blockDim.x);
   DevScalars* sc = a.sc;
   const float cexp = block_cexp(sc, s_cexp);
+  if (!a.x0) depth = 0;  // (there is an x_0 whenever the moments were taken)
   int stored = depth;
   for (int t = 1; t <= depth; ++t) {
     const float4* src = t == 1 ? a.x0 : a.spec_x + size_t(t - 2) * size_t(a.cap);
@@ -349,13 +378,13 @@ __device__ __forceinline__ int speculative_steps(const FilterArgs& a, int depth,
     int32_t* z = a.spec_z + size_t(t - 1) * size_t(a.cap);
     // each point's own iterate and slots are loaded one trip ahead, so that
     // only the neighbour loads wait on the point before them
+    const int k0 = run.x + int(threadIdx.x);
     StepHead next{};
-    if (gtid < n) next = step_head<true>(a, src, gtid);
-    for (int k = gtid; k < n; k += gstride) {
+    if (k0 < run.y) next = step_head(a, src, k0);
+    for (int k = k0; k < run.y; k += stride) {
       const StepHead h = next;
-      if (k + gstride < n) next = step_head<true>(a, src, k + gstride);
-      const float4 xo =
-          t == 1 ? eq5_step<true, true>(a, src, k, n, cexp, h) : eq5_step<false, true>(a, src, k, n, cexp, h);
+      if (k + stride < run.y) next = step_head(a, src, k + stride);
+      const float4 xo = t == 1 ? eq5_step<true>(a, src, k, n, cexp, h) : eq5_step<false>(a, src, k, n, cexp, h);
       dst[k] = xo;
       z[k] = int32_t(sq3(xo));
     }
@@ -373,7 +402,7 @@ __device__ __forceinline__ int speculative_steps(const FilterArgs& a, int depth,
       }
     }
   }
-  if (gtid == 0) sc->spec_done = stored;
+  if (int(blockIdx.x) == first && threadIdx.x == 0) sc->spec_done = stored;
   return stored;
 }
 

@@ -273,11 +273,14 @@ __device__ __forceinline__ void ne_moments_body(const MomentArgs& ma, int bid, i
   float* atf = &s_atf[DT == 1 ? warp : 0][0];
   const uint32_t hbase = uint32_t(__cvta_generic_to_shared(ath));
 
-  const int nwarps = nblk * kNeWarps;
-  for (int base = (bid * kNeWarps + warp) * 32; base < n; base += nwarps * 32) {
+  // uint8: each block takes a run of consecutive points, whose neighbours then lie in
+  // this SM's L1 (step_run); float: the blocks take turns, as their sums always did
+  const int2 run = DT == 0 ? step_run(n, bid, nblk, ma.per_sm) : make_int2(bid * kNeThreads, n);
+  const int stride = DT == 0 ? kNeThreads : nblk * kNeThreads;
+  for (int base = run.x + warp * 32; base < run.y; base += stride) {
     const int k = base + lane;
     bool has = false;
-    if (k < n) has = DT == 0 ? point_patch_u8(ma, k, lane, ath) : point_patch_f32(ma, k, lane, atf);
+    if (k < run.y) has = DT == 0 ? point_patch_u8(ma, k, lane, ath) : point_patch_f32(ma, k, lane, atf);
     if (!has) {
       if (DT == 0) {
         uint2* row = reinterpret_cast<uint2*>(ath + lane * kHRow);
@@ -638,14 +641,13 @@ __global__ void __launch_bounds__(kFinThreads) k_ne_finalize(int dtype, const do
   finalize_block(dtype, f64_partials, nblocks, sc, sigma_out);
 }
 
-// One block per SM (the dynamic shared memory keeps a second one out): block 0
-// computes sigma_est on an SM of its own, the others meanwhile take the first
+// One block per SM (1024 threads of 64 registers fill its register file, so the
+// rest of the SM's memory is L1 for the steps): block 0 computes sigma_est on an SM of its own, the others meanwhile take the first
 // filter steps, which need the graph and the colours only.  With a.fuse they
 // then also select and filter: they stop stepping once sigma_est is published
 // (or after kSpecMax steps, then waiting for it) and run the selection over
 // the stored steps (select_filter), so no second launch follows.
 constexpr int kSpecThreads = 1024;
-constexpr int kSpecPadBytes = 100 * 1024;  // shared memory that makes a second block not fit on an SM
 
 // FUSE: the selection and filter follow in the same launch (a.fuse); a kernel
 // of its own, so that the plain launch carries none of their registers.
@@ -681,7 +683,7 @@ __global__ void __launch_bounds__(kSpecThreads, 1)
   }
   __syncthreads();
   if (!s_ok) return;
-  select_filter<kSpecThreads>(a, S, 1, gridDim.x - 1, &sc->spec_barrier, epoch);
+  select_filter<kSpecThreads>(a, S, 1, gridDim.x - 1, &sc->spec_barrier, epoch, 1);
 }
 
 // Segmented estimate launch (one block per SM, cooperative): block f < count
@@ -758,11 +760,6 @@ cudaError_t launch_ne_moments_seg(const MomentArgs* a, int count, int dtype, int
 cudaError_t launch_ne_finalize_seg(const FilterArgs* spec, const double* const* f64_partials, const int* nblocks,
                                    int count, int num_sms, cudaStream_t stream) {
   if (count < 1 || count > kSegMax || num_sms < 2 * count) return cudaErrorInvalidValue;
-  static std::atomic<unsigned long long> configured{0};  // the shared-memory limit is set once per device
-  cudaError_t e = once_per_device(configured, [] {
-    return cudaFuncSetAttribute(k_ne_finalize_spec_seg, cudaFuncAttributeMaxDynamicSharedMemorySize, kSpecPadBytes);
-  });
-  if (e != cudaSuccess) return e;
   EstimateSeg es;
   es.count = count;
   // the step blocks in proportion to the frames' points, at least one each
@@ -782,8 +779,7 @@ cudaError_t launch_ne_finalize_seg(const FilterArgs* spec, const double* const* 
     given += b;
     es.first[f + 1] = given;
   }
-  return launch_kernel(k_ne_finalize_spec_seg, dim3(count + pool), dim3(kSpecThreads), kSpecPadBytes, stream, true,
-                       es);
+  return launch_kernel(k_ne_finalize_spec_seg, dim3(count + pool), dim3(kSpecThreads), 0, stream, true, es);
 }
 
 cudaError_t launch_gather_colors(const ColorArgs& a, int n, cudaStream_t stream) {
@@ -815,7 +811,11 @@ int ne_moment_blocks(int n, int num_sms, int dtype) {
 cudaError_t launch_ne_moments(const MomentArgs& a, int dtype, int num_sms, cudaStream_t stream) {
   if (a.n <= 0) return cudaSuccess;
   const int grid = ne_moment_blocks(a.n, num_sms, dtype);
-  if (dtype == 0) return launch_kernel(k_ne_moments<0>, dim3(grid), dim3(kNeThreads), 0, stream, false, a);
+  if (dtype == 0) {
+    MomentArgs m = a;
+    m.per_sm = grid % num_sms == 0 ? grid / num_sms : 1;
+    return launch_kernel(k_ne_moments<0>, dim3(grid), dim3(kNeThreads), 0, stream, false, m);
+  }
   return launch_kernel(k_ne_moments<1>, dim3(grid), dim3(kNeThreads), 0, stream, false, a);
 }
 
@@ -824,19 +824,10 @@ cudaError_t launch_ne_finalize(int dtype, const double* f64_partials, int nblock
   if (!spec || spec->spec_depth <= 0 || spec->n <= 0 || num_sms < 2)
     return launch_kernel(k_ne_finalize, dim3(1), dim3(kFinThreads), 0, stream, false, dtype, f64_partials, nblocks,
                          sc, sigma_out);
-  static std::atomic<unsigned long long> configured{0};  // the shared-memory limit is set once per device
-  const cudaError_t e = once_per_device(configured, [] {
-    cudaError_t r = cudaFuncSetAttribute(k_ne_finalize_spec<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         kSpecPadBytes);
-    if (r == cudaSuccess)
-      r = cudaFuncSetAttribute(k_ne_finalize_spec<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSpecPadBytes);
-    return r;
-  });
-  if (e != cudaSuccess) return e;
   if (spec->fuse)
-    return launch_kernel(k_ne_finalize_spec<true>, dim3(num_sms), dim3(kSpecThreads), kSpecPadBytes, stream, true,
+    return launch_kernel(k_ne_finalize_spec<true>, dim3(num_sms), dim3(kSpecThreads), 0, stream, true,
                          dtype, f64_partials, nblocks, sc, sigma_out, *spec);
-  return launch_kernel(k_ne_finalize_spec<false>, dim3(num_sms), dim3(kSpecThreads), kSpecPadBytes, stream, true,
+  return launch_kernel(k_ne_finalize_spec<false>, dim3(num_sms), dim3(kSpecThreads), 0, stream, true,
                        dtype, f64_partials, nblocks, sc, sigma_out, *spec);
 }
 

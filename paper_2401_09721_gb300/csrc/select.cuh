@@ -19,9 +19,9 @@
 //             the search stops at the first t with J(t) >= J(t-1), keeping
 //             q* = t-1.
 //   output    the kept iterate is gathered back to input order (optional).
-// Data written earlier in the same launch by other blocks (stored steps, the
-// iterates, keep flags, sigma_est) is read through L2 only (ld.global.cg):
-// the L1 caches of different SMs are not coherent within a grid.
+// Data written earlier in the same launch by other blocks is read after a grid
+// barrier that orders it (filter_step.cuh): the iterates through L1, what a step
+// reads once (stored steps' sums, keep flags, sigma_est) from L2.
 // Sums of squares are fixed-point integers (2^-8), so the reduction is exact
 // and independent of the order in which blocks add.  Grid barriers have a 2 s
 // wait limit; a block that gives up latches kFlagTimeout and every block
@@ -380,11 +380,12 @@ constexpr int kSums = 3 + 2 * kSpecMax;  // kept y^2, all y^2, kept count, then 
 
 // The selection and filter for the blocks [first, first + members) of a
 // cooperative grid of THREADS-thread blocks, from S stored steps (0: none),
-// grid barriers on *bar (epoch: the barriers this grid has passed on it);
+// grid barriers on *bar (epoch: the barriers this grid has passed on it), per_sm
+// blocks on an SM;
 // NX further neighbour slots per point (window w > 1: NX = 6 (w - 1)).
 template <int THREADS, int NX = 0>
 __device__ __forceinline__ void select_filter(const FilterArgs& a, int S, int first, uint32_t members,
-                                              uint32_t* bar, uint32_t& epoch) {
+                                              uint32_t* bar, uint32_t& epoch, int per_sm) {
   __shared__ unsigned long long s_red[(kSums + 1) * (THREADS / 32)];
   __shared__ int s_ok;
   const int n = a.n;
@@ -614,14 +615,15 @@ __device__ __forceinline__ void select_filter(const FilterArgs& a, int S, int fi
   const int q_limit = s_ctl[1];
   int q_final = s_ctl[2];
   const bool stopped = s_ctl[3] != 0;
+  const int2 run = step_run(n, int(blockIdx.x) - first, int(members), per_sm);
   bool copy_best = false;  // this step's source is the best iterate so far: copy it to xbest
   for (int t = S + 1; t <= q_limit && !stopped; ++t) {
-    const float4* __restrict__ src =
+    const float4* src =
         t == 1 && a.x0 ? a.x0
                        : (S > 0 && t == S + 1) ? a.spec_x + size_t(S - 1) * size_t(a.cap) : ((t & 1) ? a.xbuf0 : a.xbuf1);
-    float4* __restrict__ dst = (t & 1) ? a.xbuf1 : a.xbuf0;
+    float4* dst = (t & 1) ? a.xbuf1 : a.xbuf0;
     unsigned long long loc = 0;
-    for (int k = gtid; k < n; k += gstride) {
+    for (int k = run.x + int(threadIdx.x); k < run.y; k += THREADS) {
       const StepHead h = step_head(a, src, k);
       const float4 xo =
           t == 1 ? eq5_step_nx<NX, true>(a, src, k, n, cexp, h) : eq5_step_nx<NX, false>(a, src, k, n, cexp, h);
