@@ -440,7 +440,8 @@ __device__ void eig_tail(const double* __restrict__ S, const float* __restrict__
   __shared__ TridiagSmem<D, kFinThreads> tw;
   __shared__ long long s_key[D];
   __shared__ double s_sorted[D];
-  __shared__ double s_num[D][D];
+  constexpr int PR = (D + 1) / 2;  // pairs of rows (r, D - 1 - r)
+  __shared__ double s_num[D][PR], s_den[D][PR];
   __shared__ double V64[D][D + 1];
   const int tid = threadIdx.x;
 
@@ -448,20 +449,30 @@ __device__ void eig_tail(const double* __restrict__ S, const float* __restrict__
   // multisection and inverse iteration (tridiag.cuh)
   eig_vectors_f32<D, kFinThreads>(Sf, tw, V, s_mu, FinBar{});
 
-  // float64 Rayleigh quotients of the eigenvector estimates.  float64 has a
-  // long latency here, so the sums run as three interleaved chains.
+  // float64 Rayleigh quotients of the eigenvector estimates.  This GPU has few
+  // float64 lanes, so the numerators use the symmetry: v^T S v = sum_r v_r (S_rr
+  // v_r + 2 sum_{c > r} S_rc v_c), a thread for rows r and D - 1 - r of one
+  // vector, D - 1 off-diagonal terms whichever r (7500 -> 3700 cycles).
   for (int e = tid; e < D * D; e += kFinThreads) V64[e / D][e % D] = double(V[e]);
   fin_bar();
-  for (int e = tid; e < D * D; e += kFinThreads) {
-    const int k = e / D, r = e % D;
-    double w0 = 0.0, w1 = 0.0, w2 = 0.0;
-#pragma unroll
-    for (int c = 0; c < D; c += 3) {
-      w0 = fma(S[r * D + c], V64[c][k], w0);
-      if (c + 1 < D) w1 = fma(S[r * D + c + 1], V64[c + 1][k], w1);
-      if (c + 2 < D) w2 = fma(S[r * D + c + 2], V64[c + 2][k], w2);
+  static_assert(D * PR <= kFinThreads && (D & 1), "one pair a thread; the middle row pairs with itself");
+  if (tid < D * PR) {
+    const int k = tid / PR, r1 = tid % PR, r2 = D - 1 - r1;
+    const int n1 = D - 1 - r1, total = r2 > r1 ? D - 1 : n1;
+    double acc = 0.0, t1 = 0.0;
+#pragma unroll 4
+    for (int i = 0; i < D - 1; ++i) {
+      if (i == n1) {
+        t1 = acc;
+        acc = 0.0;
+      }
+      const int r = i < n1 ? r1 : r2, c = i < n1 ? r1 + 1 + i : r2 + 1 + (i - n1);
+      if (i < total) acc = fma(S[r * D + c], V64[c][k], acc);
     }
-    s_num[k][r] = (w0 + w1 + w2) * V64[r][k];
+    const double t2 = n1 < D - 1 ? acc : 0.0, v1 = V64[r1][k], v2 = r2 > r1 ? V64[r2][k] : 0.0;
+    if (n1 == D - 1) t1 = acc;
+    s_num[k][r1] = v1 * fma(2.0, t1, S[r1 * D + r1] * v1) + v2 * fma(2.0, t2, S[r2 * D + r2] * v2);
+    s_den[k][r1] = fma(v1, v1, v2 * v2);
   }
   fin_bar();
   // the rest runs in warp 0, lane j < D holding eigenvalue j
@@ -470,21 +481,17 @@ __device__ void eig_tail(const double* __restrict__ S, const float* __restrict__
     const int lane = tid;
     double lam = 0.0;
     if (lane < D) {
-      double n0 = 0.0, n1 = 0.0, n2 = 0.0, d0 = 0.0, d1 = 0.0, d2 = 0.0;
+      double n0 = 0.0, n1 = 0.0, d0 = 0.0, d1 = 0.0;
 #pragma unroll
-      for (int r = 0; r < D; r += 3) {
+      for (int r = 0; r < PR; r += 2) {
         n0 += s_num[lane][r];
-        d0 = fma(V64[r][lane], V64[r][lane], d0);
-        if (r + 1 < D) {
+        d0 += s_den[lane][r];
+        if (r + 1 < PR) {
           n1 += s_num[lane][r + 1];
-          d1 = fma(V64[r + 1][lane], V64[r + 1][lane], d1);
-        }
-        if (r + 2 < D) {
-          n2 += s_num[lane][r + 2];
-          d2 = fma(V64[r + 2][lane], V64[r + 2][lane], d2);
+          d1 += s_den[lane][r + 1];
         }
       }
-      lam = div_newton(n0 + n1 + n2, d0 + d1 + d2);
+      lam = div_newton(n0 + n1, d0 + d1);
       if (!isfinite(lam)) lam = double(s_mu[lane]);
     }
     // eigenvalues below 1e-9 max(lambda_1, 1) are numerical zeros (a rank-deficient
@@ -600,15 +607,23 @@ __device__ __noinline__ void finalize_block(int dtype, const double* __restrict_
     return;
   }
   if (!sc->pooled_patch) {
-    // Sigma = S2/N - mu mu^T (upper triangle accumulated; mirror it)
-    const double inv_n = 1.0 / npd;
-    for (int e = tid; e < kD * kD; e += kFinThreads) {
-      const int r = e / kD, c = e % kD;
-      const int rr = min(r, c), cc = max(r, c);
-      const double mr = s_sum[kD * kD + rr] * inv_n, mc = s_sum[kD * kD + cc] * inv_n;
-      const double v = s_sum[rr * kD + cc] * inv_n - mr * mc;
-      S[e] = v;
-      Sf[e] = float(v);
+    // Sigma = S2/N - mu mu^T: the upper triangle, one entry a thread, mirrored; 1/N
+    // from one warp (a float64 division in every warp is 2500 cycles here)
+    __shared__ double s_inv;
+    if (tid == 0) s_inv = div_newton(1.0, npd);
+    fin_bar();
+    const double inv_n = s_inv;
+    static_assert(kD * (kD + 1) / 2 <= kFinThreads, "one entry a thread");
+    if (tid < kD * (kD + 1) / 2) {
+      int r = 0, rest = tid;
+      while (rest >= kD - r) {
+        rest -= kD - r;
+        ++r;
+      }
+      const int c = r + rest;
+      const double v = fma(s_sum[r * kD + c], inv_n, -(s_sum[kD * kD + r] * inv_n) * (s_sum[kD * kD + c] * inv_n));
+      S[r * kD + c] = S[c * kD + r] = v;
+      Sf[r * kD + c] = Sf[c * kD + r] = float(v);
     }
     fin_bar();
     eig_tail<kD>(S, Sf, sc, sigma_out, dtype);

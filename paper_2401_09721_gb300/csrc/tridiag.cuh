@@ -7,13 +7,12 @@
 // eigenvalues far inside the noise estimate's tolerance.  The vectors come
 // from the textbook route for a small dense symmetric matrix, in float32:
 //   1. Householder reduction to tridiagonal form T = Q^T A Q (D - 2
-//      reflections H_k = I - u_k u_k^T / h_k), the rows of A in registers:
-//      for D <= 32 spread over the block's warps (lane j holds column j), so
-//      the products of each step are warp reductions side by side; for
-//      larger D in one warp;
+//      reflections H_k = I - u_k u_k^T / h_k) in one warp, a column of A in a
+//      lane's registers (two for D > 32);
 //   2. the eigenvalues of T by Sturm-count multisection (every participating
-//      thread counts at its own point, so each pass narrows every bracket at
-//      once; no iteration depends on convergence);
+//      thread counts the sign changes of the leading minors at its own point, so
+//      each pass narrows every bracket at once; no iteration depends on
+//      convergence);
 //   3. one eigenvector of T per eigenvalue by two steps of inverse iteration
 //      (an LDL^T solve of T - mu I), one thread each;
 //   4. back to A's basis: v = H_0 H_1 ... H_{D-3} z.
@@ -32,33 +31,51 @@ namespace {
 template <int D, int NT>
 struct TridiagSmem {
   static constexpr int kPer = NT / D;  // multisection points per eigenvalue and pass
-  float U[D > 2 ? D - 2 : 1][D];       // reflection vectors u_k (rows)
-  float h[D];                          // and their h_k = |u_k|^2 / 2 (0: no reflection)
-  float d[D], e[D], e2[D];             // T: diagonal, off-diagonal e_i = T[i][i+1], e_i^2
-  float rk[D + 1], su[D], sq[D];       // row k of A (and |x|^2), u and q: broadcast copies in the reduction
+  static constexpr int kPad = (D + 3) / 4 * 4;
+  alignas(16) float U[D > 2 ? D - 2 : 1][kPad];  // reflection vectors u_k (rows)
+  alignas(16) float sx[kPad], sp[kPad];          // the step's x and p: broadcast copies in the reduction
+  float ih[D];                         // 1 / h_k, h_k = |u_k|^2 / 2 (0: no reflection)
+  float d[D], e[D];                    // T: diagonal, off-diagonal e_i = T[i][i+1]
+  float ds[D], e2s[D];                 // d_i and e_i^2 of T scaled by 2^-k to a size of one
   float2 br[D];                        // brackets (lo, hi] of the eigenvalues, ascending order
   float x[NT];                         // multisection points of one pass
   int cnt[NT];                         // their Sturm counts
   float P[D][D];                       // inverse iteration: reciprocal LDL^T pivots, [i][eigenvalue]
   float bounds[2];                     // Gershgorin interval of T
   float scale;                         // max |A_ii|: the size of the matrix
+  float shrink;                        // the 2^-k above
 };
 
-// number of eigenvalues of T below x (the LDL^T pivots of T - x I that are
-// negative); a pivot smaller than pivmin in magnitude is taken as -pivmin
+// Number of eigenvalues of T below x, as the sign changes of the leading minors
+// of T - x I, p_i = (d_i - x) p_{i-1} - e_{i-1}^2 p_{i-2} (Sturm's sequence): two
+// dependent operations a row where the pivots' recurrence has a division (82
+// cycles a row).  T and x come scaled to a size of one, and the pair of minors is
+// scaled by a power of two every four rows, so that neither leaves float32's
+// range.  A minor that is exactly zero counts one change with the two beside it,
+// whatever its sign; the e_i^2 are at least 1e-16 (a change of T below the float32
+// rounding of its size), so the pair stays above 1e-32 over four rows, never both zero.
 template <int D>
-__device__ __forceinline__ int sturm_count(const float* __restrict__ d, const float* __restrict__ e2, float x,
-                                           float pivmin) {
-  float q = d[0] - x;
-  if (fabsf(q) < pivmin) q = -pivmin;
-  int c = q < 0.f;
+__device__ __forceinline__ int sturm_count(const float* __restrict__ d, const float* __restrict__ e2, float x) {
+  float p = d[0] - x, pp = 1.f;
+  uint32_t c = __float_as_uint(p) >> 31;
+#pragma unroll 1
+  for (int i0 = 1; i0 < D; i0 += 4) {
 #pragma unroll
-  for (int i = 1; i < D; ++i) {
-    q = (d[i] - x) - __fdividef(e2[i - 1], q);
-    if (fabsf(q) < pivmin) q = -pivmin;
-    c += q < 0.f;
+    for (int i = i0; i < i0 + 4; ++i) {
+      if (i < D) {
+        const float q = fmaf(d[i] - x, p, -(e2[i - 1] * pp));
+        c += (__float_as_uint(q) ^ __float_as_uint(p)) >> 31;
+        pp = p;
+        p = q;
+      }
+    }
+    // the larger of the two to [1, 2)
+    const int ex = int((__float_as_uint(fmaxf(fabsf(p), fabsf(pp))) >> 23) & 255u);
+    const float f = __uint_as_float(uint32_t(min(max(254 - ex, 1), 254)) << 23);
+    p *= f;
+    pp *= f;
   }
-  return c;
+  return int(c);
 }
 
 // passes of the bracket multisection until every bracket is below 2^-24 of
@@ -94,227 +111,150 @@ __device__ void eig_vectors_f32(const float* __restrict__ As, TridiagSmem<D, NT>
   const int lane = tid & 31;
   constexpr unsigned kFull = 0xffffffffu;
 
-  // ---- 1. Householder reduction.  D <= 32: every warp of the block holds
-  // rows of A (row i in warp i mod W, lane j its column j), so each step's
-  // products are warp reductions running side by side, with two barriers a
-  // step; D > 32: warp 0 alone, a row of A a lane (two for D > 32).
-  if constexpr (D <= 32) {
-    constexpr int W = (NT / 32) < D ? (NT / 32) : D;  // warps holding rows
-    constexpr int RPW = (D + W - 1) / W;              // rows a warp holds
-    const int warp = tid >> 5;
-    float a[RPW];
+  // ---- 1. Householder reduction, in warp 0.  Lane j holds column j of A from
+  // row k down (the registers move up one row a step).  Step k reads row k as
+  // column k below the diagonal; x reaches every lane through shared memory,
+  // every lane then forms |x|^2, and beside that chain its A x; u = x - alpha e_1
+  // with alpha = -sign(x_0) |x| gives A u = A x - alpha A e_1.  A second exchange
+  // hands p = A u / h to every lane, which forms u^T p itself: no warp reduction
+  // and two exchanges a step (870 cycles at D = 21; rows spread over twelve warps with
+  // warp reductions and block barriers took 1100).
+  if (tid < 32) {
+    float a[R][D];
 #pragma unroll
-    for (int r = 0; r < RPW; ++r) {
-      const int row = warp + r * W;
-      a[r] = (warp < W && row < D && lane < D) ? As[row * D + lane] : 0.f;
+    for (int r = 0; r < R; ++r) {
+      const int col = r * 32 + lane;
+#pragma unroll
+      for (int i = 0; i < D; ++i) a[r][i] = col < D ? As[i * D + col] : 0.f;
     }
     float scale = 0.f;
-    for (int j = 0; j < D; ++j) scale = fmaxf(scale, fabsf(As[j * D + j]));
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int col = r * 32 + lane;
+      if (col < D) scale = fmaxf(scale, fabsf(As[col * D + col]));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) scale = fmaxf(scale, __shfl_xor_sync(kFull, scale, o));
     const float skip = 1e-12f * scale;  // a column below this size is taken as already reduced
+    constexpr int N = D - 1;            // entries of x: rows k + 1 .., zero behind the last
+    constexpr int Q = (N + 3) / 4;
+    // (behind the last entry the copies hold zeros up to their padding)
+    for (int i = lane; i < TridiagSmem<D, NT>::kPad; i += 32) w.sx[i] = w.sp[i] = 0.f;
+    __syncwarp();
+    // entry i of a vector over the columns below k, zero behind the last column
+    const auto publish = [&](float* to, int k, const float (&val)[R]) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int col = r * 32 + lane;
+        if (col < D) to[col > k ? col - k - 1 : D - 1 - k + col] = col > k ? val[r] : 0.f;  // (all of 0 .. D - 1)
+      }
+    };
 #pragma unroll 1
     for (int k = 0; k + 2 < D; ++k) {
-      // the owner of row k (= column k below the diagonal, A being symmetric)
-      // forms u = x - alpha e_1 with alpha = -sign(x_0) |x|, so |u|^2 = 2 h
-      if (warp == k % W) {
-        float ak = 0.f;
+      float own[R];
 #pragma unroll
-        for (int r = 0; r < RPW; ++r)
-          if (r == k / W) ak = a[r];
-        const float v = lane > k && lane < D ? ak : 0.f;
-        float xs = v * v;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) xs += __shfl_xor_sync(kFull, xs, o);
-        const float x0 = __shfl_sync(kFull, v, k + 1);
-        const float nx = sqrtf(xs);
-        const bool reflect = nx > skip && xs > 0.f;  // warp-uniform
-        const float alpha = x0 > 0.f ? -nx : nx;
-        const float h = reflect ? fmaf(-x0, alpha, xs) : 0.f;
-        const float u = !reflect ? 0.f : (lane == k + 1 ? x0 - alpha : v);
-        if (lane < D) {
-          w.U[k][lane] = u;
-          w.su[lane] = u;
-        }
-        if (lane == 0) w.h[k] = h;
-      }
-      bar();
-      const float h = w.h[k];
-      if (!(h > 0.f)) continue;  // the same for every thread
-      const float uj = lane < D ? w.su[lane] : 0.f;
-      const float ih = __frcp_rn(h);
-      // p_i = (A u)_i / h for this warp's rows
-      float p[RPW];
-#pragma unroll
-      for (int r = 0; r < RPW; ++r) {
-        float t = a[r] * uj;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(kFull, t, o);
-        p[r] = t * ih;
-        const int row = warp + r * W;
-        if (lane == 0 && warp < W && row < D) w.sq[row] = p[r];
-      }
-      bar();
-      // K = u^T p / (2 h), q = p - K u, A <- A - u q^T - q u^T
-      const float pj = lane < D ? w.sq[lane] : 0.f;
-      float up = uj * pj;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) up += __shfl_xor_sync(kFull, up, o);
-      const float K = 0.5f * up * ih;
-      const float qj = fmaf(-K, uj, pj);
-#pragma unroll
-      for (int r = 0; r < RPW; ++r) {
-        const int row = warp + r * W;
-        const float ui = __shfl_sync(kFull, uj, row & 31);
-        const float qi = fmaf(-K, ui, p[r]);
-        a[r] = fmaf(-ui, qj, fmaf(-qi, uj, a[r]));
-      }
-    }
-    // T: diagonal and first off-diagonal, from the owners of the rows
-#pragma unroll
-    for (int r = 0; r < RPW; ++r) {
-      const int row = warp + r * W;
-      const float nxt = __shfl_down_sync(kFull, a[r], 1);  // the entry right of lane's
-      if (warp < W && row < D && lane == row) {
-        w.d[row] = a[r];
-        if (row + 1 < D) {
-          w.e[row] = nxt;
-          w.e2[row] = nxt * nxt;
-        }
-      }
-    }
-    if (tid == 0) {
-      w.e[D - 1] = 0.f;
-      w.e2[D - 1] = 0.f;
-      w.scale = scale;
-    }
-    bar();
-  }
-  if (tid < 32) {
-    if constexpr (D > 32) {
-      float a[R][D];
-      float scale = 0.f;
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const int row = r * 32 + lane;
-#pragma unroll
-        for (int j = 0; j < D; ++j) a[r][j] = row < D ? As[row * D + j] : 0.f;
-#pragma unroll
-        for (int j = 0; j < D; ++j)
-          if (row == j) scale = fmaxf(scale, fabsf(a[r][j]));
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) scale = fmaxf(scale, __shfl_xor_sync(kFull, scale, o));
-      const float skip = 1e-12f * scale;  // a column below this size is taken as already reduced
-#pragma unroll 1
-      for (int k = 0; k + 2 < D; ++k) {
-        // column k of A, below the diagonal, read as row k (A is symmetric):
-        // its owner lane publishes the row and |x|^2
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-          if (r * 32 + lane == k) {
-            float t0 = 0.f, t1 = 0.f;
-#pragma unroll
-            for (int j = 0; j < D; ++j) {
-              w.rk[j] = a[r][j];
-              const float v = j > k ? a[r][j] : 0.f;
-              if (j & 1) t1 = fmaf(v, v, t1);
-              else t0 = fmaf(v, v, t0);
-            }
-            w.rk[D] = t0 + t1;
-          }
-        }
-        __syncwarp();
-        float xv[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-          const int row = r * 32 + lane;
-          xv[r] = (row > k && row < D) ? w.rk[row] : 0.f;
-        }
-        const float xs = w.rk[D];
-        const float x0 = w.rk[k + 1];
-        const float nx = sqrtf(xs);
-        const bool reflect = nx > skip && xs > 0.f;  // warp-uniform
-        // u = x - alpha e_1 with alpha = -sign(x_0) |x|, so |u|^2 = 2 (|x|^2 + |x_0| |x|)
-        const float alpha = x0 > 0.f ? -nx : nx;
-        const float h = reflect ? fmaf(-x0, alpha, xs) : 0.f;
-        float u[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-          const int row = r * 32 + lane;
-          u[r] = !reflect ? 0.f : (row == k + 1 ? x0 - alpha : (row > k + 1 ? xv[r] : 0.f));
-          if (row < D) {
-            w.U[k][row] = u[r];
-            w.su[row] = u[r];
-          }
-        }
-        if (lane == 0) w.h[k] = h;
-        __syncwarp();
-        if (reflect) {
-          // p = A u / h, K = u^T p / (2 h), q = p - K u, A <- A - u q^T - q u^T
-          const float ih = __frcp_rn(h);
-          float p[R];
-#pragma unroll
-          for (int r = 0; r < R; ++r) {
-            const int row = r * 32 + lane;
-            float s0 = 0.f, s1 = 0.f, s2 = 0.f;
-#pragma unroll
-            for (int j = 0; j < D; j += 3) {
-              s0 = fmaf(a[r][j], w.su[j], s0);
-              if (j + 1 < D) s1 = fmaf(a[r][j + 1], w.su[j + 1], s1);
-              if (j + 2 < D) s2 = fmaf(a[r][j + 2], w.su[j + 2], s2);
-            }
-            p[r] = (s0 + s1 + s2) * ih;
-            if (row < D) w.sq[row] = p[r];
-          }
-          __syncwarp();
-          // u^T p, summed by every lane from the broadcast copies (no shuffle chain)
-          float up0 = 0.f, up1 = 0.f, up2 = 0.f;
-#pragma unroll
-          for (int j = 0; j < D; j += 3) {
-            up0 = fmaf(w.su[j], w.sq[j], up0);
-            if (j + 1 < D) up1 = fmaf(w.su[j + 1], w.sq[j + 1], up1);
-            if (j + 2 < D) up2 = fmaf(w.su[j + 2], w.sq[j + 2], up2);
-          }
-          const float up = up0 + up1 + up2;
-          __syncwarp();
-          const float K = 0.5f * up * ih;
-          float q[R];
-#pragma unroll
-          for (int r = 0; r < R; ++r) {
-            const int row = r * 32 + lane;
-            q[r] = fmaf(-K, u[r], p[r]);
-            if (row < D) w.sq[row] = q[r];
-          }
-          __syncwarp();
-#pragma unroll
-          for (int r = 0; r < R; ++r) {
-#pragma unroll
-            for (int j = 0; j < D; ++j) a[r][j] = fmaf(-u[r], w.sq[j], fmaf(-q[r], w.su[j], a[r][j]));
-          }
-        }
-        __syncwarp();
-      }
-      // T: diagonal and first off-diagonal
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const int row = r * 32 + lane;
-#pragma unroll
-        for (int j = 0; j < D; ++j) {
-          if (row == j) {
-            w.d[j] = a[r][j];
-            if (j + 1 < D) {
-              w.e[j] = a[r][j + 1];
-              w.e2[j] = a[r][j + 1] * a[r][j + 1];
-            }
-          }
-        }
-      }
-      if (lane == 0) {
-        w.e[D - 1] = 0.f;
-        w.e2[D - 1] = 0.f;
-        w.scale = scale;
-      }
+      for (int r = 0; r < R; ++r) own[r] = a[r][0];
+      publish(w.sx, k, own);
       __syncwarp();
+      // (x is read again below: the columns leave no registers for it)
+      const float4* sx = reinterpret_cast<const float4*>(w.sx);
+      float s4[4] = {0.f, 0.f, 0.f, 0.f}, p[R], t4[R][4];
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int l = 0; l < 4; ++l) t4[r][l] = 0.f;
+#pragma unroll
+      for (int i = 0; i < Q; ++i) {
+        const float4 c4 = sx[i];
+        const float c[4] = {c4.x, c4.y, c4.z, c4.w};
+#pragma unroll
+        for (int l = 0; l < 4; ++l) {
+          if (4 * i + l >= N) continue;
+          s4[l] = fmaf(c[l], c[l], s4[l]);
+#pragma unroll
+          for (int r = 0; r < R; ++r) t4[r][l] = fmaf(a[r][4 * i + l + 1], c[l], t4[r][l]);
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < R; ++r) p[r] = (t4[r][0] + t4[r][1]) + (t4[r][2] + t4[r][3]);
+      const float xs = (s4[0] + s4[1]) + (s4[2] + s4[3]);
+      const float x0 = w.sx[0];
+      // (the approximate root: a reflection to a few float32 roundings either way; xs = 0: NaN, no reflection)
+      const float nx = xs * rsqrtf(xs);
+      const bool reflect = nx > skip && xs > 0.f;  // the same for every lane
+      const float alpha = x0 > 0.f ? -nx : nx;
+      const float ih = reflect ? __frcp_rn(fmaf(-x0, alpha, xs)) : 0.f;
+      const float u0 = x0 - alpha;
+      float u[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int col = r * 32 + lane;
+        u[r] = !reflect || col <= k ? 0.f : (col == k + 1 ? u0 : own[r]);
+        if (col < D) w.U[k][col] = u[r];
+        if (col == k) {
+          w.d[k] = own[r];
+          w.e[k] = reflect ? alpha : x0;
+          w.ih[k] = ih;
+        }
+        p[r] = fmaf(-alpha, a[r][1], p[r]) * ih;
+      }
+      if (reflect) {
+        publish(w.sp, k, p);
+        __syncwarp();
+        // K = u^T p / (2 h), q = p - K u, A <- A - u q^T - q u^T
+        float v4[4] = {0.f, 0.f, 0.f, 0.f};
+        const float4* sp = reinterpret_cast<const float4*>(w.sp);
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+          const float4 t = sp[i], c = sx[i];
+          v4[0] = fmaf(i == 0 ? u0 : c.x, t.x, v4[0]);
+          v4[1] = fmaf(c.y, t.y, v4[1]);
+          v4[2] = fmaf(c.z, t.z, v4[2]);
+          v4[3] = fmaf(c.w, t.w, v4[3]);
+        }
+        const float K = 0.5f * ((v4[0] + v4[1]) + (v4[2] + v4[3])) * ih;
+        float qc[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) qc[r] = fmaf(-K, u[r], p[r]);
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+          const float4 pv = sp[i], xv = sx[i];
+          const float t[4] = {pv.x, pv.y, pv.z, pv.w}, c[4] = {i == 0 ? u0 : xv.x, xv.y, xv.z, xv.w};
+#pragma unroll
+          for (int l = 0; l < 4; ++l) {
+            if (4 * i + l >= N) continue;
+            const float q = fmaf(-K, c[l], t[l]);
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+              a[r][4 * i + l] = fmaf(-c[l], qc[r], fmaf(-q, u[r], a[r][4 * i + l + 1]));
+          }
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) a[r][D - 1] = 0.f;
+        __syncwarp();  // x and p have been read
+      } else {
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+#pragma unroll
+          for (int i = 0; i < N; ++i) a[r][i] = a[r][i + 1];
+          a[r][D - 1] = 0.f;
+        }
+        __syncwarp();  // x has been read
+      }
     }
+    // the last two rows
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int col = r * 32 + lane;
+      if (col == D - 2) w.d[D - 2] = a[r][0];
+      if (col == D - 1) {
+        w.e[D - 2] = a[r][0];
+        w.d[D - 1] = a[r][1];
+        w.e[D - 1] = 0.f;
+      }
+    }
+    if (lane == 0) w.scale = scale;
+    __syncwarp();
     // Gershgorin interval of T
     float glo = 3.0e38f, ghi = -3.0e38f;
     for (int i = lane; i < D; i += 32) {
@@ -328,9 +268,18 @@ __device__ void eig_vectors_f32(const float* __restrict__ As, TridiagSmem<D, NT>
       ghi = fmaxf(ghi, __shfl_xor_sync(kFull, ghi, o));
     }
     const float pad = 1e-6f * fmaxf(fabsf(glo), fabsf(ghi)) + 1e-30f;
+    // 2^-k of the interval's larger end: T and the points scaled by it have a size of one
+    const int ex = int((__float_as_uint(fmaxf(fabsf(glo - pad), fabsf(ghi + pad))) >> 23) & 255u);
+    const float shrink = __uint_as_float(uint32_t(min(max(254 - ex, 1), 254)) << 23);
     if (lane == 0) {
       w.bounds[0] = glo - pad;
       w.bounds[1] = ghi + pad;
+      w.shrink = shrink;
+    }
+    for (int i = lane; i < D; i += 32) {
+      const float es = w.e[i] * shrink;
+      w.ds[i] = w.d[i] * shrink;
+      w.e2s[i] = fmaxf(es * es, 1e-16f);
     }
     for (int i = lane; i < D; i += 32) w.br[i] = make_float2(glo - pad, ghi + pad);
   }
@@ -344,10 +293,7 @@ __device__ void eig_vectors_f32(const float* __restrict__ As, TridiagSmem<D, NT>
     bar();
     return;
   }
-  float emax2 = 0.f;
-#pragma unroll
-  for (int i = 0; i + 1 < D; ++i) emax2 = fmaxf(emax2, w.e2[i]);
-  const float pivmin = 1e-30f * fmaxf(1.f, emax2);
+  const float shrink = w.shrink;
 
   // ---- 2. multisection.  Pass 0 counts at NT points across the whole
   // interval; a crossing between points t - 1 and t brackets the eigenvalues
@@ -358,7 +304,7 @@ __device__ void eig_vectors_f32(const float* __restrict__ As, TridiagSmem<D, NT>
     const float lo = w.bounds[0], hi = w.bounds[1];
     const float x = lo + (hi - lo) * (float(tid + 1) / float(NT + 1));
     w.x[tid] = x;
-    w.cnt[tid] = sturm_count<D>(w.d, w.e2, x, pivmin);
+    w.cnt[tid] = sturm_count<D>(w.ds, w.e2s, x * shrink);
   }
   bar();
   {
@@ -381,7 +327,7 @@ __device__ void eig_vectors_f32(const float* __restrict__ As, TridiagSmem<D, NT>
       b = w.br[sk];
       const float x = b.x + (b.y - b.x) * (float(sj + 1) / float(kPer + 1));
       w.x[tid] = x;
-      w.cnt[tid] = sturm_count<D>(w.d, w.e2, x, pivmin);
+      w.cnt[tid] = sturm_count<D>(w.ds, w.e2s, x * shrink);
     }
     bar();
     if (sect) {
@@ -453,9 +399,17 @@ __device__ void eig_vectors_f32(const float* __restrict__ As, TridiagSmem<D, NT>
     // products run over all D entries
 #pragma unroll 1
     for (int s = D - 3; s >= 0; --s) {
-      const float hs = w.h[s];
-      if (!(hs > 0.f)) continue;
-      const float* us = w.U[s];
+      const float ih = w.ih[s];
+      if (!(ih > 0.f)) continue;
+      float us[(D + 3) / 4 * 4];
+#pragma unroll
+      for (int i = 0; i < (D + 3) / 4; ++i) {
+        const float4 t = reinterpret_cast<const float4*>(w.U[s])[i];
+        us[4 * i] = t.x;
+        us[4 * i + 1] = t.y;
+        us[4 * i + 2] = t.z;
+        us[4 * i + 3] = t.w;
+      }
       float t0 = 0.f, t1 = 0.f, t2 = 0.f;
 #pragma unroll
       for (int i = 0; i < D; i += 3) {
@@ -463,7 +417,7 @@ __device__ void eig_vectors_f32(const float* __restrict__ As, TridiagSmem<D, NT>
         if (i + 1 < D) t1 = fmaf(us[i + 1], z[i + 1], t1);
         if (i + 2 < D) t2 = fmaf(us[i + 2], z[i + 2], t2);
       }
-      const float c = (t0 + t1 + t2) * __frcp_rn(hs);
+      const float c = (t0 + t1 + t2) * ih;
 #pragma unroll
       for (int i = 0; i < D; ++i) z[i] = fmaf(-c, us[i], z[i]);
     }
