@@ -342,7 +342,7 @@ fgbd_status fgbd_set_batch_shape(int32_t device, int64_t mean_points, const fgbd
  *   sigma:      weight bandwidth; 0 means sigma_g of the graph.
  *   checkpoint: keep every checkpoint-th iterate for the backward call and
  *               recompute the others there (0 or 1: keep all); memory about
- *               (100 + 16 (q / checkpoint + checkpoint + 1)) bytes per point,
+ *               (88 + 16 (q / checkpoint + checkpoint + 1)) bytes per point,
  *               allocated on the first call that needs more (that call
  *               synchronises the device).
  * The call records q, alpha, sigma for fgbd_filter_backward.

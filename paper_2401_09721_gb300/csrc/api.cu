@@ -67,7 +67,7 @@ struct fgbd_ctx {
   float4* d_ckpt = nullptr;   // x_0, x_c, x_2c, ... (c = checkpoint interval)
   float4* d_seg = nullptr;    // x_{t0+1} .. x_{t0+c-1} of one segment (backward)
   float4* d_pp[2] = {};       // ping-pong for steps and for the adjoint
-  double* d_part = nullptr;   // per step and block: dL/dalpha, dL/dsigma terms
+  double2* d_part = nullptr;   // per block: dL/dalpha, dL/dsigma sums
   int d_q = -1, d_c = 1, d_n = 0, d_grid = 0;
   float d_alpha = 0.5f;
   double d_sigma = 0.0;
@@ -298,10 +298,10 @@ int filter_grid_for(const fgbd_ctx* ctx, int n) {
 fgbd_status diff_workspace(fgbd_ctx* ctx, int n, int q, int c, int grid) {
   const size_t N = size_t(std::max(n, 1));
   const size_t nck = size_t(q / c + 1);
-  const size_t sizes[] = {N * kK * 4, N * kK * 4, N * kK * 4, N * kK * 4, N * 4,  // nb, R, RT, d2, e
-                          nck * N * 16, size_t(c > 1 ? c - 1 : 1) * N * 16,     // checkpoints, segment
-                          N * 16, N * 16,                                       // ping-pong
-                          size_t(std::max(q, 1)) * size_t(grid) * 2 * 8};       // partials
+  const size_t sizes[] = {N * 8, N * 16, N * 16, N * 8, N * 16, N * 8, N * 16,  // rows (DiffBufs)
+                          nck * N * 16, size_t(c > 1 ? c - 1 : 1) * N * 16,    // checkpoints, segment
+                          N * 16, N * 16,                                      // ping-pong
+                          size_t(grid) * 16};                                  // partials
   size_t total = 0;
   for (size_t b : sizes) total = align_up(total, 256) + b;
   total = align_up(total, 256);
@@ -321,22 +321,20 @@ fgbd_status diff_workspace(fgbd_ctx* ctx, int n, int q, int c, int grid) {
   }
   char* base = static_cast<char*>(ctx->dmem);
   size_t off = 0;
-  void* ptrs[10];
-  for (int k = 0; k < 10; ++k) {
+  void* ptrs[12];
+  for (int k = 0; k < 12; ++k) {
     off = align_up(off, 256);
     ptrs[k] = base + off;
     off += sizes[k];
   }
-  ctx->db.nb = static_cast<int32_t*>(ptrs[0]);
-  ctx->db.R = static_cast<float*>(ptrs[1]);
-  ctx->db.RT = static_cast<float*>(ptrs[2]);
-  ctx->db.d2 = static_cast<float*>(ptrs[3]);
-  ctx->db.e = static_cast<float*>(ptrs[4]);
-  ctx->d_ckpt = static_cast<float4*>(ptrs[5]);
-  ctx->d_seg = static_cast<float4*>(ptrs[6]);
-  ctx->d_pp[0] = static_cast<float4*>(ptrs[7]);
-  ctx->d_pp[1] = static_cast<float4*>(ptrs[8]);
-  ctx->d_part = static_cast<double*>(ptrs[9]);
+  ctx->db = DiffBufs{static_cast<float2*>(ptrs[0]), static_cast<float4*>(ptrs[1]), static_cast<int4*>(ptrs[2]),
+                     static_cast<float2*>(ptrs[3]), static_cast<float4*>(ptrs[4]), static_cast<float2*>(ptrs[5]),
+                     static_cast<float4*>(ptrs[6])};
+  ctx->d_ckpt = static_cast<float4*>(ptrs[7]);
+  ctx->d_seg = static_cast<float4*>(ptrs[8]);
+  ctx->d_pp[0] = static_cast<float4*>(ptrs[9]);
+  ctx->d_pp[1] = static_cast<float4*>(ptrs[10]);
+  ctx->d_part = static_cast<double2*>(ptrs[11]);
   return FGBD_OK;
 }
 
@@ -1386,16 +1384,17 @@ fgbd_status fgbd_filter_forward(fgbd_ctx* ctx, const float* rgb_in, int32_t q, d
   if (ws != FGBD_OK) return ws;
   const float a = float(alpha);
   if (n > 0) {
-    FGBD_LAUNCH(ctx, "diff_rows", st, launch_diff_rows(n, ctx->params.bits, sigma, ctx->gb, ctx->sc, ctx->db,
-                                                       ctx->num_sms, st));
-    FGBD_LAUNCH(ctx, "diff_gather", st, launch_diff_gather(n, rgb_in, ctx->gb.perm1, ctx->d_ckpt, ctx->num_sms, st));
+    FGBD_LAUNCH(ctx, "diff_rows", st, launch_diff_rows(n, ctx->params.bits, sigma, rgb_in, ctx->gb, ctx->sc, ctx->db,
+                                                       ctx->d_ckpt, ctx->num_sms, st));
     const float4* cur = ctx->d_ckpt;
     for (int t = 0; t < q; ++t) {
       float4* dst = ((t + 1) % c == 0) ? ctx->d_ckpt + size_t((t + 1) / c) * size_t(n) : ctx->d_pp[(t + 1) & 1];
-      FGBD_LAUNCH(ctx, "diff_step", st, launch_diff_step(n, a, ctx->db, cur, dst, ctx->num_sms, st));
+      FGBD_LAUNCH(ctx, "diff_step", st, launch_diff_step(n, a, ctx->gb, ctx->db, cur, dst,
+                                                         t + 1 == q ? rgb_out : nullptr, ctx->num_sms, st));
       cur = dst;
     }
-    FGBD_LAUNCH(ctx, "diff_scatter", st, launch_diff_scatter(n, cur, ctx->gb.perm1, rgb_out, ctx->num_sms, st));
+    if (q == 0)
+      FGBD_LAUNCH(ctx, "diff_scatter", st, launch_diff_scatter(n, cur, ctx->gb.perm1, rgb_out, ctx->num_sms, st));
   }
   ctx->d_q = q;
   ctx->d_c = c;
@@ -1422,7 +1421,8 @@ fgbd_status fgbd_filter_backward(fgbd_ctx* ctx, const float* grad_out, float* gr
   const float a = ctx->d_alpha;
   int parts = 0;
   if (n > 0) {
-    FGBD_LAUNCH(ctx, "diff_gather", st, launch_diff_gather(n, grad_out, ctx->gb.perm1, ctx->d_pp[0], ctx->num_sms, st));
+    FGBD_LAUNCH(ctx, "diff_rows_t", st, launch_diff_rows_t(n, ctx->params.bits, ctx->d_sigma, grad_out, ctx->gb,
+                                                           ctx->sc, ctx->db, ctx->d_pp[0], ctx->num_sms, st));
     int ui = 0;
     int seg_t0 = -1;  // first step of the segment held in d_seg
     for (int t = q - 1; t >= 0; --t) {
@@ -1436,7 +1436,7 @@ fgbd_status fgbd_filter_backward(fgbd_ctx* ctx, const float* grad_out, float* gr
           const float4* cur = ctx->d_ckpt + size_t(t0 / c) * size_t(n);
           for (int s = t0; s < t; ++s) {
             float4* dst = ctx->d_seg + size_t(s - t0) * size_t(n);
-            FGBD_LAUNCH(ctx, "diff_step", st, launch_diff_step(n, a, ctx->db, cur, dst, ctx->num_sms, st));
+            FGBD_LAUNCH(ctx, "diff_step", st, launch_diff_step(n, a, ctx->gb, ctx->db, cur, dst, nullptr, ctx->num_sms, st));
             cur = dst;
           }
           seg_t0 = t0;
@@ -1444,14 +1444,15 @@ fgbd_status fgbd_filter_backward(fgbd_ctx* ctx, const float* grad_out, float* gr
         xt = ctx->d_seg + size_t(t - t0 - 1) * size_t(n);
       }
       FGBD_LAUNCH(ctx, "diff_back_step", st,
-                  launch_diff_back_step(n, a, ctx->d_sigma, ctx->db, xt, ctx->d_pp[ui], ctx->d_pp[ui ^ 1], ctx->sc,
-                                        ctx->d_part + size_t(t) * size_t(grid) * 2, ctx->num_sms, st));
+                  launch_diff_back_step(n, a, t == q - 1, ctx->gb, ctx->db, xt, ctx->d_pp[ui], ctx->d_pp[ui ^ 1],
+                                        t == 0 ? grad_in : nullptr, ctx->d_part, ctx->num_sms, st));
       ui ^= 1;
     }
-    FGBD_LAUNCH(ctx, "diff_scatter", st, launch_diff_scatter(n, ctx->d_pp[ui], ctx->gb.perm1, grad_in, ctx->num_sms, st));
-    parts = q * grid;
+    if (q == 0)
+      FGBD_LAUNCH(ctx, "diff_scatter", st, launch_diff_scatter(n, ctx->d_pp[0], ctx->gb.perm1, grad_in, ctx->num_sms, st));
+    parts = q > 0 ? grid : 0;
   }
-  FGBD_LAUNCH(ctx, "diff_reduce", st, launch_diff_reduce(parts, ctx->d_part, grad_params, st));
+  FGBD_LAUNCH(ctx, "diff_reduce", st, launch_diff_reduce(parts, a, ctx->d_sigma, ctx->sc, ctx->d_part, grad_params, st));
   return FGBD_OK;
 }
 

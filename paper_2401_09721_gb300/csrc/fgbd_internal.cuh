@@ -394,26 +394,30 @@ cudaError_t launch_filter_seg(const FilterArgs* a, int count, int threads, int f
 int filter_seg_max_per_sm(int threads);  // resident blocks per SM of that kernel
 
 // Differentiable filter: rows of R = D^-1 W for given alpha, sigma, and their transpose
-struct DiffBufs {
-  int32_t* nb;  // [n][6] neighbour ids (sorted order), -1 unused
-  float* R;     // [n][6] R_ij
-  float* RT;    // [n][6] R_ji: weight of i in the row of its t-th neighbour
-  float* d2;    // [n][6] squared distances
-  float* e;     // [n] sum_j R_ij d_ij^2
+struct DiffBufs {  // one value a neighbour slot: C1 (i - 1, i + 1) in the float2, C2/C3 in the float4
+  float2* r2;   // [n] R_ij; -1: no neighbour
+  float4* r4;   // [n]
+  int4* rec;    // [n] packed code, smallest squared distance, 1 / sum of weights (bits)
+  float2* rt2;  // [n] R_ji: weight of i in the row of its neighbour (backward)
+  float4* rt4;  // [n]
+  float2* g2;   // [n] R_ij (d_ij^2 - sum_k R_ik d_ik^2) (backward)
+  float4* g4;   // [n]
 };
 int diff_grid(int n, int num_sms);
-cudaError_t launch_diff_rows(int n, int bits, double sigma, const GraphBufs& gb, const DevScalars* sc,
-                             const DiffBufs& db, int num_sms, cudaStream_t stream);
-cudaError_t launch_diff_gather(int n, const float* rgb, const int32_t* perm1, float4* x, int num_sms,
-                               cudaStream_t stream);
+cudaError_t launch_diff_rows(int n, int bits, double sigma, const float* rgb, const GraphBufs& gb,
+                             const DevScalars* sc, const DiffBufs& db, float4* x, int num_sms, cudaStream_t stream);
+cudaError_t launch_diff_rows_t(int n, int bits, double sigma, const float* grad, const GraphBufs& gb,
+                               const DevScalars* sc, const DiffBufs& db, float4* u, int num_sms, cudaStream_t stream);
 cudaError_t launch_diff_scatter(int n, const float4* x, const int32_t* perm1, float* out, int num_sms,
                                 cudaStream_t stream);
-cudaError_t launch_diff_step(int n, float alpha, const DiffBufs& db, const float4* src, float4* dst, int num_sms,
-                             cudaStream_t stream);
-cudaError_t launch_diff_back_step(int n, float alpha, double sigma, const DiffBufs& db, const float4* x,
-                                  const float4* u, float4* u_out, const DevScalars* sc, double* partial,
+// out / grad_in: the result in input order (the last step), or null
+cudaError_t launch_diff_step(int n, float alpha, const GraphBufs& gb, const DiffBufs& db, const float4* src,
+                             float4* dst, float* out, int num_sms, cudaStream_t stream);
+cudaError_t launch_diff_back_step(int n, float alpha, bool first, const GraphBufs& gb, const DiffBufs& db,
+                                  const float4* x, const float4* u, float4* u_out, float* grad_in, double2* partial,
                                   int num_sms, cudaStream_t stream);
-cudaError_t launch_diff_reduce(int count, const double* partial, double* grad, cudaStream_t stream);
+cudaError_t launch_diff_reduce(int count, float alpha, double sigma, const DevScalars* sc, const double2* partial,
+                               double* grad, cudaStream_t stream);
 
 // CSR export in input order
 cudaError_t launch_csr_degree(int n, const GraphBufs& gb, int64_t* deg_out, cudaStream_t stream);
