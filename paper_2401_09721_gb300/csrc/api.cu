@@ -1559,10 +1559,9 @@ fgbd_status fgbd_graph_csr_copy(fgbd_ctx* ctx, int64_t* row_ptr, int32_t* col, f
   if (!row_ptr) return FGBD_OK;
   if (col_capacity < *nnz_host || (*nnz_host > 0 && !col)) return FGBD_EINVAL;
   const int n = ctx->n;
-  FGBD_LAUNCH(ctx, "csr_degree", st, launch_csr_degree(n, ctx->gb, row_ptr, st));
-  FGBD_LAUNCH(ctx, "csr_scan", st, launch_scan_i64(row_ptr, int64_t(n) + 1, ctx->scan_tmp, st));
-  FGBD_LAUNCH(ctx, "csr_fill", st,
-              launch_csr_fill(n, ctx->params.bits, ctx->gb, row_ptr, col, w, col_capacity, ctx->sc, st));
+  FGBD_LAUNCH(ctx, "csr_row_ptr", st, launch_csr_row_ptr(n, ctx->gb, row_ptr, ctx->scan_tmp, ctx->sc, st));
+  FGBD_LAUNCH(ctx, "csr_fill", st, launch_csr_fill(n, ctx->params.bits, ctx->gb, row_ptr, ctx->scan_tmp, col, w,
+                                                   col_capacity, ctx->sc, st));
   FGBD_CUDA(ctx, cudaStreamSynchronize(st));
   return FGBD_OK;
 }
@@ -1603,16 +1602,12 @@ fgbd_status fgbd_graph_export(fgbd_ctx* ctx, fgbd_graph** out, void* stream) {
   const int n = ctx->n;
   cudaError_t e = cudaSuccess;
   {
-    LaunchScope s1(ctx, "csr_degree", st);
-    e = launch_csr_degree(n, ctx->gb, gr->row_ptr, st);
+    LaunchScope s1(ctx, "csr_row_ptr", st);
+    e = launch_csr_row_ptr(n, ctx->gb, gr->row_ptr, ctx->scan_tmp, ctx->sc, st);
   }
   if (e == cudaSuccess) {
-    LaunchScope s2(ctx, "csr_scan", st);
-    e = launch_scan_i64(gr->row_ptr, int64_t(n) + 1, ctx->scan_tmp, st);
-  }
-  if (e == cudaSuccess) {
-    LaunchScope s3(ctx, "csr_fill", st);
-    e = launch_csr_fill(n, ctx->params.bits, ctx->gb, gr->row_ptr, gr->col, gr->w, gr->nnz, ctx->sc, st);
+    LaunchScope s2(ctx, "csr_fill", st);
+    e = launch_csr_fill(n, ctx->params.bits, ctx->gb, gr->row_ptr, ctx->scan_tmp, gr->col, gr->w, gr->nnz, ctx->sc, st);
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) {

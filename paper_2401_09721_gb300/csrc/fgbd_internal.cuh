@@ -420,10 +420,11 @@ cudaError_t launch_diff_reduce(int count, float alpha, double sigma, const DevSc
                                double* grad, cudaStream_t stream);
 
 // CSR export in input order
-cudaError_t launch_csr_degree(int n, const GraphBufs& gb, int64_t* deg_out, cudaStream_t stream);
-cudaError_t launch_scan_i64(int64_t* data, int64_t count, int64_t* block_tmp, cudaStream_t stream);
-cudaError_t launch_csr_fill(int n, int bits, const GraphBufs& gb, const int64_t* row_ptr, int32_t* col,
-                            float* w, int64_t col_capacity, const DevScalars* sc, cudaStream_t stream);
+// row_ptr[0..n]; block_tmp: a word per 1024 rows and one more, which the fill reads
+cudaError_t launch_csr_row_ptr(int n, const GraphBufs& gb, int64_t* row_ptr, int64_t* block_tmp,
+                               const DevScalars* sc, cudaStream_t stream);
+cudaError_t launch_csr_fill(int n, int bits, const GraphBufs& gb, const int64_t* row_ptr, const int64_t* block_tmp,
+                            int32_t* col, float* w, int64_t col_capacity, const DevScalars* sc, cudaStream_t stream);
 cudaError_t launch_spread_export(int n, const int2* rank12, const float* spread, const uint8_t* keep8,
                                  float* spread_out, uint8_t* keep_out, cudaStream_t stream);
 
