@@ -426,10 +426,14 @@ class GraphFilter(torch.autograd.Function):
         if getattr(context, "_diff_token", None) != fctx.token:
             raise RuntimeError("the context ran another filter forward since this one; backward needs its state")
         grad_in = torch.empty_like(grad_out)
-        gp = torch.zeros(2, dtype=torch.float64, device=grad_out.device)
+        gp = torch.empty(2, dtype=torch.float64, device=grad_out.device)
         fgbd_filter_backward(context.handle, grad_out.contiguous(), grad_in, gp, context.n)
-        like = lambda v, m: None if m is None else v.to(device=m[0], dtype=m[1]).reshape(m[2])
-        ga, gs = like(gp[0], fctx.alpha_meta), like(gp[1], fctx.sigma_meta)
+        metas = (fctx.alpha_meta, fctx.sigma_meta)
+        # one copy, and so one wait, for the parameters on the host
+        host = gp.cpu() if any(m is not None and m[0].type == "cpu" for m in metas) else None
+        like = lambda k, m: None if m is None else (
+            (host if m[0].type == "cpu" else gp)[k].to(device=m[0], dtype=m[1]).reshape(m[2]))
+        ga, gs = like(0, metas[0]), like(1, metas[1])
         return grad_in, ga, gs, None, None, None
 
 
