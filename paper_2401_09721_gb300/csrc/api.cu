@@ -74,8 +74,8 @@ struct fgbd_ctx {
   uint64_t d_gen = 0;
   bool d_valid = false;
   // filter steps stored by the noise-estimate launch (see filter_step.cuh)
-  float4* spec_x = nullptr;   // [kSpecMax][cap]
-  int32_t* spec_z = nullptr;  // [kSpecMax][cap]
+  float4* spec_x = nullptr;   // [spec_rows(cap)][cap]
+  int32_t* spec_z = nullptr;  // [spec_rows(cap)][cap]
   uint8_t* keep8 = nullptr;   // [cap]
   int spec_depth = 0;         // steps stored for noise_rgb on the current graph (0: none)
   // fgbd_run replays: CUDA graphs of whole runs, keyed by their arguments
@@ -449,7 +449,7 @@ fgbd_status do_estimate(fgbd_ctx* ctx, const void* rgb, int32_t dtype, double* s
   }
   // the same launch stores the first filter steps of these colours on the other SMs
   FilterArgs spec = filter_args(ctx, 0, 0, nullptr, fuse ? fuse_out : nullptr, fuse ? fuse_out_dtype : 0, dtype);
-  spec.spec_depth = speculate ? std::min(kSpecMax, int(ctx->params.q_max)) : 0;
+  spec.spec_depth = speculate ? std::min(fuse ? kSpecSure : spec_rows(ctx->capacity), int(ctx->params.q_max)) : 0;
   ctx->spec_depth = n > 0 && ctx->num_sms >= 2 ? spec.spec_depth : 0;
   const bool fused = fuse && ctx->spec_depth > 0;
   spec.fuse = fused ? 1 : 0;
@@ -618,7 +618,7 @@ fgbd_status seg_chunk(const std::vector<fgbd_ctx*>& ctxs, const std::vector<fgbd
     // the state fgbd_run's calls leave (n is set first: filter_args reads it)
     c->n = n;
     spec[f] = filter_args(c, 0, 0, nullptr, nullptr, 0, dtype);
-    spec[f].spec_depth = std::min(kSpecMax, int(c->params.q_max));
+    spec[f].spec_depth = std::min(kSpecSure, int(c->params.q_max));
     sel[f] = filter_args(c, 0, 0, nullptr, k.rgb_out, k.out_dtype, dtype);
     sel[f].spec_depth = spec[f].spec_depth;
     f64[f] = c->f64part;
@@ -875,8 +875,8 @@ fgbd_status fgbd_ctx_create(int64_t capacity, const fgbd_params* params, fgbd_ct
       {reinterpret_cast<void**>(&ctx->gb.pk), C * 4},
       {reinterpret_cast<void**>(&ctx->gb.ord23), 2 * align_up(C, 64) * 4},
       {reinterpret_cast<void**>(&ctx->gb.c4), C * 16},
-      {reinterpret_cast<void**>(&ctx->spec_x), size_t(kSpecMax) * align_up(C, 64) * 16},
-      {reinterpret_cast<void**>(&ctx->spec_z), size_t(kSpecMax) * align_up(C, 64) * 4},
+      {reinterpret_cast<void**>(&ctx->spec_x), size_t(spec_rows(int64_t(C))) * align_up(C, 64) * 16},
+      {reinterpret_cast<void**>(&ctx->spec_z), size_t(spec_rows(int64_t(C))) * align_up(C, 64) * 4},
       {reinterpret_cast<void**>(&ctx->keep8), C},
       {reinterpret_cast<void**>(&ctx->y8), C * 4},
       {reinterpret_cast<void**>(&ctx->yf), C * 16},
@@ -916,8 +916,8 @@ fgbd_status fgbd_ctx_create(int64_t capacity, const fgbd_params* params, fgbd_ct
   ctx->sb.keys_c2 = static_cast<uint32_t*>(keys0);
   ctx->sb.keys_c3 = static_cast<uint32_t*>(keys1);
   // the sort's rows and their scratch (8 + 8 bytes a point and code) lie in the
-  // three stored filter steps, which are written after the graph is built
-  static_assert(kSpecMax >= 3 && sizeof(float4) == sizeof(uint2) + 2 * sizeof(uint32_t), "one row of spec_x a code");
+  // first three stored filter steps, which are written after the graph is built
+  static_assert(kSpecSure >= 3 && sizeof(float4) == sizeof(uint2) + 2 * sizeof(uint32_t), "one row of spec_x a code");
   const size_t Ca = align_up(C, 64);
   ctx->sb.tmp_stride = int(Ca);
   for (int c = 0; c < 3; ++c) {
@@ -1215,7 +1215,7 @@ fgbd_status fgbd_run_batch(fgbd_ctx* const* ctxs, const int32_t* const* xyz, con
       const bool seg = shape.seg_frames > 0 && seg_eligible(cv, keys);
       for (int f = 0; f < count; ++f) {
         mark_run_done(ctxs[f], keys[f], bg.launches[f]);
-        if (seg) ctxs[f]->spec_depth = std::min(kSpecMax, int(ctxs[f]->params.q_max));
+        if (seg) ctxs[f]->spec_depth = std::min(kSpecSure, int(ctxs[f]->params.q_max));
       }
       return FGBD_OK;
     }

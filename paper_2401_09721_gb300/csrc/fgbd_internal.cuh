@@ -33,7 +33,16 @@ constexpr int kNeThreads = 256;
 constexpr int kNeGroup = 32;                       // float colours: moment blocks whose sums their last block adds up
 constexpr int kNeGroups = 32;                      // at most kNeGroup * kNeGroups moment blocks
 constexpr int kFilterThreads = 512;
-constexpr int kSpecMax = 3;                        // filter steps taken while sigma_est is computed
+// Filter steps taken while sigma_est is computed: kSpecSure of them whatever that
+// takes, and in contexts of up to kSpecSmall points as many as fit beside the eigen
+// step (28 us), up to kSpecMax.  A step of 20,000 points takes 3 us there, and a grid
+// barrier and as much again in the selection: with powers of 5 and 6 frames of 3,000
+// and 20,000 points take 70 and 68 us, 84 and 81 with three stored steps.  One of
+// 100,000 takes 4 us and the frames of that size stop earlier: 106 us, 104 with three.
+constexpr int kSpecSure = 3;
+constexpr int kSpecMax = 8;
+constexpr int kSpecSmall = 1 << 16;
+constexpr int spec_rows(int64_t cap) { return cap <= kSpecSmall ? kSpecMax : kSpecSure; }
 constexpr uint32_t kCoordMask = 0x3FFFFFFFu;       // low 30 bits: packed C1 code
 // The two high bits of a sorted point's packed code (pk, and x.w of an iterate)
 // mark a missing link to its C1 neighbour k - 1 / k + 1: set by the link step
@@ -70,6 +79,7 @@ struct DevScalars {
   uint32_t spec_barrier;        // grid barrier of the speculative filter steps
   int32_t spec_done;            // filter steps stored by the noise-estimate kernel
   uint32_t sigma_ready;         // set (release) once sigma_est of this estimate is written
+  uint32_t sigma_near;          // set when it is a few microseconds away: no further speculative step
   uint32_t spec_go[kSpecMax + 1];  // after stored step t: 1 to take another before selecting
   float fslr_thr[4];            // the FSLR threshold of this sigma_est as the selection uses it (once fslr_ready)
   uint32_t fslr_ready;          // set by the eigen step with sigma_est
@@ -362,8 +372,8 @@ struct FilterArgs {
   int spec_depth;          // 0: none
   const float4* x0;        // x_0 (r, g, b, packed code): float colours themselves, or as the moments launch wrote
                            // it into xbuf0; null: from y8, pk
-  float4* spec_x;          // [kSpecMax][cap]: x_1 .. x_S
-  int32_t* spec_z;         // [kSpecMax][cap]: per point sum_c x_q^2, fixed point
+  float4* spec_x;          // [spec_rows(cap)][cap]: x_1 .. x_S
+  int32_t* spec_z;         // [spec_rows(cap)][cap]: per point sum_c x_q^2, fixed point
   int cap;                 // row stride of spec_x / spec_z, a multiple of 64
   int fuse;                // noise-estimate launch: select and filter too, once sigma_est is known
   uint8_t* keep8;          // select mode: the FSLR keep flag of every sorted point

@@ -9,8 +9,9 @@
 namespace fgbd {
 namespace {
 
-// NX further neighbour slots per point: 0 at window 1, 6 (w - 1) at window w
-template <int NX>
+// NX further neighbour slots per point: 0 at window 1, 6 (w - 1) at window w;
+// DEEP: contexts that store more than kSpecSure steps
+template <int NX, bool DEEP = false>
 __global__ void __launch_bounds__(kFilterThreads, 2) k_filter(FilterArgs a) {
   pdl_wait();
   // the stored steps count only if the noise-estimate launch finished them
@@ -21,7 +22,7 @@ __global__ void __launch_bounds__(kFilterThreads, 2) k_filter(FilterArgs a) {
   }
   __syncthreads();
   uint32_t epoch = 0;
-  select_filter<kFilterThreads, NX>(a, s_S, 0, gridDim.x, &a.sc->barrier, epoch, 2);
+  select_filter<kFilterThreads, NX, DEEP>(a, s_S, 0, gridDim.x, &a.sc->barrier, epoch, 2);
 }
 
 // Segmented (window 1): frame f's blocks [start[f], start[f + 1]) select and
@@ -220,8 +221,13 @@ int filter_grid(int n, int num_sms, int nx) {
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_filter<extra_slots(3)>, kFilterThreads, 0);
   else if (nx == extra_slots(2))
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_filter<extra_slots(2)>, kFilterThreads, 0);
-  else
+  else {
+    int deep = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_filter<0>, kFilterThreads, 0);
+    if (e == cudaSuccess)
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&deep, k_filter<0, true>, kFilterThreads, 0);
+    per_sm = std::min(per_sm, deep);
+  }
   if (e != cudaSuccess || per_sm < 1) per_sm = 1;
   const int need = std::max(1, (n + kFilterThreads - 1) / kFilterThreads);
   return std::max(1, std::min(need, per_sm * num_sms));
@@ -233,6 +239,8 @@ cudaError_t launch_filter(const FilterArgs& a, int grid, cudaStream_t stream) {
   if (a.nx == extra_slots(3))
     return launch_kernel(k_filter<extra_slots(3)>, dim3(grid), dim3(kFilterThreads), 0, stream, true, a);
   if (a.nx != 0) return cudaErrorInvalidValue;
+  if (a.spec_depth > kSpecSure)
+    return launch_kernel(k_filter<0, true>, dim3(grid), dim3(kFilterThreads), 0, stream, true, a);
   return launch_kernel(k_filter<0>, dim3(grid), dim3(kFilterThreads), 0, stream, true, a);
 }
 

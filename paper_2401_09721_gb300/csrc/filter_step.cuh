@@ -357,13 +357,13 @@ __device__ __forceinline__ float4 eq5_step_nx(const FilterArgs& a, const float4*
 // fixed point (the selection subtracts these sums from those of y^2 for
 // Eq. 6), by the blocks [first, first + members) of a
 // cooperative grid (they need the graph and the colours only, not sigma_est):
-// `depth` steps, or, with `until_sigma`, fewer once sigma_est is published
-// (sc->sigma_ready).  Block `first` reads that flag before each grid barrier
-// and leaves its answer in sc->spec_go[t], which every block reads after the
+// `sure` steps, and then more, up to `depth`, until *stop is set.  Block
+// `first` reads that flag before each grid barrier and leaves its answer in
+// sc->spec_go[t], which every block reads after the
 // barrier, so all blocks stop after the same step.  sc->spec_done = the steps
 // stored; returns that number, or -1 after a barrier timeout.
 __device__ __forceinline__ int speculative_steps(const FilterArgs& a, int depth, int first, uint32_t members,
-                                                 bool until_sigma, uint32_t& epoch, int* s_ok, float* s_cexp,
+                                                 int sure, const uint32_t* stop, uint32_t& epoch, int* s_ok, float* s_cexp,
                                                  int* s_go) {
   const int n = a.n;
   const int2 run = step_run(n, int(blockIdx.x) - first, int(members), 1);
@@ -388,8 +388,8 @@ __device__ __forceinline__ int speculative_steps(const FilterArgs& a, int depth,
       dst[k] = xo;
       z[k] = int32_t(sq3(xo));
     }
-    const bool ask = until_sigma && t < depth;
-    if (ask && blockIdx.x == first && threadIdx.x == 0) sc->spec_go[t] = ld_acquire_u32(&sc->sigma_ready) ? 0u : 1u;
+    const bool ask = t >= sure && t < depth;
+    if (ask && blockIdx.x == first && threadIdx.x == 0) sc->spec_go[t] = ld_acquire_u32(stop) ? 0u : 1u;
     if (!grid_barrier(&sc->spec_barrier, &sc->status, members, epoch, s_ok, sc)) return -1;
     if (ask) {
       if (threadIdx.x == 0) *s_go = int(ld_acquire_u32(&sc->spec_go[t]));

@@ -448,6 +448,7 @@ __device__ void eig_tail(const double* __restrict__ S, const float* __restrict__
   // float32 eigenvector estimates: Householder tridiagonalisation, Sturm
   // multisection and inverse iteration (tridiag.cuh)
   eig_vectors_f32<D, kFinThreads>(Sf, tw, V, s_mu, FinBar{});
+  if (tid == 0) atomicExch(&sc->sigma_near, 1u);  // (8 us to go)
 
   // float64 Rayleigh quotients of the eigenvector estimates.  This GPU has few
   // float64 lanes, so the numerators use the symmetry: v^T S v = sum_r v_r (S_rr
@@ -602,6 +603,7 @@ __device__ __noinline__ void finalize_block(int dtype, const double* __restrict_
       sc->ne_valid = 1;
       if (sigma_out) *sigma_out = 0.0;
       __threadfence();
+      atomicExch(&sc->sigma_near, 1u);
       atomicExch(&sc->sigma_ready, 1u);
     }
     return;
@@ -679,7 +681,8 @@ __global__ void __launch_bounds__(kSpecThreads, 1)
     return;
   }
   uint32_t epoch = 0;
-  const int S = speculative_steps(a, a.spec_depth, 1, gridDim.x - 1, FUSE, epoch, &s_ok, &s_cexp, &s_go);
+  const int S = speculative_steps(a, a.spec_depth, 1, gridDim.x - 1, FUSE ? 1 : kSpecSure,
+                                  FUSE ? &sc->sigma_ready : &sc->sigma_near, epoch, &s_ok, &s_cexp, &s_go);
   if (!FUSE || S < 0) return;
   // sigma_est of block 0 (a bounded wait)
   if (threadIdx.x == 0) {
@@ -727,7 +730,7 @@ __global__ void __launch_bounds__(kSpecThreads, 1) k_ne_finalize_spec_seg(const 
   while (f + 1 < e.count && e.first[f + 1] <= b) ++f;
   uint32_t epoch = 0;
   speculative_steps(e.spec[f], e.spec[f].spec_depth, e.count + e.first[f], uint32_t(e.first[f + 1] - e.first[f]),
-                    false, epoch, &s_ok, &s_cexp, &s_go);
+                    kSpecSure, nullptr, epoch, &s_ok, &s_cexp, &s_go);
 }
 
 // testing: the float64 quotient of the eigen step beside CUDA's own division

@@ -7,7 +7,7 @@
 //             keep8; the kept power sum y^2 and the kept count are reduced, and
 //             so are the stored steps' per-point power sums x_q^2;
 //             x_0 = y is written unless it is there or steps are stored.
-//   J(1..S)   from those sums, by thread 0 of every block (the same values
+//   J(1..S)   from those sums, by warp 0 of every block (the same values
 //             everywhere: the sums are exact integers).
 //   step t    x_t = x_{t-1}/2 + (sum_j e_j x_{t-1}[j]) / (2 sum_j e_j) with
 //             e_j = exp(-(d2_j - min_j d2_j) / sigma_g^2) (eq5_step): the rows
@@ -354,39 +354,19 @@ __device__ __forceinline__ void output_quads(const FilterArgs& a, int kept, int 
   }
 }
 
-// Sums of several 64-bit values over the block (two's complement: exact in any order)
-template <int K, int THREADS>
-__device__ __forceinline__ void block_sums(unsigned long long (&v)[K], unsigned long long* s_red) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int i = 0; i < K; ++i) v[i] = warp_sum(v[i]);
-  if (lane == 0) {
-#pragma unroll
-    for (int i = 0; i < K; ++i) s_red[i * (THREADS / 32) + warp] = v[i];
-  }
-  __syncthreads();
-  if (threadIdx.x < K) {
-    unsigned long long t = 0;
-    for (int w = 0; w < THREADS / 32; ++w) t += s_red[threadIdx.x * (THREADS / 32) + w];
-    s_red[K * (THREADS / 32) + threadIdx.x] = t;
-  }
-  __syncthreads();
-#pragma unroll
-  for (int i = 0; i < K; ++i) v[i] = s_red[K * (THREADS / 32) + i];
-  __syncthreads();
-}
-
-constexpr int kSums = 3 + 2 * kSpecMax;  // kept y^2, all y^2, kept count, then per stored step kept and all x_q^2
-
 // The selection and filter for the blocks [first, first + members) of a
 // cooperative grid of THREADS-thread blocks, from S stored steps (0: none),
 // grid barriers on *bar (epoch: the barriers this grid has passed on it), per_sm
 // blocks on an SM;
 // NX further neighbour slots per point (window w > 1: NX = 6 (w - 1)).
-template <int THREADS, int NX = 0>
+// DEEP: up to kSpecMax stored steps (else kSpecSure).
+template <int THREADS, int NX = 0, bool DEEP = false>
 __device__ __forceinline__ void select_filter(const FilterArgs& a, int S, int first, uint32_t members,
                                               uint32_t* bar, uint32_t& epoch, int per_sm) {
-  __shared__ unsigned long long s_red[(kSums + 1) * (THREADS / 32)];
+  constexpr int W = THREADS / 32;
+  static_assert(kSpecMax <= W && 3 + 2 * kSpecMax <= THREADS, "a warp or more a stored step, a thread a sum");
+  constexpr int kSums = DEEP ? 5 : 3 + 2 * kSpecSure;
+  __shared__ unsigned long long s_red[kSums * W];
   __shared__ int s_ok;
   const int n = a.n;
   const int gtid = (int(blockIdx.x) - first) * THREADS + int(threadIdx.x);
@@ -417,67 +397,112 @@ __device__ __forceinline__ void select_filter(const FilterArgs& a, int S, int fi
   // ---- phase 0: keep flags and the Eq. 6 sums; x_0 = y unless the steps are stored.
   // Four consecutive points per thread and trip, read with 16-byte loads that
   // are all issued before the first is used.
+  // The stored steps' power sums follow from the same flags.  Up to kSpecSure steps:
+  // a thread takes its own quads again and holds the sums of every step.  DEEP: a
+  // few warps a step, from the flags in shared memory, and two sums a thread, so
+  // that eight steps cost as little as three (a 20,000-point frame with six or
+  // seven steps: 13 us, where taking four of them after a grid barrier each took
+  // 26).  On large frames, with two trips a block and three steps, the barriers
+  // between flags and sums cost 2 us (1M points: 23.2 -> 25.7), so they keep the first.
+  // acc: kept y^2, all y^2, kept count; then kept and all x_q^2 (DEEP: of this warp's step)
   unsigned long long acc[kSums] = {};
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const bool write_x0 = !S && !a.x0;
   const bool phase0 = select || write_x0;
-  for (int k0 = 4 * gtid; phase0 && k0 < n; k0 += 4 * gstride) {
-    const bool full = k0 + 4 <= n;
-    float4 x[4];
-    x0_quad(a, k0, full, write_x0, x);
-    float sp[4] = {0.f, 0.f, 0.f, 0.f};
-    if (select) {
-      if (full) {
-        const float4 v = *reinterpret_cast<const float4*>(a.spread + k0);
-        sp[0] = v.x;
-        sp[1] = v.y;
-        sp[2] = v.z;
-        sp[3] = v.w;
-      } else {
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-          if (k0 + i < n) sp[i] = a.spread[k0 + i];
-      }
-    }
-    if (write_x0) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        if (full || k0 + i < n) a.xbuf0[k0 + i] = x[i];
-    }
-    if (select) {
+  // (DEEP: blocks take equal runs of quads; with quads by thread number, three of
+  // four blocks of a frame below a wave would have none)
+  constexpr int kKeepTrips = DEEP ? 4 : 1;  // quads of keep flags a thread leaves between two barriers
+  __shared__ uint32_t s_keep[DEEP ? kKeepTrips * THREADS : 1];
+  const int quads = (n + 3) / 4, share = (quads + int(members) - 1) / int(members);
+  const int qa = DEEP ? min(quads, (int(blockIdx.x) - first) * share) : gtid - int(threadIdx.x);
+  const int qb = DEEP ? min(quads, qa + share) : quads;
+  const int tile = DEEP ? kKeepTrips * THREADS : int(members) * THREADS;
+  for (int qt = qa; phase0 && qt < qb; qt += tile) {
+    const int qe = DEEP ? min(qb, qt + tile) : min(qb, qt + THREADS);
+    for (int quad = qt + int(threadIdx.x); quad < qe; quad += THREADS) {
+      const int k0 = 4 * quad;
       uint32_t kw = 0;
+      const bool full = k0 + 4 <= n;
+      float4 x[4];
+      x0_quad(a, k0, full, write_x0, x);
+      float sp[4] = {0.f, 0.f, 0.f, 0.f};
+      if (select) {
+        if (full) {
+          const float4 v = *reinterpret_cast<const float4*>(a.spread + k0);
+          sp[0] = v.x;
+          sp[1] = v.y;
+          sp[2] = v.z;
+          sp[3] = v.w;
+        } else {
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        if (!full && k0 + i >= n) continue;
-        bool keep;
-        if (a.all_points || sp[i] <= t_lo) keep = true;
-        else if (sp[i] > t_hi) keep = false;
-        else keep = keep_ff_nx<NX>(a, k0 + i, thr);
-        kw |= uint32_t(keep) << (8 * i);
-        const unsigned long long q2 = sq3(x[i]);
-        acc[1] += q2;
-        if (keep) {
-          acc[0] += q2;
-          acc[2] += 1;
+          for (int i = 0; i < 4; ++i)
+            if (k0 + i < n) sp[i] = a.spread[k0 + i];
         }
       }
-      if (full) {
-        *reinterpret_cast<uint32_t*>(a.keep8 + k0) = kw;
-      } else {
+      if (write_x0) {
 #pragma unroll
         for (int i = 0; i < 4; ++i)
-          if (k0 + i < n) a.keep8[k0 + i] = uint8_t((kw >> (8 * i)) & 1u);
+          if (full || k0 + i < n) a.xbuf0[k0 + i] = x[i];
       }
+      if (select) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          if (!full && k0 + i >= n) continue;
+          bool keep;
+          if (a.all_points || sp[i] <= t_lo) keep = true;
+          else if (sp[i] > t_hi) keep = false;
+          else keep = keep_ff_nx<NX>(a, k0 + i, thr);
+          kw |= uint32_t(keep) << (8 * i);
+          const unsigned long long q2 = sq3(x[i]);
+          acc[1] += q2;
+          if (keep) {
+            acc[0] += q2;
+            acc[2] += 1;
+          }
+        }
+        if (full) {
+          *reinterpret_cast<uint32_t*>(a.keep8 + k0) = kw;
+        } else {
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (k0 + i < n) a.keep8[k0 + i] = uint8_t((kw >> (8 * i)) & 1u);
+        }
+      }
+      if constexpr (DEEP) s_keep[quad - qt] = kw;
+    }
+    if (DEEP && S > 0) {
+      const int wq = W / S;  // warps a stored step
+      __syncthreads();
+      if (warp < wq * S) {
+        const int32_t* zr = a.spec_z + size_t(warp % S) * size_t(a.cap);
+#pragma unroll 4
+        for (int quad = qt + 32 * (warp / S) + lane; quad < qe; quad += 32 * wq) {
+          const int kz = 4 * quad;
+          int4 z = make_int4(0, 0, 0, 0);
+          if (kz + 4 <= n) {
+            z = __ldcg(reinterpret_cast<const int4*>(zr + kz));
+          } else {
+            z.x = __ldcg(zr + kz);
+            if (kz + 1 < n) z.y = __ldcg(zr + kz + 1);
+            if (kz + 2 < n) z.z = __ldcg(zr + kz + 2);
+          }
+          const uint32_t f = s_keep[quad - qt];
+          acc[4] += (unsigned long long)((long long)z.x + z.y + z.z + z.w);
+          acc[3] += (unsigned long long)((long long)(f & 1u ? z.x : 0) + (f & 0x100u ? z.y : 0) +
+                                         (f & 0x10000u ? z.z : 0) + (f & 0x1000000u ? z.w : 0));
+        }
+      }
+      __syncthreads();
     }
   }
-  // the stored steps' power sums (a second pass over this thread's own points and keep flags)
-  if (S > 0) {
-    for (int k0 = 4 * gtid; k0 < n; k0 += 4 * gstride) {
+  if constexpr (!DEEP) {
+    for (int k0 = 4 * gtid; S > 0 && k0 < n; k0 += 4 * gstride) {
       const bool full = k0 + 4 <= n;
       uint32_t kw = 0;
-      int32_t z[kSpecMax][4] = {};
+      int32_t z[kSpecSure][4] = {};
       if (full) kw = *reinterpret_cast<const uint32_t*>(a.keep8 + k0);
 #pragma unroll
-      for (int q = 0; q < kSpecMax; ++q) {
+      for (int q = 0; q < kSpecSure; ++q) {
         if (q < S) {
           const int32_t* zr = a.spec_z + size_t(q) * size_t(a.cap) + k0;
           if (full) {
@@ -502,7 +527,7 @@ __device__ __forceinline__ void select_filter(const FilterArgs& a, int S, int fi
       for (int i = 0; i < 4; ++i) {
         const bool keep = (kw >> (8 * i)) & 1u;
 #pragma unroll
-        for (int q = 0; q < kSpecMax; ++q) {
+        for (int q = 0; q < kSpecSure; ++q) {
           if (q < S) {
             const unsigned long long zz = (unsigned long long)(long long)z[q][i];
             acc[4 + 2 * q] += zz;
@@ -513,18 +538,25 @@ __device__ __forceinline__ void select_filter(const FilterArgs& a, int S, int fi
     }
   }
   if (select) {
-    block_sums<kSums, THREADS>(acc, s_red);
-    if (threadIdx.x == 0) {
-      if (acc[0]) atomicAdd(&sc->ysq_keep, acc[0]);
-      if (acc[1]) atomicAdd(&sc->ysq_all, acc[1]);
-      if (acc[2]) atomicAdd(&sc->n_keep, acc[2]);
 #pragma unroll
-      for (int q = 0; q < kSpecMax; ++q) {
-        if (q < S) {
-          atomicAdd(reinterpret_cast<unsigned long long*>(&sc->spec_keep[q + 1]), acc[3 + 2 * q]);
-          atomicAdd(reinterpret_cast<unsigned long long*>(&sc->spec_all[q + 1]), acc[4 + 2 * q]);
-        }
+    for (int i = 0; i < kSums; ++i) {
+      acc[i] = warp_sum(acc[i]);
+      if (lane == 0) s_red[i * W + warp] = acc[i];
+    }
+    __syncthreads();
+    const int t = threadIdx.x;
+    if (t < 3 + 2 * S) {
+      // sum t: over the warps, or (DEEP, a stored step's) over those that took it
+      unsigned long long v = 0;
+      if (!DEEP || t < 3) {
+        for (int w = 0; w < W; ++w) v += s_red[t * W + w];
+      } else {
+        for (int w = (t - 3) >> 1; w < W / S * S; w += S) v += s_red[(4 - (t & 1)) * W + w];
       }
+      unsigned long long* to = t == 0 ? &sc->ysq_keep : t == 1 ? &sc->ysq_all : &sc->n_keep;
+      if (t >= 3)
+        to = reinterpret_cast<unsigned long long*>(t & 1 ? &sc->spec_keep[(t - 1) / 2] : &sc->spec_all[(t - 2) / 2]);
+      if (v) atomicAdd(to, v);
     }
   }
   if (phase0 && !grid_barrier(bar, &sc->status, members, epoch, &s_ok, sc)) return;
@@ -537,77 +569,78 @@ __device__ __forceinline__ void select_filter(const FilterArgs& a, int S, int fi
   __shared__ int s_ctl[6];  // keep_all, q_limit, q_final, stop, q_best, copy the last iterate
   __shared__ float s_cexp;
   const bool global = select && a.q_global;
-  double sigma = 0.0, nsel = 1.0, J_prev = 0.0, J_best = 0.0;  // thread 0 only
   // J(t) = |sigma^2 - lost_t / (3 N_sel)| with lost_t the exact fixed-point sum of
   // y^2 - x_t^2: sigma^2 and 2^-kSqShift / (3 N_sel) are formed once, so each J
-  // is one fused multiply-add (float64 operations have a long latency here)
-  double sig2 = 0.0, inv3n = 0.0;  // thread 0 only
-  int q_best = 0;                                               // thread 0 only
-  unsigned long long ysq = 0;
-  if (threadIdx.x == 0) {
-    // every scalar this thread reads, loaded together (one round trip to L2)
+  // is one fused multiply-add (float64 operations have a long latency here).  What
+  // the later steps' J needs stays in shared memory, not in every thread's registers.
+  __shared__ double s_sig2, s_inv3n, s_J_prev, s_J_best;
+  __shared__ unsigned long long s_ysq;
+  if (warp == 0) {
+    // lane t: J(t) of the stored step t, all side by side; the scalars loaded
+    // together (one round trip to L2)
+    static_assert(kSpecMax < 32, "a lane a stored step");
     const uint32_t c_ready = sc->cexp_ready;
     const float c_val = sc->cexp;
-    unsigned long long nkt = 0, ysk = 0, ysa = 0, sk[kSpecMax] = {}, sa[kSpecMax] = {};
-    if (select) {
-      sigma = __ldcg(a.sigma_src);
-      nkt = ld_relaxed_u64(&sc->n_keep);
-      ysk = ld_relaxed_u64(&sc->ysq_keep);
-      ysa = ld_relaxed_u64(&sc->ysq_all);
-#pragma unroll
-      for (int q = 0; q < kSpecMax; ++q) {
-        if (q < S) {
-          sk[q] = ld_relaxed_u64(reinterpret_cast<const unsigned long long*>(&sc->spec_keep[q + 1]));
-          sa[q] = ld_relaxed_u64(reinterpret_cast<const unsigned long long*>(&sc->spec_all[q + 1]));
-        }
-      }
-    }
-    s_cexp = c_ready ? c_val : step_cexp(sc);
     const int q_fixed = a.q_src ? min(max(*a.q_src, 0), kQCap) : a.q_fixed;
     const int q_limit = n == 0 ? 0 : (select ? a.q_max : q_fixed);
-    int keep_all = 0, q_final = 0, stopped = 0;
+    int keep_all = 0, q_final = 0, stopped = 0, q_best = 0;
     if (select) {
+      const double sigma = __ldcg(a.sigma_src);
+      const unsigned long long nkt = ld_relaxed_u64(&sc->n_keep);
+      const unsigned long long ysk = ld_relaxed_u64(&sc->ysq_keep);
+      const unsigned long long ysa = ld_relaxed_u64(&sc->ysq_all);
+      unsigned long long xk = 0, xa = 0;
+      if (lane >= 1 && lane <= S) {
+        xk = ld_relaxed_u64(reinterpret_cast<const unsigned long long*>(&sc->spec_keep[lane]));
+        xa = ld_relaxed_u64(reinterpret_cast<const unsigned long long*>(&sc->spec_all[lane]));
+      }
       keep_all = nkt == 0;  // no point left: every point is used
-      nsel = keep_all ? double(n) : double(nkt);
-      ysq = keep_all ? ysa : ysk;
-      sig2 = sigma * sigma;
-      inv3n = (1.0 / double(1 << kSqShift)) / (3.0 * nsel);
-      J_prev = sig2;  // J(0): nothing filtered yet
-      J_best = J_prev;
-      if (gtid == 0) sc->J[0] = J_prev;
-#pragma unroll
-      for (int t = 1; t <= kSpecMax; ++t) {
-        if (t > min(S, q_limit)) break;
-        // sum of y^2 - x_t^2 over the points of Eq. 6: exact in two's complement
-        const double lost = double((long long)(ysq - (keep_all ? sa[t - 1] : sk[t - 1])));
-        const double J = fabs(fma(-lost, inv3n, sig2));
-        if (gtid == 0) {
-          sc->J[t] = J;
-          sc->n_J = t + 1;
-        }
-        if (global) {
-          if (J < J_best) {
-            J_best = J;
+      const double nsel = keep_all ? double(n) : double(nkt);
+      const unsigned long long ysq = keep_all ? ysa : ysk;
+      const double sig2 = sigma * sigma;
+      const double inv3n = (1.0 / double(1 << kSqShift)) / (3.0 * nsel);
+      // sum of y^2 - x_t^2 over the points of Eq. 6: exact in two's complement
+      const double lost = double((long long)(ysq - (keep_all ? xa : xk)));
+      const int m = min(S, q_limit);
+      double J = fabs(fma(-lost, inv3n, sig2));
+      if (lane == 0) J = sig2;  // J(0): nothing filtered yet
+      const double before = __shfl_up_sync(0xffffffffu, J, 1);
+      const uint32_t up = __ballot_sync(0xffffffffu, !global && lane >= 1 && lane <= m && J >= before);
+      stopped = up != 0;
+      const int last = stopped ? __ffs(int(up)) - 1 : m;  // the last J of the search so far
+      q_final = stopped ? last - 1 : m;
+      const double J_prev = __shfl_sync(0xffffffffu, J, q_final);
+      double J_best = sig2;
+      if (global) {
+        for (int t = 1; t <= m; ++t) {
+          const double Jt = __shfl_sync(0xffffffffu, J, t);
+          if (Jt < J_best) {
+            J_best = Jt;
             q_best = t;
           }
-          q_final = t;
-          continue;
         }
-        if (J >= J_prev) {
-          q_final = t - 1;
-          stopped = 1;
-          break;
-        }
-        J_prev = J;
-        q_final = t;
+      }
+      if (lane == 0) {
+        s_sig2 = sig2;
+        s_inv3n = inv3n;
+        s_J_prev = J_prev;
+        s_J_best = J_best;
+        s_ysq = ysq;
+      }
+      if (int(blockIdx.x) == first) {
+        if (lane <= last) sc->J[lane] = J;
+        if (lane == 0 && last > 0) sc->n_J = last + 1;
       }
     }
-    s_ctl[0] = keep_all;
-    s_ctl[1] = q_limit;
-    s_ctl[2] = q_final;
-    s_ctl[3] = stopped;
-    s_ctl[4] = q_best;
-    s_ctl[5] = 0;
+    if (lane == 0) {
+      s_cexp = c_ready ? c_val : step_cexp(sc);
+      s_ctl[0] = keep_all;
+      s_ctl[1] = q_limit;
+      s_ctl[2] = q_final;
+      s_ctl[3] = stopped;
+      s_ctl[4] = q_best;
+      s_ctl[5] = 0;
+    }
   }
   __syncthreads();
   const float cexp = s_cexp;
@@ -640,24 +673,23 @@ __device__ __forceinline__ void select_filter(const FilterArgs& a, int S, int fi
     if (select) {
       if (threadIdx.x == 0) {
         const unsigned long long ss = ld_relaxed_u64(&sc->sumsq[t]);
-        const double lost = double((long long)(ysq - ss));
-        const double J = fabs(fma(-lost, inv3n, sig2));
+        const double lost = double((long long)(s_ysq - ss));
+        const double J = fabs(fma(-lost, s_inv3n, s_sig2));
         if (gtid == 0) {
           sc->J[t] = J;
           sc->n_J = t + 1;
         }
         if (global) {
-          const bool better = J < J_best;
+          const bool better = J < s_J_best;
           if (better) {
-            J_best = J;
-            q_best = t;
+            s_J_best = J;
+            s_ctl[4] = t;
           }
           s_ctl[3] = 0;
-          s_ctl[4] = q_best;
           s_ctl[5] = better;
         } else {
-          s_ctl[3] = J >= J_prev;
-          if (!(J >= J_prev)) J_prev = J;
+          s_ctl[3] = J >= s_J_prev;
+          if (!(J >= s_J_prev)) s_J_prev = J;
         }
       }
       __syncthreads();
