@@ -45,6 +45,7 @@ struct fgbd_ctx {
   float4* xbest = nullptr;  // the global reading of the q search: the best iterate (else null)
   float4* w4 = nullptr;     // window 1: normalised Eq. 4 weights of the slots (FilterArgs::w4, w2)
   float2* w2 = nullptr;
+  int32_t* dmin = nullptr;  // windows w > 1: FilterArgs::dmin
   double* f64part = nullptr;
   int f64_blocks = 0;
   WideNe wne{};  // noise-estimate scratch of windows w > 1 (unused at window 1)
@@ -285,6 +286,7 @@ FilterArgs filter_args(fgbd_ctx* ctx, int mode, int q_fixed, const double* sigma
   a.xbest = ctx->xbest;
   a.w4 = ctx->w4;
   a.w2 = ctx->w2;
+  a.dmin = ctx->dmin;
   return a;
 }
 
@@ -891,6 +893,7 @@ fgbd_status fgbd_ctx_create(int64_t capacity, const fgbd_params* params, fgbd_ct
       {reinterpret_cast<void**>(&ctx->pc), wide ? 0 : C * 8},
       {reinterpret_cast<void**>(&ctx->w4), wide ? 0 : C * 16},
       {reinterpret_cast<void**>(&ctx->w2), wide ? 0 : C * 8},
+      {reinterpret_cast<void**>(&ctx->dmin), wide ? C * 4 : 0},
       {reinterpret_cast<void**>(&ctx->wne.part), wide ? size_t(w_blocks) * wP * 8 : 0},
       {reinterpret_cast<void**>(&ctx->wne.tot), wide ? wP * 8 : 0},
       {reinterpret_cast<void**>(&ctx->wne.S), wide ? wD * wD * 8 : 0},

@@ -392,6 +392,7 @@ struct FilterArgs {
   // w2), written by step 1 and read by every later step of the same graph
   float4* w4;
   float2* w2;
+  int32_t* dmin;           // windows w > 1: each point's smallest squared distance, left by step 1
 };
 constexpr int kKeptBest = 64;  // kept_buf value of the iterate copied to xbest
 cudaError_t launch_filter(const FilterArgs& a, int grid, cudaStream_t stream);
