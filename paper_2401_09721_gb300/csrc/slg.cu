@@ -854,15 +854,19 @@ __device__ __forceinline__ void link_body(const LinkArgs& la, int bx, int gx, in
   }
 }
 
+// Resident blocks per SM, and so registers a thread (48): with 6 (40) the loop spilled,
+// and 16 segmented frames of 20k-100k points took 39 us, now 33; with 4 35, with 8 41.
+constexpr int kLinkPerSm = 5;
+
 template <bool SAME_LINE>
-__global__ void __launch_bounds__(kLinkThreads, 6) k_link(LinkArgs a) {
+__global__ void __launch_bounds__(kLinkThreads, kLinkPerSm) k_link(LinkArgs a) {
   pdl_wait();
   link_body<SAME_LINE>(a, blockIdx.x, gridDim.x, blockIdx.y);
 }
 
 // segmented: frame f's blocks are three runs of equal length, one per code
 template <bool SAME_LINE>
-__global__ void __launch_bounds__(kLinkThreads, 6) k_link_seg(const __grid_constant__ Seg<LinkArgs> s) {
+__global__ void __launch_bounds__(kLinkThreads, kLinkPerSm) k_link_seg(const __grid_constant__ Seg<LinkArgs> s) {
   pdl_wait();
   const int f = seg_frame(s, blockIdx.x);
   const int local = blockIdx.x - s.start[f], gx = (s.start[f + 1] - s.start[f]) / 3;
