@@ -368,11 +368,12 @@ MomentArgs moment_args(const fgbd_ctx* ctx, int n) {
   return MomentArgs{n, ctx->params.bits, ctx->pc, ctx->yf, ctx->x0, ctx->gb.c4, ctx->spread, ctx->f64part, sorted, 1, ctx->sc};
 }
 
-// `zeroed`: the caller has already zeroed the scalar regions this call fills.
+// The scalars from n_edges up to the offset `zero_to` are zeroed (the build's; a
+// whole run's regions are adjacent and zeroed together).
 // `rgb` (a whole run): the colours of the frame, which the link launch then takes
 // into the C1 order (do_estimate and the filter find them gathered).
-fgbd_status do_build(fgbd_ctx* ctx, const int32_t* xyz, int64_t n64, cudaStream_t st, bool zeroed = false,
-                     const void* rgb = nullptr, int32_t dtype = FGBD_U8) {
+fgbd_status do_build(fgbd_ctx* ctx, const int32_t* xyz, int64_t n64, cudaStream_t st,
+                     size_t zero_to = offsetof(DevScalars, build_end_), const void* rgb = nullptr, int32_t dtype = FGBD_U8) {
   if (n64 < 0 || n64 > ctx->capacity) return FGBD_EINVAL;
   if (n64 > 0 && !xyz) return FGBD_EINVAL;
   const int n = int(n64);
@@ -384,14 +385,22 @@ fgbd_status do_build(fgbd_ctx* ctx, const int32_t* xyz, int64_t n64, cudaStream_
   ctx->n = n;
   ctx->graph_gen += 1;
   cudaError_t e = cudaSuccess;
-  if (!zeroed) zero_region(ctx, offsetof(DevScalars, n_edges), offsetof(DevScalars, build_end_), st, &e);
+  const size_t zero_from = offsetof(DevScalars, n_edges);
+  const bool direct = n > 0 && n <= kDirectMax;  // one launch sorts, and zeroes too
+  if (!direct) zero_region(ctx, zero_from, zero_to, st, &e);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "memset");
   if (n > 0) {
-    FGBD_LAUNCH(ctx, "slg_hist", st, launch_coord_hist(xyz, n, bits, ctx->sc, ctx->num_sms, st));
     const BucketArgs ba =
         bucket_args(xyz, n, bits, ord_stride(ctx), ctx->sb, ctx->gb, ctx->sc, scatter_fill(ctx->num_sms));
-    FGBD_LAUNCH(ctx, "slg_scatter", st, launch_bucket_scatter(ba, st));
-    FGBD_LAUNCH(ctx, "slg_sort", st, launch_bucket_sort(ba, st));
+    if (direct) {
+      const ZeroArgs z{reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(ctx->sc) + zero_from),
+                       (zero_to - zero_from) / 4};
+      FGBD_LAUNCH(ctx, "slg_sort", st, launch_direct_sort(ba, z, st));
+    } else {
+      FGBD_LAUNCH(ctx, "slg_hist", st, launch_coord_hist(xyz, n, bits, ctx->sc, ctx->num_sms, st));
+      FGBD_LAUNCH(ctx, "slg_scatter", st, launch_bucket_scatter(ba, st));
+      FGBD_LAUNCH(ctx, "slg_sort", st, launch_bucket_sort(ba, st));
+    }
     const bool same_line = (ctx->params.variant & FGBD_VARIANT_SAME_LINE) != 0;
     if (ctx->params.window == 1)
       FGBD_LAUNCH(ctx, "slg_link", st,
@@ -493,11 +502,9 @@ fgbd_status do_select(fgbd_ctx* ctx, const void* rgb, int32_t dtype, const doubl
 
 fgbd_status direct_run(fgbd_ctx* ctx, const fgbd_ctx::RunKey& k, cudaStream_t st) {
   if (k.n < 0 || k.n > ctx->capacity) return FGBD_EINVAL;
-  // the build, noise and selection regions of the scalars are adjacent: one launch zeroes them
-  cudaError_t e = cudaSuccess;
-  zero_region(ctx, offsetof(DevScalars, n_edges), offsetof(DevScalars, sel_end_), st, &e);
-  if (e != cudaSuccess) return cuda_fail(ctx, e, "memset");
-  fgbd_status s = do_build(ctx, static_cast<const int32_t*>(k.xyz), k.n, st, true, k.rgb_in, k.in_dtype);
+  // the build, noise and selection regions of the scalars are zeroed together
+  fgbd_status s = do_build(ctx, static_cast<const int32_t*>(k.xyz), k.n, st, offsetof(DevScalars, sel_end_), k.rgb_in,
+                           k.in_dtype);
   if (s != FGBD_OK) return s;
   // with FGBD_FLAG_FUSED_SELECT the estimate launch selects and filters too
   const bool fuse = (ctx->params.flags & FGBD_FLAG_FUSED_SELECT) != 0 && ctx->params.window == 1;
@@ -734,7 +741,8 @@ fgbd_status stream_batch(const std::vector<fgbd_ctx*>& ctxs, const std::vector<f
   for (int f = 0; f < count; ++f) {
     fgbd_ctx* c = ctxs[f];
     const fgbd_ctx::RunKey& k = keys[f];
-    fgbd_status s = do_build(c, static_cast<const int32_t*>(k.xyz), k.n, c->side, false, k.rgb_in, k.in_dtype);
+    fgbd_status s = do_build(c, static_cast<const int32_t*>(k.xyz), k.n, c->side, offsetof(DevScalars, build_end_), k.rgb_in,
+                             k.in_dtype);
     if (s == FGBD_OK)
       s = do_estimate(c, k.rgb_in, k.in_dtype, nullptr, c->side, false, false, nullptr, FGBD_U8, false, k.n > 0);
     if (s != FGBD_OK) return s;
@@ -1161,7 +1169,7 @@ fgbd_status fgbd_run_reuse(fgbd_ctx* ctx, const int32_t* xyz, int64_t n, const v
   if (!ctx->ever_selected) return FGBD_ESTATE;
   DeviceGuard g(ctx->device);
   const cudaStream_t st = as_stream(stream);
-  const fgbd_status s = do_build(ctx, xyz, n, st, false, rgb_in, in_dtype);
+  const fgbd_status s = do_build(ctx, xyz, n, st, offsetof(DevScalars, build_end_), rgb_in, in_dtype);
   if (s != FGBD_OK) return s;
   cudaError_t e = cudaSuccess;
   zero_region(ctx, offsetof(DevScalars, ysq_keep), offsetof(DevScalars, sel_end_), st, &e);

@@ -286,6 +286,9 @@ BucketArgs bucket_args(const int32_t* xyz, int n, int bits, int cap, const SortB
 constexpr int scatter_fill(int num_sms) { return 2 * num_sms; }  // two resident blocks per SM
 cudaError_t launch_bucket_scatter(const BucketArgs& a, cudaStream_t stream);
 cudaError_t launch_bucket_sort(const BucketArgs& a, cudaStream_t stream);
+// a frame of up to kDirectMax points in one launch, from the coordinates; it also zeroes z
+constexpr int kDirectMax = 8192;
+cudaError_t launch_direct_sort(const BucketArgs& a, const ZeroArgs& z, cudaStream_t stream);
 cudaError_t launch_orders_export(int n, int cap, const GraphBufs& gb, int32_t* out, cudaStream_t stream);
 // segmented launches: one launch for frames 0..count-1 (count <= kSegMax), each
 // frame with the blocks its one-frame launch would have
