@@ -32,7 +32,7 @@ SIGMAS = (10.0, 20.0, 30.0, 40.0, 50.0)
 N_POINTS = 1_000_000
 BITS = 10
 L2_FLUSH_BYTES = 512 << 20
-SPEC_STEPS = 3          # filter steps the noise-estimate launch stores (kSpecMax)
+SPEC_STEPS = 3          # filter steps the noise-estimate launch stores (kSpecSure)
 FALLBACK_HBM_GBS = 6800.0
 
 

@@ -145,10 +145,9 @@ fgbd_status fgbd_params_default(fgbd_params* p);
 
 /* Create a context on the current CUDA device for frames of up to `capacity`
  * points (1 <= capacity < 2^30) and allocate all its device memory (about
- * 205 bytes per point), zeroed once.  `params` may be NULL for the defaults.
+ * 197 bytes per point; 297 up to 65536 points), zeroed once.  `params` may be NULL for the defaults.
  * On success *out owns the context; release it with fgbd_ctx_destroy.  A
- * window w > 1 adds 24 (w - 1) bytes per point (less the 24 of the stored
- * window-1 filter weights) and a few MB of noise-estimate scratch.
+ * window w > 1 takes 169 + 24 (w - 1) bytes per point and a few MB of noise-estimate scratch.
  * Errors: FGBD_EINVAL (bad capacity or parameters), FGBD_ENOTIMPL (window
  * above FGBD_MAX_WINDOW, or FGBD_VARIANT_UNSORTED_PATCH with window > 1),
  * FGBD_ENOMEM, FGBD_ECUDA. */

@@ -75,7 +75,7 @@ struct fgbd_ctx {
   uint64_t d_gen = 0;
   bool d_valid = false;
   // filter steps stored by the noise-estimate launch (see filter_step.cuh)
-  float4* spec_x = nullptr;   // [spec_rows(cap)][cap]
+  float4* spec_x = nullptr;   // [spec_rows(cap)][cap] (kSpecSure rows at windows w > 1)
   int32_t* spec_z = nullptr;  // [spec_rows(cap)][cap]
   uint8_t* keep8 = nullptr;   // [cap]
   int spec_depth = 0;         // steps stored for noise_rgb on the current graph (0: none)
@@ -874,6 +874,7 @@ fgbd_status fgbd_ctx_create(int64_t capacity, const fgbd_params* params, fgbd_ct
     void** ptr;
     size_t bytes;
   };
+  const size_t steps = size_t(wide ? kSpecSure : spec_rows(int64_t(C)));  // (wider windows store none: the sort's rows lie there)
   void* keys0 = nullptr;
   void* keys1 = nullptr;
   const Item items[] = {
@@ -885,8 +886,8 @@ fgbd_status fgbd_ctx_create(int64_t capacity, const fgbd_params* params, fgbd_ct
       {reinterpret_cast<void**>(&ctx->gb.pk), C * 4},
       {reinterpret_cast<void**>(&ctx->gb.ord23), 2 * align_up(C, 64) * 4},
       {reinterpret_cast<void**>(&ctx->gb.c4), C * 16},
-      {reinterpret_cast<void**>(&ctx->spec_x), size_t(spec_rows(int64_t(C))) * align_up(C, 64) * 16},
-      {reinterpret_cast<void**>(&ctx->spec_z), size_t(spec_rows(int64_t(C))) * align_up(C, 64) * 4},
+      {reinterpret_cast<void**>(&ctx->spec_x), steps * align_up(C, 64) * 16},
+      {reinterpret_cast<void**>(&ctx->spec_z), steps * align_up(C, 64) * 4},
       {reinterpret_cast<void**>(&ctx->keep8), C},
       {reinterpret_cast<void**>(&ctx->y8), C * 4},
       {reinterpret_cast<void**>(&ctx->yf), C * 16},

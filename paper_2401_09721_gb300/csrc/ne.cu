@@ -662,7 +662,7 @@ __global__ void __launch_bounds__(kFinThreads) k_ne_finalize(int dtype, const do
 // rest of the SM's memory is L1 for the steps): block 0 computes sigma_est on an SM of its own, the others meanwhile take the first
 // filter steps, which need the graph and the colours only.  With a.fuse they
 // then also select and filter: they stop stepping once sigma_est is published
-// (or after kSpecMax steps, then waiting for it) and run the selection over
+// (or after kSpecSure steps, then waiting for it) and run the selection over
 // the stored steps (select_filter), so no second launch follows.
 constexpr int kSpecThreads = 1024;
 

@@ -5,13 +5,14 @@
 // offset (dz, dy, dx), then by index), three colour channels each.  The FSLR
 // spread of every point (Section 2.4) comes from the same pass.  Four launches:
 //
-//   k_ne_moments_wide  batches of points staged as a transposed patch block in
-//                      shared memory; each thread owns one 3x3 tile (node a,
-//                      node b >= a) of sum a a^T or the three sums a of one
-//                      node.  uint8 colours: int8 entries c - 128 and exact
-//                      dp4a sums in int64; float colours: float32 sums per
-//                      batch, then float64.  Each block writes its partial
-//                      sums (no atomics, so the totals do not depend on timing).
+//   k_ne_moments_wide  batches of points staged in shared memory.  uint8 colours:
+//                      float16 entries c - 128, the Gram matrix by tensor-core
+//                      products (gram_mma.cuh), exact, in int64.  Float
+//                      colours: each thread owns one 3x3 tile (node a, node
+//                      b >= a) of sum a a^T or the three sums a of one node,
+//                      float32 sums per batch, then float64.  Each block writes
+//                      its partial sums (no atomics, so the totals do not
+//                      depend on timing).
 //   k_ne_wide_reduce   the partials summed entry by entry in a fixed order.
 //   k_ne_wide_eigvec   one block: Sigma = S2/N - mu mu^T in float64, then
 //                      float32 eigenvector estimates by a Householder
