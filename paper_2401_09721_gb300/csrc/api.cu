@@ -365,7 +365,7 @@ ColorArgs color_args(const fgbd_ctx* ctx, const void* rgb, int32_t dtype) {
 
 MomentArgs moment_args(const fgbd_ctx* ctx, int n) {
   const int sorted = (ctx->params.variant & FGBD_VARIANT_UNSORTED_PATCH) == 0 ? 1 : 0;
-  return MomentArgs{n, ctx->params.bits, ctx->pc, ctx->yf, ctx->x0, ctx->gb.c4, ctx->spread, ctx->f64part, sorted, 1, ctx->sc};
+  return MomentArgs{n, ctx->params.bits, ctx->pc, ctx->yf, ctx->x0, ctx->gb.c4, ctx->spread, ctx->f64part, sorted, 1, 1, ctx->sc};
 }
 
 // The scalars from n_edges up to the offset `zero_to` are zeroed (the build's; a

@@ -255,6 +255,7 @@ struct MomentArgs {
   double* f64_partials;
   int sorted_patches;
   int per_sm;        // blocks of the launch on an SM, where they fill the GPU (else 1)
+  int shares;        // float: shares of the points, one or two a block (ne_moment_shares)
   struct DevScalars* sc;
 };
 struct ZeroArgs {
@@ -319,6 +320,7 @@ cudaError_t launch_ne_moments(const MomentArgs& a, int dtype, int num_sms, cudaS
 cudaError_t launch_ne_finalize(int dtype, const double* f64_partials, int nblocks,
                                DevScalars* sc, double* sigma_out, const FilterArgs* spec, int num_sms,
                                cudaStream_t stream);
+int ne_moment_shares(int n, int num_sms);
 int ne_moment_blocks(int n, int num_sms, int dtype);
 // testing: div_newton and CUDA's division of n operand pairs
 cudaError_t launch_debug_div(const double* a, const double* b, double* q_newton, double* q_div, int64_t n,

@@ -274,88 +274,108 @@ __device__ __forceinline__ void ne_moments_body(const MomentArgs& ma, int bid, i
   const uint32_t hbase = uint32_t(__cvta_generic_to_shared(ath));
 
   // uint8: each block takes a run of consecutive points, whose neighbours then lie in
-  // this SM's L1 (step_run); float: the blocks take turns, as their sums always did
-  const int2 run = DT == 0 ? step_run(n, bid, nblk, ma.per_sm) : make_int2(bid * kNeThreads, n);
-  const int stride = DT == 0 ? kNeThreads : nblk * kNeThreads;
-  for (int base = run.x + warp * 32; base < run.y; base += stride) {
-    const int k = base + lane;
-    bool has = false;
-    if (k < run.y) has = DT == 0 ? point_patch_u8(ma, k, lane, ath) : point_patch_f32(ma, k, lane, atf);
-    if (!has) {
+  // this SM's L1 (step_run).  Float: the points are shared out over ma.shares shares,
+  // four an SM, that take turns every 256 points, and a warp's float32 sums cover up
+  // to four of its turns: what they round depends on the shares, so these stay as they
+  // are while fewer blocks are resident (three an SM, without spills).  A block takes
+  // its own share and, from the other end, one of those left over, where the turns are
+  // fewest (217k points: 27 us, a launch of all the shares as blocks 34).
+#pragma unroll 1
+  for (int pass = 0; pass < (DT == 1 ? 2 : 1); ++pass) {
+    const int share = pass == 0 ? bid : 2 * nblk - 1 - bid;
+    if (DT == 1 && share >= ma.shares) break;
+    const int2 run = DT == 0 ? step_run(n, bid, nblk, ma.per_sm) : make_int2(share * kNeThreads, n);
+    const int stride = DT == 0 ? kNeThreads : ma.shares * kNeThreads;
+    for (int base = run.x + warp * 32; base < run.y; base += stride) {
+      const int k = base + lane;
+      bool has = false;
+      if (k < run.y) has = DT == 0 ? point_patch_u8(ma, k, lane, ath) : point_patch_f32(ma, k, lane, atf);
+      if (!has) {
+        if (DT == 0) {
+          uint2* row = reinterpret_cast<uint2*>(ath + lane * kHRow);
+#pragma unroll
+          for (int j = 0; j < kK + 1; ++j) row[j] = make_uint2(0u, 0u);
+        } else {
+#pragma unroll
+          for (int r = 0; r < kD; ++r) atf[r * kRowFloats + lane] = 0.f;
+        }
+      }
+      if (DT == 1) npatch += __popc(__ballot_sync(0xffffffffu, has));
+      __syncwarp();
       if (DT == 0) {
-        uint2* row = reinterpret_cast<uint2*>(ath + lane * kHRow);
 #pragma unroll
-        for (int j = 0; j < kK + 1; ++j) row[j] = make_uint2(0u, 0u);
+        for (int ks = 0; ks < 2; ++ks) {
+          uint32_t lo[4], hi[4];
+          ldsm_x4_trans(gram_patch_addr(hbase, 16 * ks, 0, kHRow, lane), lo);
+          ldsm_x4_trans(gram_patch_addr(hbase, 16 * ks, 16, kHRow, lane), hi);
+          mma_16816(gc[0], lo, lo[0], lo[2]);
+          mma_16816(gc[1], lo, lo[1], lo[3]);
+          mma_16816(gc[2], lo, hi[0], hi[2]);
+          mma_16816(gc[3], lo, hi[1], hi[3]);
+          mma_16816(gc[4], hi, hi[0], hi[2]);
+          mma_16816(gc[5], hi, hi[1], hi[3]);
+        }
+        if (++since_flush == kGramFlushPatches / 32) {
+          flush8(gc, lane, s_tot8);
+          since_flush = 0;
+        }
       } else {
-#pragma unroll
-        for (int r = 0; r < kD; ++r) atf[r * kRowFloats + lane] = 0.f;
-      }
-    }
-    if (DT == 1) npatch += __popc(__ballot_sync(0xffffffffu, has));
-    __syncwarp();
-    if (DT == 0) {
-#pragma unroll
-      for (int ks = 0; ks < 2; ++ks) {
-        uint32_t lo[4], hi[4];
-        ldsm_x4_trans(gram_patch_addr(hbase, 16 * ks, 0, kHRow, lane), lo);
-        ldsm_x4_trans(gram_patch_addr(hbase, 16 * ks, 16, kHRow, lane), hi);
-        mma_16816(gc[0], lo, lo[0], lo[2]);
-        mma_16816(gc[1], lo, lo[1], lo[3]);
-        mma_16816(gc[2], lo, hi[0], hi[2]);
-        mma_16816(gc[3], lo, hi[1], hi[3]);
-        mma_16816(gc[4], hi, hi[0], hi[2]);
-        mma_16816(gc[5], hi, hi[1], hi[3]);
-      }
-      if (++since_flush == kGramFlushPatches / 32) {
-        flush8(gc, lane, s_tot8);
-        since_flush = 0;
-      }
-    } else {
-      if (lane < kTiles) {
+        if (lane < kTiles) {
 #pragma unroll 2
-        for (int p = 0; p < 32; p += 4) {
-          float4 a[3], b[3];
+          for (int p = 0; p < 32; p += 4) {
+            float4 a[3], b[3];
 #pragma unroll
-          for (int i = 0; i < 3; ++i) {
-            a[i] = *reinterpret_cast<const float4*>(atf + (r0 + i) * kRowFloats + p);
-            b[i] = *reinterpret_cast<const float4*>(atf + (c0 + i) * kRowFloats + p);
-          }
-#pragma unroll
-          for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) {
-              float t = accf[3 * i + j];
-              t = fmaf(a[i].x, b[j].x, t);
-              t = fmaf(a[i].y, b[j].y, t);
-              t = fmaf(a[i].z, b[j].z, t);
-              accf[3 * i + j] = fmaf(a[i].w, b[j].w, t);
+            for (int i = 0; i < 3; ++i) {
+              a[i] = *reinterpret_cast<const float4*>(atf + (r0 + i) * kRowFloats + p);
+              b[i] = *reinterpret_cast<const float4*>(atf + (c0 + i) * kRowFloats + p);
             }
-        }
-      }
-      if (lane < kD) {
-        float sum = 0.f;
 #pragma unroll
-        for (int p = 0; p < 32; p += 4) {
-          const float4 a = *reinterpret_cast<const float4*>(atf + lane * kRowFloats + p);
-          sum += a.x;
-          sum += a.y;
-          sum += a.z;
-          sum += a.w;
-        }
-        acc1f += sum;
-      }
-      if (++since_flush == 4) {
+            for (int i = 0; i < 3; ++i)
 #pragma unroll
-        for (int i = 0; i < 9; ++i) {
-          accd[i] += double(accf[i]);
-          accf[i] = 0.f;
+              for (int j = 0; j < 3; ++j) {
+                float t = accf[3 * i + j];
+                t = fmaf(a[i].x, b[j].x, t);
+                t = fmaf(a[i].y, b[j].y, t);
+                t = fmaf(a[i].z, b[j].z, t);
+                accf[3 * i + j] = fmaf(a[i].w, b[j].w, t);
+              }
+          }
         }
-        acc1d += double(acc1f);
-        acc1f = 0.f;
-        since_flush = 0;
+        if (lane < kD) {
+          float sum = 0.f;
+#pragma unroll
+          for (int p = 0; p < 32; p += 4) {
+            const float4 a = *reinterpret_cast<const float4*>(atf + lane * kRowFloats + p);
+            sum += a.x;
+            sum += a.y;
+            sum += a.z;
+            sum += a.w;
+          }
+          acc1f += sum;
+        }
+        if (++since_flush == 4) {
+#pragma unroll
+          for (int i = 0; i < 9; ++i) {
+            accd[i] += double(accf[i]);
+            accf[i] = 0.f;
+          }
+          acc1d += double(acc1f);
+          acc1f = 0.f;
+          since_flush = 0;
+        }
       }
+      __syncwarp();
     }
-    __syncwarp();
+    if (DT == 1) {
+#pragma unroll
+      for (int i = 0; i < 9; ++i) {
+        accd[i] += double(accf[i]);
+        accf[i] = 0.f;
+      }
+      acc1d += double(acc1f);
+      acc1f = 0.f;
+      since_flush = 0;
+    }
   }
   // combine the warps of the block
   if (DT == 0) {
@@ -373,9 +393,9 @@ __device__ __forceinline__ void ne_moments_body(const MomentArgs& ma, int bid, i
   double* own = reinterpret_cast<double*>(atf);
   if (lane < kTiles) {
 #pragma unroll
-    for (int i = 0; i < 9; ++i) own[9 * lane + i] = accd[i] + double(accf[i]);
+    for (int i = 0; i < 9; ++i) own[9 * lane + i] = accd[i];
   }
-  if (lane < kD) own[9 * kTiles + lane] = acc1d + double(acc1f);
+  if (lane < kD) own[9 * kTiles + lane] = acc1d;
   if (lane == 0) own[9 * kTiles + kD] = double(npatch);
   __syncthreads();
   double* row = f64_partials + size_t(bid) * kNeSums;
@@ -765,6 +785,7 @@ cudaError_t launch_ne_moments_seg(const MomentArgs* a, int count, int dtype, int
   const int fill = ne_moment_blocks(INT_MAX, num_sms, dtype);
   for (int f = 0; f < count; ++f) {
     sg.a[f] = a[f];
+    sg.a[f].shares = ne_moment_shares(a[f].n, num_sms);
     blocks[f] = a[f].n > 0 ? ne_moment_blocks(a[f].n, num_sms, dtype) : 0;
     if (dtype == 0 && blocks[f] > 0)
       blocks[f] = std::max(1, std::min(blocks[f], int(double(fill) * double(a[f].n) / total)));
@@ -806,6 +827,12 @@ cudaError_t launch_gather_colors(const ColorArgs& a, int n, cudaStream_t stream)
   return launch_kernel(k_gather_colors, dim3(grid), dim3(256), 0, stream, false, a, n);
 }
 
+// float colours: the shares of the points (k_ne_moments), at most two a block
+int ne_moment_shares(int n, int num_sms) {
+  const int need = int((int64_t(n) + kNeThreads - 1) / kNeThreads);
+  return std::max(1, std::min({need, num_sms * 4, kNeGroup * kNeGroups}));
+}
+
 int ne_moment_blocks(int n, int num_sms, int dtype) {
   // resident blocks per SM, queried once (the same code runs on every device of one build)
   struct PerSm {
@@ -823,7 +850,8 @@ int ne_moment_blocks(int n, int num_sms, int dtype) {
   }();
   const int need = int((int64_t(n) + kNeThreads - 1) / kNeThreads);
   if (dtype == 0) return std::max(1, std::min(need, num_sms * per_sm.u8));
-  return std::max(1, std::min({need, num_sms * per_sm.f32, kNeGroup * kNeGroups}));
+  const int shares = ne_moment_shares(n, num_sms);
+  return std::max(1, std::min(shares, std::max(num_sms * per_sm.f32, (shares + 1) / 2)));
 }
 
 cudaError_t launch_ne_moments(const MomentArgs& a, int dtype, int num_sms, cudaStream_t stream) {
@@ -834,7 +862,9 @@ cudaError_t launch_ne_moments(const MomentArgs& a, int dtype, int num_sms, cudaS
     m.per_sm = grid % num_sms == 0 ? grid / num_sms : 1;
     return launch_kernel(k_ne_moments<0>, dim3(grid), dim3(kNeThreads), 0, stream, false, m);
   }
-  return launch_kernel(k_ne_moments<1>, dim3(grid), dim3(kNeThreads), 0, stream, false, a);
+  MomentArgs m = a;
+  m.shares = ne_moment_shares(a.n, num_sms);
+  return launch_kernel(k_ne_moments<1>, dim3(grid), dim3(kNeThreads), 0, stream, false, m);
 }
 
 cudaError_t launch_ne_finalize(int dtype, const double* f64_partials, int nblocks, DevScalars* sc,
