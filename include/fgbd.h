@@ -300,7 +300,9 @@ fgbd_status fgbd_run_batch(fgbd_ctx* const* ctxs, const int32_t* const* xyz, con
 typedef struct fgbd_batch_shape {
   int32_t seg_frames;            /* frames per segmented launch, 1..16; 0: per-frame streams.  Default: 16
                                     below 2^18 points a frame, 0 above (fgbd_tune_batch: -1 when the batch
-                                    cannot be segmented, and nothing was tuned) */
+                                    cannot be segmented, and nothing was tuned).  Until something is set for
+                                    them, frames of 2^18 to 2^21 points run segmented, four a launch; a 0
+                                    that is set means streams */
   int32_t scatter_threads;       /* threads of a block of the row scatter (a tile of up to 4096 points): 256, 512 (default) or 1024 */
   int32_t filter_threads;        /* threads per block of the selection/filter: 256 or 512 (default) */
   int32_t filter_blocks_per_sm;  /* its blocks per SM (default 2; capped by what fits) */

@@ -680,12 +680,8 @@ int size_class(const std::vector<fgbd_ctx::RunKey>& keys) {
   return int(std::floor(std::log2(std::max(mean, 1.0))));
 }
 
-// Untuned: segmented launches of up to kSegMax frames for frames below 2^18
-// points, whose stages are short and whose working sets (about 180 bytes a
-// point) fit the L2 together; per-frame streams above, where a frame's own
-// working set fills the L2 and running the frames stage by stage would evict
-// each frame's data between its stages (measured on 16 frames of 200k-1.2M
-// points: 4.41 ms segmented against 3.45 ms on streams).
+// The shape reported for a class that nothing was set for: segmented launches of up
+// to kSegMax frames below 2^18 points, 0 above.
 BatchShape default_shape(int cls) {
   BatchShape b;
   b.seg_frames = cls < 18 ? kSegMax : 0;
@@ -697,6 +693,25 @@ BatchShape shape_for(int device, int cls) {
   for (const TunedShape& t : g_shapes)
     if (t.device == device && t.size_class == cls) return t.shape;
   return default_shape(cls);
+}
+
+// What a batch of `count` frames runs.  Where nothing was set, frames of 2^18 to 2^21
+// points go four a launch: each kernel of a single frame already fills the GPU, so on
+// streams the frames overlap little and wait for one another's cooperative launches,
+// and 16 frames a launch evict each other's data from L2 between the stages.  16
+// frames of 200k-1.2M points: 2343 us, on streams 2694, 16 a launch 2646; 2 frames
+// 225 (290), 8 frames of 283k 510 (726), of 1.15M 1736 (1890).  Larger frames were
+// not measured and stay on streams, as does a single frame.
+BatchShape run_shape(int device, int cls, int count) {
+  std::lock_guard<std::mutex> lock(g_shape_mutex);
+  for (const TunedShape& t : g_shapes)
+    if (t.device == device && t.size_class == cls) return t.shape;
+  BatchShape b = default_shape(cls);
+  if (cls >= 18 && cls < 21 && count >= 2) {
+    b.seg_frames = 4;
+    b.scatter_threads = 1024;
+  }
+  return b;
 }
 
 void store_shape(int device, int cls, const BatchShape* shape) {
@@ -1208,7 +1223,7 @@ fgbd_status fgbd_run_batch(fgbd_ctx* const* ctxs, const int32_t* const* xyz, con
   for (int f = 0; f < count; ++f) keys.push_back({xyz[f], n[f], rgb_in[f], in_dtype[f], rgb_out[f], out_dtype[f]});
   bool timing = false;
   for (int f = 0; f < count; ++f) timing |= ctxs[f]->timing;
-  const BatchShape shape = shape_for(lead->device, size_class(keys));
+  const BatchShape shape = run_shape(lead->device, size_class(keys), count);
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
     cudaGetLastError();
