@@ -703,8 +703,9 @@ __device__ __forceinline__ void select_filter(const FilterArgs& a, int S, int fi
       q_final = t;
     }
   }
-  // where the kept iterate is
-  int kept = (S > 0 && q_final <= S) ? (q_final == 0 ? -1 : 2 + q_final - 1) : (q_final & 1);
+  // where the kept iterate is (power 0: the colours themselves, since x_0 is in no
+  // iterate buffer where the steps read it elsewhere)
+  int kept = q_final == 0 ? -1 : q_final <= S ? 2 + q_final - 1 : (q_final & 1);
   if (global) {
     const int qb = s_ctl[4];
     if (qb == 0) kept = -1;
