@@ -944,13 +944,17 @@ fgbd_status fgbd_ctx_create(int64_t capacity, const fgbd_params* params, fgbd_ct
   ctx->sb.keys_c3 = static_cast<uint32_t*>(keys1);
   // the sort's rows and their scratch (8 + 8 bytes a point and code) lie in the
   // first three stored filter steps, which are written after the graph is built
-  static_assert(kSpecSure >= 3 && sizeof(float4) == sizeof(uint2) + 2 * sizeof(uint32_t), "one row of spec_x a code");
+  static_assert(kSpecSure >= 3 && sizeof(float4) == 2 * sizeof(uint2), "one row of spec_x a code");
   const size_t Ca = align_up(C, 64);
-  ctx->sb.tmp_stride = int(Ca);
   for (int c = 0; c < 3; ++c) {
     ctx->sb.row_pts[c] = reinterpret_cast<uint2*>(ctx->spec_x + size_t(c) * Ca);
-    ctx->sb.row_tmp[c] = reinterpret_cast<uint32_t*>(ctx->sb.row_pts[c] + Ca);
+    ctx->sb.row_tmp[c] = ctx->sb.row_pts[c] + Ca;
   }
+  // and the line counters of split rows (less than a byte a point) in an iterate buffer, which
+  // they fit from the first capacity that holds such a row on
+  static_assert(line_words(kRowSplit + 1) * 4 <= size_t(kRowSplit + 1) * sizeof(float4), "and grow more slowly than it");
+  ctx->sb.lines = reinterpret_cast<uint32_t*>(ctx->x1);
+  ctx->sb.line_slots = line_slots(capacity);
   ctx->gb.nx = nx;
   ctx->gb.cx_stride = int(align_up(C, 64));
   if (!(p.variant & FGBD_VARIANT_SIGMA_PAIR)) ctx->gb.node_sig = nullptr;

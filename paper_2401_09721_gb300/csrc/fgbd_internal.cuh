@@ -70,6 +70,9 @@ struct DevScalars {
   uint32_t cexp_ready;          // set by the first moments launch on this graph
   uint32_t row_used[3][kMaxRadix];  // row scatter: places of every x, y and z row handed out so far
   uint32_t row_ext[3][2];           // per coordinate: 2^b - 1 minus its smallest value, and its largest
+  // codes with rows above kRowSplit points (k_bucket_sort): blocks take turns by tickets, and
+  // how many of those rows have their counters cleared, and of their points are counted and placed
+  uint32_t sort_ticket[3], rows_cleared[3], lines_counted[3], lines_placed[3];
   uint32_t build_end_;
   // ---- noise estimate region
   unsigned long long n_patches;
@@ -135,8 +138,9 @@ static_assert(offsetof(DevScalars, n_edges) < offsetof(DevScalars, build_end_) &
 // that are only used after the graph is built (the stored filter steps).
 struct SortBufs {
   uint2* row_pts[3];     // per code [cap]: (input index, code) of every point, row by row
-  uint32_t* row_tmp[3];  // per code [2][tmp_stride]: scratch of the long-item sort (codes, then indices)
-  int tmp_stride;
+  uint2* row_tmp[3];     // per code [cap]: the points of split rows line by line; the long-item sort's scratch
+  uint32_t* lines;       // [3][line_slots][2][kMaxRadix]: the line counters of split rows (kRowSplit)
+  int line_slots;
   uint32_t* keys_c2;     // [cap] the C2 codes along C2
   uint32_t* keys_c3;     // [cap] the C3 codes along C3
 };
@@ -160,6 +164,13 @@ struct GraphBufs {
 // number of further neighbour slots at window w
 __host__ __device__ constexpr int extra_slots(int w) { return 6 * (w - 1); }
 
+// A row of more points than this is put line by line before it is sorted (k_bucket_sort).
+// Its counters, [2][kMaxRadix] points a line (counted, then placed), are those number
+// (first place) / (kRowSplit + 1) of its code: two such rows start further apart than that.
+constexpr int kRowSplit = 32768;
+constexpr int line_slots(int64_t cap) { return int(cap / (kRowSplit + 1)) + 1; }
+constexpr size_t line_words(int64_t cap) { return size_t(3) * size_t(line_slots(cap)) * 2 * kMaxRadix; }
+
 // The row scatter and the bucket sort of one frame (codes 0 C1, 1 C2, 2 C3).
 struct BucketArgs {
   int n;
@@ -168,8 +179,9 @@ struct BucketArgs {
   int window;              // output positions per block of the sort
   const int32_t* xyz;
   uint2* row_pts[3];       // SortBufs
-  uint32_t* row_tmp[3];
-  int tmp_stride;
+  uint2* row_tmp[3];
+  uint32_t* lines;
+  int line_slots;
   uint32_t* keys_out[3];   // code c of the points along code c
   int32_t* order_out[3];   // the input indices along each code
   int32_t* rank12;         // GraphBufs::rank12, as [n][2]
@@ -580,6 +592,12 @@ __device__ __forceinline__ unsigned long long global_ns() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
+}
+
+__device__ __forceinline__ uint32_t ld_acquire_u32(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
 }
 
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;  // 2 s for any device-side wait

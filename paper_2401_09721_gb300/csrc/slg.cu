@@ -307,7 +307,8 @@ __global__ void __launch_bounds__(THREADS, ScatterShape<THREADS>::kMinBlocks)
 // the lines (points of one second coordinate; their starts come from a
 // histogram of the row) that start in it, so every point has one owner and an
 // item holds at most window + kRowMax points unless one line repeats voxels
-// thousands of times.  The item's points go into kSortBuckets buckets by the
+// thousands of times.  The points of rows above kRowSplit are put line by line first
+// (next_split_window).  The item's points go into kSortBuckets buckets by the
 // leading bits of their code (relative to the item's first row, and to the
 // second coordinate's extent), and inside a bucket each point's place is the
 // number of smaller (code, index) pairs.  Repeated voxels that overfill the item
@@ -355,18 +356,24 @@ __device__ __forceinline__ void emit_sorted(const BucketArgs& a, int c, uint32_t
   if (c < 2) a.rank12[2 * size_t(idx) + c] = int32_t(r);
 }
 
-// The places of an item's rows and the second coordinates [mid0, mid1) it owns in
-// them: its small rows (side by side, all of them), and up to two large ones.
+// Where an item's points are: its small rows, all of them side by side, and of up to two
+// large rows the lines [mid0, mid1) that it owns, which take the places from line0.  A
+// split row's are at those places of row_tmp; of another row they are among all its
+// points in row_pts.
 struct ItemRows {
-  uint32_t from[3], to[3], mid0[3], mid1[3];
+  uint32_t out0, total;  // the item's places
+  uint32_t from, to;
+  uint32_t big_from[2], big_to[2], mid0[2], mid1[2], line0[2];
+  bool split[2];
 };
 
 // The points of an item that do not fit shared memory (repeated voxels), by a
 // least-significant-digit radix sort of (code, input index), kBucketThreads
-// points at a time, between the scratch half of the code's row array and the
-// output arrays (this item's `total` places from `out0`).
-__device__ __noinline__ void item_radix_sort(const BucketArgs& a, int c, uint32_t out0, uint32_t total, ItemRows rows,
-                                             uint32_t* smem) {
+// points at a time, between row_tmp and the output arrays (this item's `total`
+// places from `out0`).
+template <bool SPLIT>
+__device__ __noinline__ void item_radix_sort(const BucketArgs& a, int c, const ItemRows& rows, uint32_t* smem) {
+  const uint32_t out0 = rows.out0, total = rows.total;
   constexpr int kPairs = kBucketThreads / 64;
   uint32_t* s_cnt = smem;                        // [kPairs][kMaxRadix]
   uint32_t* s_run = s_cnt + kPairs * kMaxRadix;  // [kMaxRadix]
@@ -374,22 +381,28 @@ __device__ __noinline__ void item_radix_sort(const BucketArgs& a, int c, uint32_
   __shared__ uint32_t s_n, s_sw[32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int b = a.bits, n = a.n;
-  uint32_t* key[2] = {a.row_tmp[c] + out0, a.keys_out[c] + out0};
-  uint32_t* val[2] = {a.row_tmp[c] + size_t(a.tmp_stride) + out0, reinterpret_cast<uint32_t*>(a.order_out[c]) + out0};
-  if (tid == 0) s_n = 0u;
-  __syncthreads();
-  // the item's points: its small rows, and of its large rows the points on its lines
-  for (int g = 0; g < 3; ++g)
-    for (uint32_t i = rows.from[g] + tid; i < rows.to[g]; i += kBucketThreads) {
+  uint2* tmp = a.row_tmp[c] + out0;
+  uint32_t* keys = a.keys_out[c] + out0;
+  int32_t* order = a.order_out[c] + out0;
+  const auto load = [&](int buf, uint32_t i) {
+    return buf == 0 ? __ldcg(tmp + i) : make_uint2(uint32_t(__ldcg(order + i)), __ldcg(keys + i));
+  };
+  // the item's points into row_tmp: its small rows at their places, of a large row that is
+  // not split the points on its lines at theirs, in any order
+  for (uint32_t i = rows.from + tid; i < rows.to; i += kBucketThreads) tmp[i - out0] = a.row_pts[c][i];
+  for (int g = 0; g < 2; ++g) {
+    if (SPLIT && rows.split[g]) continue;
+    if (tid == 0) s_n = rows.line0[g] - out0;
+    __syncthreads();
+    for (uint32_t i = rows.big_from[g] + tid; i < rows.big_to[g]; i += kBucketThreads) {
       const uint2 e = a.row_pts[c][i];
       const uint32_t mid = (e.y >> b) & ((1u << b) - 1u);
       if (mid < rows.mid0[g] || mid >= rows.mid1[g]) continue;
       const uint32_t p = atomicAdd(&s_n, 1u);
-      if (p < total) {
-        key[0][p] = e.y;
-        val[0][p] = e.x;
-      }
+      if (p < total) tmp[p] = e;
     }
+    __syncthreads();
+  }
   __syncthreads();
   int cur = 0;
   const int idx_bits = max(1, 32 - __clz(n - 1));
@@ -401,13 +414,13 @@ __device__ __noinline__ void item_radix_sort(const BucketArgs& a, int c, uint32_
     const int shift = by_idx ? 10 * pass : b * (pass - idx_passes);
     const int dbits = by_idx ? 10 : b;
     const uint32_t dm = (1u << dbits) - 1u;
-    const uint32_t *ks = key[cur], *vs = val[cur];
-    uint32_t *kd = key[cur ^ 1], *vd = val[cur ^ 1];
     // every digit's first place
     s_run[tid] = 0u;
     __syncthreads();
-    for (uint32_t i = tid; i < total; i += kBucketThreads)
-      atomicAdd(&s_run[((by_idx ? __ldcg(vs + i) : __ldcg(ks + i)) >> shift) & dm], 1u);
+    for (uint32_t i = tid; i < total; i += kBucketThreads) {
+      const uint2 e = load(cur, i);
+      atomicAdd(&s_run[((by_idx ? e.x : e.y) >> shift) & dm], 1u);
+    }
     __syncthreads();
     uint32_t run = s_run[tid];
     run = block_exclusive(run, s_sw);
@@ -418,8 +431,8 @@ __device__ __noinline__ void item_radix_sort(const BucketArgs& a, int c, uint32_
       __syncthreads();
       const uint32_t pos = c0 + uint32_t(tid);
       const bool valid = pos < total;
-      const uint32_t k = valid ? __ldcg(ks + pos) : 0u, v = valid ? __ldcg(vs + pos) : 0u;
-      const uint32_t d = ((by_idx ? v : k) >> shift) & dm;
+      const uint2 e = valid ? load(cur, pos) : make_uint2(0u, 0u);
+      const uint32_t d = ((by_idx ? e.x : e.y) >> shift) & dm;
       const uint32_t rk = warp_rank(valid, d, dbits, wh, half, lane);
       __syncthreads();
       // thread d: the warps' offsets of digit d, and the digit's points in this chunk
@@ -434,8 +447,12 @@ __device__ __noinline__ void item_radix_sort(const BucketArgs& a, int c, uint32_
       if (valid) {
         const uint32_t p = s_run[d] + ((wh[d] >> half) & 0xffffu) + rk;
         if (p < total) {
-          kd[p] = k;
-          vd[p] = v;
+          if (cur == 0) {
+            keys[p] = e.y;
+            order[p] = int32_t(e.x);
+          } else {
+            tmp[p] = e;
+          }
         }
       }
       __syncthreads();
@@ -444,8 +461,10 @@ __device__ __noinline__ void item_radix_sort(const BucketArgs& a, int c, uint32_
     __syncthreads();
     cur ^= 1;
   }
-  for (uint32_t i = tid; i < total; i += kBucketThreads)
-    emit_sorted(a, c, out0 + i, __ldcg(key[cur] + i), __ldcg(val[cur] + i));
+  for (uint32_t i = tid; i < total; i += kBucketThreads) {
+    const uint2 e = load(cur, i);
+    emit_sorted(a, c, out0 + i, e.y, e.x);
+  }
 }
 
 // A code's bucket: the leading bits of the code with the unused high bits of
@@ -522,7 +541,17 @@ __device__ __forceinline__ void rank_item(const BucketArgs& a, int c, const Buck
   }
 }
 
-__device__ __forceinline__ void bucket_sort_body(const BucketArgs& a, int item, int c) {
+// the line counters of code c's split row that starts at place `first`
+__device__ __forceinline__ uint32_t* line_counters(const BucketArgs& a, int c, uint32_t first) {
+  return a.lines + (size_t(c) * size_t(a.line_slots) + first / uint32_t(kRowSplit + 1)) * size_t(2 * kMaxRadix);
+}
+
+// One window of a code.  SPLIT: the code has rows above kRowSplit points, which lie line by
+// line in row_tmp, the points of every line counted; false (and nothing done) if it has
+// such rows and they do not.
+template <bool SPLIT>
+__device__ __forceinline__ bool sort_window(const BucketArgs& a, int item, int c) {
+  const uint32_t* start = a.sc->row_start[row_coord(c)];
   extern __shared__ __align__(16) uint32_t smem[];
   // (code in the high, index in the low half; four entries of padding for the ranking loads)
   unsigned long long* s_pt = reinterpret_cast<unsigned long long*>(smem);     // [kItemMax + 4]
@@ -531,23 +560,22 @@ __device__ __forceinline__ void bucket_sort_body(const BucketArgs& a, int item, 
   __shared__ uint32_t s_lo, s_hi, s_row0, s_row1;  // the small rows' places, the first and the last row
   __shared__ uint32_t s_big[2];                    // 1 + the large row that starts before / in the window
   __shared__ uint32_t s_mid0, s_mid1;              // a large row's own lines [mid0, mid1)
-  __shared__ uint32_t s_first, s_last;             // and the places they take, of both rows
+  __shared__ uint32_t s_first[2], s_last;          // and the first places they take; the end of both rows'
   const int tid = threadIdx.x, lane = tid & 31;
   const int b = a.bits, radix = 1 << b, n = a.n;
   const uint32_t m = uint32_t(radix) - 1u;
   const DevScalars* sc = a.sc;
   const uint2* pts = a.row_pts[c];
-  const uint32_t* start = sc->row_start[row_coord(c)];
   const uint32_t w0 = uint32_t(item) * uint32_t(a.window), w1 = w0 + uint32_t(a.window);
   const uint32_t rs = tid < radix ? start[tid] : 0u, re = tid < radix ? min(start[tid + 1], uint32_t(n)) : 0u;
   const int mc = mid_coord(c);
-  const uint32_t mid0 = m - sc->row_ext[mc][0], mid1 = sc->row_ext[mc][1];
   reinterpret_cast<uint4*>(s_cnt)[tid] = make_uint4(0u, 0u, 0u, 0u);
   if (tid == 0) {
-    s_lo = s_row0 = s_first = 0xffffffffu;
+    s_lo = s_row0 = s_first[0] = s_first[1] = 0xffffffffu;
     s_hi = s_row1 = s_big[0] = s_big[1] = s_last = 0u;
   }
-  __syncthreads();
+  if (SPLIT) __syncthreads();
+  else if (__syncthreads_or(re > rs && re - rs > uint32_t(kRowSplit))) return false;
   {
     uint32_t lo = 0xffffffffu, hi = 0u, row = 0xffffffffu;
     if (re > rs) {
@@ -579,25 +607,34 @@ __device__ __forceinline__ void bucket_sort_body(const BucketArgs& a, int item, 
   // the small rows lie side by side: [lo, lo + cnt_small), lo = 0 if there are none
   const uint32_t lo = s_hi ? s_lo : 0u, cnt_small = s_hi - lo;
   const uint32_t big[2] = {s_big[0], s_big[1]};
-  if (!cnt_small && !big[0] && !big[1]) return;
-  const BucketOf bucket = bucket_of(s_row0, s_row1, mid0, mid1, b);
+  if (!cnt_small && !big[0] && !big[1]) return true;
   uint32_t out0 = cnt_small ? lo : 0xffffffffu, out1 = s_hi;  // the item's places [out0, out1)
-  uint32_t b0[2] = {0u, 0u}, b1[2] = {0u, 0u}, l0[2] = {0u, 0u}, l1[2] = {0u, 0u};  // large rows: places, own lines
+  // large rows: where their points are read (split ones: the own lines' places), own lines
+  uint32_t b0[2] = {0u, 0u}, b1[2] = {0u, 0u}, l0[2] = {0u, 0u}, l1[2] = {0u, 0u};
+  bool split[2] = {false, false};
   if (big[0] | big[1]) {
 #pragma unroll
     for (int g = 0; g < 2; ++g) {
       if (!big[g]) continue;
       b0[g] = start[big[g] - 1u];
       b1[g] = min(start[big[g]], uint32_t(n));
-      // the row's line histogram, and the lines that start in the window
-#pragma unroll 4
-      for (uint32_t i = b0[g] + tid; i < b1[g]; i += kBucketThreads) atomicAdd(&s_cnt[(pts[i].y >> b) & m], 1u);
+      if (SPLIT) split[g] = b1[g] - b0[g] > uint32_t(kRowSplit);
       if (tid == 0) {
         s_mid0 = 0xffffffffu;
         s_mid1 = 0u;
       }
-      __syncthreads();
-      const uint32_t v = s_cnt[tid];
+      uint32_t v;  // the points of line tid
+      if (SPLIT && split[g]) {
+        __syncthreads();
+        v = __ldcg(line_counters(a, c, b0[g]) + tid);
+      } else {
+        // the row's line histogram
+#pragma unroll 4
+        for (uint32_t i = b0[g] + tid; i < b1[g]; i += kBucketThreads) atomicAdd(&s_cnt[(pts[i].y >> b) & m], 1u);
+        __syncthreads();
+        v = s_cnt[tid];
+      }
+      // and the lines that start in the window
       const uint32_t at = b0[g] + block_exclusive(v, s_w[g]);
       s_cnt[tid] = 0u;
       const bool own = v && at >= w0 && at < w1;
@@ -608,53 +645,72 @@ __device__ __forceinline__ void bucket_sort_body(const BucketArgs& a, int item, 
         atomicMax(&s_mid1, hi_w);
       }
       if (own) {
-        atomicMin(&s_first, at);
-        atomicMax(&s_last, at + v);
+        atomicMin(&s_first[g], at);
+        atomicMax(&s_last, min(at + v, uint32_t(n)));
       }
       __syncthreads();
       l0[g] = s_mid0;
       l1[g] = s_mid1;
+      if (SPLIT && split[g]) {
+        b0[g] = min(s_first[g], uint32_t(n));
+        b1[g] = l1[g] ? min(s_last, uint32_t(n)) : 0u;  // (of the two rows', this one's is the largest so far)
+      }
       __syncthreads();
     }
-    out0 = min(out0, s_first);
+    out0 = min(out0, min(s_first[0], s_first[1]));
     out1 = max(out1, s_last);
-    if (out0 >= out1) return;  // one long line crosses the window
+    if (out0 >= out1) return true;  // one long line crosses the window
   }
   const uint32_t total = out1 - out0;
+  uint32_t mid0 = m - sc->row_ext[mc][0], mid1 = sc->row_ext[mc][1];
+  if (s_row0 == s_row1 && (l1[0] | l1[1])) {
+    // a part of one row: its buckets share out the own lines only
+    mid0 = l1[0] ? l0[0] : l0[1];
+    mid1 = (l1[0] ? l1[0] : l1[1]) - 1u;
+  }
+  const BucketOf bucket = bucket_of(s_row0, s_row1, mid0, mid1, b);
   const auto owned = [&](int g, uint32_t k) {
     const uint32_t mid = (k >> b) & m;
     return mid >= l0[g] && mid < l1[g];
   };
-  // (by value: nothing of the loops below is kept in memory for the rare radix sort)
-#define FGBD_ITEM_RADIX_SORT()                                                                                  \
-  item_radix_sort(a, c, out0, min(total, uint32_t(n) - min(out0, uint32_t(n))),                                 \
-                  ItemRows{{lo, b0[0], b0[1]},                                                                  \
-                           {lo + cnt_small, l1[0] ? b1[0] : 0u, l1[1] ? b1[1] : 0u},                            \
-                           {0u, l0[0], l0[1]},                                                                  \
-                           {1u << b, l1[0], l1[1]}},                                                            \
-                  smem)
-  if (total > uint32_t(kItemMax)) {
-    FGBD_ITEM_RADIX_SORT();
-    return;
-  }
   const auto count = [&](uint32_t k) { return count_in(s_cnt, bucket(k)); };
+  bool fits = total <= uint32_t(kItemMax);
+  if (fits) {
 #pragma unroll 4
-  for (uint32_t i = lo + tid; i < lo + cnt_small; i += kBucketThreads) count(pts[i].y);
+    for (uint32_t i = lo + tid; i < lo + cnt_small; i += kBucketThreads) count(pts[i].y);
 #pragma unroll
-  for (int g = 0; g < 2; ++g)
-    if (l1[g])
+    for (int g = 0; g < 2; ++g)
+      if (l1[g])
 #pragma unroll 4
-      for (uint32_t i = b0[g] + tid; i < b1[g]; i += kBucketThreads) {
-        const uint32_t k = pts[i].y;
-        if (owned(g, k)) count(k);
-      }
-  __syncthreads();
-  const uint32_t most = bucket_starts(s_cnt, s_w[2]);
-  if (__syncthreads_or(most > kBucketMax)) {
-    FGBD_ITEM_RADIX_SORT();
-    return;
+        for (uint32_t i = b0[g] + tid; i < b1[g]; i += kBucketThreads) {
+          const uint32_t k = (SPLIT && split[g] ? __ldcg(a.row_tmp[c] + i) : pts[i]).y;
+          if (owned(g, k)) count(k);
+        }
+    __syncthreads();
+    fits = !__syncthreads_or(bucket_starts(s_cnt, s_w[2]) > kBucketMax);
   }
-#undef FGBD_ITEM_RADIX_SORT
+  if (!fits) {
+    // (through shared memory: nothing of the loops around is kept on the stack for this)
+    __shared__ ItemRows s_rows;
+    if (tid == 0) {
+      s_rows.out0 = out0;
+      s_rows.total = total;
+      s_rows.from = lo;
+      s_rows.to = lo + cnt_small;
+#pragma unroll
+      for (int g = 0; g < 2; ++g) {
+        s_rows.big_from[g] = b0[g];
+        s_rows.big_to[g] = l1[g] ? b1[g] : 0u;
+        s_rows.mid0[g] = l0[g];
+        s_rows.mid1[g] = l1[g];
+        s_rows.line0[g] = s_first[g];
+        if (SPLIT) s_rows.split[g] = split[g];
+      }
+    }
+    __syncthreads();
+    item_radix_sort<SPLIT>(a, c, s_rows, smem);
+    return true;
+  }
   const auto put = [&](uint2 e) {
     const uint32_t p = count(e.y);
     if (p < uint32_t(kItemMax)) s_pt[p] = ((unsigned long long)e.y << 32) | e.x;
@@ -666,15 +722,165 @@ __device__ __forceinline__ void bucket_sort_body(const BucketArgs& a, int item, 
     if (l1[g])
 #pragma unroll 4
       for (uint32_t i = b0[g] + tid; i < b1[g]; i += kBucketThreads) {
-        const uint2 e = pts[i];
+        const uint2 e = SPLIT && split[g] ? __ldcg(a.row_tmp[c] + i) : pts[i];
         if (owned(g, e.y)) put(e);
       }
   if (tid < 4) s_pt[total + tid] = ~0ull;
   __syncthreads();
   rank_item(a, c, bucket, s_pt, s_cnt, out0, total);
+  return true;
 }
 
-__global__ void __launch_bounds__(kBucketThreads, 2) k_bucket_sort(BucketArgs a) {
+// Thread 0 waits until *counter reaches `target` (a bounded wait); false for every thread if it gave up.
+__device__ __forceinline__ bool wait_count(const BucketArgs& a, const uint32_t* counter, uint32_t target, int* s_ok) {
+  if (threadIdx.x == 0) {
+    const unsigned long long t0 = global_ns(), limit = a.sc->wait_limit_ns;
+    int ok = 1;
+    while (ld_acquire_u32(counter) < target) {
+      if (global_ns() - t0 > limit) {
+        atomicOr(&a.sc->status, kFlagTimeout);
+        ok = 0;
+        break;
+      }
+      __nanosleep(64);
+    }
+    *s_ok = ok;
+  }
+  __syncthreads();
+  return *s_ok != 0;
+}
+
+// what this block's threads have written, published as `add` on *counter
+__device__ __forceinline__ void publish_count(uint32_t* counter, uint32_t add) {
+  __syncthreads();
+  if (threadIdx.x == 0 && add) {
+    __threadfence();
+    atomicAdd(counter, add);
+  }
+}
+
+// A code with rows above kRowSplit points (walls and floors along an axis).  Left as they
+// are, every window of such a row reads the whole row three times to find its own lines,
+// and the graph of a plane of 1M points took 580 us.  Instead the row's points are counted
+// by line and put line by line into row_tmp, a window's positions at a time, before the
+// windows are sorted: 115-120 us (91 for a sphere of 1M points).  The rows are split from
+// 32768 points on because the three steps before the sort cost 20-40 us: rows of 8,000 and
+// 10,000 points (1M in all) 110 and 122 us as they are, 169 and 181 split; of 31,000 160 and
+// 165; of 100,000 (800,000 in all) 164 as they are, 115 split.
+// The code's blocks take tickets: first the rows' counters are cleared, then the windows'
+// points counted, then placed, then the windows sorted.  A block waits only for parts whose
+// tickets were drawn before its own, that is by blocks already running, and those wait only
+// for still earlier ones: whatever number of blocks is resident, the waits end.  (A launch
+// of its own between the row scatter and the sort would cost frames without such rows
+// 2-3 us.  All three codes' windows by common tickets, plain ones between the steps: 10 us
+// slower than with the other codes' blocks beside them.)
+
+// The next window to sort, or -1: none is left, or a wait gave up.
+__device__ __noinline__ int next_split_window(const BucketArgs& a, int c) {
+  const int items = (a.n + a.window - 1) / a.window;  // (the code's blocks)
+  const uint32_t* start = a.sc->row_start[row_coord(c)];
+  extern __shared__ __align__(16) uint32_t smem[];
+  uint32_t* s_n = smem;                 // [kMaxRadix] this window's points of a line
+  uint32_t* s_at = s_n + kMaxRadix;     // [kMaxRadix] and their first place
+  __shared__ uint32_t s_big[2], s_ticket, s_rows, s_points, s_scan[32];
+  __shared__ int s_ok;
+  const int tid = threadIdx.x;
+  const int b = a.bits, n = a.n;
+  const uint32_t m = (1u << b) - 1u;
+  DevScalars* sc = a.sc;
+  // the row of this thread, if it is split
+  const uint32_t rs = tid <= int(m) ? start[tid] : 0u, re = tid <= int(m) ? min(start[tid + 1], uint32_t(n)) : 0u;
+  const bool mine = re > rs && re - rs > uint32_t(kRowSplit);
+  if (tid == 0) s_rows = s_points = 0u;
+  __syncthreads();
+  if (mine) {
+    atomicAdd(&s_rows, 1u);
+    atomicAdd(&s_points, re - rs);
+  }
+  __syncthreads();
+  const uint32_t rows = s_rows, points = s_points;
+  for (;;) {
+    __syncthreads();
+    if (tid == 0) s_ticket = atomicAdd(&sc->sort_ticket[c], 1u);
+    if (tid < 2) s_big[tid] = 0u;
+    __syncthreads();
+    const uint32_t phase = s_ticket / uint32_t(items), item = s_ticket % uint32_t(items);
+    if (phase >= 3u)
+      return phase == 3u && wait_count(a, &sc->lines_placed[c], points, &s_ok) ? int(item) : -1;
+    // the split rows that overlap the window: 1 + the one that starts before it, and in it
+    const uint32_t w0 = item * uint32_t(a.window), w1 = w0 + uint32_t(a.window);
+    if (mine && rs < w1 && re > w0) s_big[rs < w0 ? 0 : 1] = uint32_t(tid) + 1u;
+    __syncthreads();
+    if (phase == 0u) {
+      if (s_big[1]) {
+        uint32_t* cnt = line_counters(a, c, start[s_big[1] - 1u]);
+        for (int i = tid; i < 2 * kMaxRadix; i += kBucketThreads) cnt[i] = 0u;
+      }
+      publish_count(&sc->rows_cleared[c], s_big[1] ? 1u : 0u);
+      continue;
+    }
+    if (phase == 1u ? !wait_count(a, &sc->rows_cleared[c], rows, &s_ok)
+                    : !wait_count(a, &sc->lines_counted[c], points, &s_ok))
+      return -1;
+    uint32_t done = 0u;
+    for (int g = 0; g < 2; ++g) {
+      if (!s_big[g]) continue;
+      const uint32_t first = start[s_big[g] - 1u];
+      const uint32_t from = max(first, w0), to = min(min(start[s_big[g]], uint32_t(n)), w1);
+      uint32_t* cnt = line_counters(a, c, first);
+      const uint2* pts = a.row_pts[c];
+      static_assert(kWindowMax <= 4 * kBucketThreads && kMaxRadix == kBucketThreads, "four points, one line a thread");
+      s_n[tid] = 0u;
+      __syncthreads();
+      uint2 e[4];
+      uint32_t r[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const uint32_t i = from + uint32_t(j * kBucketThreads + tid);
+        e[j] = i < to ? pts[i] : make_uint2(0u, 0u);
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (from + uint32_t(j * kBucketThreads + tid) < to) r[j] = atomicAdd(&s_n[(e[j].y >> b) & m], 1u);
+      __syncthreads();
+      const uint32_t v = s_n[tid];
+      if (phase == 1u) {
+        if (v) atomicAdd(cnt + tid, v);
+      } else {
+        const uint32_t at = first + block_exclusive(__ldcg(cnt + tid), s_scan);
+        s_at[tid] = v ? at + atomicAdd(cnt + kMaxRadix + tid, v) : 0u;
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (from + uint32_t(j * kBucketThreads + tid) < to) {
+            const uint32_t p = s_at[(e[j].y >> b) & m] + r[j];
+            if (p < uint32_t(n)) a.row_tmp[c][p] = e[j];
+          }
+      }
+      done += to > from ? to - from : 0u;
+      __syncthreads();
+    }
+    publish_count(phase == 1u ? &sc->lines_counted[c] : &sc->lines_placed[c], done);
+  }
+}
+
+// (calls of their own: inlined, they cost the other frames' sort its registers: 5 us at 1M points)
+__device__ __noinline__ void sort_split_window(const BucketArgs& a, int item, int c) { sort_window<true>(a, item, c); }
+
+__device__ __noinline__ void sort_split_rows(const BucketArgs& a, int c) {
+  for (;;) {
+    const int item = next_split_window(a, c);
+    if (item < 0) return;
+    sort_split_window(a, item, c);
+  }
+}
+
+// one block for every window of a code
+__device__ __forceinline__ void bucket_sort_body(const BucketArgs& a, int block, int c) {
+  if (!sort_window<false>(a, block, c)) sort_split_rows(a, c);
+}
+
+__global__ void __launch_bounds__(kBucketThreads, 2) k_bucket_sort(const __grid_constant__ BucketArgs a) {
   pdl_wait();
   bucket_sort_body(a, blockIdx.x, blockIdx.y);
 }
@@ -687,7 +893,7 @@ __global__ void __launch_bounds__(kBucketThreads, 2) k_bucket_sort(BucketArgs a)
 constexpr int kDirectPer = kDirectMax / kBucketThreads;
 static_assert(kDirectMax <= kItemMax && kDirectPer * kBucketThreads == kDirectMax, "one item, whole points a thread");
 
-__global__ void __launch_bounds__(kBucketThreads, 1) k_direct_sort(BucketArgs a, ZeroArgs z) {
+__global__ void __launch_bounds__(kBucketThreads, 1) k_direct_sort(const __grid_constant__ BucketArgs a, ZeroArgs z) {
   pdl_wait();
   const int tid = threadIdx.x, lane = tid & 31;
   if (blockIdx.x >= 3) {
@@ -761,8 +967,10 @@ __global__ void __launch_bounds__(kBucketThreads, 1) k_direct_sort(BucketArgs a,
       if (i < n) a.row_pts[c][i] = make_uint2(uint32_t(i), code[j]);
     }
     __syncthreads();
-    item_radix_sort(a, c, 0u, uint32_t(n), ItemRows{{0u, 0u, 0u}, {uint32_t(n), 0u, 0u}, {0u, 0u, 0u}, {1u << b, 0u, 0u}},
-                    smem);
+    __shared__ ItemRows s_all;
+    if (tid == 0) s_all = ItemRows{0u, uint32_t(n), 0u, uint32_t(n)};
+    __syncthreads();
+    item_radix_sort<false>(a, c, s_all, smem);
     return;
   }
 #pragma unroll
@@ -1251,7 +1459,8 @@ BucketArgs bucket_args(const int32_t* xyz, int n, int bits, int cap, const SortB
     a.row_pts[c] = sb.row_pts[c];
     a.row_tmp[c] = sb.row_tmp[c];
   }
-  a.tmp_stride = sb.tmp_stride;
+  a.lines = sb.lines;
+  a.line_slots = sb.line_slots;
   a.keys_out[0] = gb.pk;
   a.keys_out[1] = sb.keys_c2;
   a.keys_out[2] = sb.keys_c3;

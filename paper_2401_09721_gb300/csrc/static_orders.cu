@@ -19,6 +19,7 @@ using namespace fgbd;
 namespace {
 
 constexpr size_t kMaxPts = FGBD_STATIC_MAX_POINTS;
+static_assert(kMaxPts <= kRowSplit, "no row is split: no line counters, and no wait (the scalars hold no limit)");
 constexpr size_t align256(size_t v) { return (v + 255) / 256 * 256; }
 
 // byte offsets inside the scratch array
@@ -26,7 +27,7 @@ constexpr size_t kOffScalars = 0;
 constexpr size_t kOffKeys2 = align256(kOffScalars + sizeof(DevScalars));
 constexpr size_t kOffKeys3 = align256(kOffKeys2 + kMaxPts * 4);
 constexpr size_t kOffRows = align256(kOffKeys3 + kMaxPts * 4);      // [3][points] of (index, code)
-constexpr size_t kOffTmp = align256(kOffRows + 3 * kMaxPts * 8);    // [3][2][points]
+constexpr size_t kOffTmp = align256(kOffRows + 3 * kMaxPts * 8);    // [3][points]
 constexpr size_t kOffPerm1 = align256(kOffTmp + 3 * kMaxPts * 8);
 constexpr size_t kOffRank12 = align256(kOffPerm1 + kMaxPts * 4);
 constexpr size_t kOffPk = align256(kOffRank12 + kMaxPts * 8);
@@ -88,10 +89,9 @@ extern "C" fgbd_status fgbd_scan_orders_static(const int32_t* xyz, int64_t n64, 
     SortBufs sb{};
     sb.keys_c2 = reinterpret_cast<uint32_t*>(base + kOffKeys2);
     sb.keys_c3 = reinterpret_cast<uint32_t*>(base + kOffKeys3);
-    sb.tmp_stride = int(kMaxPts);
     for (size_t c = 0; c < 3; ++c) {
       sb.row_pts[c] = reinterpret_cast<uint2*>(base + kOffRows) + c * kMaxPts;
-      sb.row_tmp[c] = reinterpret_cast<uint32_t*>(base + kOffTmp) + c * 2 * kMaxPts;
+      sb.row_tmp[c] = reinterpret_cast<uint2*>(base + kOffTmp) + c * kMaxPts;
     }
     GraphBufs gb{};
     gb.perm1 = reinterpret_cast<int32_t*>(base + kOffPerm1);
