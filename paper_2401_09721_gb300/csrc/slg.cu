@@ -311,8 +311,9 @@ __global__ void __launch_bounds__(THREADS, ScatterShape<THREADS>::kMinBlocks)
 // (next_split_window).  The item's points go into kSortBuckets buckets by the
 // leading bits of their code (relative to the item's first row, and to the
 // second coordinate's extent), and inside a bucket each point's place is the
-// number of smaller (code, index) pairs.  Repeated voxels that overfill the item
-// or a bucket are ordered by a radix sort through global memory instead.
+// number of smaller (code, index) pairs.  Where that leaves many points in a bucket the
+// buckets follow the rows instead (item_by_rows).  Repeated voxels that overfill the item
+// or a bucket are ordered by a radix sort through global memory.
 // Measured (1M body points, b = 10): 38 us for the three codes, of which the
 // prologue 7, counting 6, placing 5, ranking and writing 17; it is bound by its
 // instructions (22 M a launch) and by the barriers between its phases.  With the
@@ -328,7 +329,8 @@ constexpr int kWindowMax = 4096;
 constexpr int kItemMax = kWindowMax + kRowMax;
 constexpr int kSortBucketBits = 13;
 constexpr int kSortBuckets = 1 << kSortBucketBits;  // 16-bit counters, two a word
-constexpr uint32_t kBucketMax = 512;                // larger buckets are not ranked by counting
+constexpr uint32_t kBucketCoarse = 256;             // larger ones: the buckets follow the rows instead (item_by_rows)
+constexpr uint32_t kBucketMax = 512;                // larger ones still are not ranked by counting
 constexpr size_t kBucketSmem = sizeof(uint2) * (size_t(kItemMax) + 4) + sizeof(uint16_t) * size_t(kSortBuckets);
 static_assert(kSortBuckets == 8 * kBucketThreads && kMaxRadix <= kBucketThreads, "eight buckets, one row a thread");
 static_assert(kItemMax < 65536, "16-bit places inside an item");
@@ -356,14 +358,18 @@ __device__ __forceinline__ void emit_sorted(const BucketArgs& a, int c, uint32_t
   if (c < 2) a.rank12[2 * size_t(idx) + c] = int32_t(r);
 }
 
-// Where an item's points are: its small rows, all of them side by side, and of up to two
-// large rows the lines [mid0, mid1) that it owns, which take the places from line0.  A
-// split row's are at those places of row_tmp; of another row they are among all its
-// points in row_pts.
+// An item as its slower paths take it.  Its points: its small rows, all of them side by
+// side, and of up to two large rows the lines [mid0, mid1) that it owns, which take the
+// places [line0, line1).  A split row's are at those places of row_tmp; of another row
+// they are among all its points in row_pts.
 struct ItemRows {
-  uint32_t out0, total;  // the item's places
-  uint32_t from, to;
-  uint32_t big_from[2], big_to[2], mid0[2], mid1[2], line0[2];
+  const uint32_t* start;             // the code's row starts
+  uint32_t ext0, ext1;               // the extent of the second coordinate
+  uint32_t out0, total;              // the item's places
+  uint32_t from, to;                 // the small rows
+  uint32_t big[2];                   // 1 + the large row (0: none)
+  uint32_t big_from[2], big_to[2];   // where its points are read
+  uint32_t mid0[2], mid1[2], line0[2], line1[2];
   bool split[2];
 };
 
@@ -519,7 +525,8 @@ __device__ __forceinline__ uint32_t bucket_starts(uint32_t* s_cnt, uint32_t* s_w
 }
 
 // The placed points of an item (four entries of padding behind them) to their places from out0.
-__device__ __forceinline__ void rank_item(const BucketArgs& a, int c, const BucketOf& bucket,
+template <typename Bucket>
+__device__ __forceinline__ void rank_item(const BucketArgs& a, int c, const Bucket& bucket,
                                           const unsigned long long* s_pt, const uint32_t* s_cnt, uint32_t out0,
                                           uint32_t total) {
   // counter k is now the end of bucket k.  The points before a bucket are
@@ -541,6 +548,76 @@ __device__ __forceinline__ void rank_item(const BucketArgs& a, int c, const Buck
   }
 }
 
+// Buckets that follow the item's rows: a row has as many of them as points, over the
+// second coordinate's extent (a large row over the item's lines), so they stay small where
+// the rows lie far apart (two bodies, one above the other) or a few stray points make
+// the extent many times that of the rest.
+struct BucketByRow {
+  const ItemRows& it;
+  int b, n;
+  uint32_t scale;  // buckets a place, 2^-16
+  __device__ __forceinline__ uint32_t operator()(uint32_t k) const {
+    const uint32_t m = (1u << b) - 1u, row = k >> (2 * b);
+    uint32_t at = it.start[row], end = min(it.start[row + 1], uint32_t(n)), mid0 = it.ext0, span = it.ext1 - it.ext0;
+#pragma unroll
+    for (int g = 0; g < 2; ++g)
+      if (row + 1u == it.big[g]) {
+        at = it.line0[g];
+        end = it.line1[g];
+        mid0 = it.mid0[g];
+        span = it.mid1[g] - 1u - mid0;
+      }
+    const uint32_t in_row = ((((k >> b) & m) - mid0) << b) | (k & m);
+    const int bits = 32 - __clz(int(span)) + b;
+    const uint32_t place = at - it.out0 + uint32_t(((unsigned long long)(end - at) * in_row) >> bits);
+    return min(uint32_t(((unsigned long long)place * scale) >> 16), uint32_t(kSortBuckets - 1));
+  }
+};
+
+// An item whose buckets were too large: with buckets that follow its rows, or by the radix
+// sort if repeated voxels overfill those too.  (Two spheres of 200,000 points apart along
+// an axis: the sort 84 us with the items across the gap by the radix sort, 22 so; a block
+// of 20^3 voxels and two points in the grid's corners: the graph 90 -> 39.)  Counting a
+// second time pays from buckets of some 256 points on: a box surface of 300,000 points,
+// whose edges fill buckets of 256, 97 us, with a limit of 128 108; a sphere of 100,000
+// points with two stray ones 43 and 35.
+template <bool SPLIT>
+__device__ __noinline__ void item_by_rows(const BucketArgs& a, int c, const ItemRows& rows, uint32_t* smem) {
+  unsigned long long* s_pt = reinterpret_cast<unsigned long long*>(smem);
+  uint32_t* s_cnt = reinterpret_cast<uint32_t*>(s_pt + kItemMax + 4);
+  __shared__ uint32_t s_w[32];
+  const int tid = threadIdx.x, b = a.bits;
+  const uint32_t m = (1u << b) - 1u;
+  if (rows.total <= uint32_t(kItemMax)) {
+    const BucketByRow bucket{rows, b, a.n, (uint32_t(kSortBuckets) << 16) / rows.total};
+    const auto points = [&](auto&& f) {
+      for (uint32_t i = rows.from + tid; i < rows.to; i += kBucketThreads) f(a.row_pts[c][i]);
+      for (int g = 0; g < 2; ++g)
+        for (uint32_t i = rows.big_from[g] + tid; i < rows.big_to[g]; i += kBucketThreads) {
+          const uint2 e = SPLIT && rows.split[g] ? __ldcg(a.row_tmp[c] + i) : a.row_pts[c][i];
+          const uint32_t mid = (e.y >> b) & m;
+          if (mid >= rows.mid0[g] && mid < rows.mid1[g]) f(e);
+        }
+    };
+    __syncthreads();
+    reinterpret_cast<uint4*>(s_cnt)[tid] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+    points([&](uint2 e) { count_in(s_cnt, bucket(e.y)); });
+    __syncthreads();
+    if (!__syncthreads_or(bucket_starts(s_cnt, s_w) > kBucketMax)) {
+      points([&](uint2 e) {
+        const uint32_t p = count_in(s_cnt, bucket(e.y));
+        if (p < uint32_t(kItemMax)) s_pt[p] = ((unsigned long long)e.y << 32) | e.x;
+      });
+      if (tid < 4) s_pt[rows.total + tid] = ~0ull;
+      __syncthreads();
+      rank_item(a, c, bucket, s_pt, s_cnt, rows.out0, rows.total);
+      return;
+    }
+  }
+  item_radix_sort<SPLIT>(a, c, rows, smem);
+}
+
 // the line counters of code c's split row that starts at place `first`
 __device__ __forceinline__ uint32_t* line_counters(const BucketArgs& a, int c, uint32_t first) {
   return a.lines + (size_t(c) * size_t(a.line_slots) + first / uint32_t(kRowSplit + 1)) * size_t(2 * kMaxRadix);
@@ -560,7 +637,7 @@ __device__ __forceinline__ bool sort_window(const BucketArgs& a, int item, int c
   __shared__ uint32_t s_lo, s_hi, s_row0, s_row1;  // the small rows' places, the first and the last row
   __shared__ uint32_t s_big[2];                    // 1 + the large row that starts before / in the window
   __shared__ uint32_t s_mid0, s_mid1;              // a large row's own lines [mid0, mid1)
-  __shared__ uint32_t s_first[2], s_last;          // and the first places they take; the end of both rows'
+  __shared__ uint32_t s_first[2], s_last[2];       // and the places they take
   const int tid = threadIdx.x, lane = tid & 31;
   const int b = a.bits, radix = 1 << b, n = a.n;
   const uint32_t m = uint32_t(radix) - 1u;
@@ -572,7 +649,7 @@ __device__ __forceinline__ bool sort_window(const BucketArgs& a, int item, int c
   reinterpret_cast<uint4*>(s_cnt)[tid] = make_uint4(0u, 0u, 0u, 0u);
   if (tid == 0) {
     s_lo = s_row0 = s_first[0] = s_first[1] = 0xffffffffu;
-    s_hi = s_row1 = s_big[0] = s_big[1] = s_last = 0u;
+    s_hi = s_row1 = s_big[0] = s_big[1] = s_last[0] = s_last[1] = 0u;
   }
   if (SPLIT) __syncthreads();
   else if (__syncthreads_or(re > rs && re - rs > uint32_t(kRowSplit))) return false;
@@ -646,19 +723,19 @@ __device__ __forceinline__ bool sort_window(const BucketArgs& a, int item, int c
       }
       if (own) {
         atomicMin(&s_first[g], at);
-        atomicMax(&s_last, min(at + v, uint32_t(n)));
+        atomicMax(&s_last[g], min(at + v, uint32_t(n)));
       }
       __syncthreads();
       l0[g] = s_mid0;
       l1[g] = s_mid1;
       if (SPLIT && split[g]) {
         b0[g] = min(s_first[g], uint32_t(n));
-        b1[g] = l1[g] ? min(s_last, uint32_t(n)) : 0u;  // (of the two rows', this one's is the largest so far)
+        b1[g] = s_last[g];
       }
       __syncthreads();
     }
     out0 = min(out0, min(s_first[0], s_first[1]));
-    out1 = max(out1, s_last);
+    out1 = max(out1, max(s_last[0], s_last[1]));
     if (out0 >= out1) return true;  // one long line crosses the window
   }
   const uint32_t total = out1 - out0;
@@ -687,12 +764,15 @@ __device__ __forceinline__ bool sort_window(const BucketArgs& a, int item, int c
           if (owned(g, k)) count(k);
         }
     __syncthreads();
-    fits = !__syncthreads_or(bucket_starts(s_cnt, s_w[2]) > kBucketMax);
+    fits = !__syncthreads_or(bucket_starts(s_cnt, s_w[2]) > kBucketCoarse);
   }
   if (!fits) {
     // (through shared memory: nothing of the loops around is kept on the stack for this)
     __shared__ ItemRows s_rows;
     if (tid == 0) {
+      s_rows.start = start;
+      s_rows.ext0 = m - sc->row_ext[mc][0];
+      s_rows.ext1 = sc->row_ext[mc][1];
       s_rows.out0 = out0;
       s_rows.total = total;
       s_rows.from = lo;
@@ -703,12 +783,14 @@ __device__ __forceinline__ bool sort_window(const BucketArgs& a, int item, int c
         s_rows.big_to[g] = l1[g] ? b1[g] : 0u;
         s_rows.mid0[g] = l0[g];
         s_rows.mid1[g] = l1[g];
+        s_rows.big[g] = l1[g] ? s_big[g] : 0u;
         s_rows.line0[g] = s_first[g];
+        s_rows.line1[g] = s_last[g];
         if (SPLIT) s_rows.split[g] = split[g];
       }
     }
     __syncthreads();
-    item_radix_sort<SPLIT>(a, c, s_rows, smem);
+    item_by_rows<SPLIT>(a, c, s_rows, smem);
     return true;
   }
   const auto put = [&](uint2 e) {
@@ -959,18 +1041,30 @@ __global__ void __launch_bounds__(kBucketThreads, 1) k_direct_sort(const __grid_
     if (j * kBucketThreads + tid < n) count_in(s_cnt, bucket(code[j]));
   __syncthreads();
   const uint32_t most = bucket_starts(s_cnt, s_w);
-  if (__syncthreads_or(most > kBucketMax)) {
-    // repeated voxels: the radix sort reads the points as the row scatter leaves them
+  if (__syncthreads_or(most > kBucketCoarse)) {
+    // the slower paths read the points and the row starts as the row scatter leaves them
+    __shared__ uint32_t s_start[kMaxRadix + 1];
+    __shared__ ItemRows s_all;
+    s_start[tid] = 0u;
+    if (tid == 0) {
+      s_start[kMaxRadix] = uint32_t(n);
+      s_all = ItemRows{s_start, s_lo[1], s_hi[1], 0u, uint32_t(n), 0u, uint32_t(n)};
+    }
+    __syncthreads();
 #pragma unroll
     for (int j = 0; j < kDirectPer; ++j) {
       const int i = j * kBucketThreads + tid;
-      if (i < n) a.row_pts[c][i] = make_uint2(uint32_t(i), code[j]);
+      if (i < n) {
+        a.row_pts[c][i] = make_uint2(uint32_t(i), code[j]);
+        atomicAdd(&s_start[code[j] >> (2 * b)], 1u);
+      }
     }
     __syncthreads();
-    __shared__ ItemRows s_all;
-    if (tid == 0) s_all = ItemRows{0u, uint32_t(n), 0u, uint32_t(n)};
+    const uint32_t first = block_exclusive(s_start[tid], s_w);
     __syncthreads();
-    item_radix_sort<false>(a, c, s_all, smem);
+    s_start[tid] = first;
+    __syncthreads();
+    item_by_rows<false>(a, c, s_all, smem);
     return;
   }
 #pragma unroll
