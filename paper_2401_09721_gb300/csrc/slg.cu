@@ -337,14 +337,9 @@ static_assert(kItemMax < 65536, "16-bit places inside an item");
 
 // Stable rank of one key among the equal digits of its warp (lanes in order),
 // added to the warp's digit counter (16-bit half `half` of the pair word).
-__device__ __forceinline__ uint32_t warp_rank(bool valid, uint32_t d, int bits, uint32_t* wh, int half, int lane) {
-  uint32_t peers = __ballot_sync(0xffffffffu, valid);
-  for (int b = 0; b < bits; ++b) {
-    const bool bit = (d >> b) & 1u;
-    const uint32_t on = __ballot_sync(0xffffffffu, bit);
-    peers &= bit ? on : ~on;
-  }
-  const int leader = peers ? __ffs(peers) - 1 : lane;
+__device__ __forceinline__ uint32_t warp_rank(bool valid, uint32_t d, uint32_t* wh, int half, int lane) {
+  const uint32_t peers = __match_any_sync(0xffffffffu, valid ? d : 0xffffffffu);
+  const int leader = __ffs(peers) - 1;
   uint32_t old = 0;
   if (valid && lane == leader) old = (atomicAdd(&wh[d], uint32_t(__popc(peers)) << half) >> half) & 0xffffu;
   return __shfl_sync(0xffffffffu, old, leader) + __popc(peers & ((1u << lane) - 1u));
@@ -373,103 +368,252 @@ struct ItemRows {
   bool split[2];
 };
 
-// The points of an item that do not fit shared memory (repeated voxels), by a
-// least-significant-digit radix sort of (code, input index), kBucketThreads
-// points at a time, between row_tmp and the output arrays (this item's `total`
-// places from `out0`).
+// The points of an item that repeated voxels make too long or too crowded: into the
+// order of their input indices, through a bitmap of the indices in shared memory, then by
+// stable radix passes over the coordinates in which they differ (of the points of one voxel
+// none), between row_tmp and the output arrays (the item's places).  One block, bound
+// by its instructions and its scattered stores.  The graph of 100,000 points in one voxel
+// takes 269 us, with radix passes over the index and all of the code 1410; of 20,000 beside
+// a sphere of as many 229 and 330.  (Its steps are calls of their own: inlined,
+// they cost the windows' sort its registers, 5 us at 1M points.)
+constexpr int kRadixPer = 4;             // points a thread at a time
+constexpr int kBitmapWords = 24 * 1024;  // input indices a time, 32 a word
+static_assert(sizeof(uint32_t) * kBitmapWords <= kBucketSmem, "the bitmap fits the shared memory of an item");
+
+// the digit of a code: its bits [shift, shift + bits)
+struct Digit {
+  int shift, bits;
+  __device__ __forceinline__ uint32_t operator()(uint32_t code) const { return (code >> shift) & ((1u << bits) - 1u); }
+};
+
+// place i of an item in row_tmp (buf 0) or the output arrays (buf 1)
+__device__ __forceinline__ uint2 radix_load(const BucketArgs& a, int c, uint32_t out0, int buf, uint32_t i) {
+  i += out0;
+  return buf == 0 ? __ldcg(a.row_tmp[c] + i) : make_uint2(uint32_t(__ldcg(a.order_out[c] + i)), __ldcg(a.keys_out[c] + i));
+}
+__device__ __forceinline__ void radix_store(const BucketArgs& a, int c, const ItemRows& rows, int buf, uint32_t i, uint2 e) {
+  if (i >= rows.total) return;
+  i += rows.out0;
+  if (buf == 0) {
+    a.row_tmp[c][i] = e;
+  } else {
+    a.keys_out[c][i] = e.y;
+    a.order_out[c][i] = int32_t(e.x);
+  }
+}
+
+// The item's points into the output arrays: its small rows at their places, of a large row
+// the points on its lines at theirs, in any order; and the bits in which their codes differ.
 template <bool SPLIT>
-__device__ __noinline__ void item_radix_sort(const BucketArgs& a, int c, const ItemRows& rows, uint32_t* smem) {
-  const uint32_t out0 = rows.out0, total = rows.total;
-  constexpr int kPairs = kBucketThreads / 64;
-  uint32_t* s_cnt = smem;                        // [kPairs][kMaxRadix]
-  uint32_t* s_run = s_cnt + kPairs * kMaxRadix;  // [kMaxRadix]
-  static_assert(sizeof(uint32_t) * (kPairs + 1) * kMaxRadix <= sizeof(uint2) * kItemMax, "the counters fit the item's points");
-  __shared__ uint32_t s_n, s_sw[32];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int b = a.bits, n = a.n;
-  uint2* tmp = a.row_tmp[c] + out0;
-  uint32_t* keys = a.keys_out[c] + out0;
-  int32_t* order = a.order_out[c] + out0;
-  const auto load = [&](int buf, uint32_t i) {
-    return buf == 0 ? __ldcg(tmp + i) : make_uint2(uint32_t(__ldcg(order + i)), __ldcg(keys + i));
-  };
-  // the item's points into row_tmp: its small rows at their places, of a large row that is
-  // not split the points on its lines at theirs, in any order
-  for (uint32_t i = rows.from + tid; i < rows.to; i += kBucketThreads) tmp[i - out0] = a.row_pts[c][i];
+__device__ __noinline__ void radix_gather(const BucketArgs& a, int c, const ItemRows& rows, uint32_t* s_vary) {
+  __shared__ uint32_t s_n;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int b = a.bits;
+  const uint2* pts = a.row_pts[c];
+#pragma unroll 4
+  for (uint32_t i = rows.from + tid; i < rows.to; i += kBucketThreads) radix_store(a, c, rows, 1, i - rows.out0, pts[i]);
   for (int g = 0; g < 2; ++g) {
-    if (SPLIT && rows.split[g]) continue;
-    if (tid == 0) s_n = rows.line0[g] - out0;
+    const uint32_t to = rows.big_to[g];
+    if (SPLIT && rows.split[g]) {
+#pragma unroll 4
+      for (uint32_t i = rows.big_from[g] + tid; i < to; i += kBucketThreads)
+        radix_store(a, c, rows, 1, i - rows.out0, __ldcg(a.row_tmp[c] + i));
+      continue;
+    }
+    if (tid == 0) s_n = rows.line0[g];
     __syncthreads();
-    for (uint32_t i = rows.big_from[g] + tid; i < rows.big_to[g]; i += kBucketThreads) {
-      const uint2 e = a.row_pts[c][i];
+    for (uint32_t i0 = rows.big_from[g] + uint32_t(tid & ~31); i0 < to; i0 += kBucketThreads) {
+      const bool in = i0 + lane < to;
+      const uint2 e = pts[in ? i0 + lane : i0];
       const uint32_t mid = (e.y >> b) & ((1u << b) - 1u);
-      if (mid < rows.mid0[g] || mid >= rows.mid1[g]) continue;
-      const uint32_t p = atomicAdd(&s_n, 1u);
-      if (p < total) tmp[p] = e;
+      const bool own = in && mid >= rows.mid0[g] && mid < rows.mid1[g];
+      const uint32_t who = __ballot_sync(0xffffffffu, own);
+      uint32_t p = 0u;
+      if (lane == 0 && who) p = atomicAdd(&s_n, uint32_t(__popc(who)));
+      p = __shfl_sync(0xffffffffu, p, 0) + __popc(who & ((1u << lane) - 1u));
+      if (own) radix_store(a, c, rows, 1, p - rows.out0, e);
     }
     __syncthreads();
+  }
+  if (tid == 0) *s_vary = 0u;
+  __syncthreads();
+  const uint32_t* keys = a.keys_out[c] + rows.out0;
+  const uint32_t k0 = __ldcg(keys);
+  uint32_t v = 0u;
+#pragma unroll 4
+  for (uint32_t i = tid; i < rows.total; i += kBucketThreads) v |= __ldcg(keys + i) ^ k0;
+  v = __reduce_or_sync(0xffffffffu, v);
+  if (lane == 0) atomicOr(s_vary, v);
+  __syncthreads();
+}
+
+// words of the bitmap of the indices from i0 on
+__device__ __forceinline__ uint32_t bitmap_words(int n, uint32_t i0) {
+  return min((uint32_t(n) - i0 + 31u) / 32u, uint32_t(kBitmapWords));
+}
+
+// The input indices i0 .. i0 + 32 kBitmapWords - 1 of the item's points (in order_out) as a bitmap.
+__device__ __noinline__ void fill_bitmap(const BucketArgs& a, int c, const ItemRows& rows, uint32_t i0, uint32_t* s_bits) {
+  const uint32_t words = bitmap_words(a.n, i0);
+  for (uint32_t i = threadIdx.x; i < words; i += kBucketThreads) s_bits[i] = 0u;
+  __syncthreads();
+  const int32_t* order = a.order_out[c] + rows.out0;
+#pragma unroll 4
+  for (uint32_t i = threadIdx.x; i < rows.total; i += kBucketThreads) {
+    const uint32_t at = uint32_t(__ldcg(order + i)) - i0;
+    if (at < 32u * words) atomicOr(&s_bits[at >> 5], 1u << (at & 31u));
   }
   __syncthreads();
-  int cur = 0;
-  const int idx_bits = max(1, 32 - __clz(n - 1));
-  const int idx_passes = (idx_bits + 9) / 10;
+}
+
+// A bitmap's indices in ascending order into row_tmp, from the item's place `base` on; the place
+// behind them.  A warp writes out a run of words, 32 bits of one word at a time.
+__device__ __noinline__ uint32_t write_bitmap(const BucketArgs& a, int c, const ItemRows& rows, uint32_t i0, uint32_t base,
+                                              const uint32_t* s_bits) {
+  __shared__ uint32_t s_sw[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t words = bitmap_words(a.n, i0), run = (words + 31u) / 32u;  // of a warp
+  const uint32_t from = min(words, warp * run), to = min(words, from + run);
+  uint32_t mine = 0u;
+  for (uint32_t i = from + lane; i < to; i += 32u) mine += __popc(s_bits[i]);
+  mine = __reduce_add_sync(0xffffffffu, mine);
+  if (lane == 0) s_sw[warp] = mine;
+  __syncthreads();
+  uint32_t p = base + warps_before(s_sw, lane, warp);
+  for (uint32_t w0 = from; w0 < to; w0 += 32u) {
+    const uint32_t word = w0 + lane < to ? s_bits[w0 + lane] : 0u;
+    for (uint32_t todo = __ballot_sync(0xffffffffu, word != 0u); todo; todo &= todo - 1u) {
+      const int l = __ffs(todo) - 1;
+      const uint32_t w = __shfl_sync(0xffffffffu, word, l), at = p + __popc(w & ((1u << lane) - 1u));
+      if (((w >> lane) & 1u) && at < rows.total) a.row_tmp[c][rows.out0 + at].x = i0 + 32u * (w0 + uint32_t(l)) + lane;
+      p += __popc(w);
+    }
+  }
+  base += __reduce_add_sync(0xffffffffu, s_sw[lane]);
+  __syncthreads();
+  return base;
+}
+
+// The points into row_tmp in the order of their input indices, with their codes.
+__device__ __noinline__ void place_by_index(const BucketArgs& a, int c, const ItemRows& rows, uint32_t* s_bits) {
+  uint32_t base = 0u;
+  for (uint32_t i0 = 0u; i0 < uint32_t(a.n); i0 += 32u * kBitmapWords) {
+    fill_bitmap(a, c, rows, i0, s_bits);
+    base = write_bitmap(a, c, rows, i0, base, s_bits);
+  }
+  const uint32_t m = (1u << a.bits) - 1u;
+  for (uint32_t i = threadIdx.x; i < rows.total; i += kBucketThreads) {
+    uint2* e = a.row_tmp[c] + rows.out0 + i;
+    const uint32_t idx = __ldcg(&e->x);
+    if (idx >= uint32_t(a.n)) continue;
+    const int32_t* q = a.xyz + 3 * size_t(idx);
+    e->y = code_of(c, uint32_t(q[0]) & m, uint32_t(q[1]) & m, uint32_t(q[2]) & m, a.bits);
+  }
+  __syncthreads();
+}
+
+// Every digit's first place into s_run (points of one digit side by side are counted together).
+__device__ __noinline__ void radix_count(const BucketArgs& a, int c, const ItemRows& rows, Digit digit, int cur,
+                                         uint32_t* s_run) {
+  __shared__ uint32_t s_sw[32];
+  const int tid = threadIdx.x, lane = tid & 31;
+  s_run[tid] = 0u;
+  __syncthreads();
+#pragma unroll 4
+  for (uint32_t i0 = uint32_t(tid & ~31); i0 < rows.total; i0 += kBucketThreads) {
+    const bool in = i0 + lane < rows.total;
+    const uint32_t d = digit(radix_load(a, c, rows.out0, cur, in ? i0 + lane : i0).y);
+    const uint32_t valid = __ballot_sync(0xffffffffu, in);
+    if (__all_sync(0xffffffffu, d == __shfl_sync(0xffffffffu, d, 0))) {
+      if (lane == 0) atomicAdd(&s_run[d], uint32_t(__popc(valid)));
+    } else if (in) {
+      atomicAdd(&s_run[d], 1u);
+    }
+  }
+  __syncthreads();
+  const uint32_t run = block_exclusive(s_run[tid], s_sw);
+  __syncthreads();
+  s_run[tid] = run;
+  __syncthreads();
+}
+
+// The points from buffer cur to their digits' places in the other, those of one digit in the
+// order they have.
+__device__ __noinline__ void radix_place(const BucketArgs& a, int c, const ItemRows& rows, Digit digit, int cur,
+                                         uint32_t* smem) {
+  constexpr int kPairs = kBucketThreads / 64;
+  uint32_t* s_run = smem;                         // [kMaxRadix] each digit's next place
+  uint32_t* s_at = s_run + kMaxRadix;             // [kMaxRadix] its first place among the points at hand
+  uint32_t* s_cnt = s_at + kMaxRadix;             // [kPairs][kMaxRadix] two warps a word
+  uint2* s_e = reinterpret_cast<uint2*>(s_cnt + kPairs * kMaxRadix);  // [kRadixPer][kBucketThreads] digit by digit
+  static_assert(sizeof(uint32_t) * (kPairs + 2) * kMaxRadix + sizeof(uint2) * kRadixPer * kBucketThreads <= kBucketSmem,
+                "they fit the shared memory of an item");
+  __shared__ uint32_t s_sw[32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   uint32_t* wh = s_cnt + (warp >> 1) * kMaxRadix;
   const int half = 16 * (warp & 1);
-  for (int pass = 0; pass < idx_passes + 3; ++pass) {
-    const bool by_idx = pass < idx_passes;
-    const int shift = by_idx ? 10 * pass : b * (pass - idx_passes);
-    const int dbits = by_idx ? 10 : b;
-    const uint32_t dm = (1u << dbits) - 1u;
-    // every digit's first place
-    s_run[tid] = 0u;
-    __syncthreads();
-    for (uint32_t i = tid; i < total; i += kBucketThreads) {
-      const uint2 e = load(cur, i);
-      atomicAdd(&s_run[((by_idx ? e.x : e.y) >> shift) & dm], 1u);
-    }
-    __syncthreads();
-    uint32_t run = s_run[tid];
-    run = block_exclusive(run, s_sw);
-    __syncthreads();
-    s_run[tid] = run;
-    for (uint32_t c0 = 0; c0 < total; c0 += kBucketThreads) {
-      for (int i = tid; i < kPairs * kMaxRadix; i += kBucketThreads) s_cnt[i] = 0u;
-      __syncthreads();
-      const uint32_t pos = c0 + uint32_t(tid);
-      const bool valid = pos < total;
-      const uint2 e = valid ? load(cur, pos) : make_uint2(0u, 0u);
-      const uint32_t d = ((by_idx ? e.x : e.y) >> shift) & dm;
-      const uint32_t rk = warp_rank(valid, d, dbits, wh, half, lane);
-      __syncthreads();
-      // thread d: the warps' offsets of digit d, and the digit's points in this chunk
-      uint32_t w0 = 0u;
+  for (uint32_t c0 = 0; c0 < rows.total; c0 += kRadixPer * kBucketThreads) {
+    for (int i = tid; i < kPairs * kMaxRadix / 4; i += kBucketThreads)
+      reinterpret_cast<uint4*>(s_cnt)[i] = make_uint4(0u, 0u, 0u, 0u);
+    const uint32_t count = min(rows.total - c0, uint32_t(kRadixPer * kBucketThreads));
+    const uint32_t pos = uint32_t(warp * 32 * kRadixPer + lane);  // a warp's points side by side
+    uint2 e[kRadixPer];
+    uint32_t rk[kRadixPer];
 #pragma unroll
-      for (int w = 0; w < kPairs; ++w) {
-        const uint32_t q = s_cnt[w * kMaxRadix + tid];
-        s_cnt[w * kMaxRadix + tid] = w0 | ((w0 + (q & 0xffffu)) << 16);
-        w0 += (q & 0xffffu) + (q >> 16);
+    for (int j = 0; j < kRadixPer; ++j)
+      e[j] = pos + 32u * j < count ? radix_load(a, c, rows.out0 + c0, cur, pos + 32u * j) : make_uint2(0u, 0u);
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kRadixPer; ++j) rk[j] = warp_rank(pos + 32u * j < count, digit(e[j].y), wh, half, lane);
+    __syncthreads();
+    // thread d: the warps' offsets of digit d, and the digit's points at hand
+    uint32_t w0 = 0u;
+#pragma unroll 4
+    for (int w = 0; w < kPairs; ++w) {
+      const uint32_t q = s_cnt[w * kMaxRadix + tid];
+      s_cnt[w * kMaxRadix + tid] = w0 | ((w0 + (q & 0xffffu)) << 16);
+      w0 += (q & 0xffffu) + (q >> 16);
+    }
+    s_at[tid] = block_exclusive(w0, s_sw);
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kRadixPer; ++j)
+      if (pos + 32u * j < count) {
+        const uint32_t d = digit(e[j].y);
+        s_e[s_at[d] + ((wh[d] >> half) & 0xffffu) + rk[j]] = e[j];
       }
-      __syncthreads();
-      if (valid) {
-        const uint32_t p = s_run[d] + ((wh[d] >> half) & 0xffffu) + rk;
-        if (p < total) {
-          if (cur == 0) {
-            keys[p] = e.y;
-            order[p] = int32_t(e.x);
-          } else {
-            tmp[p] = e;
-          }
-        }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kRadixPer; ++j) {
+      const uint32_t p = uint32_t(j * kBucketThreads + tid);
+      if (p < count) {
+        const uint2 v = s_e[p];
+        const uint32_t d = digit(v.y);
+        radix_store(a, c, rows, cur ^ 1, s_run[d] + p - s_at[d], v);
       }
-      __syncthreads();
-      s_run[tid] += w0;
     }
     __syncthreads();
+    s_run[tid] += w0;
+  }
+  __syncthreads();
+}
+
+template <bool SPLIT>
+__device__ __forceinline__ void item_radix_sort(const BucketArgs& a, int c, const ItemRows& rows, uint32_t* smem) {
+  __shared__ uint32_t s_vary;
+  radix_gather<SPLIT>(a, c, rows, &s_vary);
+  place_by_index(a, c, rows, smem);
+  int cur = 0;
+  for (int f = 0; f < 3; ++f) {
+    const Digit digit{a.bits * f, a.bits};
+    if (digit(s_vary) == 0u) continue;
+    radix_count(a, c, rows, digit, cur, smem);
+    radix_place(a, c, rows, digit, cur, smem);
     cur ^= 1;
   }
-  for (uint32_t i = tid; i < total; i += kBucketThreads) {
-    const uint2 e = load(cur, i);
-    emit_sorted(a, c, out0 + i, e.y, e.x);
+  for (uint32_t i = threadIdx.x; i < rows.total; i += kBucketThreads) {
+    const uint2 e = radix_load(a, c, rows.out0, cur, i);
+    emit_sorted(a, c, rows.out0 + i, e.y, e.x);
   }
 }
 
@@ -582,7 +726,7 @@ struct BucketByRow {
 // whose edges fill buckets of 256, 97 us, with a limit of 128 108; a sphere of 100,000
 // points with two stray ones 43 and 35.
 template <bool SPLIT>
-__device__ __noinline__ void item_by_rows(const BucketArgs& a, int c, const ItemRows& rows, uint32_t* smem) {
+__device__ __noinline__ bool rank_by_rows(const BucketArgs& a, int c, const ItemRows& rows, uint32_t* smem) {
   unsigned long long* s_pt = reinterpret_cast<unsigned long long*>(smem);
   uint32_t* s_cnt = reinterpret_cast<uint32_t*>(s_pt + kItemMax + 4);
   __shared__ uint32_t s_w[32];
@@ -612,10 +756,15 @@ __device__ __noinline__ void item_by_rows(const BucketArgs& a, int c, const Item
       if (tid < 4) s_pt[rows.total + tid] = ~0ull;
       __syncthreads();
       rank_item(a, c, bucket, s_pt, s_cnt, rows.out0, rows.total);
-      return;
+      return true;
     }
   }
-  item_radix_sort<SPLIT>(a, c, rows, smem);
+  return false;
+}
+
+template <bool SPLIT>
+__device__ __noinline__ void item_by_rows(const BucketArgs& a, int c, const ItemRows& rows, uint32_t* smem) {
+  if (!rank_by_rows<SPLIT>(a, c, rows, smem)) item_radix_sort<SPLIT>(a, c, rows, smem);
 }
 
 // the line counters of code c's split row that starts at place `first`
@@ -626,8 +775,9 @@ __device__ __forceinline__ uint32_t* line_counters(const BucketArgs& a, int c, u
 // One window of a code.  SPLIT: the code has rows above kRowSplit points, which lie line by
 // line in row_tmp, the points of every line counted; false (and nothing done) if it has
 // such rows and they do not.
+enum class Window { kDone, kHasSplitRows, kCrowded };
 template <bool SPLIT>
-__device__ __forceinline__ bool sort_window(const BucketArgs& a, int item, int c) {
+__device__ __forceinline__ Window sort_window(const BucketArgs& a, int item, int c, ItemRows& s_rows) {
   const uint32_t* start = a.sc->row_start[row_coord(c)];
   extern __shared__ __align__(16) uint32_t smem[];
   // (code in the high, index in the low half; four entries of padding for the ranking loads)
@@ -652,7 +802,7 @@ __device__ __forceinline__ bool sort_window(const BucketArgs& a, int item, int c
     s_hi = s_row1 = s_big[0] = s_big[1] = s_last[0] = s_last[1] = 0u;
   }
   if (SPLIT) __syncthreads();
-  else if (__syncthreads_or(re > rs && re - rs > uint32_t(kRowSplit))) return false;
+  else if (__syncthreads_or(re > rs && re - rs > uint32_t(kRowSplit))) return Window::kHasSplitRows;
   {
     uint32_t lo = 0xffffffffu, hi = 0u, row = 0xffffffffu;
     if (re > rs) {
@@ -684,7 +834,7 @@ __device__ __forceinline__ bool sort_window(const BucketArgs& a, int item, int c
   // the small rows lie side by side: [lo, lo + cnt_small), lo = 0 if there are none
   const uint32_t lo = s_hi ? s_lo : 0u, cnt_small = s_hi - lo;
   const uint32_t big[2] = {s_big[0], s_big[1]};
-  if (!cnt_small && !big[0] && !big[1]) return true;
+  if (!cnt_small && !big[0] && !big[1]) return Window::kDone;
   uint32_t out0 = cnt_small ? lo : 0xffffffffu, out1 = s_hi;  // the item's places [out0, out1)
   // large rows: where their points are read (split ones: the own lines' places), own lines
   uint32_t b0[2] = {0u, 0u}, b1[2] = {0u, 0u}, l0[2] = {0u, 0u}, l1[2] = {0u, 0u};
@@ -736,7 +886,7 @@ __device__ __forceinline__ bool sort_window(const BucketArgs& a, int item, int c
     }
     out0 = min(out0, min(s_first[0], s_first[1]));
     out1 = max(out1, max(s_last[0], s_last[1]));
-    if (out0 >= out1) return true;  // one long line crosses the window
+    if (out0 >= out1) return Window::kDone;  // one long line crosses the window
   }
   const uint32_t total = out1 - out0;
   uint32_t mid0 = m - sc->row_ext[mc][0], mid1 = sc->row_ext[mc][1];
@@ -768,7 +918,6 @@ __device__ __forceinline__ bool sort_window(const BucketArgs& a, int item, int c
   }
   if (!fits) {
     // (through shared memory: nothing of the loops around is kept on the stack for this)
-    __shared__ ItemRows s_rows;
     if (tid == 0) {
       s_rows.start = start;
       s_rows.ext0 = m - sc->row_ext[mc][0];
@@ -790,8 +939,7 @@ __device__ __forceinline__ bool sort_window(const BucketArgs& a, int item, int c
       }
     }
     __syncthreads();
-    item_by_rows<SPLIT>(a, c, s_rows, smem);
-    return true;
+    return Window::kCrowded;
   }
   const auto put = [&](uint2 e) {
     const uint32_t p = count(e.y);
@@ -810,7 +958,7 @@ __device__ __forceinline__ bool sort_window(const BucketArgs& a, int item, int c
   if (tid < 4) s_pt[total + tid] = ~0ull;
   __syncthreads();
   rank_item(a, c, bucket, s_pt, s_cnt, out0, total);
-  return true;
+  return Window::kDone;
 }
 
 // Thread 0 waits until *counter reaches `target` (a bounded wait); false for every thread if it gave up.
@@ -947,7 +1095,11 @@ __device__ __noinline__ int next_split_window(const BucketArgs& a, int c) {
 }
 
 // (calls of their own: inlined, they cost the other frames' sort its registers: 5 us at 1M points)
-__device__ __noinline__ void sort_split_window(const BucketArgs& a, int item, int c) { sort_window<true>(a, item, c); }
+__device__ __noinline__ void sort_split_window(const BucketArgs& a, int item, int c) {
+  extern __shared__ __align__(16) uint32_t smem[];
+  __shared__ ItemRows s_rows;
+  if (sort_window<true>(a, item, c, s_rows) == Window::kCrowded) item_by_rows<true>(a, c, s_rows, smem);
+}
 
 __device__ __noinline__ void sort_split_rows(const BucketArgs& a, int c) {
   for (;;) {
@@ -959,7 +1111,11 @@ __device__ __noinline__ void sort_split_rows(const BucketArgs& a, int c) {
 
 // one block for every window of a code
 __device__ __forceinline__ void bucket_sort_body(const BucketArgs& a, int block, int c) {
-  if (!sort_window<false>(a, block, c)) sort_split_rows(a, c);
+  extern __shared__ __align__(16) uint32_t smem[];
+  __shared__ ItemRows s_rows;
+  const Window w = sort_window<false>(a, block, c, s_rows);
+  if (w == Window::kCrowded) item_by_rows<false>(a, c, s_rows, smem);
+  else if (w == Window::kHasSplitRows) sort_split_rows(a, c);
 }
 
 __global__ void __launch_bounds__(kBucketThreads, 2) k_bucket_sort(const __grid_constant__ BucketArgs a) {
