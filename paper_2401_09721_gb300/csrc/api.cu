@@ -590,6 +590,13 @@ bool seg_eligible(const std::vector<fgbd_ctx*>& ctxs, const std::vector<fgbd_ctx
   return true;
 }
 
+// Mean points of the frames from which on they select and filter one after another: a
+// step moves 72 bytes a point, so the steps of one frame of 1M points stay in L2 and those
+// of four frames side by side evict each other's.  8 body frames of 1M points with a power
+// of 64 9.98 ms side by side, 8.16 one after another (on streams 8.40), with a power of 2
+// 1.35 and 1.40; of 700,000 (spheres) 6.64 and 6.81, 1.32 and 1.42.
+constexpr int64_t kSelectAlone = 7 << 17;
+
 // Frames [i0, i1) of the batch (i1 - i0 <= kSegMax), enqueued on `st`.
 fgbd_status seg_chunk(const std::vector<fgbd_ctx*>& ctxs, const std::vector<fgbd_ctx::RunKey>& keys, int i0,
                       int i1, const BatchShape& shape, cudaStream_t st) {
@@ -641,8 +648,13 @@ fgbd_status seg_chunk(const std::vector<fgbd_ctx*>& ctxs, const std::vector<fgbd
   if (same_line) lead->launches += 1;  // and the line flags
   FGBD_LAUNCH(lead, "seg_moments", st, launch_ne_moments_seg(m, F, dtype, num_sms, st));
   FGBD_LAUNCH(lead, "seg_estimate", st, launch_ne_finalize_seg(spec, f64, nblk, F, num_sms, st));
-  FGBD_LAUNCH(lead, "seg_select", st,
-              launch_filter_seg(sel, F, shape.filter_threads, shape.filter_per_sm, num_sms, st));
+  if (points >= double(F) * double(kSelectAlone)) {
+    for (int f = 0; f < F; ++f)
+      FGBD_LAUNCH(lead, "filter_select", st, launch_filter(sel[f], filter_grid_for(ctxs[i0 + f], sel[f].n), st));
+  } else {
+    FGBD_LAUNCH(lead, "seg_select", st,
+                launch_filter_seg(sel, F, shape.filter_threads, shape.filter_per_sm, num_sms, st));
+  }
   for (int f = 0; f < F; ++f) {
     fgbd_ctx* c = ctxs[i0 + f];
     mark_run_done(c, keys[i0 + f], 0);
