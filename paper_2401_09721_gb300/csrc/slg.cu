@@ -330,7 +330,6 @@ constexpr int kItemMax = kWindowMax + kRowMax;
 constexpr int kSortBucketBits = 13;
 constexpr int kSortBuckets = 1 << kSortBucketBits;  // 16-bit counters, two a word
 constexpr uint32_t kBucketCoarse = 256;             // larger ones: the buckets follow the rows instead (item_by_rows)
-constexpr uint32_t kBucketMax = 512;                // larger ones still are not ranked by counting
 constexpr size_t kBucketSmem = sizeof(uint2) * (size_t(kItemMax) + 4) + sizeof(uint16_t) * size_t(kSortBuckets);
 static_assert(kSortBuckets == 8 * kBucketThreads && kMaxRadix <= kBucketThreads, "eight buckets, one row a thread");
 static_assert(kItemMax < 65536, "16-bit places inside an item");
@@ -373,10 +372,10 @@ struct ItemRows {
 // stable radix passes over the coordinates in which they differ (of the points of one voxel
 // none), between row_tmp and the output arrays (the item's places).  One block, bound
 // by its instructions and its scattered stores.  The graph of 100,000 points in one voxel
-// takes 269 us, with radix passes over the index and all of the code 1410; of 20,000 beside
-// a sphere of as many 229 and 330.  (Its steps are calls of their own: inlined,
+// takes 266 us, with radix passes over the index and all of the code 1410; of 20,000 beside
+// a sphere of as many 234 and 330.  (Its steps are calls of their own: inlined,
 // they cost the windows' sort its registers, 5 us at 1M points.)
-constexpr int kRadixPer = 4;             // points a thread at a time
+constexpr int kRadixPer = 2;             // points a thread at a time
 constexpr int kBitmapWords = 24 * 1024;  // input indices a time, 32 a word
 static_assert(sizeof(uint32_t) * kBitmapWords <= kBucketSmem, "the bitmap fits the shared memory of an item");
 
@@ -599,7 +598,7 @@ __device__ __noinline__ void radix_place(const BucketArgs& a, int c, const ItemR
 }
 
 template <bool SPLIT>
-__device__ __forceinline__ void item_radix_sort(const BucketArgs& a, int c, const ItemRows& rows, uint32_t* smem) {
+__device__ __noinline__ void item_radix_sort(const BucketArgs& a, int c, const ItemRows& rows, uint32_t* smem) {
   __shared__ uint32_t s_vary;
   radix_gather<SPLIT>(a, c, rows, &s_vary);
   place_by_index(a, c, rows, smem);
@@ -718,53 +717,132 @@ struct BucketByRow {
   }
 };
 
-// An item whose buckets were too large: with buckets that follow its rows, or by the radix
-// sort if repeated voxels overfill those too.  (Two spheres of 200,000 points apart along
-// an axis: the sort 84 us with the items across the gap by the radix sort, 22 so; a block
-// of 20^3 voxels and two points in the grid's corners: the graph 90 -> 39.)  Counting a
-// second time pays from buckets of some 256 points on: a box surface of 300,000 points,
-// whose edges fill buckets of 256, 97 us, with a limit of 128 108; a sphere of 100,000
-// points with two stray ones 43 and 35.
-template <bool SPLIT>
-__device__ __noinline__ bool rank_by_rows(const BucketArgs& a, int c, const ItemRows& rows, uint32_t* smem) {
-  unsigned long long* s_pt = reinterpret_cast<unsigned long long*>(smem);
-  uint32_t* s_cnt = reinterpret_cast<uint32_t*>(s_pt + kItemMax + 4);
-  __shared__ uint32_t s_w[32];
-  const int tid = threadIdx.x, b = a.bits;
-  const uint32_t m = (1u << b) - 1u;
-  if (rows.total <= uint32_t(kItemMax)) {
-    const BucketByRow bucket{rows, b, a.n, (uint32_t(kSortBuckets) << 16) / rows.total};
-    const auto points = [&](auto&& f) {
-      for (uint32_t i = rows.from + tid; i < rows.to; i += kBucketThreads) f(a.row_pts[c][i]);
-      for (int g = 0; g < 2; ++g)
-        for (uint32_t i = rows.big_from[g] + tid; i < rows.big_to[g]; i += kBucketThreads) {
-          const uint2 e = SPLIT && rows.split[g] ? __ldcg(a.row_tmp[c] + i) : a.row_pts[c][i];
-          const uint32_t mid = (e.y >> b) & m;
-          if (mid >= rows.mid0[g] && mid < rows.mid1[g]) f(e);
-        }
-    };
-    __syncthreads();
-    reinterpret_cast<uint4*>(s_cnt)[tid] = make_uint4(0u, 0u, 0u, 0u);
-    __syncthreads();
-    points([&](uint2 e) { count_in(s_cnt, bucket(e.y)); });
-    __syncthreads();
-    if (!__syncthreads_or(bucket_starts(s_cnt, s_w) > kBucketMax)) {
-      points([&](uint2 e) {
-        const uint32_t p = count_in(s_cnt, bucket(e.y));
-        if (p < uint32_t(kItemMax)) s_pt[p] = ((unsigned long long)e.y << 32) | e.x;
-      });
-      if (tid < 4) s_pt[rows.total + tid] = ~0ull;
-      __syncthreads();
-      rank_item(a, c, bucket, s_pt, s_cnt, rows.out0, rows.total);
-      return true;
+// The item's points in s_pt by a bitonic sort of (code, index), in the form whose merges begin
+// with mirrored pairs, so that every exchange is ascending and places behind the last
+// point need not exist.  A warp's pairs of up to 64 places lie in 64 places of its own.
+__device__ __noinline__ void bitonic_item(unsigned long long* s_pt, uint32_t total) {
+  const uint32_t tid = threadIdx.x;
+  const auto exchange = [&](uint32_t lo, uint32_t hi) {
+    if (hi >= total) return;
+    const unsigned long long x = s_pt[lo], y = s_pt[hi];
+    if (y < x) {
+      s_pt[lo] = y;
+      s_pt[hi] = x;
     }
+  };
+  const int top = 32 - __clz(int(total - 1u));  // 2^top places hold the points
+  const uint32_t pairs = total > 1u ? 1u << (top - 1) : 0u;
+  for (int k = 1; k <= top; ++k) {
+    // blocks of 2^k places: mirrored pairs, then pairs 2^j apart
+    if (k > 6) __syncthreads();
+    for (uint32_t t = tid; t < pairs; t += kBucketThreads) {
+      const uint32_t in = t & ((1u << (k - 1)) - 1u), at = (t >> (k - 1)) << k;
+      exchange(at + in, at + (1u << k) - 1u - in);
+    }
+    int j = k - 2;
+    for (; j > 5; --j) {
+      __syncthreads();
+      for (uint32_t t = tid; t < pairs; t += kBucketThreads) {
+        const uint32_t lo = ((t >> j) << (j + 1)) + (t & ((1u << j) - 1u));
+        exchange(lo, lo + (1u << j));
+      }
+    }
+    if (k > 6) __syncthreads();
+    for (; j >= 0; --j) {
+      __syncwarp();
+      for (uint32_t t = tid; t < pairs; t += kBucketThreads) {
+        const uint32_t lo = ((t >> j) << (j + 1)) + (t & ((1u << j) - 1u));
+        exchange(lo, lo + (1u << j));
+      }
+    }
+    __syncwarp();
   }
-  return false;
+  __syncthreads();
 }
 
+// An item whose buckets were too large: with buckets that follow its rows; what is then
+// still crowded, by repeated voxels, through the bitonic sort or, where the points differ in
+// one coordinate at most, through the bitmap (5,000 points in one voxel: the graph 39 us, by
+// the bitonic sort 74); and an item that does not fit, through the bitmap.
+// (Two spheres of 200,000 points apart along an axis: the sort 84 us with the items across
+// the gap by a radix sort, 22 so; a block of 20^3 voxels and two points in the grid's
+// corners: the graph 90 -> 39.)  Counting a second time pays from buckets of some 256
+// points on: a box surface of 300,000 points, whose edges fill buckets of 256, 97 us, with
+// a limit of 128 108; a sphere of 100,000 points with two stray ones 43 and 35.  The
+// bitonic sort takes the place of a point's comparisons with more than kCrowded others on
+// average: the graph of 2,000 voxels 500 times each takes 314 us, with comparisons 458; of
+// 4,096 voxels 244 times each 450 and 347.
+constexpr uint32_t kCrowded = 320;
 template <bool SPLIT>
 __device__ __noinline__ void item_by_rows(const BucketArgs& a, int c, const ItemRows& rows, uint32_t* smem) {
-  if (!rank_by_rows<SPLIT>(a, c, rows, smem)) item_radix_sort<SPLIT>(a, c, rows, smem);
+  if (rows.total > uint32_t(kItemMax)) {
+    item_radix_sort<SPLIT>(a, c, rows, smem);
+    return;
+  }
+  unsigned long long* s_pt = reinterpret_cast<unsigned long long*>(smem);
+  uint32_t* s_cnt = reinterpret_cast<uint32_t*>(s_pt + kItemMax + 4);
+  __shared__ uint32_t s_w[32], s_sq, s_and, s_or;
+  const int tid = threadIdx.x, b = a.bits;
+  const uint32_t m = (1u << b) - 1u;
+  const BucketByRow bucket{rows, b, a.n, (uint32_t(kSortBuckets) << 16) / rows.total};
+  const auto points = [&](auto&& f) {
+    for (uint32_t i = rows.from + tid; i < rows.to; i += kBucketThreads) f(a.row_pts[c][i]);
+    for (int g = 0; g < 2; ++g)
+      for (uint32_t i = rows.big_from[g] + tid; i < rows.big_to[g]; i += kBucketThreads) {
+        const uint2 e = SPLIT && rows.split[g] ? __ldcg(a.row_tmp[c] + i) : a.row_pts[c][i];
+        const uint32_t mid = (e.y >> b) & m;
+        if (mid >= rows.mid0[g] && mid < rows.mid1[g]) f(e);
+      }
+  };
+  __syncthreads();
+  reinterpret_cast<uint4*>(s_cnt)[tid] = make_uint4(0u, 0u, 0u, 0u);
+  if (tid == 0) {
+    s_sq = s_or = 0u;
+    s_and = ~0u;
+  }
+  __syncthreads();
+  uint32_t all = ~0u, any = 0u;  // the bits that all, and any of the codes have
+  points([&](uint2 e) {
+    count_in(s_cnt, bucket(e.y));
+    all &= e.y;
+    any |= e.y;
+  });
+  all = __reduce_and_sync(0xffffffffu, all);
+  any = __reduce_or_sync(0xffffffffu, any);
+  if ((tid & 31) == 0) {
+    atomicAnd(&s_and, all);
+    atomicOr(&s_or, any);
+  }
+  __syncthreads();
+  // the comparisons that ranking would make (at most kItemMax squared, below 2^27)
+  uint32_t sq = 0u;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint32_t w = s_cnt[4 * tid + i];
+    sq += (w & 0xffffu) * (w & 0xffffu) + (w >> 16) * (w >> 16);
+  }
+  sq = __reduce_add_sync(0xffffffffu, sq);
+  if ((tid & 31) == 0) atomicAdd(&s_sq, sq);
+  bucket_starts(s_cnt, s_w);
+  __syncthreads();
+  points([&](uint2 e) {
+    const uint32_t p = count_in(s_cnt, bucket(e.y));
+    if (p < uint32_t(kItemMax)) s_pt[p] = ((unsigned long long)e.y << 32) | e.x;
+  });
+  if (tid < 4) s_pt[rows.total + tid] = ~0ull;
+  __syncthreads();
+  if (s_sq <= kCrowded * rows.total) {
+    rank_item(a, c, bucket, s_pt, s_cnt, rows.out0, rows.total);
+    return;
+  }
+  const uint32_t vary = s_and ^ s_or;
+  if (((vary & m) != 0u) + (((vary >> b) & m) != 0u) + (vary >> (2 * b) != 0u) < 2) {
+    item_radix_sort<SPLIT>(a, c, rows, smem);
+    return;
+  }
+  bitonic_item(s_pt, rows.total);
+  for (uint32_t i = tid; i < rows.total; i += kBucketThreads)
+    emit_sorted(a, c, rows.out0 + i, uint32_t(s_pt[i] >> 32), uint32_t(s_pt[i]));
 }
 
 // the line counters of code c's split row that starts at place `first`

@@ -1,5 +1,5 @@
 """Orders of points that repeat voxels thousands of times, which the sort takes through a
-bitmap of the input indices: one voxel and a few, among others and alone, in the input's
+bitonic sort or a bitmap of the input indices: one voxel and a few, among others and alone, in the input's
 order and shuffled, in rows that are split by lines and not, more input indices than one
 bitmap holds, on both sides of the frame size that one launch sorts, and in a segmented
 batch.  Equal codes are ordered by input index (Section 2.2).  And what that costs."""
@@ -34,12 +34,18 @@ def points(kind, rng):
         return np.concatenate([np.repeat(np.array([[7, 7, 7], [8, 7, 7], [7, 7, 8]]), 15000, axis=0), others(500, 64)]), 6
     if kind == "wide":         # indices of two bitmaps
         return np.concatenate([others(880000, 128), np.full((30000, 3), 3)]), 7
-    if kind == "many":         # buckets of equal points just above and below what is ranked by counting
+    if kind == "many":         # buckets of equal points
         return np.concatenate([np.repeat(rng.integers(0, 1024, size=(20, 3)), 500 + 2 * np.arange(20), axis=0),
                                others(9000, 1024)]), 10
+    if kind == "crowded":      # equal points around what is ranked by comparisons, on a line and not
+        spread = np.repeat(rng.integers(0, 1024, size=(100, 3)), np.arange(270, 370), axis=0)
+        line = np.repeat(np.stack([np.arange(100), np.full(100, 3), np.full(100, 4)], 1), np.arange(270, 370), axis=0)
+        return np.concatenate([spread, line]), 10
+    if kind == "pairs":        # an item of the largest size, and a frame of two voxels
+        return np.array([[3, 4, 5], [900, 4, 5]])[rng.integers(0, 2, size=11264)], 10
 
 
-KINDS = ["one", "small", "beside", "few", "runs", "wide", "many"]
+KINDS = ["one", "small", "beside", "few", "runs", "wide", "many", "crowded", "pairs"]
 
 
 @pytest.mark.parametrize("shuffle", [False, True])
