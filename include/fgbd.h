@@ -268,16 +268,18 @@ fgbd_status fgbd_run_reuse(fgbd_ctx* ctx, const int32_t* xyz, int64_t n, const v
  *   count: 0..FGBD_BATCH_MAX; the contexts must be distinct and on one device.
  * Segmented batches: when every frame has at least one point, window 1, the
  * same ablation switches and the same input colour type, each stage may run as
- * one launch over up to 16 frames (the sort passes, the link, the colour
- * gather, the moments: every frame's blocks in one grid; the noise estimate:
- * one eigen block per frame while the other SMs, shared out by frame size,
- * take the frames' speculative filter steps; the selection and filter: one
- * cooperative launch in which each frame's blocks, shared out by frame size,
- * synchronise among themselves).  Whether a batch that can be segmented is,
- * how many frames a launch takes and the block shapes of the row scatter and
- * of the selection/filter are those fgbd_tune_batch chose for this device and
- * frame size (or fgbd_set_batch_shape set; by default segmented below 2^18
- * points a frame); they do not change any result.  Other batches run every
+ * one launch over up to 16 frames (the histograms, the row scatter, the sort,
+ * the link with the colours, the moments: every frame's blocks in one grid; the
+ * noise estimate: one eigen block per frame while the other SMs, shared out by
+ * frame size, take the frames' speculative filter steps; the selection and
+ * filter: one cooperative launch in which each frame's blocks, shared out by
+ * frame size, synchronise among themselves, or, for frames of 7 * 2^17 points
+ * and more on average, one launch a frame).  Whether a batch that can be
+ * segmented is, how many frames a launch takes and the block shapes of the row
+ * scatter and of the selection/filter are those fgbd_tune_batch chose for this
+ * device and frame size (or fgbd_set_batch_shape set); where neither did, 16
+ * frames a launch below 2^18 points a frame, four from there to 2^21, streams
+ * above.  They do not change any result.  Other batches run every
  * frame on a stream of its own, forked from `stream` and joined back into it,
  * the cooperative selection/filter launches one frame after another.
  * Either way results, stats and errors are per context, exactly as after
@@ -298,10 +300,10 @@ fgbd_status fgbd_run_batch(fgbd_ctx* const* ctxs, const int32_t* const* xyz, con
 
 /* How a batch runs (no counterpart in the paper). */
 typedef struct fgbd_batch_shape {
-  int32_t seg_frames;            /* frames per segmented launch, 1..16; 0: per-frame streams.  Default: 16
-                                    below 2^18 points a frame, 0 above (fgbd_tune_batch: -1 when the batch
-                                    cannot be segmented, and nothing was tuned).  Until something is set for
-                                    them, frames of 2^18 to 2^21 points run segmented, four a launch; a 0
+  int32_t seg_frames;            /* frames per segmented launch, 1..16; 0: per-frame streams.  Reported
+                                    where nothing is set: 16 below 2^18 points a frame, 0 above, although
+                                    frames of 2^18 to 2^21 points then run four a launch (fgbd_tune_batch:
+                                    -1 when the batch cannot be segmented, and nothing was tuned).  A 0
                                     that is set means streams */
   int32_t scatter_threads;       /* threads of a block of the row scatter (a tile of up to 4096 points): 256, 512 (default) or 1024 */
   int32_t filter_threads;        /* threads per block of the selection/filter: 256 or 512 (default) */
@@ -326,9 +328,12 @@ fgbd_status fgbd_tune_batch(fgbd_ctx* const* ctxs, const int32_t* const* xyz, co
                             const void* const* rgb_in, const int32_t* in_dtype, void* const* rgb_out,
                             const int32_t* out_dtype, int32_t count, void* stream, fgbd_batch_shape* chosen);
 
-/* The shapes a segmented batch of frames of about `mean_points` points on CUDA
- * device `device` uses, into *out (host); set them (or, with shape NULL, go
- * back to the defaults) with fgbd_set_batch_shape.  Errors: FGBD_EINVAL. */
+/* The shapes set for batches of frames of about `mean_points` points on CUDA
+ * device `device`, or the defaults of fgbd_batch_shape, into *out (host); set
+ * them (or, with shape NULL, go back to what runs where nothing is set) with
+ * fgbd_set_batch_shape.  To keep what runs where nothing is set, pass NULL, not
+ * the defaults read here: a default of 0 frames that is set means streams.
+ * Errors: FGBD_EINVAL. */
 fgbd_status fgbd_get_batch_shape(int32_t device, int64_t mean_points, fgbd_batch_shape* out);
 fgbd_status fgbd_set_batch_shape(int32_t device, int64_t mean_points, const fgbd_batch_shape* shape);
 

@@ -570,10 +570,11 @@ fgbd_status capture_run(fgbd_ctx* ctx, const fgbd_ctx::RunKey& k, cudaStream_t s
 // instead of 8 per frame, every frame's short latency-bound kernels
 // side by side in one grid, the estimate launch with one eigen block per
 // frame, and one cooperative selection/filter for all frames (each frame's
-// blocks synchronise among themselves).  Each frame's blocks run the same
-// code with the same block counts as its one-frame kernels (or, for the
-// block shapes the tuner may change, code whose results do not depend on the
-// shape), so the outputs equal fgbd_run's bit for bit.
+// blocks synchronise among themselves; large frames one after another, kSelectAlone).
+// Each frame's blocks run the code of its one-frame kernels, with the same block counts
+// where a result depends on them (the float32 sums of edge lengths and of float colours'
+// moments; everywhere else the sums are exact integers), so the outputs equal
+// fgbd_run's bit for bit.
 
 bool seg_eligible(const std::vector<fgbd_ctx*>& ctxs, const std::vector<fgbd_ctx::RunKey>& keys) {
   const fgbd_ctx* c0 = ctxs[0];

@@ -63,7 +63,7 @@ struct DevScalars {
   // ---- graph build region
   unsigned long long n_edges;   // distinct undirected edges E
   unsigned long long dist_fx;   // sum of edge lengths, fixed point 2^-kDistShift
-  alignas(16) uint32_t chist[3][kMaxRadix];  // histograms of x, y and z (read as uint4)
+  alignas(16) uint32_t chist[3][kMaxRadix];  // histograms of x, y and z
   unsigned long long node_fx;   // node-mean reading: sum over points of their mean edge length (fixed point)
   unsigned long long node_cnt;  // and the points that have edges
   float cexp;                   // the Eq. 4 exponent scale log2(e) / sigma_g^2 of this graph, once cexp_ready
@@ -303,8 +303,11 @@ cudaError_t launch_bucket_sort(const BucketArgs& a, cudaStream_t stream);
 constexpr int kDirectMax = 8192;
 cudaError_t launch_direct_sort(const BucketArgs& a, const ZeroArgs& z, cudaStream_t stream);
 cudaError_t launch_orders_export(int n, int cap, const GraphBufs& gb, int32_t* out, cudaStream_t stream);
-// segmented launches: one launch for frames 0..count-1 (count <= kSegMax), each
-// frame with the blocks its one-frame launch would have
+// segmented launches: one launch for frames 0..count-1 (count <= kSegMax).  The histogram,
+// the sort, the link and the float moments give each frame the blocks its one-frame launch
+// would have; the row scatter and the uint8 moments its share of the blocks that fill the
+// GPU, which changes no result (the order inside a row is the sort's, the moments are
+// exact integers)
 HistArgs hist_args(const int32_t* xyz, int n, int bits, DevScalars* sc);
 LinkArgs link_args(int n, int bits, int cap, const GraphBufs& gb, const SortBufs& sb, DevScalars* sc,
                    const ColorArgs& colors);

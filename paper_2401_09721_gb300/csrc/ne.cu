@@ -64,13 +64,7 @@ constexpr int kHRow = 40;
 constexpr int kHPatches = 32;
 constexpr int kRowFloats = 36;  // 32 float entries and padding: rows start on 16 bytes, four banks apart
 
-// Per point: FSLR spread over the point and its neighbours (written to
-// spread[k]) and, for a point with exactly 6 neighbours, its patch (the point
-// then its neighbours by (d^2, dz, dy, dx, index)) written to the warp's patch
-// block: row `lane` of float16 (uint8), column `lane` of float32 rows (float).
-// Returns whether a patch was written.  Equal distances are ordered by sorted id
-// alone: the C1 order is that of (z, y, x, input index).
-// a patch place per neighbour, four bits each: its rank in the strict order (d^2,
+// A patch place per neighbour, four bits each: its rank in the strict order (d^2,
 // sorted id) from the 15 pairwise comparisons.  Starts from the link order, which
 // the "w/o sort" ablation keeps: C1 prev, C1 next, C2 prev, C2 next, C3 prev, C3
 // next.
@@ -105,6 +99,13 @@ __device__ __forceinline__ uint2 patch_node(uint32_t c, uint32_t last) {
   const __half2 hb = __hsub2(*reinterpret_cast<const __half2*>(&b), off);
   return make_uint2(*reinterpret_cast<const uint32_t*>(&ha), *reinterpret_cast<const uint32_t*>(&hb));
 }
+
+// Per point: FSLR spread over the point and its neighbours (written to
+// spread[k]) and, for a point with exactly 6 neighbours, its patch (the point
+// then its neighbours by (d^2, dz, dy, dx, index)) written to the warp's patch
+// block: row `lane` of float16 (uint8), column `lane` of float32 rows (float).
+// Returns whether a patch was written.  Equal distances are ordered by sorted id
+// alone: the C1 order is that of (z, y, x, input index).
 
 // uint8 colours
 __device__ __forceinline__ bool point_patch_u8(const MomentArgs& ma, int k, int lane, __half* ath) {
@@ -211,6 +212,13 @@ __device__ __forceinline__ bool point_patch_f32(const MomentArgs& ma, int k, int
   return true;
 }
 
+// the six Gram blocks into the block's int64 sums (sum a a^T, sum a, the patch count)
+__device__ __forceinline__ void flush8(float (&gc)[6][4], int lane, unsigned long long* tot) {
+#pragma unroll
+  for (int t = 0; t < 6; ++t)
+    gram_flush_nodes<kK + 1>(gc[t], t / 4, t < 4 ? t : t - 2, lane, tot, tot + kD * kD, tot + kD * kD + kD);
+}
+
 // Warp-synchronous: each warp takes 32 points at a time, stages their patches
 // in its own shared-memory block and accumulates the moments with __syncwarp
 // only.  The kernel is bound by its instructions (64 % of the issue slots used at 1M
@@ -229,13 +237,6 @@ __device__ __forceinline__ bool point_patch_f32(const MomentArgs& ma, int k, int
 // group's sums in block order, so that the eigen step reads a few rows instead of
 // one a block (adding 608 rows there, one load after another, made the estimate
 // launch 146 us at 217k points; with the groups it is 41 us).
-// the six Gram blocks into the block's int64 sums (sum a a^T, sum a, the patch count)
-__device__ __forceinline__ void flush8(float (&gc)[6][4], int lane, unsigned long long* tot) {
-#pragma unroll
-  for (int t = 0; t < 6; ++t)
-    gram_flush_nodes<kK + 1>(gc[t], t / 4, t < 4 ? t : t - 2, lane, tot, tot + kD * kD, tot + kD * kD + kD);
-}
-
 template <int DT>
 __device__ __forceinline__ void ne_moments_body(const MomentArgs& ma, int bid, int nblk) {
   const int n = ma.n;

@@ -561,7 +561,7 @@ __device__ __forceinline__ void select_filter(const FilterArgs& a, int S, int fi
   }
   if (phase0 && !grid_barrier(bar, &sc->status, members, epoch, &s_ok, sc)) return;
 
-  // J(0..S) from the stored terms, by thread 0 of each block (every block
+  // J(0..S) from the stored terms, by warp 0 of each block, a lane a step (every block
   // reaches the same values: the sums are exact integers).  Under the global
   // reading (a.q_global) the search never stops early and q* is the argmin of
   // J over 0..q_max (the smaller q among equal values); a new best iterate

@@ -1711,7 +1711,10 @@ int coord_hist_blocks(int n, int num_sms) {
   return n <= 0 ? 0 : std::max(1, std::min((n + kSortTile - 1) / kSortTile, 2 * num_sms));
 }
 int link_gx(int n, int num_sms) {
-  // the three codes' blocks together fill the GPU once (6 resident blocks of 256 threads per SM)
+  // up to two blocks per SM for each of the three codes.  Five of those six are resident at a
+  // time (kLinkPerSm), so above 311,000 points a sixth of the blocks starts as others end.
+  // The number of blocks decides which edge lengths a thread adds in float32, so it is the
+  // same in both paths.
   return std::max(1, std::min((n + kLinkThreads * kLinkPerLane - 1) / (kLinkThreads * kLinkPerLane), num_sms * 2));
 }
 int line_flag_blocks(int n, int num_sms) { return n <= 0 ? 0 : std::min((n + 255) / 256, num_sms * 8); }
