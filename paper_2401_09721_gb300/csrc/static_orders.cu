@@ -1,4 +1,4 @@
-// fgbd_scan_orders_static: the scan-order radix sort without any device allocation.
+// fgbd_scan_orders_static: the scan orders without any device allocation.
 //
 // Some callers cannot call cudaMalloc at the moment they need the scan orders:
 // a real-time frame loop where an allocation would stall the frame, plug-ins
