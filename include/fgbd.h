@@ -273,8 +273,9 @@ fgbd_status fgbd_run_reuse(fgbd_ctx* ctx, const int32_t* xyz, int64_t n, const v
  * noise estimate: one eigen block per frame while the other SMs, shared out by
  * frame size, take the frames' speculative filter steps; the selection and
  * filter: one cooperative launch in which each frame's blocks, shared out by
- * frame size, synchronise among themselves, or, for frames of 7 * 2^17 points
- * and more on average, one launch a frame).  Whether a batch that can be
+ * frame size, synchronise among themselves, and for frames of 7 * 2^17 points
+ * and more on average a second one that takes their steps from the ninth on one
+ * frame after another).  Whether a batch that can be
  * segmented is, how many frames a launch takes and the block shapes of the row
  * scatter and of the selection/filter are those fgbd_tune_batch chose for this
  * device and frame size (or fgbd_set_batch_shape set); where neither did, 16

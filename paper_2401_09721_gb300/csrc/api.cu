@@ -570,7 +570,8 @@ fgbd_status capture_run(fgbd_ctx* ctx, const fgbd_ctx::RunKey& k, cudaStream_t s
 // instead of 8 per frame, every frame's short latency-bound kernels
 // side by side in one grid, the estimate launch with one eigen block per
 // frame, and one cooperative selection/filter for all frames (each frame's
-// blocks synchronise among themselves; large frames one after another, kSelectAlone).
+// blocks synchronise among themselves; the later steps of large frames one frame after
+// another, kStepAlone).
 // Each frame's blocks run the code of its one-frame kernels, with the same block counts
 // where a result depends on them (the float32 sums of edge lengths and of float colours'
 // moments; everywhere else the sums are exact integers), so the outputs equal
@@ -591,12 +592,16 @@ bool seg_eligible(const std::vector<fgbd_ctx*>& ctxs, const std::vector<fgbd_ctx
   return true;
 }
 
-// Mean points of the frames from which on they select and filter one after another: a
-// step moves 72 bytes a point, so the steps of one frame of 1M points stay in L2 and those
-// of four frames side by side evict each other's.  8 body frames of 1M points with a power
-// of 64 9.98 ms side by side, 8.16 one after another (on streams 8.40), with a power of 2
-// 1.35 and 1.40; of 700,000 (spheres) 6.64 and 6.81, 1.32 and 1.42.
-constexpr int64_t kSelectAlone = 7 << 17;
+// Mean points of the frames from which on they take only the first steps side by side
+// and the others one frame after another (k_filter_rest_seg): a step moves 72 bytes a
+// point, so the steps of one frame of 1M points stay in L2 and those of four frames evict
+// each other's.  8 body frames of 1M points with powers of 64 9.01 ms side by side, 7.73 so
+// (on streams 8.4); with powers of 1 and 4 1.33 and 1.59 either way (all of each search one
+// frame after another 1.40 and 1.67).  Powers of 9, just behind the line, cost 2 %: 8 spheres
+// 2.22 and 2.28; with the line at 12 steps those of 64 take 1.5 % more.  Frames of 700,000
+// points (spheres) are as fast side by side: 6.64 ms with powers of 64, 6.81 one by one.
+constexpr int64_t kStepAlone = 7 << 17;
+constexpr int kStepsTogether = 8;
 
 // Frames [i0, i1) of the batch (i1 - i0 <= kSegMax), enqueued on `st`.
 fgbd_status seg_chunk(const std::vector<fgbd_ctx*>& ctxs, const std::vector<fgbd_ctx::RunKey>& keys, int i0,
@@ -649,13 +654,12 @@ fgbd_status seg_chunk(const std::vector<fgbd_ctx*>& ctxs, const std::vector<fgbd
   if (same_line) lead->launches += 1;  // and the line flags
   FGBD_LAUNCH(lead, "seg_moments", st, launch_ne_moments_seg(m, F, dtype, num_sms, st));
   FGBD_LAUNCH(lead, "seg_estimate", st, launch_ne_finalize_seg(spec, f64, nblk, F, num_sms, st));
-  if (points >= double(F) * double(kSelectAlone)) {
-    for (int f = 0; f < F; ++f)
-      FGBD_LAUNCH(lead, "filter_select", st, launch_filter(sel[f], filter_grid_for(ctxs[i0 + f], sel[f].n), st));
-  } else {
-    FGBD_LAUNCH(lead, "seg_select", st,
-                launch_filter_seg(sel, F, shape.filter_threads, shape.filter_per_sm, num_sms, st));
-  }
+  const bool large = F > 1 && points >= double(F) * double(kStepAlone);
+  if (large)
+    for (int f = 0; f < F; ++f) sel[f].step_cap = kStepsTogether;
+  FGBD_LAUNCH(lead, "seg_select", st,
+              launch_filter_seg(sel, F, shape.filter_threads, shape.filter_per_sm, num_sms, st));
+  if (large) FGBD_LAUNCH(lead, "seg_rest", st, launch_filter_rest_seg(sel, F, num_sms, st));
   for (int f = 0; f < F; ++f) {
     fgbd_ctx* c = ctxs[i0 + f];
     mark_run_done(c, keys[i0 + f], 0);

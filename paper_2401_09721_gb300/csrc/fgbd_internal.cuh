@@ -101,6 +101,8 @@ struct DevScalars {
   long long spec_keep[kSpecMax + 1];  // over the kept points: sum of x_q^2 (fixed point), stored steps q = 1..
   long long spec_all[kSpecMax + 1];   // the same over every point
   uint32_t barrier;
+  uint32_t barrier_rest;        // of the launch that takes the search up again
+  int32_t resume_t;             // the step after which a segmented launch left the search to it (0: it did not)
   uint32_t sel_end_;
   // ---- results of the selection
   double J[kQCap + 1];
@@ -374,6 +376,7 @@ struct FilterArgs {
   int q_fixed;           // mode 1
   const int32_t* q_src;  // mode 1: if set, q is read here on the device (and q_sel is left as it is)
   int q_max;             // mode 0
+  int step_cap;          // segmented launch: the step after which it leaves the search (0: none)
   double fslr_factor;
   int all_points;        // Eq. 6 over every point (the limited region is off)
   const double* sigma_src;  // sigma_est to use (device)
@@ -423,6 +426,8 @@ cudaError_t launch_output(const FilterArgs& a, cudaStream_t stream);  // the kep
 cudaError_t launch_filter_seg(const FilterArgs* a, int count, int threads, int filter_per_sm, int num_sms,
                               cudaStream_t stream);
 int filter_seg_max_per_sm(int threads);  // resident blocks per SM of that kernel
+// the searches that it left (FilterArgs::step_cap), one frame after another with the whole GPU
+cudaError_t launch_filter_rest_seg(const FilterArgs* a, int count, int num_sms, cudaStream_t stream);
 
 // Differentiable filter: rows of R = D^-1 W for given alpha, sigma, and their transpose
 struct DiffBufs {  // one value a neighbour slot: C1 (i - 1, i + 1) in the float2, C2/C3 in the float4

@@ -39,7 +39,21 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_filter_seg(const __
   }
   __syncthreads();
   uint32_t epoch = 0;
-  select_filter<THREADS, 0>(a, s_S, s.start[f], uint32_t(s.start[f + 1] - s.start[f]), &a.sc->barrier, epoch, 1);
+  select_filter<THREADS, 0, false, SearchPart::kCapped>(a, s_S, s.start[f], uint32_t(s.start[f + 1] - s.start[f]),
+                                                        &a.sc->barrier, epoch, 1);
+}
+
+// The frames whose search that launch left (resume_t), one after another with every block.
+__global__ void __launch_bounds__(kFilterThreads, 2) k_filter_rest_seg(const __grid_constant__ Seg<FilterArgs> s) {
+  pdl_wait();
+  for (int f = 0; f < s.count; ++f) {
+    const FilterArgs& a = s.a[f];
+    if (a.sc->resume_t == 0) continue;
+    __syncthreads();  // the frame before has left the shared scalars
+    uint32_t epoch = 0;
+    const int S = min(int(a.sc->spec_done), a.spec_depth);
+    select_filter<kFilterThreads, 0, false, SearchPart::kRest>(a, S, 0, gridDim.x, &a.sc->barrier_rest, epoch, 2);
+  }
 }
 
 __global__ void __launch_bounds__(256) k_output(FilterArgs a) {
@@ -283,6 +297,21 @@ cudaError_t launch_filter_seg(const FilterArgs* a, int count, int threads, int f
   const int grid = seg_layout(sg, blocks, count);
   if (threads == 256) return launch_kernel(k_filter_seg<256>, dim3(grid), dim3(256), 0, stream, true, sg);
   return launch_kernel(k_filter_seg<512>, dim3(grid), dim3(512), 0, stream, true, sg);
+}
+
+cudaError_t launch_filter_rest_seg(const FilterArgs* a, int count, int num_sms, cudaStream_t stream) {
+  if (count < 1 || count > kSegMax) return cudaErrorInvalidValue;
+  int per_sm = 0;
+  const cudaError_t e =
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_filter_rest_seg, kFilterThreads, 0);
+  if (e != cudaSuccess) return e;
+  Seg<FilterArgs> sg;
+  for (int f = 0; f < count; ++f) {
+    if (a[f].nx != 0) return cudaErrorInvalidValue;
+    sg.a[f] = a[f];
+  }
+  sg.count = count;
+  return launch_kernel(k_filter_rest_seg, dim3(std::max(1, per_sm) * num_sms), dim3(kFilterThreads), 0, stream, true, sg);
 }
 
 cudaError_t launch_output(const FilterArgs& a, cudaStream_t stream) {

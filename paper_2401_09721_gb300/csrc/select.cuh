@@ -359,8 +359,10 @@ __device__ __forceinline__ void output_quads(const FilterArgs& a, int kept, int 
 // grid barriers on *bar (epoch: the barriers this grid has passed on it), per_sm
 // blocks on an SM;
 // NX further neighbour slots per point (window w > 1: NX = 6 (w - 1)).
-// DEEP: up to kSpecMax stored steps (else kSpecSure).
-template <int THREADS, int NX = 0, bool DEEP = false>
+// DEEP: up to kSpecMax stored steps (else kSpecSure).  PART: the whole search, or (a
+// segmented launch) leave it after step a.step_cap if it has not ended, or take it up there.
+enum class SearchPart { kWhole, kCapped, kRest };
+template <int THREADS, int NX = 0, bool DEEP = false, SearchPart PART = SearchPart::kWhole>
 __device__ __forceinline__ void select_filter(const FilterArgs& a, int S, int first, uint32_t members,
                                               uint32_t* bar, uint32_t& epoch, int per_sm) {
   constexpr int W = THREADS / 32;
@@ -372,11 +374,12 @@ __device__ __forceinline__ void select_filter(const FilterArgs& a, int S, int fi
   const int gtid = (int(blockIdx.x) - first) * THREADS + int(threadIdx.x);
   const int gstride = int(members) * THREADS;
   DevScalars* sc = a.sc;
-  const bool select = a.mode == 0;
+  constexpr bool kRest = PART == SearchPart::kRest;
+  const bool select = kRest || a.mode == 0;
   // Block-uniform scalars, computed by thread 0: the FSLR threshold 2 sigma_est
   // as a float32 band [t_lo, t_hi] (outside it float32 decides) and as float-float.
   __shared__ float s_thr[4];
-  if (threadIdx.x == 0 && select) {
+  if (threadIdx.x == 0 && select && !kRest) {
     if (a.sigma_src == &sc->sigma_est && sc->fslr_ready) {
       // as the eigen step formed them with sigma_est (fslr_band, the same arithmetic)
 #pragma unroll
@@ -388,7 +391,7 @@ __device__ __forceinline__ void select_filter(const FilterArgs& a, int S, int fi
   __syncthreads();
   float t_lo = 0.f, t_hi = 0.f;
   FF thr = {0.f, 0.f};
-  if (select) {
+  if (select && !kRest) {
     t_lo = s_thr[0];
     t_hi = s_thr[1];
     thr = {s_thr[2], s_thr[3]};
@@ -408,7 +411,7 @@ __device__ __forceinline__ void select_filter(const FilterArgs& a, int S, int fi
   unsigned long long acc[kSums] = {};
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const bool write_x0 = !S && !a.x0;
-  const bool phase0 = select || write_x0;
+  const bool phase0 = !kRest && (select || write_x0);
   // (DEEP: blocks take equal runs of quads; with quads by thread number, three of
   // four blocks of a frame below a wave would have none)
   constexpr int kKeepTrips = DEEP ? 4 : 1;  // quads of keep flags a thread leaves between two barriers
@@ -496,7 +499,7 @@ __device__ __forceinline__ void select_filter(const FilterArgs& a, int S, int fi
     }
   }
   if constexpr (!DEEP) {
-    for (int k0 = 4 * gtid; S > 0 && k0 < n; k0 += 4 * gstride) {
+    for (int k0 = 4 * gtid; !kRest && S > 0 && k0 < n; k0 += 4 * gstride) {
       const bool full = k0 + 4 <= n;
       uint32_t kw = 0;
       int32_t z[kSpecSure][4] = {};
@@ -537,7 +540,7 @@ __device__ __forceinline__ void select_filter(const FilterArgs& a, int S, int fi
       }
     }
   }
-  if (select) {
+  if (select && !kRest) {
 #pragma unroll
     for (int i = 0; i < kSums; ++i) {
       acc[i] = warp_sum(acc[i]);
@@ -609,7 +612,12 @@ __device__ __forceinline__ void select_filter(const FilterArgs& a, int S, int fi
       stopped = up != 0;
       const int last = stopped ? __ffs(int(up)) - 1 : m;  // the last J of the search so far
       q_final = stopped ? last - 1 : m;
-      const double J_prev = __shfl_sync(0xffffffffu, J, q_final);
+      double J_prev = __shfl_sync(0xffffffffu, J, q_final);
+      if (kRest) {
+        stopped = 0;
+        q_final = sc->resume_t;
+        J_prev = sc->J[q_final];
+      }
       double J_best = sig2;
       if (global) {
         for (int t = 1; t <= m; ++t) {
@@ -627,7 +635,7 @@ __device__ __forceinline__ void select_filter(const FilterArgs& a, int S, int fi
         s_J_best = J_best;
         s_ysq = ysq;
       }
-      if (int(blockIdx.x) == first) {
+      if (!kRest && int(blockIdx.x) == first) {
         if (lane <= last) sc->J[lane] = J;
         if (lane == 0 && last > 0) sc->n_J = last + 1;
       }
@@ -650,10 +658,11 @@ __device__ __forceinline__ void select_filter(const FilterArgs& a, int S, int fi
   const bool stopped = s_ctl[3] != 0;
   const int2 run = step_run(n, int(blockIdx.x) - first, int(members), per_sm);
   bool copy_best = false;  // this step's source is the best iterate so far: copy it to xbest
-  for (int t = S + 1; t <= q_limit && !stopped; ++t) {
+  for (int t = (kRest ? q_final : S) + 1; t <= q_limit && !stopped; ++t) {
     const float4* src =
         t == 1 && a.x0 ? a.x0
-                       : (S > 0 && t == S + 1) ? a.spec_x + size_t(S - 1) * size_t(a.cap) : ((t & 1) ? a.xbuf0 : a.xbuf1);
+                       : (!kRest && S > 0 && t == S + 1) ? a.spec_x + size_t(S - 1) * size_t(a.cap)
+                                                         : ((t & 1) ? a.xbuf0 : a.xbuf1);
     float4* dst = (t & 1) ? a.xbuf1 : a.xbuf0;
     unsigned long long loc = 0;
     for (int k = run.x + int(threadIdx.x); k < run.y; k += THREADS) {
@@ -699,6 +708,10 @@ __device__ __forceinline__ void select_filter(const FilterArgs& a, int S, int fi
       }
       q_final = t;
       copy_best = s_ctl[5] != 0;
+      if (PART == SearchPart::kCapped && t == a.step_cap && t < q_limit) {
+        if (gtid == 0) sc->resume_t = t;
+        return;
+      }
     } else {
       q_final = t;
     }
